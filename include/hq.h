@@ -86,7 +86,7 @@ typedef struct {
     int64_t N_pad;      /* N rounded up to 128; padding rows are zero */
     int64_t bytes;      /* size of the blob */
     int32_t max_abs_b;  /* largest |B| entry, for the accumulator-range check */
-    int32_t reserved;
+    int32_t reserved;   /* 1: the one-limb section of the split fold follows (see hq_weight_prepare); 0: it does not */
 } hq_weight_desc;
 
 int hq_version(void);
@@ -114,6 +114,10 @@ hq_status hq_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t c
  * blob       host buffer of hq_weight_blob_bytes(...) bytes; copy it to the device as is.
  * s_w        host [N] per-output-channel scales (for DOUBLE: scales of H^T W).
  * desc       filled on success.
+ * FOLDED 4-bit weights with blocks of 32 .. 512 channels get a second section of half the first one's size: one-limb
+ *   weights with four of the log2(had_block) factors of H_raw applied, for the fused layer calls, which give the other
+ *   factors to the codes (same integers, half the tensor work).  A blob_bytes that holds only the first section is taken
+ *   as well; the layer then always runs on two limbs.
  * Errors: FOLDED/DOUBLE with C % had_block != 0; FOLDED whose integers need more than 2 limbs -> HQ_ERR_OVERFLOW_RISK. */
 int64_t hq_weight_blob_bytes(int64_t N, int32_t RS, int64_t C, int32_t w_bits, int32_t had_block,
                              hq_weight_mode mode);
@@ -148,6 +152,9 @@ hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t
 
 /* ---- Fused layer: transform -> quantize -> integer product -> rescale in one call (Eq. 12 / Eq. 14). ----
  * Codes and scales live in `workspace` (device, hq_workspace_size bytes); the code container is desc->container.
+ * hq_workspace_size: codes (row pitch rounded up to 16 bytes), then the scales at the next multiple of 256; if that is
+ * more than HQ_NOALLOC_SCRATCH_BYTES, also rows * cols bytes for the split-fold codes.  A workspace that holds only codes
+ * and scales is enough for every layer: the product then runs on the two-limb weights, with the same results.
  * alpha is derived from the descriptor.  y pitch ldy elements.
  * The product kernel is launched so that it may begin (set-up, first weight tile) while the transform kernel is still
  * running; it waits for the transform before it touches codes or activation scales.  Work enqueued on the stream before

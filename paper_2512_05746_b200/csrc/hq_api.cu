@@ -3,6 +3,7 @@
 #include <mutex>
 
 #include "hq_common.cuh"
+#include "hq_fwht.cuh"
 
 // Scratch of hq_qlinear_noalloc: part of the library's device image, one copy per GPU that loads the library.
 // In host code this name is only a handle for cudaGetSymbolAddress, never a device pointer.
@@ -11,7 +12,7 @@ static __device__ __align__(256) unsigned char hq_noalloc_scratch[HQ_NOALLOC_SCR
 namespace hq {
 hq_status launch_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t cols, int64_t ldx, int had_block,
                                 int bits, hq_scale_mode mode, const float* static_scale, void* codes,
-                                hq_container cont, int64_t ld_codes, float* scales, cudaStream_t st);
+                                hq_container cont, int64_t ld_codes, float* scales, cudaStream_t st, SplitOut* zo = nullptr);
 hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64_t M, int64_t K, int64_t lda,
                        const hq_weight_desc* desc, const void* w_dev, const float* scale_a, int scale_a_is_scalar,
                        const float* scale_w, const float* bias, float alpha, int32_t* acc_out, void* y,
@@ -26,21 +27,23 @@ hq_status launch_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t 
                                const float* gamma, const float* beta, float eps, int had_block, int bits,
                                hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont,
                                int64_t ld_codes, float* scales, void* scratch, size_t scratch_bytes, cudaStream_t st,
-                               int silu, const void* pre_bias, const void* x2, int64_t split);
+                               int silu, const void* pre_bias, const void* x2, int64_t split, SplitOut* zo = nullptr);
 hq_status launch_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, int64_t ldx2, int64_t split, hq_dtype xdt,
                                     int64_t rows, int64_t cols, int had_block, int bits, hq_scale_mode mode,
                                     const float* static_scale, void* codes, hq_container cont, int64_t ld_codes,
-                                    float* scales, cudaStream_t st);
+                                    float* scales, cudaStream_t st, SplitOut* zo = nullptr);
 hq_status launch_ln_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t cols, int64_t ldx, const float* weight,
                           const float* bias, int64_t rows_per_group, float eps, int had_block, int bits,
                           hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont, int64_t ld_codes,
-                          float* scales, cudaStream_t st);
+                          float* scales, cudaStream_t st, SplitOut* zo = nullptr);
 hq_status launch_hadamard_quant_width(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C,
                                       int had_block_w, int bits, const float* static_scale, void* z, float* scale_out,
                                       cudaStream_t st);
 hq_status launch_hadamard_quant_width2(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C,
                                        int had_block_w, int bits, const float* static_scale, void* z_limbs,
                                        float* scale_out, cudaStream_t st);
+
+int sm_count();             // hq_gemm.cu: SM count of the current device
 
 namespace {
 int64_t code_pitch(int64_t cols, hq_container cont) {
@@ -50,6 +53,70 @@ int64_t code_pitch(int64_t cols, hq_container cont) {
 int64_t scales_offset(int64_t rows, int64_t cols, hq_container cont) {
     return (rows * code_pitch(cols, cont) + 255) / 256 * 256;
 }
+// Codes and scales; behind them, where the caller's workspace has room for it, the split-fold codes z of the layer.
+int64_t codes_bytes(int64_t rows, int64_t cols, hq_container cont) {
+    return scales_offset(rows, cols, cont) + (rows > 0 ? rows : 1) * int64_t(sizeof(float));
+}
+int64_t split_offset(int64_t rows, int64_t cols, hq_container cont) { return (codes_bytes(rows, cols, cont) + 255) / 256 * 256; }
+int64_t split_bytes(int64_t rows, int64_t cols, hq_container cont) {
+    return split_offset(rows, cols, cont) + rows * code_pitch(cols, HQ_CODES_INT8);
+}
+
+// What a fused layer call cannot do without: its codes and scales.
+hq_status layer_bytes(int64_t rows, int64_t cols, hq_container cont, size_t* bytes) {
+    if (cont != HQ_CODES_NIBBLE && cont != HQ_CODES_INT8) return HQ_ERR_INVALID_ARG;
+    if (rows < 0 || cols <= 0) return HQ_ERR_SHAPE;
+    *bytes = size_t(codes_bytes(rows, cols, cont));
+    return HQ_OK;
+}
+
+// The intermediate of a fused layer call in its workspace, and the operands its product runs on: the codes and the weights
+// as prepared, or (after the transform kernel has said that it wrote them) the split-fold codes and the one-limb weights
+// behind the two-limb ones in the blob.  The sums are the same integers either way.
+struct LayerCodes {
+    unsigned char* codes;
+    float* scales;
+    int64_t ld;
+    SplitOut z{};
+    hq_weight_desc split_desc;
+    const void* split_w;
+
+    // rows x cols codes whose product has out_rows rows
+    LayerCodes(const hq_weight_desc* desc, const void* w_dev, int a_bits, int64_t rows, int64_t cols, int64_t out_rows,
+               hq_container cont, void* workspace, size_t ws_bytes)
+        : codes(static_cast<unsigned char*>(workspace)),
+          scales(reinterpret_cast<float*>(codes + scales_offset(rows, cols, cont))), ld(code_pitch(cols, cont)) {
+        if (split_applies(desc, a_bits, cols) && split_pays(desc, rows, cols, out_rows) && ws_bytes >= size_t(split_bytes(rows, cols, cont))) {
+            z.z = codes + split_offset(rows, cols, cont);
+            z.ld = code_pitch(cols, HQ_CODES_INT8);
+            split_desc = *desc;
+            split_desc.limbs = 1;
+            split_desc.container = HQ_CODES_INT8;
+            split_w = static_cast<const unsigned char*>(w_dev) + desc->N_pad * 2 * desc->RS * desc->C_pad;
+        }
+    }
+    static bool split_applies(const hq_weight_desc* desc, int a_bits, int64_t cols) {
+        if (desc->reserved != kBlobHasSplit || desc->limbs != 2 || desc->C != cols) return false;
+        const int klog = ilog2(desc->had_block);
+        return split_block_ok(klog) && split_fits(klog, a_bits) && cols < 131072;
+    }
+    // One limb halves the column tiles, and the transform kernel computes and writes a second byte per code.  A tile of 256
+    // rows and 256 operand rows takes about 0.28 us per 128 bytes of the reduction on a pair of SMs (four MMAs of 134
+    // cycles), whichever the limbs, so what counts is the rounds of tiles that are saved; the second byte costs 0.7 us plus
+    // its traffic at about 5.2 TB/s.  Measured (two limbs / one): 8192 x 1152 -> 4608 57.9 / 44.2 us, 64 x 32 x 32 x 512 3x3
+    // 176 / 117 us; where no round is saved it only costs: 256 x 256 -> 256 6.1 / 6.8 us, 2 x 8 x 8 x 1024 3x3 26.8 / 27.8.
+    static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows) {
+        const int64_t pairs = sm_count() / 2, m = (out_rows + 255) / 256;
+        const int64_t two = (m * (desc->N_pad / 128) + pairs - 1) / pairs, one = (m * ((desc->N_pad + 255) / 256) + pairs - 1) / pairs;
+        const double saved_us = 0.28 * double(two - one) * double(desc->RS * desc->C_pad / 128);
+        return saved_us > 0.7 + double(rows) * double(cols) / 5.2e6;
+    }
+    const void* a() const { return z.written ? z.z : codes; }
+    int64_t lda() const { return z.written ? z.ld : ld; }
+    hq_container container(hq_container cont) const { return z.written ? HQ_CODES_INT8 : cont; }
+    const hq_weight_desc* desc(const hq_weight_desc* d) const { return z.written ? &split_desc : d; }
+    const void* w(const void* w_dev) const { return z.written ? split_w : w_dev; }
+};
 }  // namespace
 }  // namespace hq
 
@@ -80,7 +147,10 @@ extern "C" hq_status hq_workspace_size(int64_t rows, int64_t cols, hq_container 
     if (bytes == nullptr) return HQ_ERR_INVALID_ARG;
     if (cont != HQ_CODES_NIBBLE && cont != HQ_CODES_INT8) return HQ_ERR_INVALID_ARG;
     if (rows < 0 || cols <= 0) return HQ_ERR_SHAPE;
-    *bytes = size_t(hq::scales_offset(rows, cols, cont)) + size_t(rows > 0 ? rows : 1) * sizeof(float);
+    // Codes and scales.  Layers beyond HQ_NOALLOC_SCRATCH_BYTES also get room for the split-fold codes; smaller ones hold
+    // too few tiles to gain from one-limb weights and keep the size at which the no-allocation entry point takes them.
+    *bytes = size_t(hq::codes_bytes(rows, cols, cont));
+    if (*bytes > size_t(HQ_NOALLOC_SCRATCH_BYTES)) *bytes = size_t(hq::split_bytes(rows, cols, cont));
     return HQ_OK;
 }
 
@@ -94,16 +164,15 @@ extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t 
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const hq_container cont = hq_container(desc->container);
     size_t need = 0;
-    hq_status s = hq_workspace_size(M, K, cont, &need);
+    hq_status s = layer_bytes(M, K, cont, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned char* codes = static_cast<unsigned char*>(workspace);
-    float* scales = reinterpret_cast<float*>(codes + scales_offset(M, K, cont));
-    const int64_t ldc = code_pitch(K, cont);
-    s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, codes, cont, ldc, scales, st);
+    LayerCodes lc(desc, w_dev, a_bits, M, K, M, cont, workspace, ws_bytes);
+    s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
+                              &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(codes, cont, a_bits, M, K, ldc, desc, w_dev, scales, mode == HQ_SCALE_STATIC, scale_w, bias,
+    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, K, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
                         hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true);
 }
 
@@ -117,17 +186,15 @@ extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const hq_container cont = hq_container(desc->container);
     size_t need = 0;
-    hq_status s = hq_workspace_size(M, K, cont, &need);
+    hq_status s = layer_bytes(M, K, cont, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned char* codes = static_cast<unsigned char*>(workspace);
-    float* scales = reinterpret_cast<float*>(codes + scales_offset(M, K, cont));
-    const int64_t ldc = code_pitch(K, cont);
+    LayerCodes lc(desc, w_dev, a_bits, M, K, M, cont, workspace, ws_bytes);
     s = launch_ln_quant(x, xdt, M, K, ldx, ln_weight, ln_bias, rows_per_group, eps, desc->had_block, a_bits, HQ_SCALE_PER_ROW,
-                        nullptr, codes, cont, ldc, scales, st);
+                        nullptr, lc.codes, cont, lc.ld, lc.scales, st, &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(codes, cont, a_bits, M, K, ldc, desc, w_dev, scales, 0, scale_w, bias, hq_alpha_for(desc), nullptr,
+    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, K, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, 0, scale_w, bias, hq_alpha_for(desc), nullptr,
                         y, ydt, ldy, dev_status, st, true);
 }
 
@@ -145,18 +212,19 @@ static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split
     const hq_container cont = hq_container(desc->container);
     const int64_t rows = Nb * H * W;
     size_t need = 0;
-    hq_status s = hq_workspace_size(rows, C, cont, &need);
+    hq_status s = layer_bytes(rows, C, cont, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned char* codes = static_cast<unsigned char*>(workspace);
-    float* scales = reinterpret_cast<float*>(codes + scales_offset(rows, C, cont));
-    s = launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, desc->had_block, a_bits, mode, static_scale, codes,
-                             cont, ldc, scales, scratch, scratch_bytes, st, 1, pre_bias, x2, split);
+    // per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb
+    LayerCodes lc(desc, w_dev, a_bits, rows, C, rows / (stride == 2 ? 4 : 1), cont, workspace,
+                  mode == HQ_SCALE_STATIC || R * S == 1 ? ws_bytes : 0);
+    s = launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, desc->had_block, a_bits, mode, static_scale,
+                             lc.codes, cont, ldc, lc.scales, scratch, scratch_bytes, st, 1, pre_bias, x2, split, &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qconv2d(codes, cont, a_bits, Nb, H, W, C, desc, w_dev, R, S, stride, pad, scales,
+    return launch_qconv2d(lc.a(), lc.container(cont), a_bits, Nb, H, W, C, lc.desc(desc), lc.w(w_dev), R, S, stride, pad, lc.scales,
                           mode == HQ_SCALE_STATIC, scale_w, bias, hq_alpha_for(desc), nullptr, y, ydt, dev_status, st, true);
 }
 
@@ -200,18 +268,16 @@ extern "C" hq_status hq_gn_qlinear(const void* x, hq_dtype xdt, int64_t Nb, int6
     const hq_container cont = hq_container(desc->container);
     const int64_t M = Nb * rows_per_sample;
     size_t need = 0;
-    hq_status s = hq_workspace_size(M, C, cont, &need);
+    hq_status s = layer_bytes(M, C, cont, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned char* codes = static_cast<unsigned char*>(workspace);
-    float* scales = reinterpret_cast<float*>(codes + scales_offset(M, C, cont));
-    const int64_t ldc = code_pitch(C, cont);
+    LayerCodes lc(desc, w_dev, a_bits, M, C, M, cont, workspace, ws_bytes);
     s = launch_gn_silu_quant(x, xdt, Nb, rows_per_sample, 1, C, groups, gamma, beta, eps, desc->had_block, a_bits,
-                             HQ_SCALE_PER_ROW, nullptr, codes, cont, ldc, scales, scratch, scratch_bytes, st, silu != 0,
-                             nullptr, nullptr, 0);
+                             HQ_SCALE_PER_ROW, nullptr, lc.codes, cont, lc.ld, lc.scales, scratch, scratch_bytes, st,
+                             silu != 0, nullptr, nullptr, 0, &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(codes, cont, a_bits, M, C, ldc, desc, w_dev, scales, 0, scale_w, bias, hq_alpha_for(desc), nullptr,
+    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, C, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, 0, scale_w, bias, hq_alpha_for(desc), nullptr,
                         y, ydt, ldy, dev_status, st, true);
 }
 
@@ -227,21 +293,23 @@ static hq_status qconv_impl(const void* x, const void* x2, int64_t split, hq_dty
     const hq_container cont = hq_container(desc->container);
     const int64_t rows = Nb * H * W;
     size_t need = 0;
-    hq_status s = hq_workspace_size(rows, C, cont, &need);
+    hq_status s = layer_bytes(rows, C, cont, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned char* codes = static_cast<unsigned char*>(workspace);
-    float* scales = reinterpret_cast<float*>(codes + scales_offset(rows, C, cont));
+    // per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb
+    LayerCodes lc(desc, w_dev, a_bits, rows, C, rows / (stride == 2 ? 4 : 1), cont, workspace,
+                  mode == HQ_SCALE_STATIC || R * S == 1 ? ws_bytes : 0);
     if (x2 != nullptr)
         s = launch_hadamard_quant_cat(x, split, x2, C - split, split, xdt, rows, C, desc->had_block, a_bits, mode, static_scale,
-                                      codes, cont, ldc, scales, st);
+                                      lc.codes, cont, ldc, lc.scales, st, &lc.z);
     else
-        s = launch_hadamard_quant(x, xdt, rows, C, C, desc->had_block, a_bits, mode, static_scale, codes, cont, ldc, scales, st);
+        s = launch_hadamard_quant(x, xdt, rows, C, C, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
+                              &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qconv2d(codes, cont, a_bits, Nb, H, W, C, desc, w_dev, R, S, stride, pad, scales,
+    return launch_qconv2d(lc.a(), lc.container(cont), a_bits, Nb, H, W, C, lc.desc(desc), lc.w(w_dev), R, S, stride, pad, lc.scales,
                           mode == HQ_SCALE_STATIC, scale_w, bias, hq_alpha_for(desc), nullptr, y, ydt, dev_status, st, true);
 }
 
@@ -282,7 +350,7 @@ extern "C" hq_status hq_qconv_width(const void* x, hq_dtype xdt, int64_t Nb, int
         if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
         const int64_t rows2 = Nb * H * W;
         size_t need2 = 0;
-        hq_status s2 = hq_workspace_size(rows2, 2 * C, HQ_CODES_INT8, &need2);
+        hq_status s2 = layer_bytes(rows2, 2 * C, HQ_CODES_INT8, &need2);
         if (s2 != HQ_OK) return s2;
         if (ws_bytes < need2) return HQ_ERR_WORKSPACE;
         if ((2 * C) % 16 != 0) return HQ_ERR_ALIGNMENT;
@@ -298,7 +366,7 @@ extern "C" hq_status hq_qconv_width(const void* x, hq_dtype xdt, int64_t Nb, int
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const int64_t rows = Nb * H * W;
     size_t need = 0;
-    hq_status s = hq_workspace_size(rows, C, HQ_CODES_INT8, &need);
+    hq_status s = layer_bytes(rows, C, HQ_CODES_INT8, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     if (C % 16 != 0) return HQ_ERR_ALIGNMENT;              // densely packed pixels for the convolution's TMA boxes
@@ -344,17 +412,17 @@ extern "C" hq_status hq_qlinear_noalloc(const void* x, hq_dtype xdt, int64_t M, 
     if (desc == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     const hq_container cont = hq_container(desc->container);
     size_t need = 0;
-    hq_status s = hq_workspace_size(M, K, cont, &need);
+    hq_status s = layer_bytes(M, K, cont, &need);
     if (s != HQ_OK) return s;
     if (need > size_t(HQ_NOALLOC_SCRATCH_BYTES)) return HQ_ERR_SCRATCH_LIMIT;
     unsigned char* codes = nullptr;
     s = noalloc_scratch_address(&codes);
     if (s != HQ_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    float* scales = reinterpret_cast<float*>(codes + scales_offset(M, K, cont));
-    const int64_t ldc = code_pitch(K, cont);
-    s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, codes, cont, ldc, scales, st);
+    LayerCodes lc(desc, w_dev, a_bits, M, K, M, cont, codes, HQ_NOALLOC_SCRATCH_BYTES);
+    s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
+                              &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(codes, cont, a_bits, M, K, ldc, desc, w_dev, scales, mode == HQ_SCALE_STATIC, scale_w, bias,
+    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, K, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
                         hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true);
 }

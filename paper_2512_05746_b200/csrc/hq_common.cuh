@@ -25,6 +25,11 @@ enum : int32_t {
     kStatusUnpackWait = 0x500,   // unpack warps / MMA issuer waited on the staging ring
 };
 
+// Where the transform kernel may leave the codes' share of the split fold (split_codes in hq_fwht.cuh) beside the codes;
+// `written`: it did.
+constexpr int32_t kBlobHasSplit = 1;      // hq_weight_desc::reserved: the one-limb section follows the two-limb one
+struct SplitOut { uint8_t* z; int64_t ld; bool written; };
+
 #define HQ_CUDA_OK(expr) do { cudaError_t e__ = (expr); if (e__ != cudaSuccess) return HQ_ERR_CUDA; } while (0)
 
 #ifdef __CUDACC__

@@ -172,4 +172,70 @@ __device__ __forceinline__ void pack_codes(const f32x2 (&v)[E / 2], float inv, i
     }
 }
 
+// ---- the transform of Eq. 12's weight side, shared between weights and codes -----------------------------------
+// The folded product sum_i q_i (H_raw W)_i needs weights of w_bits + k bits: two int8 limbs, twice the tensor work.  H_raw
+// is a Kronecker product over the index bits, H_raw = prod of the factors of bits A times those of the bits not in A, and
+// symmetric, so the same integers come out of z = (factors of A) q against B' = (factors of the other bits) W.  Four bits
+// stay with 4-bit weights (|B'| <= 7 * 16), the other k - 4 go to the codes (|z| <= 2^(a_bits-1) * 2^(k-4)): where both fit
+// a signed byte, ONE limb carries the whole product.  A is the k - 4 lowest of the order {2, 3, 4, 1, 0}: the index bits
+// that a thread's 32 consecutive codes, four to a word, hold between words and then inside a word.
+constexpr int kSplitWeightBits = 4;                    // index bits whose factors stay with the weights
+__host__ __device__ constexpr bool split_block_ok(int klog) { return klog >= 5 && klog <= 9; }
+__host__ __device__ constexpr int split_code_bit(int i) { return i < 3 ? 2 + i : 4 - i; }       // 2, 3, 4, 1, 0
+// Whether z fits a signed byte for codes of a_bits bits (every row of H_raw but the first has as many -1 as +1).
+__host__ __device__ constexpr bool split_fits(int klog, int a_bits) { return a_bits - 1 + klog - kSplitWeightBits <= 7; }
+
+// u: 32 consecutive codes as bytes, biased by 128 >> A so that every sum below stays in its byte; on return z as signed
+// bytes.  A byte-wise butterfly is two additions per word pair: a + b, and a - b + (the bias to come); inside a word the
+// shifted copy comes from a multiplication by 2^16 +- 1 or 2^8 +- 1.  1.3 to 2 instructions per code.
+template <int A>
+__device__ __forceinline__ void split_butterflies(uint32_t (&u)[8]) {
+    constexpr uint32_t kOnes = 0x01010101u;
+#pragma unroll
+    for (int i = 0; i < A; ++i) {
+        const uint32_t bias = kOnes * uint32_t((128 >> A) << (i + 1));     // the bias after this stage
+        if (i < 3) {
+            const int h = 1 << i;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                if (!(w & h)) {
+                    const uint32_t a = u[w], b = u[w | h];
+                    u[w] = a + b;
+                    u[w | h] = a + bias - b;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                // bytes 2, 3 of s and d: e0 + e2, e1 + e3 and e0 - e2, e1 - e3 (bit 0: bytes 1, 3: e0 + e1, e2 + e3, ...)
+                const uint32_t s = u[w] * (i == 3 ? 0x00010001u : 0x00000101u);
+                const uint32_t d = u[w] * (i == 3 ? 0x0000FFFFu : 0x000000FFu) + bias;
+                u[w] = __byte_perm(s, d, i == 3 ? 0x7632 : 0x7351);
+            }
+        }
+    }
+#pragma unroll
+    for (int w = 0; w < 8; ++w) u[w] ^= 0x80808080u;
+}
+
+// z of the 32 codes in w (8 words of bytes, or 4 words of nibbles, element 2j in the low one).
+template <int KLOG, bool INT8_IN>
+__device__ __forceinline__ void split_codes(const uint32_t (&w)[INT8_IN ? 8 : 4], uint32_t (&z)[8]) {
+    constexpr int A = KLOG - kSplitWeightBits;
+    constexpr uint32_t kOnes = 0x01010101u, off = 128u >> A;
+    if (INT8_IN) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z[i] = (w[i] ^ 0x80808080u) - (128u - off) * kOnes;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t n = w[i] ^ 0x88888888u;                         // code + 8 in every nibble
+            const uint32_t ev = n & 0x0F0F0F0Fu, od = (n >> 4) & 0x0F0F0F0Fu;
+            z[2 * i] = __byte_perm(ev, od, 0x5140) + off * kOnes - 8u * kOnes;
+            z[2 * i + 1] = __byte_perm(ev, od, 0x7362) + off * kOnes - 8u * kOnes;
+        }
+    }
+    split_butterflies<A>(z);
+}
+
 }  // namespace hq

@@ -39,6 +39,8 @@ struct QuantParams {
     uint8_t* codes;
     int64_t ld_codes;
     float* scales;
+    uint8_t* z;          // optional second output: the codes with the k - 4 factors of H_raw that the weights leave to them
+    int64_t ld_z;        // (split_codes), one signed byte each, for the one-limb product
     // optional GroupNorm + SiLU applied to the values as they are loaded (gn_stats == nullptr: off)
     const float* gn_stats;   // [samples][groups][2]: mean, 1/sqrt(var + eps)
     const float* gn_gamma;   // [cols]
@@ -282,6 +284,15 @@ __global__ void __launch_bounds__(320) fwht_quant_fast(const QuantParams p) {
         if (p.scales != nullptr) {
             if (!STATIC) { if (tr == 0) p.scales[row] = scale; }
             else if (row == 0 && tr == 0) p.scales[0] = scale;
+        }
+        if constexpr (split_block_ok(KLOG)) {              // E = 32 here: the thread's codes are 32 consecutive channels
+            if (p.z != nullptr) {
+                uint32_t zw[8];
+                split_codes<KLOG, INT8_OUT>(w, zw);
+                uint4* zd = reinterpret_cast<uint4*>(p.z + row * p.ld_z + int64_t(blk) * N + E * tb);
+                zd[0] = make_uint4(zw[0], zw[1], zw[2], zw[3]);
+                zd[1] = make_uint4(zw[4], zw[5], zw[6], zw[7]);
+            }
         }
     }
 }
@@ -739,7 +750,9 @@ struct SplitArgs { const void* x2; int64_t split, ldx2; };
 static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, int64_t cols, int64_t ldx, int had_block,
                                    int bits, hq_scale_mode mode, const float* static_scale, void* codes,
                                    hq_container cont, int64_t ld_codes, float* scales, const GnArgs* gn,
-                                   cudaStream_t st, const LnArgs* ln = nullptr, const SplitArgs* sp = nullptr) {
+                                   cudaStream_t st, const LnArgs* ln = nullptr, const SplitArgs* sp = nullptr,
+                                   SplitOut* zo = nullptr) {
+    if (zo != nullptr) zo->written = false;
     if (rows == 0 && cols > 0) return HQ_OK;                       // nothing to do; pointers may be NULL
     if (x == nullptr || codes == nullptr) return HQ_ERR_INVALID_ARG;
     if (xdt != HQ_F32 && xdt != HQ_BF16) return HQ_ERR_INVALID_ARG;
@@ -812,6 +825,10 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         const size_t smem = size_t(threads / (n / E)) * size_t(n / 4 + n / 4 / jslots) * 16 + size_t((rpc + 3) & ~3) * 4 +
                             (gn != nullptr ? size_t(cols) * 8 : 0) + (ln != nullptr ? size_t(rpc) * 8 : 0);
         const int grid = int((rows + rpc - 1) / rpc);
+        if (zo != nullptr && zo->z != nullptr && split_block_ok(klog) && split_fits(klog, bits)) {
+            p.z = zo->z; p.ld_z = zo->ld;
+            zo->written = true;
+        }
         cudaError_t e = xdt == HQ_F32
                             ? dispatch_fast<float>(klog, p, cont == HQ_CODES_INT8, grid, threads, smem, st)
                             : dispatch_fast<__nv_bfloat16>(klog, p, cont == HQ_CODES_INT8, grid, threads, smem, st);
@@ -840,20 +857,20 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
 
 hq_status launch_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t cols, int64_t ldx, int had_block,
                                 int bits, hq_scale_mode mode, const float* static_scale, void* codes,
-                                hq_container cont, int64_t ld_codes, float* scales, cudaStream_t st) {
+                                hq_container cont, int64_t ld_codes, float* scales, cudaStream_t st, SplitOut* zo) {
     return launch_quant_impl(x, xdt, rows, cols, ldx, had_block, bits, mode, static_scale, codes, cont, ld_codes, scales,
-                             nullptr, st);
+                             nullptr, st, nullptr, nullptr, zo);
 }
 
 // The same on the column concatenation [x | x2] of two matrices read in place: x holds columns [0, split), x2 the rest.
 hq_status launch_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, int64_t ldx2, int64_t split, hq_dtype xdt,
                                     int64_t rows, int64_t cols, int had_block, int bits, hq_scale_mode mode,
                                     const float* static_scale, void* codes, hq_container cont, int64_t ld_codes,
-                                    float* scales, cudaStream_t st) {
+                                    float* scales, cudaStream_t st, SplitOut* zo) {
     if (x2 == nullptr) return HQ_ERR_INVALID_ARG;
     const SplitArgs sp{x2, split, ldx2};
     return launch_quant_impl(x, xdt, rows, cols, ldx, had_block, bits, mode, static_scale, codes, cont, ld_codes, scales,
-                             nullptr, st, nullptr, &sp);
+                             nullptr, st, nullptr, &sp, zo);
 }
 
 // GroupNorm statistics of an NHWC tensor (hw pixels per sample): fp64 sums per (sample, group) in `scratch` (cleared
@@ -914,7 +931,7 @@ hq_status launch_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t 
                                const float* gamma, const float* beta, float eps, int had_block, int bits,
                                hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont,
                                int64_t ld_codes, float* scales, void* scratch, size_t scratch_bytes, cudaStream_t st,
-                               int silu, const void* pre_bias, const void* x2, int64_t split) {
+                               int silu, const void* pre_bias, const void* x2, int64_t split, SplitOut* zo) {
     if (gamma == nullptr || beta == nullptr) return HQ_ERR_INVALID_ARG;
     if (H <= 0 || W <= 0) return HQ_ERR_SHAPE;
     const int64_t hw = H * W;
@@ -925,10 +942,10 @@ hq_status launch_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t 
     if (x2 != nullptr) {
         const SplitArgs sp{x2, split, C - split};
         return launch_quant_impl(x, xdt, Nb * hw, C, split, had_block, bits, mode, static_scale, codes, cont, ld_codes, scales,
-                                 &gn, st, nullptr, &sp);
+                                 &gn, st, nullptr, &sp, zo);
     }
     return launch_quant_impl(x, xdt, Nb * hw, C, C, had_block, bits, mode, static_scale, codes, cont, ld_codes, scales, &gn,
-                             st);
+                             st, nullptr, nullptr, zo);
 }
 
 // LayerNorm over each row with a per-sample affine, fused into the transform+quantize kernel (one pass: the row's
@@ -936,12 +953,12 @@ hq_status launch_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t 
 hq_status launch_ln_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t cols, int64_t ldx, const float* weight,
                           const float* bias, int64_t rows_per_group, float eps, int had_block, int bits,
                           hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont, int64_t ld_codes,
-                          float* scales, cudaStream_t st) {
+                          float* scales, cudaStream_t st, SplitOut* zo) {
     if (rows_per_group < 0 || !(eps >= 0.f)) return HQ_ERR_INVALID_ARG;
     if ((weight != nullptr && !aligned16(weight)) || (bias != nullptr && !aligned16(bias)) || cols % 4 != 0) return HQ_ERR_ALIGNMENT;
     const LnArgs ln{weight, bias, rows_per_group, eps};
     return launch_quant_impl(x, xdt, rows, cols, ldx, had_block, bits, mode, static_scale, codes, cont, ld_codes, scales,
-                             nullptr, st, &ln);
+                             nullptr, st, &ln, nullptr, zo);
 }
 
 // Width-axis transform + quantization + integer factor of Eq. 13-14: x NHWC fp32/bf16 -> z int8 NHWC.
@@ -1027,7 +1044,7 @@ extern "C" hq_status hq_ln_quant(const void* x, hq_dtype xdt, int64_t rows, int6
                                  hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont,
                                  int64_t ld_codes, float* scales, void* stream) {
     return hq::launch_ln_quant(x, xdt, rows, cols, ldx, weight, bias, rows_per_group, eps, had_block, bits, mode,
-                               static_scale, codes, cont, ld_codes, scales, static_cast<cudaStream_t>(stream));
+                               static_scale, codes, cont, ld_codes, scales, static_cast<cudaStream_t>(stream), nullptr);
 }
 
 extern "C" hq_status hq_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C,
@@ -1037,7 +1054,7 @@ extern "C" hq_status hq_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, i
                                       size_t scratch_bytes, void* stream) {
     return hq::launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, had_block, bits, mode, static_scale, codes,
                                     cont, ld_codes, scales, scratch, scratch_bytes, static_cast<cudaStream_t>(stream), 1,
-                                    pre_bias, nullptr, 0);
+                                    pre_bias, nullptr, 0, nullptr);
 }
 
 extern "C" hq_status hq_gn_silu_quant_cat(const void* x, const void* x2, int64_t C1, hq_dtype xdt, int64_t Nb, int64_t H,
@@ -1048,7 +1065,7 @@ extern "C" hq_status hq_gn_silu_quant_cat(const void* x, const void* x2, int64_t
     if (x2 == nullptr) return HQ_ERR_INVALID_ARG;
     return hq::launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, had_block, bits, mode, static_scale, codes,
                                     cont, ld_codes, scales, scratch, scratch_bytes, static_cast<cudaStream_t>(stream), 1,
-                                    pre_bias, x2, C1);
+                                    pre_bias, x2, C1, nullptr);
 }
 
 extern "C" hq_status hq_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, int64_t ldx2, int64_t cols1,
@@ -1056,7 +1073,7 @@ extern "C" hq_status hq_hadamard_quant_cat(const void* x, int64_t ldx, const voi
                                            hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont,
                                            int64_t ld_codes, float* scales, void* stream) {
     return hq::launch_hadamard_quant_cat(x, ldx, x2, ldx2, cols1, xdt, rows, cols, had_block, bits, mode, static_scale, codes,
-                                         cont, ld_codes, scales, static_cast<cudaStream_t>(stream));
+                                         cont, ld_codes, scales, static_cast<cudaStream_t>(stream), nullptr);
 }
 
 extern "C" hq_status hq_hadamard_quant_width(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C,
@@ -1078,5 +1095,5 @@ extern "C" hq_status hq_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows
                                        void* codes, hq_container cont, int64_t ld_codes, float* scales,
                                        void* stream) {
     return hq::launch_hadamard_quant(x, xdt, rows, cols, ldx, had_block, bits, mode, static_scale, codes, cont,
-                                     ld_codes, scales, static_cast<cudaStream_t>(stream));
+                                     ld_codes, scales, static_cast<cudaStream_t>(stream), nullptr);
 }

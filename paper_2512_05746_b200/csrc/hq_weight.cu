@@ -9,11 +9,16 @@
 //   K axis tap-major, each tap padded with zeros to a multiple of 128 channels; for the NIBBLE activation
 //          container every 8 consecutive channels are stored in the order 0,2,4,6,1,3,5,7, which is the order
 //          the in-kernel nibble unpack produces for the activation operand.
+// FOLDED 4-bit weights with blocks of 32 .. 512 channels carry a second section behind the first: the one-limb weights of
+// the split fold, B' = (the four factors of H_raw that stay with the weights) Q(W), whose product with the codes the fused
+// layer calls' transform kernel leaves (split_codes in hq_fwht.cuh) is the same integer.  Natural channel order whatever
+// the container; one row per output channel.
 #include <cmath>
 #include <cstring>
 #include <vector>
 
 #include "hq_common.cuh"
+#include "hq_fwht.cuh"
 
 namespace hq {
 namespace {
@@ -40,6 +45,23 @@ void fwht_inplace(T* v, int n) {
             }
 }
 
+bool split_section(int w_bits, int had_block, hq_weight_mode mode) {
+    return mode == HQ_W_FOLDED && w_bits == 4 && had_block > 1 && is_pow2(had_block) && split_block_ok(ilog2(had_block));
+}
+
+// The factors of the index bits in `mask` of H_raw, on each block of n values.
+void fwht_bits_inplace(int32_t* v, int n, int mask) {
+    for (int h = 1; h < n; h <<= 1) {
+        if (!(mask & h)) continue;
+        for (int s = 0; s < n; s += 2 * h)
+            for (int j = s; j < s + h; ++j) {
+                const int32_t a = v[j], b = v[j + h];
+                v[j] = a + b;
+                v[j + h] = a - b;
+            }
+    }
+}
+
 void quantize_channel(const double* w, int64_t count, int w_bits, int32_t* out, float* scale) {
     const int qmax = kQmax(w_bits), qmin = kQmin(w_bits);
     double amax = 0.0;
@@ -62,7 +84,8 @@ extern "C" int64_t hq_weight_blob_bytes(int64_t N, int32_t RS, int64_t C, int32_
     if (N <= 0 || RS <= 0 || C <= 0) return 0;
     const int limbs = hq::limbs_for(w_bits, had_block, mode);
     const int64_t Ck = mode == HQ_W_PLAIN_A2 ? 2 * C : C;          // channels per tap along K
-    return hq::round_up(N, hq::kTileN) * limbs * RS * hq::round_up(Ck, hq::kTileK);
+    const int64_t limb = hq::round_up(N, hq::kTileN) * RS * hq::round_up(Ck, hq::kTileK);
+    return limb * (limbs + (limbs == 2 && hq::split_section(w_bits, had_block, mode) ? 1 : 0));
 }
 
 extern "C" hq_status hq_weight_prepare(const float* w, int64_t N, int32_t RS, int64_t C, int32_t w_bits,
@@ -83,12 +106,18 @@ extern "C" hq_status hq_weight_prepare(const float* w, int64_t N, int32_t RS, in
     const int64_t Ck = a2 ? 2 * C : C;                              // channels per tap along K
     const int64_t C_pad = round_up(Ck, kTileK), N_pad = round_up(N, kTileN);
     const int64_t Kp = int64_t(RS) * C_pad;
-    const int64_t need = N_pad * limbs * Kp;
-    if (blob_bytes < need) return HQ_ERR_WORKSPACE;
+    const int64_t base = N_pad * limbs * Kp;
+    if (blob_bytes < base) return HQ_ERR_WORKSPACE;
+    // a buffer of the two-limb section's size alone is taken as well: the layer then runs on two limbs
+    const bool split = limbs == 2 && split_section(w_bits, had_block, mode) && blob_bytes >= base + N_pad * Kp;
+    const int64_t need = base + (split ? N_pad * Kp : 0);
+    int weight_mask = n - 1;                                        // index bits whose factors stay with the weights
+    if (split)
+        for (int i = 0; i < ilog2(n) - kSplitWeightBits; ++i) weight_mask &= ~(1 << split_code_bit(i));
 
     const int64_t KK = int64_t(RS) * C;
     std::vector<double> row(KK);
-    std::vector<int32_t> B(KK);
+    std::vector<int32_t> B(KK), B1(split ? KK : 0);
     int8_t* out = static_cast<int8_t*>(blob);
     std::memset(out, 0, size_t(need));
     int32_t max_abs = 0;
@@ -103,6 +132,16 @@ extern "C" hq_status hq_weight_prepare(const float* w, int64_t N, int32_t RS, in
             }
         }
         quantize_channel(row.data(), KK, w_bits, B.data(), &s_w[o]);
+        if (split) {
+            B1 = B;
+            for (int64_t b = 0; b < KK / n; ++b) fwht_bits_inplace(B1.data() + b * n, n, weight_mask);
+            for (int t = 0; t < RS; ++t)
+                for (int64_t c = 0; c < C; ++c) {
+                    const int32_t v = B1[t * C + c];                // at most 7 * 16: Q(W) of an absmax scale has no -8
+                    if (v < -128 || v > 127) return HQ_ERR_OVERFLOW_RISK;
+                    out[base + o * Kp + int64_t(t) * C_pad + c] = int8_t(v);
+                }
+        }
         if (mode == HQ_W_FOLDED && n > 1)
             for (int64_t b = 0; b < KK / n; ++b) fwht_inplace(B.data() + b * n, n);
 
@@ -137,7 +176,8 @@ extern "C" hq_status hq_weight_prepare(const float* w, int64_t N, int32_t RS, in
     }
     desc->N = N; desc->C = Ck; desc->RS = RS; desc->w_bits = w_bits; desc->had_block = had_block;
     desc->mode = int32_t(mode); desc->limbs = limbs; desc->container = int32_t(container);
-    desc->C_pad = C_pad; desc->N_pad = N_pad; desc->bytes = need; desc->max_abs_b = max_abs; desc->reserved = 0;
+    desc->C_pad = C_pad; desc->N_pad = N_pad; desc->bytes = need; desc->max_abs_b = max_abs;
+    desc->reserved = split ? kBlobHasSplit : 0;
     return HQ_OK;
 }
 
