@@ -377,7 +377,8 @@ hq_status hq_qlinear_noalloc(const void* x, hq_dtype xdt, int64_t M, int64_t K, 
  *   1  wherever a pair kernel covers the problem (also K_pad 128 or 384 and problems of few tiles, where it measures level
  *      or slower);
  *   2  (default) where it measured faster: reductions with streamed weights (K_pad > 512), convolutions, and two-limb
- *      weights at K_pad 512 on problems of at least one 256-row tile per SM.
+ *      weights at K_pad 512 on problems of at least one 256-row tile per SM; problems of few tiles with a long reduction
+ *      run on clusters of 2, 4 or 8 SMs that divide a tile's reduction (one code per byte, bf16 output).
  * Results are bit-identical in every mode.  Returns the previous mode.  Process-wide, not thread-safe. */
 int hq_set_pair_gemm(int mode);
 

@@ -100,16 +100,15 @@ struct LayerCodes {
         const int klog = ilog2(desc->had_block);
         return split_block_ok(klog) && split_fits(klog, a_bits) && cols < 131072;
     }
-    // One limb halves the column tiles, and the transform kernel computes and writes a second byte per code.  A tile of 256
-    // rows and 256 operand rows takes about 0.28 us per 128 bytes of the reduction on a pair of SMs (four MMAs of 134
-    // cycles), whichever the limbs, so what counts is the rounds of tiles that are saved; the second byte costs 0.7 us plus
-    // its traffic at about 5.2 TB/s.  Measured (two limbs / one): 8192 x 1152 -> 4608 57.9 / 44.2 us, 64 x 32 x 32 x 512 3x3
-    // 176 / 117 us; where no round is saved it only costs: 256 x 256 -> 256 6.1 / 6.8 us, 2 x 8 x 8 x 1024 3x3 26.8 / 27.8.
+    // One limb halves the column tiles (or the weights a CTA of the split kernel streams), and the transform kernel computes
+    // and writes a second byte per code, which costs 0.7 us plus its traffic at about 5.2 TB/s.  Measured (two limbs / one):
+    // 8192 x 1152 -> 4608 57.9 / 44.2 us, 64 x 32 x 32 x 512 3x3 176 / 117 us, 2 x 16 x 16 x 768 3x3 13.1 / 11.8 us; where
+    // no round of tiles is saved it only costs: 256 x 256 -> 256 6.1 / 6.8 us, 8 x 64 x 64 x 256 3x3 stride 2 16.5 / 17.6.
     static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows) {
-        const int64_t pairs = sm_count() / 2, m = (out_rows + 255) / 256;
-        const int64_t two = (m * (desc->N_pad / 128) + pairs - 1) / pairs, one = (m * ((desc->N_pad + 255) / 256) + pairs - 1) / pairs;
-        const double saved_us = 0.28 * double(two - one) * double(desc->RS * desc->C_pad / 128);
-        return saved_us > 0.7 + double(rows) * double(cols) / 5.2e6;
+        const int num_kb = int(desc->RS * desc->C_pad / 128), tile_rows = out_rows < 128 ? int(out_rows > 0 ? out_rows : 1) : 128;
+        const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us;
+        const double one = plan_product(1, out_rows, tile_rows, desc->N_pad, num_kb).us;
+        return two - one > 0.7 + double(rows) * double(cols) / 5.2e6;
     }
     const void* a() const { return z.written ? z.z : codes; }
     int64_t lda() const { return z.written ? z.ld : ld; }

@@ -30,6 +30,10 @@ enum : int32_t {
 constexpr int32_t kBlobHasSplit = 1;      // hq_weight_desc::reserved: the one-limb section follows the two-limb one
 struct SplitOut { uint8_t* z; int64_t ld; bool written; };
 
+// hq_gemm_splitk.cu: CTAs a tile's reduction is divided over (0: persistent kernels) and the estimated time of a product.
+struct ProductPlan { int ways; double us; };
+ProductPlan plan_product(int limbs, int64_t out_rows, int tile_rows, int64_t n_pad, int num_kb);
+
 #define HQ_CUDA_OK(expr) do { cudaError_t e__ = (expr); if (e__ != cudaSuccess) return HQ_ERR_CUDA; } while (0)
 
 #ifdef __CUDACC__
@@ -111,6 +115,13 @@ __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bul
 // one be scheduled once every CTA has called it or exited.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A load of what the kernel before this one wrote, for use behind griddep_wait(): through the non-coherent path (__ldg) the
+// compiler may move the load in front of the wait, which gave a layer the scale that the workspace held before.
+__device__ __forceinline__ float ld_dependent(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
 // at most one bulk store group of this thread may still be reading shared memory
 __device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }

@@ -37,6 +37,10 @@ hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, in
                                    bool after_quant);
 hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, const CUtensorMap& tmY,
                             const hq_weight_desc* desc, const void* w_dev, cudaStream_t st);
+// hq_gemm_splitk.cu: the same product with a tile's reduction divided over a cluster, for problems of few tiles
+int splitk_ways(hq_container cont, const gemm::GemmParams& g, int64_t out_rows, int tile_rows, int64_t n_pad);
+hq_status launch_qgemm_splitk(const gemm::GemmParams& g, int ways, int tile_rows, int64_t out_rows, const CUtensorMap& tmA,
+                              const hq_weight_desc* desc, const void* w_dev, cudaStream_t st);
 int g_pair_gemm = 2;       // hq_set_pair_gemm: 0 never, 1 wherever the pair kernels cover, 2 where they measured faster
 
 namespace {
@@ -298,6 +302,11 @@ hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64
     fill_epilogue(p, cont, a_bits, desc, K, scale_a, scale_a_is_scalar, scale_w, bias, alpha, acc_out, y, ydt, ldy,
                   dev_status);
 
+    if (const int ways = g_pair_gemm == 2 ? splitk_ways(cont, p, M, kBM, desc->N_pad) : 0) {
+        CUtensorMap tmA;
+        if (!encode_2d(&tmA, a_codes, uint64_t(row_bytes), uint64_t(M), uint64_t(lda), kBK, kBM, true)) return HQ_ERR_CUDA;
+        return launch_qgemm_splitk(p, ways, kBM, M, tmA, desc, w_dev, st);
+    }
     if (g_pair_gemm && pair_kernel_covers(cont, desc, M, y, ydt, ldy, acc_out, p.combine_fast != 0) &&
         (g_pair_gemm == 1 || pair_kernel_pays(desc, M)))
         return launch_qgemm_pair(a_codes, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias, alpha, y, ldy,
@@ -374,13 +383,17 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     // whole images or a whole number of row groups per image.
     const bool rows_consecutive = p.bw == Wo && p.bw * p.bh * p.bn == kBM && (p.bh == Ho || (p.bn == 1 && Ho % p.bh == 0));
     p.per_tap = per_tap ? 1 : 0;
-    p.tma_store = (!per_tap && y != nullptr && acc_out == nullptr && p.y_bf16 && p.y_vec_ok && p.combine_fast && rows_consecutive) ? 1 : 0;
+    // the split kernel stores rows itself: it only needs a tile's pixels to be consecutive, however many there are
+    const bool box_consecutive = p.bw == Wo && (p.bh == Ho || (p.bn == 1 && Ho % p.bh == 0));
+    const int ways = g_pair_gemm == 2 && box_consecutive ? splitk_ways(cont, p, Nb * Ho * Wo, box_rows, desc->N_pad) : 0;
+    p.tma_store = (ways == 0 && !per_tap && y != nullptr && acc_out == nullptr && p.y_bf16 && p.y_vec_ok && p.combine_fast && rows_consecutive) ? 1 : 0;
     if (p.tma_store && !encode_y(&tmY, y, uint64_t(desc->N), uint64_t(Nb * Ho * Wo), uint64_t(desc->N))) return HQ_ERR_CUDA;
     const uint64_t dims[4] = {uint64_t(row_bytes), uint64_t(W), uint64_t(H), uint64_t(Nb)};
     // With a traversal stride the box extent is given in input elements: stride * (pixels wanted).
     const uint32_t box[4] = {uint32_t(nib ? kBK / 2 : kBK), uint32_t(p.bw * stride), uint32_t(p.bh * stride), uint32_t(p.bn)};
     const uint32_t estr[4] = {1, uint32_t(stride), uint32_t(stride), 1};
     if (!encode_4d(&tmA, a_codes, dims, box, estr, !nib)) return HQ_ERR_CUDA;
+    if (ways > 0) return launch_qgemm_splitk(p, ways, box_rows, Nb * Ho * Wo, tmA, desc, w_dev, st);
     const uint64_t Kp = uint64_t(desc->C_pad) * desc->RS;
     if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, kBN, true)) return HQ_ERR_CUDA;
     if (g_pair_gemm && pair_stream_covers_conv(cont, p)) return launch_qconv_pair(p, tmA, tmY, desc, w_dev, st);

@@ -414,7 +414,7 @@ __device__ __forceinline__ void fast_epilogue_warp(const GemmParams& p, const Ti
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int64_t row = int64_t(row0) + tr + 8 * j;
-                sa[j] = p.sa_scalar ? __ldg(p.scale_a) : (row < total_rows ? __ldg(p.scale_a + row) : 0.f);
+                sa[j] = p.sa_scalar ? ld_dependent(p.scale_a) : (row < total_rows ? ld_dependent(p.scale_a + row) : 0.f);
             }
         }
         int row0_next = -1;
@@ -432,7 +432,7 @@ __device__ __forceinline__ void fast_epilogue_warp(const GemmParams& p, const Ti
             sa_nx[j] = sa[j];
             if (row0_next >= 0) {                        // the next tile's row scales fly while this tile is processed
                 const int64_t row = int64_t(row0_next) + tr + 8 * j;
-                sa_nx[j] = row < total_rows ? __ldg(p.scale_a + row) : 0.f;
+                sa_nx[j] = row < total_rows ? ld_dependent(p.scale_a + row) : 0.f;
             }
         }
         const uint32_t t0 = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as * kBN + wc0);
@@ -740,7 +740,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     const int r = g / p.S, sx = g - r * p.S;
                     const int hi_ = ho * p.stride + r - p.pad, wi_ = wo * p.stride + sx - p.pad;
                     if (!row_ok || hi_ < 0 || hi_ >= p.H || wi_ < 0 || wi_ >= p.W) return 0.f;
-                    return __ldg(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);
+                    return ld_dependent(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);
                 };
                 float run[64];
 #pragma unroll
@@ -811,8 +811,8 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             // the row scale of this tile was requested while the previous tile was processed
             float sa_raw = sa_next;
             if (i == 0 && want_y) {
-                if (p.sa_scalar) sa_raw = __ldg(p.scale_a);
-                else if (my_row >= 0) sa_raw = __ldg(p.scale_a + my_row);
+                if (p.sa_scalar) sa_raw = ld_dependent(p.scale_a);
+                else if (my_row >= 0) sa_raw = ld_dependent(p.scale_a + my_row);
             }
             int next_row = -1;
             if (i + 1 < walk.count && want_y && !p.sa_scalar) {
@@ -825,7 +825,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             for (int j = 0; j < 4; ++j) rows[j] = out_row_of<CONV>(p, tc, q * 32 + j * 8 + (lane >> 2));
             if (!wait_or_abort(&ctl->tfull[as], aphase, ctl, p.dev_status, kStatusAccumWait)) { ok = false; break; }
             tc_fence_after();
-            if (next_row >= 0) sa_next = __ldg(p.scale_a + next_row);
+            if (next_row >= 0) sa_next = ld_dependent(p.scale_a + next_row);
             else if (p.sa_scalar) sa_next = sa_raw;
             float sa_eff = 0.f;
             if (want_y && my_row >= 0) {

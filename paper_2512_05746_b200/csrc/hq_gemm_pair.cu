@@ -15,6 +15,7 @@
 // barrier arrivals.  Every wait is bounded.
 #include <cuda.h>
 
+#include "hq_cluster.cuh"
 #include "hq_gemm_kernel.cuh"
 
 namespace hq {
@@ -61,20 +62,6 @@ __host__ __device__ inline PairLayout pair_layout(int num_kb, int stages, int kp
     return L;
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The address of the same shared-memory object in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t map_to_cta(const void* p, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-    return a;
-}
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
     // default (CTA-scope release) semantics: what the arrival orders are this warp's tensor-memory reads, which the
     // tcgen05 fence in front of it covers; a cluster-scope release here drains the thread's whole memory pipeline
@@ -458,7 +445,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             float sa = sa_next;
             if (i == 0) {
                 const int64_t my_row = int64_t(m2) * 256 + int(rank) * 128 + q * 32 + lane;
-                sa = p.sa_scalar ? __ldg(p.scale_a) : (my_row < p.M ? __ldg(p.scale_a + my_row) : 0.f);
+                sa = p.sa_scalar ? ld_dependent(p.scale_a) : (my_row < p.M ? ld_dependent(p.scale_a + my_row) : 0.f);
             }
             if (!wait_pair(&ctl->tfull[as], uint32_t(i >> 1) & 1u, ctl, p.dev_status, kStatusAccumWait)) { ok = false; break; }
             tc_fence_after();
@@ -467,7 +454,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                 const int u2 = u + 1;
                 const int n2 = u2 / p.tiles_m2, m2n = u2 - n2 * p.tiles_m2;
                 const int64_t row2 = int64_t(m2n) * 256 + int(rank) * 128 + q * 32 + lane;
-                sa_next = row2 < p.M ? __ldg(p.scale_a + row2) : 0.f;
+                sa_next = row2 < p.M ? ld_dependent(p.scale_a + row2) : 0.f;
             }
             const float sa_eff = p.alpha * sa;
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
@@ -672,7 +659,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 __syncwarp();
             }
             const int64_t my_row = int64_t(m2) * 256 + int(rank) * 128 + q * 32 + lane;
-            const float sa = p.sa_scalar ? __ldg(p.scale_a) : (my_row < p.M ? __ldg(p.scale_a + my_row) : 0.f);
+            const float sa = p.sa_scalar ? ld_dependent(p.scale_a) : (my_row < p.M ? ld_dependent(p.scale_a + my_row) : 0.f);
             if (!wait_pair(&ctl->tfull[as], uint32_t(i >> 1) & 1u, ctl, p.dev_status, kStatusAccumWait)) { ok = false; break; }
             tc_fence_after();
             const float sa_eff = p.alpha * sa;
