@@ -133,24 +133,37 @@ def _check(status: int, what: str):
         raise HqError(status, what)
 
 
+# The helpers below run a dozen times per call, and a small layer's kernels are as short as its marshalling (a 256 x 256
+# linear: 8 us on the device): addresses and streams cross as plain integers, and torch's objects are looked up once.
+_DTYPES: dict = {}
+_stream_of_device = None
+
+
 def _dptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    if stream is None:
+    global _stream_of_device
+    if stream is not None:
+        return stream.cuda_stream
+    if _stream_of_device is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        torch.cuda.init()
+        raw, device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        _stream_of_device = lambda: raw(device())
+    return _stream_of_device()
 
 
 def _dtype_code(t):
-    import torch
-    if t.dtype == torch.float32:
-        return HQ_F32
-    if t.dtype == torch.bfloat16:
-        return HQ_BF16
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    code = _DTYPES.get(t.dtype)
+    if code is None:
+        import torch
+        _DTYPES.update({torch.float32: HQ_F32, torch.bfloat16: HQ_BF16})
+        if t.dtype not in _DTYPES:
+            raise TypeError(f"unsupported dtype {t.dtype}")
+        code = _DTYPES[t.dtype]
+    return code
 
 
 def hq_version() -> int:
@@ -250,7 +263,7 @@ def hq_qlinear(x, pw: PreparedWeight, bias, a_bits: int, y, workspace, static_sc
     mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
     _check(lib.hq_qlinear(_dptr(x), _dtype_code(x), M, K, x.stride(0), C.byref(pw.desc), _dptr(pw.blob_dev),
                           _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode, _dptr(static_scale), _dptr(y), _dtype_code(y),
-                          y.stride(0), _dptr(workspace), workspace.numel() * workspace.element_size(),
+                          y.stride(0), _dptr(workspace), workspace.nbytes,
                           _dptr(dev_status), _stream(stream)), "hq_qlinear")
 
 
@@ -275,12 +288,12 @@ def hq_qconv(x, pw: PreparedWeight, R: int, S: int, stride: int, pad: int, bias,
         _check(lib.hq_qconv_cat(_dptr(x), _dptr(x2), Cin, _dtype_code(x), Nb, H, W, Cin + x2.shape[3], C.byref(pw.desc),
                                 _dptr(pw.blob_dev), R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode,
                                 _dptr(static_scale), _dptr(y), _dtype_code(y), _dptr(workspace),
-                                workspace.numel() * workspace.element_size(), _dptr(dev_status), _stream(stream)),
+                                workspace.nbytes, _dptr(dev_status), _stream(stream)),
                "hq_qconv_cat")
         return
     _check(lib.hq_qconv(_dptr(x), _dtype_code(x), Nb, H, W, Cin, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride,
                         pad, _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode, _dptr(static_scale), _dptr(y),
-                        _dtype_code(y), _dptr(workspace), workspace.numel() * workspace.element_size(),
+                        _dtype_code(y), _dptr(workspace), workspace.nbytes,
                         _dptr(dev_status), _stream(stream)), "hq_qconv")
 
 
@@ -294,12 +307,12 @@ def hq_gn_silu_quant(x, groups: int, gamma, beta, eps: float, had_block: int, bi
         _check(lib.hq_gn_silu_quant_cat(_dptr(x), _dptr(x2), Cin, _dtype_code(x), Nb, H, W, Cin + x2.shape[3], groups,
                                         _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps, had_block, bits, mode,
                                         _dptr(static_scale), _dptr(codes), container, codes.stride(0), _dptr(scales),
-                                        _dptr(scratch), scratch.numel() * scratch.element_size(), _stream(stream)),
+                                        _dptr(scratch), scratch.nbytes, _stream(stream)),
                "hq_gn_silu_quant_cat")
         return
     _check(lib.hq_gn_silu_quant(_dptr(x), _dtype_code(x), Nb, H, W, Cin, groups, _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps, had_block,
                                 bits, mode, _dptr(static_scale), _dptr(codes), container, codes.stride(0), _dptr(scales),
-                                _dptr(scratch), scratch.numel() * scratch.element_size(), _stream(stream)),
+                                _dptr(scratch), scratch.nbytes, _stream(stream)),
            "hq_gn_silu_quant")
 
 
@@ -315,15 +328,15 @@ def hq_gn_silu_qconv(x, groups: int, gamma, beta, eps: float, pw: PreparedWeight
                                         _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps, C.byref(pw.desc), _dptr(pw.blob_dev),
                                         R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode, _dptr(static_scale),
                                         _dptr(y), _dtype_code(y), _dptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _dptr(scratch),
-                                        scratch.numel() * scratch.element_size(), _dptr(dev_status), _stream(stream)),
+                                        workspace.nbytes, _dptr(scratch),
+                                        scratch.nbytes, _dptr(dev_status), _stream(stream)),
                "hq_gn_silu_qconv_cat")
         return
     _check(lib.hq_gn_silu_qconv(_dptr(x), _dtype_code(x), Nb, H, W, Cin, groups, _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps,
                                 C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias),
                                 a_bits, mode, _dptr(static_scale), _dptr(y), _dtype_code(y), _dptr(workspace),
-                                workspace.numel() * workspace.element_size(), _dptr(scratch),
-                                scratch.numel() * scratch.element_size(), _dptr(dev_status), _stream(stream)),
+                                workspace.nbytes, _dptr(scratch),
+                                scratch.nbytes, _dptr(dev_status), _stream(stream)),
            "hq_gn_silu_qconv")
 
 
@@ -344,7 +357,7 @@ def hq_ln_qlinear(x, ln_weight, ln_bias, rows_per_group: int, eps: float, pw: Pr
     M, K = x.shape
     _check(lib.hq_ln_qlinear(_dptr(x), _dtype_code(x), M, K, x.stride(0), _dptr(ln_weight), _dptr(ln_bias), rows_per_group,
                              eps, C.byref(pw.desc), _dptr(pw.blob_dev), _dptr(pw.s_w_dev), _dptr(bias), a_bits, _dptr(y),
-                             _dtype_code(y), y.stride(0), _dptr(workspace), workspace.numel() * workspace.element_size(),
+                             _dtype_code(y), y.stride(0), _dptr(workspace), workspace.nbytes,
                              _dptr(dev_status), _stream(stream)), "hq_ln_qlinear")
 
 
@@ -368,7 +381,7 @@ def hq_qconv_width(x, pw: PreparedWeight, R: int, S: int, stride: int, pad: int,
     Nb, H, W, Cin = x.shape
     _check(lib.hq_qconv_width(_dptr(x), _dtype_code(x), Nb, H, W, Cin, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride,
                               pad, _dptr(pw.s_w_dev), _dptr(bias), a_bits, had_block_w, _dptr(static_scale), _dptr(y),
-                              _dtype_code(y), _dptr(workspace), workspace.numel() * workspace.element_size(),
+                              _dtype_code(y), _dptr(workspace), workspace.nbytes,
                               _dptr(dev_status), _stream(stream)), "hq_qconv_width")
 
 
@@ -382,8 +395,8 @@ def hq_gn_qlinear(x, Nb: int, groups: int, gamma, beta, eps: float, silu: bool, 
     M, Cin = x.shape
     _check(lib.hq_gn_qlinear(_dptr(x), _dtype_code(x), Nb, M // Nb, Cin, groups, _dptr(gamma), _dptr(beta), eps, int(silu),
                              C.byref(pw.desc), _dptr(pw.blob_dev), _dptr(pw.s_w_dev), _dptr(bias), a_bits, _dptr(y),
-                             _dtype_code(y), y.stride(0), _dptr(workspace), workspace.numel() * workspace.element_size(),
-                             _dptr(scratch), scratch.numel() * scratch.element_size(), _dptr(dev_status), _stream(stream)),
+                             _dtype_code(y), y.stride(0), _dptr(workspace), workspace.nbytes,
+                             _dptr(scratch), scratch.nbytes, _dptr(dev_status), _stream(stream)),
            "hq_gn_qlinear")
 
 
@@ -426,7 +439,7 @@ def hq_concat_channels(a, b, out, stream=None) -> None:
 def hq_groupnorm_act(x, groups: int, gamma, beta, eps: float, silu: bool, out, scratch, stream=None) -> None:
     Nb, H, W, Cc = x.shape
     _check(lib.hq_groupnorm_act(_dptr(x), Nb, H, W, Cc, groups, _dptr(gamma), _dptr(beta), eps, int(silu), _dptr(out),
-                                _dptr(scratch), scratch.numel() * scratch.element_size(), _stream(stream)), "hq_groupnorm_act")
+                                _dptr(scratch), scratch.nbytes, _stream(stream)), "hq_groupnorm_act")
 
 
 def hq_conv2d_direct(x, w, bias, R: int, stride: int, pad: int, y, stream=None) -> None:

@@ -86,7 +86,8 @@ struct LayerCodes {
                hq_container cont, void* workspace, size_t ws_bytes)
         : codes(static_cast<unsigned char*>(workspace)),
           scales(reinterpret_cast<float*>(codes + scales_offset(rows, cols, cont))), ld(code_pitch(cols, cont)) {
-        if (split_applies(desc, a_bits, cols) && split_pays(desc, rows, cols, out_rows) && ws_bytes >= size_t(split_bytes(rows, cols, cont))) {
+        if (ws_bytes >= size_t(split_bytes(rows, cols, cont)) && split_applies(desc, a_bits, cols) &&
+            split_pays(desc, rows, cols, out_rows)) {
             z.z = codes + split_offset(rows, cols, cont);
             z.ld = code_pitch(cols, HQ_CODES_INT8);
             split_desc = *desc;

@@ -740,7 +740,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     const int r = g / p.S, sx = g - r * p.S;
                     const int hi_ = ho * p.stride + r - p.pad, wi_ = wo * p.stride + sx - p.pad;
                     if (!row_ok || hi_ < 0 || hi_ >= p.H || wi_ < 0 || wi_ >= p.W) return 0.f;
-                    return ld_dependent(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);
+                    return __ldg(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);      // never a dependent launch (pdl = 0)
                 };
                 float run[64];
 #pragma unroll
