@@ -73,6 +73,16 @@ __device__ __forceinline__ f32x2 silu2(f32x2 y) {
     return mul2(y, pk2(rcp_ftz(d0), rcp_ftz(d1)));
 }
 
+// Asynchronous 16-byte copies global -> shared.
+__device__ __forceinline__ void cp_async_16(void* smem, const void* gmem) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Slot of channel quad c4 in the LayerNorm prologue's tables, and the slots of one table.
+__host__ __device__ constexpr int ln_slot(int c4) { return c4 + 4 * (c4 >> 5); }
+__host__ __device__ constexpr int ln_tab_slots(int cols) { return ln_slot(cols / 4 - 1) + 1; }
+
 __device__ __forceinline__ float4 load4(const float* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
     uint2 raw = __ldcs(reinterpret_cast<const uint2*>(p));
@@ -100,7 +110,7 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
 // over the row (statistics taken here: the row is in the registers of its threads) with a per-sample affine, 3 GroupNorm
 // alone (the normalisation in front of an attention block's QKV projection).
 template <int KLOG, int E, typename InT, bool INT8_OUT, bool STATIC, int PRO>
-__global__ void __launch_bounds__(320) fwht_quant_fast(const QuantParams p) {
+__global__ void __launch_bounds__(320, PRO == 2 && E == 32 ? 3 : 1) fwht_quant_fast(const QuantParams p) {
     constexpr bool GN = PRO == 1 || PRO == 3;          // 3: GroupNorm without the SiLU
     constexpr bool GN_SILU = PRO == 1;
     constexpr bool LN = PRO == 2;
@@ -133,13 +143,11 @@ __global__ void __launch_bounds__(320) fwht_quant_fast(const QuantParams p) {
     // sample the CTA's rows belong to (the host makes sure a CTA never straddles two samples), then y * sigmoid(y).
     float* gn_a = reinterpret_cast<float*>(rowmax + ((p.rows_per_cta + 3) & ~3));
     float* gn_b = gn_a + p.cols;
-    // LayerNorm prologue: two sums per row, gathered in shared memory (the affine vectors of the CTA's sample are read
-    // from global memory as they are used: a CTA holds only a few rows, a table of its own would cost more than it saves)
-    float* lnacc = gn_a;                               // [rows_per_cta][2]
-    if (LN) {
-        if (tid < 2 * p.rows_per_cta) lnacc[tid] = 0.f;
-        __syncthreads();
-    }
+    // LayerNorm prologue: the row sums' parts ([2][threads]) and the affine vectors of the CTA's sample ([2][cols], a slot
+    // of 64 bytes after every 128 channels so that neighbouring Hadamard blocks start in different banks).
+    float* ln_part = gn_a;
+    float4* ln_tab = reinterpret_cast<float4*>(ln_part + 2 * blockDim.x);
+    const int ln_slots = ln_tab_slots(int(p.cols));
 
     // The rows' values are requested first, so that the table below is built while they are on their way.
     using Raw = typename std::conditional<sizeof(InT) == 4, float4, uint2>::type;
@@ -153,6 +161,20 @@ __global__ void __launch_bounds__(320) fwht_quant_fast(const QuantParams p) {
                              : reinterpret_cast<const InT*>(p.x) + r * p.ldx + c0;
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) cur[i] = __ldcs(reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i)));
+    }
+    if (LN) {
+        // The affine vectors are copied asynchronously while the row statistics are taken.  Read from L2 where they are
+        // used, 16 loads per thread behind the second barrier, they made this latency-bound prologue twice as long.
+        const int64_t g = p.ln_rows_per_group > 0 ? (int64_t(blockIdx.x) * p.rows_per_cta) / p.ln_rows_per_group : 0;
+        const int quads = int(p.cols) / 4;
+        for (int f = tid; f < 2 * quads; f += blockDim.x) {
+            const bool is_b = f >= quads;
+            const int c4 = is_b ? f - quads : f;
+            const float* src = is_b ? p.ln_b : p.ln_w;
+            float4* dst = ln_tab + (is_b ? ln_slots : 0) + ln_slot(c4);
+            if (src != nullptr) cp_async_16(dst, src + g * p.cols + 4 * c4);
+            else *dst = is_b ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(1.f, 1.f, 1.f, 1.f);
+        }
     }
     if (GN) {
         const unsigned sample = blockIdx.x / unsigned(p.gn_sets_per_sample);
@@ -200,42 +222,42 @@ __global__ void __launch_bounds__(320) fwht_quant_fast(const QuantParams p) {
         }
     }
     if (LN) {
-        // mean, then the sum of squared deviations (two passes over the registers), each gathered per row through a
-        // shared-memory sum; y = (x - mean) * rstd * w[c] + b[c]
-        // four neighbouring lanes belong to one row when the row's thread count is a multiple of 4: add them up by
-        // shuffles first, so that a quarter of the threads go to shared memory
-        const bool quad = (p.threads_per_row & 3) == 0;
+        // mean, then the sum of squared deviations (two passes over the registers); y = (x - mean) * rstd * w[c] + b[c].
+        // A row's threads come in aligned runs of 2^j lanes (2^j the largest power of two that divides their number):
+        // shuffles add up a run, and every thread adds the runs' parts in the same order, so that a sum does not depend
+        // on which warp came first.
+        const int run = p.threads_per_row & -p.threads_per_row, lanes = run < 32 ? run : 32;
+        const int parts = p.threads_per_row / lanes;
+        auto row_sum = [&](float part, float* buf) {
+            for (int off = 1; off < lanes; off <<= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+            if ((tr & (lanes - 1)) == 0) buf[row_in_cta * parts + tr / lanes] = part;
+            __syncthreads();
+            float sum = 0.f;
+#pragma unroll 4
+            for (int i = 0; i < parts; ++i) sum += buf[row_in_cta * parts + i];
+            return sum;
+        };
         f32x2 acc = v[0];
 #pragma unroll
         for (int i = 1; i < P; ++i) acc = add2(acc, v[i]);
         float lo, hi;
         upk2(acc, lo, hi);
-        float part = lo + hi;
-        if (quad) { part += __shfl_xor_sync(0xffffffffu, part, 1); part += __shfl_xor_sync(0xffffffffu, part, 2); }
-        if (!quad || (tid & 3) == 0) atomicAdd(&lnacc[2 * row_in_cta], part);
-        __syncthreads();
-        const float mean = lnacc[2 * row_in_cta] / float(p.cols);
+        const float mean = row_sum(lo + hi, ln_part) / float(p.cols);
         const f32x2 mean2 = pk2(mean, mean);
         acc = pk2(0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < P; ++i) { v[i] = sub2(v[i], mean2); acc = fma2(v[i], v[i], acc); }
         upk2(acc, lo, hi);
-        part = lo + hi;
-        if (quad) { part += __shfl_xor_sync(0xffffffffu, part, 1); part += __shfl_xor_sync(0xffffffffu, part, 2); }
-        if (!quad || (tid & 3) == 0) atomicAdd(&lnacc[2 * row_in_cta + 1], part);
-        __syncthreads();
-        const float rstd = rsqrtf(lnacc[2 * row_in_cta + 1] / float(p.cols) + p.ln_eps);
+        cp_async_wait_all();                           // this thread's pieces of the table; the barrier covers the others'
+        const float rstd = rsqrtf(row_sum(lo + hi, ln_part + blockDim.x) / float(p.cols) + p.ln_eps);
         const f32x2 rstd2 = pk2(rstd, rstd);
-        const int64_t g = p.ln_rows_per_group > 0 ? (int64_t(blockIdx.x) * p.rows_per_cta) / p.ln_rows_per_group : 0;
-        const float* wrow = p.ln_w != nullptr ? p.ln_w + g * p.cols : nullptr;
-        const float* brow = p.ln_b != nullptr ? p.ln_b + g * p.cols : nullptr;
+        const float4* tab_w = ln_tab + ln_slot(blk * (N / 4)) + ln_slot(tb);
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) {
-            const int ch = blk * N + 4 * (tb + TB * i);
-            const float4 a4 = wrow != nullptr ? __ldg(reinterpret_cast<const float4*>(wrow + ch)) : make_float4(1.f, 1.f, 1.f, 1.f);
-            const float4 b4 = brow != nullptr ? __ldg(reinterpret_cast<const float4*>(brow + ch)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            v[2 * i] = valid ? fma2(mul2(v[2 * i], rstd2), pk2(a4.x, a4.y), pk2(b4.x, b4.y)) : pk2(0.f, 0.f);
-            v[2 * i + 1] = valid ? fma2(mul2(v[2 * i + 1], rstd2), pk2(a4.z, a4.w), pk2(b4.z, b4.w)) : pk2(0.f, 0.f);
+            // slot of channel quad blk N/4 + tb + TB i: the three parts never carry into one another's group of 32 quads
+            const float4 a4 = tab_w[ln_slot(TB * i)], b4 = tab_w[ln_slots + ln_slot(TB * i)];
+            v[2 * i] = fma2(mul2(v[2 * i], rstd2), pk2(a4.x, a4.y), pk2(b4.x, b4.y));
+            v[2 * i + 1] = fma2(mul2(v[2 * i + 1], rstd2), pk2(a4.z, a4.w), pk2(b4.z, b4.w));
         }
     }
     float4* grp = xch + (tid / TB) * GS;
@@ -823,7 +845,8 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         // exchange buffer: per Hadamard block n/4 float4 slots plus one slot of padding per J (J = E/2 or E/4)
         const int jslots = (klog - ilog2(E) >= ilog2(E) - 1) ? E / 2 : E / 4;
         const size_t smem = size_t(threads / (n / E)) * size_t(n / 4 + n / 4 / jslots) * 16 + size_t((rpc + 3) & ~3) * 4 +
-                            (gn != nullptr ? size_t(cols) * 8 : 0) + (ln != nullptr ? size_t(rpc) * 8 : 0);
+                            (gn != nullptr ? size_t(cols) * 8 : 0) +
+                            (ln != nullptr ? size_t(2 * threads) * 4 + size_t(2 * ln_tab_slots(int(cols))) * 16 : 0);
         const int grid = int((rows + rpc - 1) / rpc);
         if (zo != nullptr && zo->z != nullptr && split_block_ok(klog) && split_fits(klog, bits)) {
             p.z = zo->z; p.ld_z = zo->ld;
