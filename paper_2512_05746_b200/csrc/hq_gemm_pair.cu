@@ -150,12 +150,14 @@ __device__ __forceinline__ bool wait_pair(uint64_t* bar, uint32_t parity, PairCt
 // 128 wavefronts per warp and tile, 1024 per tile on the data pipe that also feeds the tensor core its operands (1024 per
 // tile) and takes the staging stores and the bulk stores' reads (520): together more than the 2144 cycles of a tile's MMAs.
 // NBUF: the warp's staging buffers (two used in turn, or one).
-template <int LIMBS, int PREG = 0, int NBUF = 2>
+// BN: operand-B rows (accumulator columns) of the tile.
+template <int LIMBS, int PREG = 0, int NBUF = 2, int BN = kBN>
 __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg, int lane, const float* prm_sw,
                                               const float* prm_b, float sa_eff, const CUtensorMap* tmY, int col0, int row0,
                                               uint32_t tempty_leader, const float (&rsw)[PREG > 0 ? PREG * 16 : 1] = {0.f},
                                               const float (&rb)[PREG > 0 ? PREG * 16 : 1] = {0.f}) {
-    constexpr int NSTEPS = LIMBS == 2 ? kBN / 2 / 2 / 16 : kBN / 2 / 16;
+    static_assert(LIMBS == 1 || BN == kBN, "narrower tiles exist with one limb");
+    constexpr int NSTEPS = LIMBS == 2 ? kBN / 2 / 2 / 16 : BN / 2 / 16;
     const uint32_t wsw = (lane >> 1) & 3;
     uint32_t hi[16], lo[16];
     tmem_ld_32x16(t_row, hi);
@@ -514,7 +516,9 @@ __device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const void* tma
 
 // KPS = 2 (even K block counts): two K blocks per ring stage, laid out [A0 | B0 | A1 | B1]: the issuing lane's barrier
 // rounds halve (a wait, a fence, eight MMAs and a commit per 64 KB stage); three stages fit.
-template <int LIMBS, bool CONV, int KPS>
+// BN: operand-B rows per tile, 256, or with one limb also 192 or 128 (the host takes the width whose rounds of tiles cost
+// least, see stream_width); a narrower tile's weight half fills only part of its place in the stage.
+template <int LIMBS, bool CONV, int KPS, int BN>
 __global__ void __launch_bounds__(kPairThreads, 1)
 qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmY, const PairStreamParams p) {
@@ -568,7 +572,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                 for (int kb0 = 0; kb0 < num_kb; kb0 += KPS) {
                     if (!wait_pair(&ctl->empty[stage], phase ^ 1, ctl, p.dev_status, kStatusEmptyWait)) { ok = false; break; }
                     const uint32_t fbar = map_to_cta(&ctl->full[stage], 0);
-                    if (rank == 0) mbar_expect_tx(&ctl->full[stage], 2u * uint32_t(KPS * kPairStageBytes));
+                    if (rank == 0) mbar_expect_tx(&ctl->full[stage], 2u * uint32_t(KPS * (kABytes + BN / 2 * kBK)));
 #pragma unroll
                     for (int k = 0; k < KPS; ++k) {
                         const int kb = kb0 + k;
@@ -580,7 +584,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                         } else {
                             tma_load_2d_pair(dst, &tmA, fbar, kb * kBK, m_tile * kBM);
                         }
-                        tma_load_2d_pair(dst + kABytes, &tmB, fbar, kb * kBK, n_tile * kBN + int(rank) * 128);
+                        tma_load_2d_pair(dst + kABytes, &tmB, fbar, kb * kBK, n_tile * BN + int(rank) * (BN / 2));
                     }
                     if (++stage == nstages) { stage = 0; phase ^= 1; }
                 }
@@ -592,7 +596,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             // A lone lane spends several cycles per instruction, and this lane's path per K block is what paces the
             // kernel: the operand descriptors advance by constants (a stage is 32 KB = 2048 descriptor units on, the
             // weights 1024 units behind the activations), and only the very first MMA of a tile overwrites.
-            const uint32_t idesc = make_idesc_i8(256, kBN);
+            const uint32_t idesc = make_idesc_i8(256, BN);
             const uint64_t desc0 = make_sw128_kmajor_desc(smem_u32(sRing));
             constexpr uint64_t kBlockUnits = kPairStageBytes >> 4, kStageUnits = KPS * kBlockUnits, kBUnits = kABytes >> 4;
             uint64_t a_desc = desc0;
@@ -636,7 +640,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         unsigned char* stg = sStage + ew * NBUF * kStagingBytes;
         float* prm_sw = sParam + ew * 2 * (kBN / 2);
         float* prm_b = prm_sw + kBN / 2;
-        constexpr int cols_per_tile = LIMBS == 2 ? kBN / 2 : kBN;
+        constexpr int cols_per_tile = LIMBS == 2 ? kBN / 2 : BN;
         constexpr int cols_per_warp = cols_per_tile / 2;
         const int wc0 = chalf * cols_per_warp;
         const uint32_t tempty_leader[2] = {map_to_cta(&ctl->tempty[0], 0), map_to_cta(&ctl->tempty[1], 0)};
@@ -665,7 +669,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             const float sa_eff = p.alpha * sa;
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
             const uint32_t t_fast = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as * kBN + wc0);
-            epilogue_pair<LIMBS, 0, NBUF>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as]);
+            epilogue_pair<LIMBS, 0, NBUF, BN>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as]);
         }
         if (lane == 0) bulk_wait_read_all();           // shared memory must outlive the copy engine's reads
     }
@@ -756,10 +760,10 @@ int max_pairs(size_t smem) {
     return slot;
 }
 
-template <int LIMBS, bool CONV, int KPS>
+template <int LIMBS, bool CONV, int KPS, int BN>
 cudaError_t launch_pair_stream(int pairs_wanted, size_t smem, cudaStream_t st, const CUtensorMap& tmA, const CUtensorMap& tmB,
                                const CUtensorMap& tmY, const PairStreamParams& p) {
-    auto kern = qgemm_pair_stream_kernel<LIMBS, CONV, KPS>;
+    auto kern = qgemm_pair_stream_kernel<LIMBS, CONV, KPS, BN>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -795,6 +799,34 @@ cudaError_t launch_pair_stream(int pairs_wanted, size_t smem, cudaStream_t st, c
     return cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmY, p);
 }
 
+// Operand-B rows per tile with one limb: the width whose rounds of tiles over the pairs cost least.  An MMA's time follows
+// its width down to 128 (68 / 51 / 35 ns at 256 / 192 / 128), but a K block's operands do not (32 / 28 / 24 KB per CTA against
+// 274 / 205 / 138 ns of MMAs: the narrower tiles are paced by the loads), so a round of them counts as 235 and 200 columns
+// instead of 192 and 128; where a narrower width changes nothing in the number of tiles it has to spare at least 30 % of the
+// wider one's columns.  Measured (256 wide / chosen): 16001 x 1024 -> 1288 23.7 / 21.8 us (192), 4096 x 2048 -> 264 10.6 / 8.4
+// (128), 16 x 16 x 16 x 768 3x3 21.7 / 18.6 (192); not taken: 20 x 32 x 32 x 256 -> 384 3x3 22.2 / 23.9 (192, as many tiles).
+int stream_width(int64_t tiles_m2, int64_t N) {
+    const int64_t pairs = sm_count() / 2, wide = (N + kBN - 1) / kBN;
+    auto rounds = [&](int64_t tiles_n) { return (tiles_m2 * tiles_n + pairs - 1) / pairs; };
+    int best = kBN;
+    int64_t cost = rounds(wide) * kBN * 95 / 100;
+    for (const int bn : {192, 128}) {
+        const int64_t tn = (N + bn - 1) / bn, c = rounds(tn) * (bn == 192 ? 235 : 200);
+        if (c < cost && (tn != wide || 10 * (wide * kBN - N) >= 3 * wide * kBN)) { best = bn; cost = c; }
+    }
+    return best;
+}
+
+template <int LIMBS, bool CONV, int KPS>
+cudaError_t launch_pair_stream_bn(int bn, int pairs_wanted, size_t smem, cudaStream_t st, const CUtensorMap& tmA,
+                                  const CUtensorMap& tmB, const CUtensorMap& tmY, const PairStreamParams& p) {
+    if constexpr (LIMBS == 1) {
+        if (bn == 192) return launch_pair_stream<1, CONV, KPS, 192>(pairs_wanted, smem, st, tmA, tmB, tmY, p);
+        if (bn == 128) return launch_pair_stream<1, CONV, KPS, 128>(pairs_wanted, smem, st, tmA, tmB, tmY, p);
+    }
+    return launch_pair_stream<LIMBS, CONV, KPS, kBN>(pairs_wanted, smem, st, tmA, tmB, tmY, p);
+}
+
 bool pair_stream_stages(PairStreamParams& p, size_t& smem, int kps) {
     for (int stages = kPairMaxStages; stages >= 3; --stages) {
         const PairStreamLayout L = pair_stream_layout(stages, kps);
@@ -825,19 +857,26 @@ hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, in
     p.M = M; p.N = int(desc->N); p.limbs = desc->limbs;
     p.num_kb = int(desc->C_pad / kBK);
     p.tiles_m2 = int((M + 255) / 256);
-    p.tiles_n = int(desc->limbs == 2 ? desc->N_pad / 128 : (desc->N_pad + 255) / 256);
+    const int bn = desc->limbs == 2 ? kBN : stream_width(p.tiles_m2, desc->N);
+    p.tiles_n = int(desc->limbs == 2 ? desc->N_pad / 128 : (desc->N + bn - 1) / bn);
     p.scale_a = scale_a; p.sa_scalar = scale_a_is_scalar; p.scale_w = scale_w; p.bias = bias; p.alpha = alpha;
     p.pdl = after_quant ? 1 : 0; p.dev_status = dev_status;
     size_t smem = 0;
-    if (!pair_stream_stages(p, smem, 1)) return HQ_ERR_UNSUPPORTED;    // two K blocks per stage measured 2 % slower here
+    // Two K blocks per ring stage measured 2 % slower here at full width; narrower tiles of a longer reduction gain 8-15 %
+    // (their MMAs leave the issuing lane less time per barrier round), shorter ones lose 4 %.
+    const int kps = bn < kBN && p.num_kb % 2 == 0 && p.num_kb >= 10 ? 2 : 1;
+    if (!pair_stream_stages(p, smem, kps)) return HQ_ERR_UNSUPPORTED;
     CUtensorMap tmA, tmB, tmY;
     if (!encode_2d(&tmA, a_codes, uint64_t(K), uint64_t(M), uint64_t(lda), kBK, kBM, true)) return HQ_ERR_CUDA;
     const uint64_t Kp = uint64_t(desc->C_pad);
-    if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, 128, true)) return HQ_ERR_CUDA;
+    if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, uint32_t(bn / 2), true)) return HQ_ERR_CUDA;
     if (!encode_y(&tmY, y, uint64_t(desc->N), uint64_t(M), uint64_t(ldy))) return HQ_ERR_CUDA;
     const int tiles = p.tiles_m2 * p.tiles_n;
-    cudaError_t e = desc->limbs == 2 ? launch_pair_stream<2, false, 1>(tiles, smem, st, tmA, tmB, tmY, p)
-                                     : launch_pair_stream<1, false, 1>(tiles, smem, st, tmA, tmB, tmY, p);
+    cudaError_t e;
+    if (desc->limbs == 2) e = launch_pair_stream<2, false, 1, kBN>(tiles, smem, st, tmA, tmB, tmY, p);
+    else if (kps == 2) e = bn == 192 ? launch_pair_stream<1, false, 2, 192>(tiles, smem, st, tmA, tmB, tmY, p)
+                                     : launch_pair_stream<1, false, 2, 128>(tiles, smem, st, tmA, tmB, tmY, p);
+    else e = launch_pair_stream_bn<1, false, 1>(bn, tiles, smem, st, tmA, tmB, tmY, p);
     return e == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
 
@@ -849,7 +888,8 @@ hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, c
     p.M = int64_t(g.Nb) * g.Ho * g.Wo; p.N = g.N; p.limbs = g.limbs;
     p.num_kb = g.kb_per_tap * g.taps;
     p.tiles_m2 = (g.tiles_m + 1) / 2;
-    p.tiles_n = g.tiles_n;
+    const int bn = g.limbs == 2 ? kBN : stream_width(p.tiles_m2, g.N);
+    p.tiles_n = g.limbs == 2 ? g.tiles_n : (g.N + bn - 1) / bn;
     p.scale_a = g.scale_a; p.sa_scalar = g.sa_scalar; p.scale_w = g.scale_w; p.bias = g.bias; p.alpha = g.alpha;
     p.pdl = g.pdl; p.dev_status = g.dev_status;
     p.kb_per_tap = g.kb_per_tap; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
@@ -859,13 +899,13 @@ hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, c
     if (!pair_stream_stages(p, smem, kps)) return HQ_ERR_UNSUPPORTED;
     CUtensorMap tmB;
     const uint64_t Kp = uint64_t(desc->C_pad) * desc->RS;
-    if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, 128, true)) return HQ_ERR_CUDA;
+    if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, uint32_t(bn / 2), true)) return HQ_ERR_CUDA;
     const int tiles = p.tiles_m2 * p.tiles_n;
     cudaError_t e;
-    if (kps == 2) e = desc->limbs == 2 ? launch_pair_stream<2, true, 2>(tiles, smem, st, tmA, tmB, tmY, p)
-                                       : launch_pair_stream<1, true, 2>(tiles, smem, st, tmA, tmB, tmY, p);
-    else e = desc->limbs == 2 ? launch_pair_stream<2, true, 1>(tiles, smem, st, tmA, tmB, tmY, p)
-                              : launch_pair_stream<1, true, 1>(tiles, smem, st, tmA, tmB, tmY, p);
+    if (kps == 2) e = desc->limbs == 2 ? launch_pair_stream_bn<2, true, 2>(bn, tiles, smem, st, tmA, tmB, tmY, p)
+                                       : launch_pair_stream_bn<1, true, 2>(bn, tiles, smem, st, tmA, tmB, tmY, p);
+    else e = desc->limbs == 2 ? launch_pair_stream_bn<2, true, 1>(bn, tiles, smem, st, tmA, tmB, tmY, p)
+                              : launch_pair_stream_bn<1, true, 1>(bn, tiles, smem, st, tmA, tmB, tmY, p);
     return e == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
 

@@ -1,0 +1,39 @@
+"""Narrower column tiles of the streamed pair kernel (one weight limb, 192 or 128 operand rows per tile): bit for bit the one-CTA
+kernel's output, at column counts that end inside a tile, at one and two K blocks per ring stage and for a convolution."""
+import pytest
+
+from paper_2512_05746_b200 import inputs
+from test_gpu_splitk import both
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,K,N", [
+    (16001, 1024, 1288),      # 192 wide, one K block per stage, ragged rows and columns
+    (4096, 2048, 264),        # 128 wide, two K blocks per stage
+    (4096, 1152, 264),        # 128 wide, an odd number of K blocks
+    (5000, 4096, 520),        # 192 wide, two K blocks per stage
+    (20000, 1280, 136),       # 192 wide, as many tiles as 256 wide ones
+    (8192, 4608, 1152),       # 192 wide, whole tiles
+])
+def test_linear_on_narrow_tiles(M, K, N):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    pw = hq.hq_weight_prepare(inputs.weights((N, K), seed=N), 8, 128, hq.HQ_W_DOUBLE, hq.HQ_CODES_INT8).to_device()
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    q = torch.randint(-128, 128, (M, K), generator=gen, device="cuda", dtype=torch.int8).view(torch.uint8)
+    sa = torch.rand((M,), generator=gen, device="cuda") + 0.5
+    b = torch.from_numpy(inputs.bias(N, seed=1)).cuda()
+    both(torch, hq, lambda y, st: hq.hq_qgemm(q, hq.HQ_CODES_INT8, 8, K, pw, scale_a=sa, bias=b, y=y, dev_status=st), (M, N))
+
+
+@pytest.mark.parametrize("Nb,H,C,Cout", [(16, 16, 768, 768), (40, 32, 256, 136), (9, 32, 640, 264)])
+def test_convolution_on_narrow_tiles(Nb, H, C, Cout):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    pw = hq.hq_weight_prepare(inputs.weights((Cout, 3, 3, C), seed=C), 4, 128, hq.HQ_W_PLAIN, hq.HQ_CODES_INT8).to_device()
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    q = torch.randint(-128, 128, (Nb, H, H, C), generator=gen, device="cuda", dtype=torch.int8).view(torch.uint8)
+    sa, b = torch.rand((1,), generator=gen, device="cuda") + 0.5, torch.from_numpy(inputs.bias(Cout, seed=1)).cuda()
+    both(torch, hq, lambda y, st: hq.hq_qconv2d(q, hq.HQ_CODES_INT8, 8, Nb, H, H, C, pw, 3, 3, 1, 1, scale_a=sa, bias=b, y=y,
+                                                dev_status=st), (Nb, H, H, Cout))
