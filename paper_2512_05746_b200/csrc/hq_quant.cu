@@ -177,10 +177,11 @@ __global__ void __launch_bounds__(320, PRO == 2 && E == 32 ? 3 : 1) fwht_quant_f
         }
     }
     if (GN) {
+        griddep_wait();                                // the statistics; x itself was complete before they were begun
         const unsigned sample = blockIdx.x / unsigned(p.gn_sets_per_sample);
         const float2* st = reinterpret_cast<const float2*>(p.gn_stats) + size_t(sample) * p.gn_groups;
         for (int c = 4 * tid; c < int(p.cols); c += 4 * blockDim.x) {      // a channel quad lies in one group
-            const float2 ms = __ldg(st + (p.gn_cg_shift >= 0 ? c >> p.gn_cg_shift : c / p.gn_cg));
+            const float2 ms = ld_dependent2(st + (p.gn_cg_shift >= 0 ? c >> p.gn_cg_shift : c / p.gn_cg));
             const float4 gm = __ldg(reinterpret_cast<const float4*>(p.gn_gamma + c));
             const float4 bt = __ldg(reinterpret_cast<const float4*>(p.gn_beta + c));
             const float4 a = make_float4(ms.y * gm.x, ms.y * gm.y, ms.y * gm.z, ms.y * gm.w);
@@ -595,6 +596,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_kernel(const InT* x, const In
     constexpr int U = 8;                               // loads in flight per thread
     __shared__ double red[2 * Q][256];
     __shared__ int s_last;
+    griddep_launch();                                  // the transform kernel may place its CTAs and request its rows
     const int tid = threadIdx.x;
     const int pieces = C / VEC;
     const int nq = pieces < 256 ? pieces : 256;        // pieces walked side by side
@@ -714,6 +716,111 @@ __global__ void __launch_bounds__(256, 4) gn_stats_kernel(const InT* x, const In
     }
 }
 
+// The same statistics with one CTA per (sample, run of whole groups): it sees every pixel of its channels, so the sums need
+// no atomics, no clearing and no ticket, and the call no memset in front (two 32 x 32 x 512 images: 6.6 us of this kernel
+// and 1.5 us of memset before).  A thread owns a 16-byte piece and takes the pixels in the sets that the kernel above adds up
+// in fp32 (eight pixels `ppl` apart), so the fp32 partial sums are the same; only the fp64 sums over them run in another
+// order.  The CTA reads `pieces` * 16 contiguous bytes of every pixel, its neighbours in the grid the rest.
+template <typename InT, int VEC>
+__global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, const InT* x2, int split, const __nv_bfloat16* pre_bias,
+                                                               int hw, int C, int groups, int run, int ppl, float* stats,
+                                                               double inv_count, double eps) {
+    constexpr int Q = VEC / 4, U = 8;
+    __shared__ double red[2 * Q][256];
+    __shared__ double piece_sum[2 * Q][256];
+    griddep_launch();
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int cg = C / groups, pieces = run * cg / VEC, lanes = 256 / pieces;      // the host keeps pieces <= 256
+    const int runs = groups / run;
+    const int sample = blockIdx.x / runs, g0 = (blockIdx.x - sample * runs) * run;
+    const int piece = tid % pieces, pl = tid / pieces;
+    const int ch = g0 * cg + piece * VEC;
+    double s1[Q], s2[Q];
+    f32x2 e_lo[Q], e_hi[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) { s1[q] = 0.0; s2[q] = 0.0; e_lo[q] = pk2(0.f, 0.f); e_hi[q] = pk2(0.f, 0.f); }
+    if (pl < lanes) {
+        if (pre_bias != nullptr) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const uint2 er = __ldg(reinterpret_cast<const uint2*>(pre_bias + int64_t(sample) * C + ch + 4 * q));
+                e_lo[q] = pk2(__uint_as_float(er.x << 16), __uint_as_float(er.x & 0xFFFF0000u));
+                e_hi[q] = pk2(__uint_as_float(er.y << 16), __uint_as_float(er.y & 0xFFFF0000u));
+            }
+        }
+        const bool second = x2 != nullptr && ch >= split;
+        const int64_t pitch = x2 == nullptr ? C : (second ? C - split : split);
+        const InT* src = (second ? x2 + (ch - split) : x + ch) + int64_t(sample) * hw * pitch;
+        const int full = hw / (U * ppl) * ppl;         // sets of eight pixels; the pixels behind them are taken one by one
+        for (int set = pl; set < full; set += lanes) {
+            const int px = set / ppl * (U * ppl) + set % ppl;
+            GnPiece<VEC> raw[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) raw[u] = gn_load(src + int64_t(px + u * ppl) * pitch, static_cast<GnPiece<VEC>*>(nullptr));
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                f32x2 a = pk2(0.f, 0.f), b = pk2(0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    f32x2 lo, hi;
+                    gn_quad(raw[u], q, lo, hi);
+                    lo = add2(lo, e_lo[q]);
+                    hi = add2(hi, e_hi[q]);
+                    a = add2(a, add2(lo, hi));
+                    b = fma2(lo, lo, fma2(hi, hi, b));
+                }
+                float a0, a1, b0, b1;
+                upk2(a, a0, a1);
+                upk2(b, b0, b1);
+                s1[q] += double(a0 + a1);
+                s2[q] += double(b0 + b1);
+            }
+        }
+        for (int px = full * U + pl; px < hw; px += lanes) {
+            const GnPiece<VEC> raw = gn_load(src + int64_t(px) * pitch, static_cast<GnPiece<VEC>*>(nullptr));
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                f32x2 lo, hi;
+                gn_quad(raw, q, lo, hi);
+                lo = add2(lo, e_lo[q]);
+                hi = add2(hi, e_hi[q]);
+                float a0, a1, b0, b1;
+                upk2(add2(lo, hi), a0, a1);
+                upk2(fma2(lo, lo, mul2(hi, hi)), b0, b1);
+                s1[q] += double(a0 + a1);
+                s2[q] += double(b0 + b1);
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) { red[2 * q][tid] = s1[q]; red[2 * q + 1][tid] = s2[q]; }
+    __syncthreads();
+    // every sum of every piece over its threads, by runs of 8, 16 or 32 lanes
+    const int w = lanes <= 8 ? 8 : (lanes <= 16 ? 16 : 32), sub = lane & (w - 1);
+    for (int j0 = warp * (32 / w); j0 < 2 * Q * pieces; j0 += 8 * (32 / w)) {
+        const int j = j0 + lane / w, k = j / pieces, pc = j - k * pieces;
+        double t = 0.0;
+        if (j < 2 * Q * pieces)
+            for (int l = sub; l < lanes; l += w) t += red[k][l * pieces + pc];
+        for (int off = w >> 1; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+        if (sub == 0 && j < 2 * Q * pieces) piece_sum[k][pc] = t;
+    }
+    __syncthreads();
+    if (tid < run) {                                   // the host keeps run <= 256
+        const int quads = cg / 4;
+        double a = 0.0, b = 0.0;
+        for (int i = 0; i < quads; ++i) {
+            const int qd = tid * quads + i, pc = qd / Q, q = qd - pc * Q;
+            a += piece_sum[2 * q][pc];
+            b += piece_sum[2 * q + 1][pc];
+        }
+        const double mean = a * inv_count;
+        double var = b * inv_count - mean * mean;
+        if (var < 0.0) var = 0.0;
+        reinterpret_cast<float2*>(stats)[int64_t(sample) * groups + g0 + tid] = make_float2(float(mean), float(1.0 / sqrt(var + eps)));
+    }
+}
+
 template <int KLOG, int E, typename InT>
 cudaError_t launch_fast(const QuantParams& p, bool int8_out, int grid, int threads, size_t smem, cudaStream_t st) {
     const bool stat = p.static_scale != nullptr;
@@ -721,6 +828,17 @@ cudaError_t launch_fast(const QuantParams& p, bool int8_out, int grid, int threa
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
             if (e != cudaSuccess) return e;
+        }
+        if (p.gn_stats != nullptr) {
+            // a dependent of the statistics kernel: its rows are on their way before it waits for the statistics (1-2 us)
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(unsigned(grid)); cfg.blockDim = dim3(unsigned(threads));
+            cfg.dynamicSmemBytes = smem; cfg.stream = st;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr; cfg.numAttrs = 1;
+            return cudaLaunchKernelEx(&cfg, kern, p);
         }
         kern<<<grid, threads, smem, st>>>(p);
         return cudaGetLastError();
@@ -896,6 +1014,24 @@ hq_status launch_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, 
                              nullptr, st, nullptr, &sp, zo);
 }
 
+// Groups per CTA of the slab kernel, or 0: the one-wave kernel takes the tensor (groups of more than 256 pieces, more samples
+// than one wave of CTAs).  The fewest groups for which the CTAs fit one wave of four per SM.  On tensors of more than 20 MB,
+// where bandwidth counts and not the latency of atomics, only if the run fills whole sectors of a pixel and the threads of a
+// piece share its sets evenly.  Statistics + transform, one-wave / slab: 2 x 32 x 32 x 512 13.7 / 6.7 us, 8 x 8 x 8 x 1024
+// 8.9 / 8.8, 64 x 32 x 32 x 512 56.8 / 55.0; not taken: 16 x 64 x 64 x 256 29.7 / 31.2 (half sectors), 64 x 16 x 16 x 768
+// 27.7 / 28.8 (32 sets over 21 threads).
+static int gn_slab_run(int64_t Nb, int64_t hw, int64_t C, int groups, int elt, int vec) {
+    const int64_t cg = C / groups;
+    for (int run = 1; run <= groups && run <= 256; ++run) {
+        if (groups % run != 0 || (run * cg) % vec != 0 || run * cg / vec > 256) continue;
+        if (Nb * (groups / run) > int64_t(sm_count()) * 4) continue;
+        const int64_t sets = (hw + 7) / 8, lanes = 256 / (run * cg / vec);
+        const bool even = 10 * sets >= 8 * lanes * ((sets + lanes - 1) / lanes);
+        return Nb * hw * C * elt <= 20000000 || (even && run * cg * elt >= 32) ? run : 0;
+    }
+    return 0;
+}
+
 // GroupNorm statistics of an NHWC tensor (hw pixels per sample): fp64 sums per (sample, group) in `scratch` (cleared
 // here), then mean and 1/sqrt(var + eps) as floats behind them.  scratch: Nb * groups * (2 doubles + 2 floats).
 hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, int64_t C, int groups, float eps,
@@ -915,7 +1051,6 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     const __nv_bfloat16* pre = static_cast<const __nv_bfloat16*>(pre_bias);
     double* sums = static_cast<double*>(scratch);
     float* stats = reinterpret_cast<float*>(sums + size_t(Nb) * groups * 2);
-    HQ_CUDA_OK(cudaMemsetAsync(scratch, 0, need, st));             // the sums and the ticket counters
     if (hw > 0x7fffffff) return HQ_ERR_UNSUPPORTED;                // the tickets count pixels in 32 bits
     // 16-byte pieces (bf16: eight channels) where the shape allows them
     if (x2 != nullptr) {                                           // channels [split, C) of every pixel live in x2
@@ -925,6 +1060,20 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     const bool wide = xdt == HQ_BF16 && C % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     const int64_t pieces = C / (wide ? 8 : 4);
     const int64_t ppl = pieces < 256 ? 256 / pieces : 1;
+    const double inv_count = 1.0 / (double(hw) * double(C / groups));
+    if (const int run = gn_slab_run(Nb, hw, C, groups, elt, wide ? 8 : 4)) {
+        const unsigned slabs = unsigned(Nb * (groups / run));
+#define HQ_SLAB(T, V) gn_stats_slab_kernel<T, V><<<slabs, 256, 0, st>>>(static_cast<const T*>(x), static_cast<const T*>(x2), int(split), pre, int(hw), \
+                                                                        int(C), groups, run, int(ppl), stats, inv_count, double(eps))
+        if (xdt == HQ_F32) HQ_SLAB(float, 4);
+        else if (wide) HQ_SLAB(__nv_bfloat16, 8);
+        else HQ_SLAB(__nv_bfloat16, 4);
+#undef HQ_SLAB
+        if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
+        *stats_out = stats;
+        return HQ_OK;
+    }
+    HQ_CUDA_OK(cudaMemsetAsync(scratch, 0, need, st));             // the sums and the ticket counters
     // one wave of CTAs (four per SM) that share the pixels of all samples evenly, in whole rounds of loads; small
     // tensors get fewer CTAs so that a thread still walks a round of eight pixels
     const int64_t total_px = Nb * hw;
@@ -932,7 +1081,6 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     int64_t ctas = int64_t(sm_count()) * 4;
     int64_t span = ((total_px + ctas - 1) / ctas + round - 1) / round * round;
     ctas = (total_px + span - 1) / span;
-    const double inv_count = 1.0 / (double(hw) * double(C / groups));
     const unsigned grid = unsigned(ctas);
     if (xdt == HQ_F32)
         gn_stats_kernel<float, 4><<<grid, 256, 0, st>>>(static_cast<const float*>(x), static_cast<const float*>(x2), int(split), pre, hw, total_px, span, int(C), groups, sums,
