@@ -109,8 +109,13 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
 // PRO: prologue applied to the values before the transform: 0 none, 1 GroupNorm + SiLU (statistics given), 2 LayerNorm
 // over the row (statistics taken here: the row is in the registers of its threads) with a per-sample affine, 3 GroupNorm
 // alone (the normalisation in front of an attention block's QKV projection).
+// Blocks per SM the registers are bounded for: three for LayerNorm on 32 values (64 registers; unbounded 26 us on 8192 x 1152,
+// two 18.4, three 15.8, four 18.2); none stated for the GroupNorm prologues (56 registers; stating one lets the compiler take
+// 84, 2.1 ms instead of 1.8 for the 44 launches of a UNet forward at batch 64); one for the plain transform (level at 256 and
+// 512 channels, 60.9 -> 54.7 us on 65536 x 1152).
+__host__ __device__ constexpr int quant_min_blocks(int pro, int e) { return pro == 2 && e == 32 ? 3 : (pro == 0 ? 1 : 0); }
 template <int KLOG, int E, typename InT, bool INT8_OUT, bool STATIC, int PRO>
-__global__ void __launch_bounds__(320, PRO == 2 && E == 32 ? 3 : 1) fwht_quant_fast(const QuantParams p) {
+__global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast(const QuantParams p) {
     constexpr bool GN = PRO == 1 || PRO == 3;          // 3: GroupNorm without the SiLU
     constexpr bool GN_SILU = PRO == 1;
     constexpr bool LN = PRO == 2;
