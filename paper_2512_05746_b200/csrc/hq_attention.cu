@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(128, (DH <= 64 ? 4 : 2)) attention_kernel(cons
     if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
 }
 
-// ---- head widths of 64 and 128: operands by TMA -----------------------------------------------------------------
+// ---- operands by TMA: head widths of 64 and 128, and of 32, 48 and 96 where the keys fill their blocks -----------------
 // Q, K and V tiles come in by bulk tensor loads in the 128-byte swizzle (rows of 64 head channels = 128 bytes; a width
 // of 128 takes two such column halves per tile), issued by one thread as soon as the MMAs that read the buffer have
 // completed: the next K block lands during the softmax, the next V block during the next S product, no registers or
@@ -327,11 +327,13 @@ __device__ __forceinline__ uint64_t make_sw128_mnmajor_desc(uint32_t smem_addr, 
     return d;
 }
 
-template <int DH>
+// LAZY: that rule; otherwise the maximum moves with every block.
+template <int DH, bool LAZY>
 __global__ void __launch_bounds__(128, (DH <= 64 ? 4 : 2))
 attention_tma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV, const AttnParams p) {
     extern __shared__ __align__(1024) unsigned char smem_attn_tma[];
-    constexpr int KB = kKeyBlock, NH = DH / 64;                // column halves per tile
+    constexpr int KB = kKeyBlock, NH = (DH + 63) / 64;         // 64-channel parts per tile (the last may reach into the next
+                                                               // head's channels, which no MMA reads)
     constexpr int kQHalf = kQTile * 128, kKVHalf = KB * 128;   // bytes of one 64-channel half of a tile
     constexpr int kTmemCols = attn_tmem_cols(DH);
     unsigned char* sQ = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_attn_tma) + 1023) & ~uintptr_t(1023));
@@ -445,7 +447,8 @@ attention_tma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
         float mx = -INFINITY;
 #pragma unroll
         for (int e = 0; e < KB; e += 2) mx = max3(mx, __uint_as_float(sreg[e]), __uint_as_float(sreg[e + 1]));
-        const float m_new = (mx - m_run) * p.scale_log2 > 8.0f ? mx : m_run;     // first block: inf > 8
+        const float m_new = LAZY ? ((mx - m_run) * p.scale_log2 > 8.0f ? mx : m_run)     // first block: inf > 8
+                                 : fmaxf(m_run, mx);
         const float mc = m_new * p.scale_log2;
         const float alpha = ex2(m_run * p.scale_log2 - mc);              // 1 when the maximum stays, 0 on the first block
         f32x2 sum2 = pk2(0.f, 0.f);
@@ -554,17 +557,17 @@ attention_tma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
 }
 
-template <int DH>
+template <int DH, bool LAZY>
 hq_status launch_attention_tma(const AttnParams& p, int Nb, cudaStream_t st) {
     CUtensorMap tmQ, tmKV;
     const uint64_t rows = uint64_t(Nb) * p.L, cols = 3 * uint64_t(p.C);
     if (!encode_2d_bf16_sw128(&tmQ, p.qkv, cols, rows, cols * 2, kQTile)) return HQ_ERR_CUDA;
     if (!encode_2d_bf16_sw128(&tmKV, p.qkv, cols, rows, cols * 2, kKeyBlock)) return HQ_ERR_CUDA;
-    const size_t smem = size_t(DH / 64) * (kQTile + 2 * kKeyBlock) * 128 + size_t(kQTile) * kKeyBlock * 2 + 1024;
-    if (cudaFuncSetAttribute(attention_tma_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+    const size_t smem = size_t((DH + 63) / 64) * (kQTile + 2 * kKeyBlock) * 128 + size_t(kQTile) * kKeyBlock * 2 + 1024;
+    if (cudaFuncSetAttribute(attention_tma_kernel<DH, LAZY>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
         return HQ_ERR_CUDA;
     const dim3 grid(unsigned((p.L + kQTile - 1) / kQTile), unsigned(p.heads), unsigned(Nb));
-    attention_tma_kernel<DH><<<grid, 128, smem, st>>>(tmQ, tmKV, p);
+    attention_tma_kernel<DH, LAZY><<<grid, 128, smem, st>>>(tmQ, tmKV, p);
     return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
 
@@ -598,12 +601,21 @@ extern "C" hq_status hq_attention(const void* qkv, int64_t Nb, int64_t L, int64_
     p.dev_status = dev_status;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
+    // Tiles by TMA for every width where the keys fill their blocks (64 x 256 tokens, 8 heads of 96: 66 -> 52 us).  In a sample's
+    // last, partly filled block the tile holds keys of the next sample, whose zero weights would meet an infinity of that
+    // sample's values: widths 64 and 128 have no other kernel, the others keep the one that stages through registers and fills
+    // with zeros for those lengths.  They move their maximum with every block, as it does: the same bits either way.
+    if (p.L % kKeyBlock == 0) {
+        if (dh == 32) return launch_attention_tma<32, false>(p, int(Nb), st);
+        if (dh == 48) return launch_attention_tma<48, false>(p, int(Nb), st);
+        if (dh == 96) return launch_attention_tma<96, false>(p, int(Nb), st);
+    }
     switch (dh) {
         case 32: e = launch_attention<32>(p, int(Nb), st); break;
         case 48: e = launch_attention<48>(p, int(Nb), st); break;
-        case 64: return launch_attention_tma<64>(p, int(Nb), st);
+        case 64: return launch_attention_tma<64, true>(p, int(Nb), st);
         case 96: e = launch_attention<96>(p, int(Nb), st); break;
-        case 128: return launch_attention_tma<128>(p, int(Nb), st);
+        case 128: return launch_attention_tma<128, true>(p, int(Nb), st);
         default: return HQ_ERR_UNSUPPORTED;      // head widths the tensor-core tile shapes here cover: 32, 48, 64, 96, 128
     }
     return e == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
