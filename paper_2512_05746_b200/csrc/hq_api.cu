@@ -81,7 +81,8 @@ struct LayerCodes {
     hq_weight_desc split_desc;
     const void* split_w;
 
-    // rows x cols codes whose product has out_rows rows
+    // rows x cols codes whose product has out_rows rows.  The caller has refused a null w_dev: split_w is never null, so the
+    // product's own check no longer sees one.
     LayerCodes(const hq_weight_desc* desc, const void* w_dev, int a_bits, int64_t rows, int64_t cols, int64_t out_rows,
                hq_container cont, void* workspace, size_t ws_bytes)
         : codes(static_cast<unsigned char*>(workspace)),
@@ -160,7 +161,7 @@ extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t 
                                 hq_dtype ydt, int64_t ldy, void* workspace, size_t ws_bytes, int32_t* dev_status,
                                 void* stream) {
     using namespace hq;
-    if (desc == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
+    if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const hq_container cont = hq_container(desc->container);
     size_t need = 0;
@@ -182,7 +183,7 @@ extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64
                                    hq_dtype ydt, int64_t ldy, void* workspace, size_t ws_bytes, int32_t* dev_status,
                                    void* stream) {
     using namespace hq;
-    if (desc == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
+    if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const hq_container cont = hq_container(desc->container);
     size_t need = 0;
@@ -207,7 +208,7 @@ static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split
                                       hq_dtype ydt, void* workspace, size_t ws_bytes, void* scratch, size_t scratch_bytes,
                                       int32_t* dev_status, void* stream) {
     using namespace hq;
-    if (desc == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
+    if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const hq_container cont = hq_container(desc->container);
     const int64_t rows = Nb * H * W;
@@ -262,7 +263,7 @@ extern "C" hq_status hq_gn_qlinear(const void* x, hq_dtype xdt, int64_t Nb, int6
                                    hq_dtype ydt, int64_t ldy, void* workspace, size_t ws_bytes, void* scratch,
                                    size_t scratch_bytes, int32_t* dev_status, void* stream) {
     using namespace hq;
-    if (desc == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
+    if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     if (Nb <= 0 || rows_per_sample <= 0) return HQ_ERR_SHAPE;
     const hq_container cont = hq_container(desc->container);
@@ -288,7 +289,7 @@ static hq_status qconv_impl(const void* x, const void* x2, int64_t split, hq_dty
                               const float* static_scale, void* y, hq_dtype ydt, void* workspace, size_t ws_bytes,
                               int32_t* dev_status, void* stream) {
     using namespace hq;
-    if (desc == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
+    if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
     const hq_container cont = hq_container(desc->container);
     const int64_t rows = Nb * H * W;
@@ -409,7 +410,7 @@ extern "C" hq_status hq_qlinear_noalloc(const void* x, hq_dtype xdt, int64_t M, 
                                         const float* bias, int a_bits, hq_scale_mode mode, const float* static_scale,
                                         void* y, hq_dtype ydt, int64_t ldy, int32_t* dev_status, void* stream) {
     using namespace hq;
-    if (desc == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
+    if (desc == nullptr || w_dev == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     const hq_container cont = hq_container(desc->container);
     size_t need = 0;
     hq_status s = layer_bytes(M, K, cont, &need);

@@ -149,3 +149,26 @@ def test_dit_layer_list():
     assert all(L["K"] % L["had_block"] == 0 and L["had_block"] == 128 for L in layers)
     big = [L for L in layers if L["M"] == 32 * 256]
     assert len(big) == 28 * 4 and {(L["K"], L["N"]) for L in big} == {(1152, 3456), (1152, 1152), (1152, 4608), (4608, 1152)}
+
+
+@pytest.mark.parametrize("had_block", [128, 1024])
+def test_fused_layers_refuse_null_weights_before_a_launch(hq, had_block):
+    """The split fold (blocks of 32 to 512) derives a second address from the weights': a null one has to be refused as it is
+    where the layer runs on the weights alone (block 1024)."""
+    K, N, M = 1152 if had_block == 128 else 2048, 4608, 8192
+    lin = hq.hq_weight_prepare(inputs.weights((N, K), seed=1), 4, had_block, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8)
+    conv = hq.hq_weight_prepare(inputs.weights((256, 3, 3, 1024), seed=1), 4, had_block, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8)
+    assert lin.desc.reserved == conv.desc.reserved == (1 if had_block == 128 else 0)
+    L, d, dc, fake, big = hq.lib, C.byref(lin.desc), C.byref(conv.desc), C.c_void_p(0x1000), 1 << 30
+    assert L.hq_qlinear(fake, 1, M, K, K, d, None, fake, None, 4, 0, None, fake, 1, N, fake, big, None, None) == 1
+    assert L.hq_ln_qlinear(fake, 1, M, K, K, None, None, 0, 1e-6, d, None, fake, None, 4, fake, 1, N, fake, big, None, None) == 1
+    assert L.hq_gn_qlinear(fake, 1, 8, M // 8, K, 32, fake, fake, 1e-5, 0, d, None, fake, None, 4, fake, 1, N, fake, big, fake,
+                           1 << 20, None, None) == 1
+    assert L.hq_qconv(fake, 1, 8, 32, 32, 1024, dc, None, 3, 3, 1, 1, fake, None, 4, 1, fake, fake, 1, fake, big, None, None) == 1
+    assert L.hq_qconv_cat(fake, fake, 0, 1, 8, 32, 32, 1024, dc, None, 3, 3, 1, 1, fake, None, 4, 1, fake, fake, 1, fake, big,
+                          None, None) == 1
+    assert L.hq_gn_silu_qconv(fake, 1, 8, 32, 32, 1024, 32, fake, fake, None, 1e-5, dc, None, 3, 3, 1, 1, fake, None, 4, 1, fake,
+                              fake, 1, fake, big, fake, 1 << 20, None, None) == 1
+    assert L.hq_gn_silu_qconv_cat(fake, fake, 0, 1, 8, 32, 32, 1024, 32, fake, fake, None, 1e-5, dc, None, 3, 3, 1, 1, fake, None, 4,
+                                  1, fake, fake, 1, fake, big, fake, 1 << 20, None, None) == 1
+    assert L.hq_qlinear_noalloc(fake, 1, 1024, K, K, d, None, fake, None, 4, 0, None, fake, 1, N, None, None) == 1
