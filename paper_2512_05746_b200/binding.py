@@ -468,7 +468,17 @@ def hq_qlinear_fused(x, pw: PreparedWeight, bias, a_bits: int, y, static_scale=N
 def hq_set_pair_gemm(mode: int) -> int:
     """Where products run on pairs of SMs (cta_group::2): 0 nowhere, 1 (or True) wherever covered, 2 (the default) where
     it measured faster (streamed weights, convolutions); returns the previous mode."""
+    global _pair_gemm_mode
+    _pair_gemm_mode = min(max(int(mode), 0), 2)
     return int(lib.hq_set_pair_gemm(int(mode)))
+
+
+_pair_gemm_mode = 2
+
+
+def pair_gemm_mode() -> int:
+    """The mode hq_set_pair_gemm set last (launches that are kept, a CUDA graph, belong to the mode they were captured in)."""
+    return _pair_gemm_mode
 
 
 def hq_mma_i8_probe_pair(pairs: int, iters: int, dev_status=None, stream=None) -> None:

@@ -327,6 +327,9 @@ class UNet:
                    out=self.eps_out)
         # one workspace for the codes and scales of whichever quantized layer is running (sized for the largest)
         self.ws = t.empty((self._ws_need,), dtype=t.uint8, device=self.dev)
+        # what the recorded calls read beside the buffers made here: `replay` looks whether it is still what it captured
+        self.layers = list(self.pw.values())
+        self.operands = [*self.f32.values(), *self.bf.values(), *self.static.values()]
         return self
 
     def set_inputs(self, x, t, y):
@@ -352,32 +355,43 @@ class UNet:
         self.torch.cuda.synchronize()
         self.hq.hq_check_status(self.status)
 
+    def _looked_up(self):
+        """Everything the recorded calls look up anew each time they run: a graph of them is what they are as long as this
+        compares equal (about 40 us; a weight put on the device again, another status word or another kernel choice differs)."""
+        tensors = [self.ws, self.scratch, self.status, self.x_in, self.t_in, self.y_in, self.eps_out, *self.operands]
+        for pw in self.layers:
+            tensors += (pw.blob_dev, pw.s_w_dev)
+        tensors = [v for v in tensors if v is not None]
+        return (self.a_bits, self.cont, self.EPS, self.cfg["groups"], self.hq.pair_gemm_mode(), self.ws.nbytes, self.scratch.nbytes,
+                tuple(self.tape), b"".join(pw.desc for pw in self.layers), list(map(self.torch.Tensor.data_ptr, tensors)))
+
     def replay(self):
         """`run()` with its launches kept as a CUDA graph.  The calls of a forward and their buffers are fixed by `build`, and
         at small batches issuing them from the host takes longer than the device needs (2 images: 2.9 ms for 2.4 ms of
-        kernels).  The first forward after a build runs the calls themselves, the second one captures them; a change of
-        `a_bits` starts over.  Inside a caller's own capture, or on another device's stream, the calls run as they are."""
+        kernels).  The first forward after a build runs the calls themselves, the second one captures them; any change of what
+        the calls look up starts over.  Inside a caller's own capture, or with another device current, the calls run as they
+        are."""
         t = self.torch
-        key = (self.a_bits, id(self.tape), len(self.tape), self.ws.data_ptr())
-        elsewhere = t.device(self.dev).index not in (None, t.cuda.current_device())
-        if elsewhere or self.calibrating or t.cuda.is_current_stream_capturing():
+        if self.calibrating or self.ws.device.index != t.cuda.current_device() or t.cuda.is_current_stream_capturing():
             self.run()
-        elif self.graph_key != key:
+            return
+        key = self._looked_up()
+        if self.graph_key != key:
             self.run()
             self.graph, self.graph_key = None, key
-        else:
-            if self.graph is None:
-                graph, stream = t.cuda.CUDAGraph(), t.cuda.Stream()
-                stream.wait_stream(t.cuda.current_stream())
-                with t.cuda.stream(stream):
-                    graph.capture_begin(capture_error_mode="thread_local")
-                    try:
-                        self.run()
-                    finally:
-                        graph.capture_end()
-                t.cuda.current_stream().wait_stream(stream)
-                self.graph = graph
-            self.graph.replay()
+            return
+        if self.graph is None:
+            graph, stream = t.cuda.CUDAGraph(), t.cuda.Stream()
+            stream.wait_stream(t.cuda.current_stream())
+            with t.cuda.stream(stream):
+                graph.capture_begin(capture_error_mode="thread_local")
+                try:
+                    self.run()
+                finally:
+                    graph.capture_end()
+            t.cuda.current_stream().wait_stream(stream)
+            self.graph = graph
+        self.graph.replay()
 
     def forward(self, x, t, y, record=None):
         """eps [Nb, S, S, in_ch] fp32.  record: a list that receives, per library call, its name and copies of the tensors

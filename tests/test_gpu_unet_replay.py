@@ -47,3 +47,39 @@ def test_forward_by_graph_is_the_forward_by_calls():
     got = out.clone()
     assert torch.equal(got, by_calls(args))
     hq.hq_check_status(net.status)
+
+
+def test_forward_follows_replaced_weights_status_and_kernel_choice():
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    from paper_2512_05746_b200.unet import UNet
+    cfg = inputs.unet_config(batch=2, latent=32, base=128, attn_resolutions=(16, 8, 4), had_block=128, classes=10)
+    net = UNet(cfg, inputs.unet_params(cfg, seed=0), hq, torch.device("cuda")).build(2)
+    I = inputs.unet_inputs(cfg, seed=0)
+    args = [torch.from_numpy(I[k]) for k in ("x", "t", "y")]
+    net.calibrate(*args)
+    for _ in range(3):
+        net.forward(*args)
+    first = net.forward(*args).clone()
+    pw, graph = net.pw["mid.attn.qkv"], net.graph
+    assert graph is not None
+    kept = pw.blob_dev, pw.s_w_dev, net.status               # their addresses are not handed out again
+    pw.to_device()
+    pw.blob_dev.zero_()                                      # other weights at another address
+    want = net.forward(*args, record=[]).clone()
+    assert not torch.equal(want, first)
+    for _ in range(3):
+        assert torch.equal(net.forward(*args), want)
+    assert net.graph is not graph
+    net.status = torch.zeros_like(net.status)
+    for _ in range(3):
+        assert torch.equal(net.forward(*args), want)
+    hq.hq_check_status(net.status)
+    graph, before = net.graph, hq.hq_set_pair_gemm(0)
+    try:
+        for _ in range(3):
+            assert torch.equal(net.forward(*args), want)
+        assert net.graph is not graph
+    finally:
+        hq.hq_set_pair_gemm(before)
+    del kept
