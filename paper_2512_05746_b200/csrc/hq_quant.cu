@@ -1019,20 +1019,40 @@ hq_status launch_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, 
                              nullptr, st, nullptr, &sp, zo);
 }
 
+// The one-wave statistics kernel: pixels per CTA (four CTAs per SM share the pixels of all samples evenly, in whole rounds of
+// loads; small tensors get fewer CTAs so that a thread still walks a round of eight pixels) and their number.
+static int64_t gn_wave_span(int64_t Nb, int64_t hw, int64_t C, int vec) {
+    const int64_t pieces = C / vec, round = 8 * (pieces < 256 ? 256 / pieces : 1), ctas = int64_t(sm_count()) * 4;
+    return ((Nb * hw + ctas - 1) / ctas + round - 1) / round * round;
+}
+static int64_t gn_wave_ctas(int64_t Nb, int64_t hw, int64_t C, int vec) {
+    const int64_t span = gn_wave_span(Nb, hw, C, vec);
+    return (Nb * hw + span - 1) / span;
+}
+
 // Groups per CTA of the slab kernel, or 0: the one-wave kernel takes the tensor (groups of more than 256 pieces, more samples
-// than one wave of CTAs).  The fewest groups for which the CTAs fit one wave of four per SM.  On tensors of more than 20 MB,
-// where bandwidth counts and not the latency of atomics, only if the run fills whole sectors of a pixel and the threads of a
-// piece share its sets evenly.  Statistics + transform, one-wave / slab: 2 x 32 x 32 x 512 13.7 / 6.7 us, 8 x 8 x 8 x 1024
-// 8.9 / 8.8, 64 x 32 x 32 x 512 56.8 / 55.0; not taken: 16 x 64 x 64 x 256 29.7 / 31.2 (half sectors), 64 x 16 x 16 x 768
-// 27.7 / 28.8 (32 sets over 21 threads).
+// than one wave of CTAs).  The fewest groups for which the CTAs fit one wave of four per SM.  Both sides are estimated, in us
+// over what they share.  A slab CTA walks its pixels in rounds of eight loads per thread, 0.85 us each however few CTAs there
+// are, and 1.4 times that where its run fills half sectors only.  The one-wave kernel spreads the bytes over the whole chip, but
+// its CTAs add their sums to one address per group in turn (20 ns each), behind a memset.  On tensors of more than 20 MB
+// bandwidth counts and not the latency of atomics: there the slabs also have to fill whole sectors, share the sets of a piece
+// evenly and be short.  Statistics + transform, one-wave / slab: 2 x 32 x 32 x 512 14.5 / 7.8 us, 1 x 64 x 64 x 512 18.5 / 11.1,
+// 1 x 64 x 64 x 2048 90 / 31, 64 x 32 x 32 x 512 56.8 / 55.0; not taken: 1 x 128 x 128 x 1024 63 / 52 from L2 but 66 / 83 from
+// memory, 1 x 256 x 256 x 512 66 / 162, 1 x 512 x 512 x 512 201 / 665, 16 x 64 x 64 x 256 29.7 / 31.2 (half sectors),
+// 64 x 16 x 16 x 768 27.7 / 28.8 (32 sets over 21 threads), one group of 256 channels on 1 x 64 x 64 18.6 / 61.
 static int gn_slab_run(int64_t Nb, int64_t hw, int64_t C, int groups, int elt, int vec) {
     const int64_t cg = C / groups;
     for (int run = 1; run <= groups && run <= 256; ++run) {
         if (groups % run != 0 || (run * cg) % vec != 0 || run * cg / vec > 256) continue;
         if (Nb * (groups / run) > int64_t(sm_count()) * 4) continue;
-        const int64_t sets = (hw + 7) / 8, lanes = 256 / (run * cg / vec);
-        const bool even = 10 * sets >= 8 * lanes * ((sets + lanes - 1) / lanes);
-        return Nb * hw * C * elt <= 20000000 || (even && run * cg * elt >= 32) ? run : 0;
+        const int64_t bytes = Nb * hw * C * elt, sets = (hw + 7) / 8, lanes = 256 / (run * cg / vec);
+        const int64_t rounds = (sets + lanes - 1) / lanes;
+        const bool full = run * cg * elt >= 32, even = 10 * sets >= 8 * lanes * rounds;
+        const int64_t per_sample = gn_wave_ctas(Nb, hw, C, vec) / Nb, adds = (per_sample > 1 ? per_sample : 1) * (cg > vec ? cg / vec : 1);
+        const double slab = (full ? 0.85 : 1.2) * double(rounds);
+        const double wave = 5.0 + 0.02 * double(adds) + 0.3 * (bytes < 20000000 ? double(bytes) * 1e-6 : 20.0);
+        const bool streams = full && even && (hw <= 4096 || bytes <= 40000000);
+        return slab < wave && (bytes <= 20000000 || streams) ? run : 0;
     }
     return 0;
 }
@@ -1079,14 +1099,8 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
         return HQ_OK;
     }
     HQ_CUDA_OK(cudaMemsetAsync(scratch, 0, need, st));             // the sums and the ticket counters
-    // one wave of CTAs (four per SM) that share the pixels of all samples evenly, in whole rounds of loads; small
-    // tensors get fewer CTAs so that a thread still walks a round of eight pixels
-    const int64_t total_px = Nb * hw;
-    const int64_t round = ppl * 8;
-    int64_t ctas = int64_t(sm_count()) * 4;
-    int64_t span = ((total_px + ctas - 1) / ctas + round - 1) / round * round;
-    ctas = (total_px + span - 1) / span;
-    const unsigned grid = unsigned(ctas);
+    const int64_t total_px = Nb * hw, span = gn_wave_span(Nb, hw, C, wide ? 8 : 4);
+    const unsigned grid = unsigned(gn_wave_ctas(Nb, hw, C, wide ? 8 : 4));
     if (xdt == HQ_F32)
         gn_stats_kernel<float, 4><<<grid, 256, 0, st>>>(static_cast<const float*>(x), static_cast<const float*>(x2), int(split), pre, hw, total_px, span, int(C), groups, sums,
                                                        stats, inv_count, double(eps));

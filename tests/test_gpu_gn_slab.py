@@ -46,3 +46,28 @@ def test_gn_statistics_of_a_run_of_groups(oracle, Nb, H, W, C, G, n, dt, c1):
     s = scales.view(Nb, H * W)[pick].reshape(-1).cpu().numpy()
     assert float(np.abs(s / s_ref - 1.0).max()) <= 1e-6
     check_codes(q, q_ref, v, f"groupnorm runs {Nb}x{H}x{W}x{C}", tie_rel=1e-6, mismatch_frac=1e-4)
+
+
+@pytest.mark.parametrize("Nb,H,W,C,G,slab", [
+    (2, 32, 32, 512, 32, True),         # 32 pixel rows on 64 CTAs
+    (1, 64, 64, 2048, 32, True),        # long runs, but the one-wave kernel's sums meet at 32 addresses
+    (1, 256, 256, 128, 32, False),      # 16 CTAs of 65536 pixels each
+    (1, 64, 64, 256, 1, False),         # one group: one CTA for the whole image
+    (1, 160, 256, 512, 32, False),      # 42 MB on 32 CTAs
+])
+def test_few_large_samples_are_not_left_to_a_few_ctas(Nb, H, W, C, G, slab):
+    """Which kernel took the statistics shows in the scratch: the one with a CTA per run of groups keeps its fp64 sums to itself."""
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    x = (torch.randn((Nb, H, W, C), generator=gen, device="cuda") + 0.5).to(torch.bfloat16)
+    gamma, beta = torch.randn((C,), generator=gen, device="cuda"), torch.randn((C,), generator=gen, device="cuda")
+    scratch = torch.full((Nb * G * 24,), 0xFF, dtype=torch.uint8, device="cuda")
+    out = torch.zeros_like(x)
+    hq.hq_groupnorm_act(x, G, gamma, beta, 1e-5, False, out, scratch)
+    assert bool((scratch[: Nb * G * 16] == 0xFF).all()) == slab
+    v = x.double().view(Nb, H * W, G, C // G)
+    want = (v - v.mean(dim=(1, 3), keepdim=True)) * (v.var(dim=(1, 3), unbiased=False, keepdim=True) + 1e-5).rsqrt()
+    want = want.view(Nb, H, W, C) * gamma.double() + beta.double()
+    # one bf16 rounding (2^-9 relative) of an fp32 value that a few roundings at the size of its terms (at most 6 |gamma|) moved
+    assert bool(((out.double() - want).abs() <= want.abs() * 2.0 ** -8 + 6 * gamma.double().abs() * 2.0 ** -20).all())
