@@ -53,6 +53,7 @@ struct QuantParams {
     int gn_cg_shift;
     // optional LayerNorm over each row with a per-sample affine, applied before the transform (ln_on != 0)
     int ln_on;
+    int ln_table;            // the affine vectors go through shared memory
     const float* ln_w;       // [groups][cols] or nullptr (= 1)
     const float* ln_b;       // [groups][cols] or nullptr (= 0)
     int64_t ln_rows_per_group;   // rows that share one affine vector pair; 0: all rows
@@ -73,9 +74,10 @@ __device__ __forceinline__ f32x2 silu2(f32x2 y) {
     return mul2(y, pk2(rcp_ftz(d0), rcp_ftz(d1)));
 }
 
-// Asynchronous 16-byte copies global -> shared.
+// Asynchronous 16-byte copies global -> shared, kept in L1: the CTAs of an SM copy the same vectors (with `.cg` the lines that all
+// CTAs ask L2 for at once made 16384 x 768 with one affine for all rows 22.6 instead of 17.4 us).
 __device__ __forceinline__ void cp_async_16(void* smem, const void* gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem)), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -107,18 +109,20 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
 //            KLOG = 12 needs one more stage than fits and takes it with a lane exchange.
 // Dynamic scales never need the clamp (|t| * qmax / max|t| rounds to at most qmax); static scales do.
 // PRO: prologue applied to the values before the transform: 0 none, 1 GroupNorm + SiLU (statistics given), 2 LayerNorm
-// over the row (statistics taken here: the row is in the registers of its threads) with a per-sample affine, 3 GroupNorm
-// alone (the normalisation in front of an attention block's QKV projection).
+// over the row (statistics taken here: the row is in the registers of its threads) with a per-sample affine copied into shared
+// memory, 3 GroupNorm alone (the normalisation in front of an attention block's QKV projection), 4 LayerNorm that reads the affine
+// vectors where it uses them (ln_table says which of the two a launch takes).
 // Blocks per SM the registers are bounded for: three for LayerNorm on 32 values (64 registers; unbounded 26 us on 8192 x 1152,
 // two 18.4, three 15.8, four 18.2); none stated for the GroupNorm prologues (56 registers; stating one lets the compiler take
 // 84, 2.1 ms instead of 1.8 for the 44 launches of a UNet forward at batch 64); one for the plain transform (level at 256 and
 // 512 channels, 60.9 -> 54.7 us on 65536 x 1152).
-__host__ __device__ constexpr int quant_min_blocks(int pro, int e) { return pro == 2 && e == 32 ? 3 : (pro == 0 ? 1 : 0); }
+__host__ __device__ constexpr int quant_min_blocks(int pro, int e) { return (pro == 2 || pro == 4) && e == 32 ? 3 : (pro == 0 ? 1 : 0); }
 template <int KLOG, int E, typename InT, bool INT8_OUT, bool STATIC, int PRO>
 __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast(const QuantParams p) {
     constexpr bool GN = PRO == 1 || PRO == 3;          // 3: GroupNorm without the SiLU
     constexpr bool GN_SILU = PRO == 1;
-    constexpr bool LN = PRO == 2;
+    constexpr bool LN = PRO == 2 || PRO == 4;
+    constexpr bool LN_TABLE = PRO == 2;
     griddep_launch();      // a GEMM launched as a programmatic dependent may start its prologue as this grid drains
     constexpr int N = 1 << KLOG;
     constexpr int LE = ilog2_c(E);
@@ -148,8 +152,8 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     // sample the CTA's rows belong to (the host makes sure a CTA never straddles two samples), then y * sigmoid(y).
     float* gn_a = reinterpret_cast<float*>(rowmax + ((p.rows_per_cta + 3) & ~3));
     float* gn_b = gn_a + p.cols;
-    // LayerNorm prologue: the row sums' parts ([2][threads]) and the affine vectors of the CTA's sample ([2][cols], a slot
-    // of 64 bytes after every 128 channels so that neighbouring Hadamard blocks start in different banks).
+    // LayerNorm prologue: the row sums' parts ([2][threads]) and, with LN_TABLE, the affine vectors of the CTA's sample ([2][cols],
+    // a slot of 64 bytes after every 128 channels so that neighbouring Hadamard blocks start in different banks).
     float* ln_part = gn_a;
     float4* ln_tab = reinterpret_cast<float4*>(ln_part + 2 * blockDim.x);
     const int ln_slots = ln_tab_slots(int(p.cols));
@@ -167,17 +171,16 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) cur[i] = __ldcs(reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i)));
     }
-    if (LN) {
-        // The affine vectors are copied asynchronously while the row statistics are taken.  Read from L2 where they are
-        // used, 16 loads per thread behind the second barrier, they made this latency-bound prologue twice as long.
-        const int64_t g = p.ln_rows_per_group > 0 ? (int64_t(blockIdx.x) * p.rows_per_cta) / p.ln_rows_per_group : 0;
+    const int64_t ln_group = LN && p.ln_rows_per_group > 0 ? (int64_t(blockIdx.x) * p.rows_per_cta) / p.ln_rows_per_group : 0;
+    if (LN_TABLE) {
+        // The affine vectors are copied asynchronously while the row statistics are taken.
         const int quads = int(p.cols) / 4;
         for (int f = tid; f < 2 * quads; f += blockDim.x) {
             const bool is_b = f >= quads;
             const int c4 = is_b ? f - quads : f;
             const float* src = is_b ? p.ln_b : p.ln_w;
             float4* dst = ln_tab + (is_b ? ln_slots : 0) + ln_slot(c4);
-            if (src != nullptr) cp_async_16(dst, src + g * p.cols + 4 * c4);
+            if (src != nullptr) cp_async_16(dst, src + ln_group * p.cols + 4 * c4);
             else *dst = is_b ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(1.f, 1.f, 1.f, 1.f);
         }
     }
@@ -254,14 +257,24 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
 #pragma unroll
         for (int i = 0; i < P; ++i) { v[i] = sub2(v[i], mean2); acc = fma2(v[i], v[i], acc); }
         upk2(acc, lo, hi);
-        cp_async_wait_all();                           // this thread's pieces of the table; the barrier covers the others'
+        if (LN_TABLE) cp_async_wait_all();             // this thread's pieces of the table; the barrier covers the others'
         const float rstd = rsqrtf(row_sum(lo + hi, ln_part + blockDim.x) / float(p.cols) + p.ln_eps);
         const f32x2 rstd2 = pk2(rstd, rstd);
         const float4* tab_w = ln_tab + ln_slot(blk * (N / 4)) + ln_slot(tb);
+        const float* wrow = p.ln_w != nullptr ? p.ln_w + ln_group * p.cols : nullptr;
+        const float* brow = p.ln_b != nullptr ? p.ln_b + ln_group * p.cols : nullptr;
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) {
             // slot of channel quad blk N/4 + tb + TB i: the three parts never carry into one another's group of 32 quads
-            const float4 a4 = tab_w[ln_slot(TB * i)], b4 = tab_w[ln_slots + ln_slot(TB * i)];
+            float4 a4 = make_float4(1.f, 1.f, 1.f, 1.f), b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (LN_TABLE) {
+                a4 = tab_w[ln_slot(TB * i)];
+                b4 = tab_w[ln_slots + ln_slot(TB * i)];
+            } else {
+                const int ch = blk * N + 4 * (tb + TB * i);
+                if (wrow != nullptr) a4 = __ldg(reinterpret_cast<const float4*>(wrow + ch));
+                if (brow != nullptr) b4 = __ldg(reinterpret_cast<const float4*>(brow + ch));
+            }
             v[2 * i] = fma2(mul2(v[2 * i], rstd2), pk2(a4.x, a4.y), pk2(b4.x, b4.y));
             v[2 * i + 1] = fma2(mul2(v[2 * i + 1], rstd2), pk2(a4.z, a4.w), pk2(b4.z, b4.w));
         }
@@ -856,6 +869,10 @@ cudaError_t launch_fast(const QuantParams& p, bool int8_out, int grid, int threa
         if (int8_out) return stat ? go(fwht_quant_fast<KLOG, E, InT, true, true, 3>) : go(fwht_quant_fast<KLOG, E, InT, true, false, 3>);
         return stat ? go(fwht_quant_fast<KLOG, E, InT, false, true, 3>) : go(fwht_quant_fast<KLOG, E, InT, false, false, 3>);
     }
+    if (p.ln_on && !p.ln_table) {
+        if (int8_out) return stat ? go(fwht_quant_fast<KLOG, E, InT, true, true, 4>) : go(fwht_quant_fast<KLOG, E, InT, true, false, 4>);
+        return stat ? go(fwht_quant_fast<KLOG, E, InT, false, true, 4>) : go(fwht_quant_fast<KLOG, E, InT, false, false, 4>);
+    }
     if (p.ln_on) {
         if (int8_out) return stat ? go(fwht_quant_fast<KLOG, E, InT, true, true, 2>) : go(fwht_quant_fast<KLOG, E, InT, true, false, 2>);
         return stat ? go(fwht_quant_fast<KLOG, E, InT, false, true, 2>) : go(fwht_quant_fast<KLOG, E, InT, false, false, 2>);
@@ -891,6 +908,18 @@ struct GnArgs { const float* stats; const float* gamma; const float* beta; int g
 struct LnArgs { const float* w; const float* b; int64_t rows_per_group; float eps; };
 
 struct SplitArgs { const void* x2; int64_t split, ldx2; };
+
+// Whether the LayerNorm prologue copies its affine vectors into shared memory (`with`: bytes a CTA takes then) or reads them from
+// L1 / L2 behind the second barrier.  The copy hides their latency, but at wide rows it costs resident CTAs: taken where the SM
+// holds as many CTAs as by registers (64 a thread, 128 on 64 values), or where every CTA has an SM to itself.  Without affine
+// vectors there is nothing to copy.  Copied / read, bf16, one affine per 256 rows: 16384 x 1152 28.3 / 30.0 us, 16384 x 768 17.5 /
+// 18.0, 65536 x 2304 212 / 238, 256 x 2048 4.1 / 4.4; read: 16384 x 1536 39 / 31, 16384 x 2048 50 / 41, 16384 x 4096 133 / 84,
+// 16384 x 8192 (block 4096) 347 / 222, and without vectors 16384 x 1152 28.1 / 25.8, 16384 x 8192 336 / 167.
+static bool ln_table(const LnArgs& ln, int64_t grid, int threads, int E, size_t with) {
+    if (ln.w == nullptr && ln.b == nullptr) return false;
+    if (with > 227 * 1024) return false;
+    return grid <= sm_count() || 228 * 1024 / (with + 1024) >= size_t(65536 / ((E == 32 ? 64 : 128) * threads));
+}
 
 static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, int64_t cols, int64_t ldx, int had_block,
                                    int bits, hq_scale_mode mode, const float* static_scale, void* codes,
@@ -967,10 +996,14 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         if (threads <= 320) {                               // otherwise the generic kernel below takes the row shape
         // exchange buffer: per Hadamard block n/4 float4 slots plus one slot of padding per J (J = E/2 or E/4)
         const int jslots = (klog - ilog2(E) >= ilog2(E) - 1) ? E / 2 : E / 4;
-        const size_t smem = size_t(threads / (n / E)) * size_t(n / 4 + n / 4 / jslots) * 16 + size_t((rpc + 3) & ~3) * 4 +
-                            (gn != nullptr ? size_t(cols) * 8 : 0) +
-                            (ln != nullptr ? size_t(2 * threads) * 4 + size_t(2 * ln_tab_slots(int(cols))) * 16 : 0);
+        size_t smem = size_t(threads / (n / E)) * size_t(n / 4 + n / 4 / jslots) * 16 + size_t((rpc + 3) & ~3) * 4 +
+                      (gn != nullptr ? size_t(cols) * 8 : 0) + (ln != nullptr ? size_t(2 * threads) * 4 : 0);
         const int grid = int((rows + rpc - 1) / rpc);
+        if (ln != nullptr) {
+            const size_t table = size_t(2 * ln_tab_slots(int(cols))) * 16;
+            p.ln_table = ln_table(*ln, grid, threads, E, smem + table);
+            if (p.ln_table) smem += table;
+        }
         if (zo != nullptr && zo->z != nullptr && split_block_ok(klog) && split_fits(klog, bits)) {
             p.z = zo->z; p.ld_z = zo->ld;
             zo->written = true;

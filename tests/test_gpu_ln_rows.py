@@ -43,3 +43,16 @@ def test_ln_row_statistics(oracle, rows, cols, n, rpg, dt, with_w, with_b):
     # the statistics and the transform in fp32 move a scale by a few units of 2^-24, as in the other prologue tests
     assert float(np.abs(out[0][1].cpu().numpy() / s_ref - 1.0).max()) <= 1e-6
     check_codes(out[0][0].cpu().numpy().view(np.int8), q_ref, v, f"layernorm rows {rows}x{cols}", tie_rel=1e-6, mismatch_frac=1e-4)
+
+
+@pytest.mark.parametrize("rows,cols,n,rpg,dt,with_w,with_b", [
+    (1024, 1536, 256, 256, "bf16", True, True),     # two CTAs fewer per SM with a table
+    (1024, 4096, 128, 0, "f32", True, True),        # one affine for all rows
+    (304, 8192, 4096, 16, "bf16", True, False),     # 64 values a thread, no addend
+    (160, 16384, 512 * 8, 0, "f32", False, True),   # the widest row, no factor
+    (4096, 1152, 128, 0, "bf16", False, False),     # neither vector
+    (321, 96, 32, 0, "f32", False, False),
+])
+def test_ln_affine_read_where_it_is_used(oracle, rows, cols, n, rpg, dt, with_w, with_b):
+    """Rows whose table of affine vectors would cost resident CTAs, and rows without any."""
+    test_ln_row_statistics(oracle, rows, cols, n, rpg, dt, with_w, with_b)
