@@ -152,14 +152,23 @@ hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t
 
 /* ---- Fused layer: transform -> quantize -> integer product -> rescale in one call (Eq. 12 / Eq. 14). ----
  * Codes and scales live in `workspace` (device, hq_workspace_size bytes); the code container is desc->container.
- * hq_workspace_size: codes (row pitch rounded up to 16 bytes), then the scales at the next multiple of 256; if that is
- * more than HQ_NOALLOC_SCRATCH_BYTES, also rows * cols bytes for the split-fold codes.  A workspace that holds only codes
- * and scales is enough for every layer: the product then runs on the two-limb weights, with the same results.
+ * The workspace holds the codes (row pitch rounded up to 16 bytes), the scales at the next multiple of 256, and behind them,
+ * at the next multiple of 256, room for the split-fold codes (rows of C bytes, pitch rounded up to 16) of a layer that runs
+ * faster on the one-limb weights.  Codes and scales alone are enough for every layer: the product then runs on the
+ * two-limb weights, with the same results.
+ *  hq_workspace_size knows the shape only: codes and scales, and where these take more than HQ_NOALLOC_SCRATCH_BYTES the
+ *    room too, whether the layer has a use for it or not (up to that size it stays the figure by which
+ *    hq_qlinear_noalloc takes a layer).
+ *  hq_layer_workspace_size knows the layer (weights, width of the codes, one static scale or one per row, stride; rows of
+ *    its input: M or Nb * H * W) and asks for the room at any size, and only where the layer then uses it.  On the current
+ *    device: the choice depends on its number of SMs.
  * alpha is derived from the descriptor.  y pitch ldy elements.
  * The product kernel is launched so that it may begin (set-up, first weight tile) while the transform kernel is still
  * running; it waits for the transform before it touches codes or activation scales.  Work enqueued on the stream before
  * the call has completed before either kernel starts, as usual. */
 hq_status hq_workspace_size(int64_t rows, int64_t cols, hq_container cont, size_t* bytes);
+hq_status hq_layer_workspace_size(const hq_weight_desc* desc, int a_bits, hq_scale_mode mode, int64_t rows, int stride,
+                                  size_t* bytes);
 hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc,
                      const void* w_dev, const float* scale_w, const float* bias, int a_bits, hq_scale_mode mode,
                      const float* static_scale, void* y, hq_dtype ydt, int64_t ldy, void* workspace,

@@ -23,7 +23,7 @@ HQ_W_PLAIN, HQ_W_FOLDED, HQ_W_DOUBLE, HQ_W_PLAIN_A2 = 0, 1, 2, 3
 WEIGHT_MODES = {"plain": HQ_W_PLAIN, "folded": HQ_W_FOLDED, "double": HQ_W_DOUBLE, "plain_a2": HQ_W_PLAIN_A2}
 
 EXPORTS = ["hq_version", "hq_status_string", "hq_check_status", "hq_hadamard_quant", "hq_weight_blob_bytes",
-           "hq_weight_prepare", "hq_qgemm", "hq_qconv2d", "hq_workspace_size", "hq_qlinear", "hq_qconv",
+           "hq_weight_prepare", "hq_qgemm", "hq_qconv2d", "hq_workspace_size", "hq_layer_workspace_size", "hq_qlinear", "hq_qconv",
            "hq_alpha_for", "hq_mma_i8_probe", "hq_qlinear_noalloc", "hq_hadamard_quant_width", "hq_qconv_width", "hq_gn_silu_quant",
            "hq_ln_quant", "hq_ln_qlinear", "hq_gn_silu_qconv", "hq_gn_qlinear", "hq_silu", "hq_add", "hq_add_rows_bcast",
            "hq_class_embed_add", "hq_timestep_embedding", "hq_upsample_nearest2x", "hq_concat_channels", "hq_groupnorm_act",
@@ -65,6 +65,7 @@ def _load():
     L.hq_qconv2d.argtypes = [p, i32, i32, i64, i64, i64, i64, C.POINTER(WeightDesc), p, i32, i32, i32, i32, p, i32,
                              p, p, C.c_float, p, p, i32, p, p]
     L.hq_workspace_size.argtypes = [i64, i64, i32, C.POINTER(C.c_size_t)]
+    L.hq_layer_workspace_size.argtypes = [C.POINTER(WeightDesc), i32, i32, i64, i32, C.POINTER(C.c_size_t)]
     L.hq_qlinear.argtypes = [p, i32, i64, i64, i64, C.POINTER(WeightDesc), p, p, p, i32, i32, p, p, i32, i64, p,
                              C.c_size_t, p, p]
     L.hq_qconv.argtypes = [p, i32, i64, i64, i64, i64, C.POINTER(WeightDesc), p, i32, i32, i32, i32, p, p, i32, i32,
@@ -112,7 +113,7 @@ def _load():
     L.hq_alpha_for.argtypes = [C.POINTER(WeightDesc)]
     L.hq_mma_i8_probe.argtypes = [i32, i32, p, p]
     for name in ("hq_check_status", "hq_hadamard_quant", "hq_weight_prepare", "hq_qgemm", "hq_qconv2d",
-                 "hq_workspace_size", "hq_qlinear", "hq_qconv", "hq_mma_i8_probe", "hq_qlinear_noalloc",
+                 "hq_workspace_size", "hq_layer_workspace_size", "hq_qlinear", "hq_qconv", "hq_mma_i8_probe", "hq_qlinear_noalloc",
                  "hq_hadamard_quant_width", "hq_qconv_width", "hq_gn_silu_quant", "hq_ln_quant", "hq_ln_qlinear", "hq_gn_silu_qconv",
                  "hq_gn_qlinear", "hq_silu", "hq_add", "hq_add_rows_bcast", "hq_class_embed_add", "hq_timestep_embedding",
                  "hq_upsample_nearest2x", "hq_concat_channels", "hq_groupnorm_act", "hq_conv2d_direct", "hq_attention",
@@ -254,6 +255,15 @@ def hq_qconv2d(a_codes, container: int, a_bits: int, Nb: int, H: int, W: int, Ci
 def hq_workspace_size(rows: int, cols: int, container: int) -> int:
     out = C.c_size_t(0)
     _check(lib.hq_workspace_size(rows, cols, container, C.byref(out)), "hq_workspace_size")
+    return int(out.value)
+
+
+def hq_layer_workspace_size(pw: PreparedWeight, a_bits: int, rows: int, static: bool = False, stride: int = 1) -> int:
+    """Bytes a fused call of this layer makes use of: codes and scales, and room for the split-fold codes where it runs on the
+    one-limb weights then.  rows: M, or Nb * H * W of the input; static: one activation scale for the whole tensor."""
+    out = C.c_size_t(0)
+    _check(lib.hq_layer_workspace_size(C.byref(pw.desc), a_bits, HQ_SCALE_STATIC if static else HQ_SCALE_PER_ROW, rows, stride,
+                                       C.byref(out)), "hq_layer_workspace_size")
     return int(out.value)
 
 

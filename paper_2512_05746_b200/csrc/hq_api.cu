@@ -81,14 +81,13 @@ struct LayerCodes {
     hq_weight_desc split_desc;
     const void* split_w;
 
-    // rows x cols codes whose product has out_rows rows.  The caller has refused a null w_dev: split_w is never null, so the
-    // product's own check no longer sees one.
-    LayerCodes(const hq_weight_desc* desc, const void* w_dev, int a_bits, int64_t rows, int64_t cols, int64_t out_rows,
+    // rows x cols codes.  The caller has refused a null w_dev: split_w is never null, so the product's own check no longer
+    // sees one.
+    LayerCodes(const hq_weight_desc* desc, const void* w_dev, int a_bits, hq_scale_mode mode, int64_t rows, int64_t cols, int stride,
                hq_container cont, void* workspace, size_t ws_bytes)
         : codes(static_cast<unsigned char*>(workspace)),
           scales(reinterpret_cast<float*>(codes + scales_offset(rows, cols, cont))), ld(code_pitch(cols, cont)) {
-        if (ws_bytes >= size_t(split_bytes(rows, cols, cont)) && split_applies(desc, a_bits, cols) &&
-            split_pays(desc, rows, cols, out_rows)) {
+        if (ws_bytes >= size_t(split_bytes(rows, cols, cont)) && split_taken(desc, a_bits, mode, rows, cols, stride)) {
             z.z = codes + split_offset(rows, cols, cont);
             z.ld = code_pitch(cols, HQ_CODES_INT8);
             split_desc = *desc;
@@ -96,6 +95,11 @@ struct LayerCodes {
             split_desc.container = HQ_CODES_INT8;
             split_w = static_cast<const unsigned char*>(w_dev) + desc->N_pad * 2 * desc->RS * desc->C_pad;
         }
+    }
+    // Per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb.
+    static bool split_taken(const hq_weight_desc* desc, int a_bits, hq_scale_mode mode, int64_t rows, int64_t cols, int stride) {
+        return (mode == HQ_SCALE_STATIC || desc->RS == 1) && split_applies(desc, a_bits, cols) &&
+               split_pays(desc, rows, cols, rows / (stride == 2 ? 4 : 1));
     }
     static bool split_applies(const hq_weight_desc* desc, int a_bits, int64_t cols) {
         if (desc->reserved != kBlobHasSplit || desc->limbs != 2 || desc->C != cols) return false;
@@ -148,10 +152,27 @@ extern "C" hq_status hq_workspace_size(int64_t rows, int64_t cols, hq_container 
     if (bytes == nullptr) return HQ_ERR_INVALID_ARG;
     if (cont != HQ_CODES_NIBBLE && cont != HQ_CODES_INT8) return HQ_ERR_INVALID_ARG;
     if (rows < 0 || cols <= 0) return HQ_ERR_SHAPE;
-    // Codes and scales.  Layers beyond HQ_NOALLOC_SCRATCH_BYTES also get room for the split-fold codes; smaller ones hold
-    // too few tiles to gain from one-limb weights and keep the size at which the no-allocation entry point takes them.
+    // Codes and scales; beyond HQ_NOALLOC_SCRATCH_BYTES also room for the split-fold codes, since the shape does not say
+    // whether the layer has a use for it.  Smaller layers gain from it as well (4096 x 1152 -> 4608 30.7 / 24.5 us), but for
+    // them this is the size at which the no-allocation entry point takes a layer: they ask hq_layer_workspace_size.
     *bytes = size_t(hq::codes_bytes(rows, cols, cont));
     if (*bytes > size_t(HQ_NOALLOC_SCRATCH_BYTES)) *bytes = size_t(hq::split_bytes(rows, cols, cont));
+    return HQ_OK;
+}
+
+// Two limbs / one, whole layer: 1024 x 1152 -> 4608 12.7 / 11.3 us, 4096 x 1152 -> 4608 30.7 / 24.5, 7000 x 1024 -> 4096 41.6 / 35.3,
+// 16 x 16 x 16 x 768 3x3 38.5 / 21.6, 15 x 32 x 32 x 512 3x3 51.4 / 33.2, 64 x 8 x 8 x 1024 3x3 48.7 / 30.4.
+extern "C" hq_status hq_layer_workspace_size(const hq_weight_desc* desc, int a_bits, hq_scale_mode mode, int64_t rows, int stride,
+                                             size_t* bytes) {
+    using namespace hq;
+    if (desc == nullptr || bytes == nullptr) return HQ_ERR_INVALID_ARG;
+    if (mode != HQ_SCALE_PER_ROW && mode != HQ_SCALE_STATIC) return HQ_ERR_INVALID_ARG;
+    if (a_bits != 3 && a_bits != 4 && a_bits != 8) return HQ_ERR_INVALID_ARG;
+    if (stride != 1 && stride != 2) return HQ_ERR_UNSUPPORTED;
+    const hq_container cont = hq_container(desc->container);
+    const hq_status s = layer_bytes(rows, desc->C, cont, bytes);
+    if (s != HQ_OK) return s;
+    if (LayerCodes::split_taken(desc, a_bits, mode, rows, desc->C, stride)) *bytes = size_t(split_bytes(rows, desc->C, cont));
     return HQ_OK;
 }
 
@@ -169,7 +190,7 @@ extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t 
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, M, K, M, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, workspace, ws_bytes);
     s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
                               &lc.z);
     if (s != HQ_OK) return s;
@@ -191,7 +212,7 @@ extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, M, K, M, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, K, 1, cont, workspace, ws_bytes);
     s = launch_ln_quant(x, xdt, M, K, ldx, ln_weight, ln_bias, rows_per_group, eps, desc->had_block, a_bits, HQ_SCALE_PER_ROW,
                         nullptr, lc.codes, cont, lc.ld, lc.scales, st, &lc.z);
     if (s != HQ_OK) return s;
@@ -219,9 +240,7 @@ static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb
-    LayerCodes lc(desc, w_dev, a_bits, rows, C, rows / (stride == 2 ? 4 : 1), cont, workspace,
-                  mode == HQ_SCALE_STATIC || R * S == 1 ? ws_bytes : 0);
+    LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes);
     s = launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, desc->had_block, a_bits, mode, static_scale,
                              lc.codes, cont, ldc, lc.scales, scratch, scratch_bytes, st, 1, pre_bias, x2, split, &lc.z);
     if (s != HQ_OK) return s;
@@ -273,7 +292,7 @@ extern "C" hq_status hq_gn_qlinear(const void* x, hq_dtype xdt, int64_t Nb, int6
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, M, C, M, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, C, 1, cont, workspace, ws_bytes);
     s = launch_gn_silu_quant(x, xdt, Nb, rows_per_sample, 1, C, groups, gamma, beta, eps, desc->had_block, a_bits,
                              HQ_SCALE_PER_ROW, nullptr, lc.codes, cont, lc.ld, lc.scales, scratch, scratch_bytes, st,
                              silu != 0, nullptr, nullptr, 0, &lc.z);
@@ -300,9 +319,7 @@ static hq_status qconv_impl(const void* x, const void* x2, int64_t split, hq_dty
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb
-    LayerCodes lc(desc, w_dev, a_bits, rows, C, rows / (stride == 2 ? 4 : 1), cont, workspace,
-                  mode == HQ_SCALE_STATIC || R * S == 1 ? ws_bytes : 0);
+    LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes);
     if (x2 != nullptr)
         s = launch_hadamard_quant_cat(x, split, x2, C - split, split, xdt, rows, C, desc->had_block, a_bits, mode, static_scale,
                                       lc.codes, cont, ldc, lc.scales, st, &lc.z);
@@ -420,7 +437,7 @@ extern "C" hq_status hq_qlinear_noalloc(const void* x, hq_dtype xdt, int64_t M, 
     s = noalloc_scratch_address(&codes);
     if (s != HQ_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, M, K, M, cont, codes, HQ_NOALLOC_SCRATCH_BYTES);
+    LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, codes, HQ_NOALLOC_SCRATCH_BYTES);
     s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
                               &lc.z);
     if (s != HQ_OK) return s;

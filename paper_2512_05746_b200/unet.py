@@ -147,8 +147,9 @@ class UNet:
     def _new(self, shape, dtype=None):
         return self.torch.empty(shape, dtype=dtype or self.torch.bfloat16, device=self.dev)
 
-    def _need_ws(self, rows, cols):
-        self._ws_need = max(self._ws_need, self.hq.hq_workspace_size(rows, cols, self.cont))
+    def _need_ws(self, pw, rows, static=False, stride=1):
+        # for 4-bit codes too, whose layers use more of it: `a_bits` may be changed after the build
+        self._ws_need = max(self._ws_need, *(self.hq.hq_layer_workspace_size(pw, b, rows, static, stride) for b in (self.a_bits, 4)))
 
     def _ws_views(self, rows, cols):
         row_bytes = cols // 2 if self.cont == self.hq.HQ_CODES_NIBBLE else cols
@@ -163,7 +164,7 @@ class UNet:
         Nb, H, W, Cin = x.shape
         Cin += x2.shape[3] if x2 is not None else 0
         pw = self.pw[name]
-        self._need_ws(Nb * H * W, Cin)
+        self._need_ws(pw, Nb * H * W, static=True, stride=stride)
         y = self._new((Nb, H // stride, W // stride, pw.desc.N))
         bias = self.f32[name + ".b"]
         ss = self.static.setdefault(name, t.ones((1,), dtype=t.float32, device=self.dev))
@@ -200,7 +201,7 @@ class UNet:
         Nb, H, W, Cin = x.shape
         Cin += x2.shape[3] if x2 is not None else 0
         pw = self.pw[name]
-        self._need_ws(Nb * H * W, Cin)
+        self._need_ws(pw, Nb * H * W)
         y = self._new((Nb, H, W, pw.desc.N))
         bias = self.f32[name + ".b"]
         self._emit("q", name, lambda: hq.hq_qconv(x, pw, 1, 1, 1, 0, bias, self.a_bits, y, self.ws, dev_status=self.status,
@@ -213,7 +214,7 @@ class UNet:
         hq = self.hq
         M, K = x.shape
         pw = self.pw[name]
-        self._need_ws(M, K)
+        self._need_ws(pw, M)
         y = self._new((M, pw.desc.N))
         bias = self.f32[name + ".b"]
         if norm:

@@ -172,3 +172,30 @@ def test_fused_layers_refuse_null_weights_before_a_launch(hq, had_block):
     assert L.hq_gn_silu_qconv_cat(fake, fake, 0, 1, 8, 32, 32, 1024, 32, fake, fake, None, 1e-5, dc, None, 3, 3, 1, 1, fake, None, 4,
                                   1, fake, fake, 1, fake, big, fake, 1 << 20, None, None) == 1
     assert L.hq_qlinear_noalloc(fake, 1, 1024, K, K, d, None, fake, None, 4, 0, None, fake, 1, N, None, None) == 1
+
+
+@pytest.mark.parametrize("rows,cols,n,mode,w_bits,container,a_bits,static,stride,taps,room", [
+    (4096, 1152, 128, "folded", 4, 1, 4, False, 1, 1, True),        # 4.5 MiB of codes, runs on one limb
+    (4096, 1152, 128, "folded", 4, 0, 3, True, 1, 1, True),         # two codes per byte
+    (65536, 1152, 128, "folded", 4, 1, 8, False, 1, 1, False),      # 8-bit codes need two limbs
+    (65536, 1024, 1024, "folded", 4, 1, 4, False, 1, 1, False),     # so do blocks above 512
+    (65536, 1152, 128, "double", 4, 1, 4, False, 1, 1, False),      # one limb anyhow
+    (256, 256, 256, "folded", 4, 1, 4, False, 1, 1, False),         # nothing to gain
+    (15 * 32 * 32, 512, 256, "folded", 4, 1, 4, True, 1, 9, True),  # 7.6 MiB
+    (64 * 32 * 32, 512, 256, "folded", 4, 1, 4, False, 1, 9, False),    # one scale per pixel under a 3x3 window
+])
+def test_layer_workspace_asks_for_what_the_layer_uses(hq, rows, cols, n, mode, w_bits, container, a_bits, static, stride, taps, room):
+    N = {1152: 4608, 256: 256}.get(cols, 1024)
+    w = inputs.weights((N, cols) if taps == 1 else (512, 3, 3, cols), seed=0)
+    pw = hq.hq_weight_prepare(w, w_bits, n, hq.WEIGHT_MODES[mode], container)
+    pitch = (cols // 2 if container == 0 else cols + 15) // 16 * 16
+    codes = (rows * pitch + 255) // 256 * 256 + 4 * rows
+    want = (codes + 255) // 256 * 256 + rows * cols if room else codes
+    assert hq.hq_layer_workspace_size(pw, a_bits, rows, static, stride) == want
+    pw.desc.reserved = 0                                            # a blob of the two-limb section alone
+    assert hq.hq_layer_workspace_size(pw, a_bits, rows, static, stride) == codes
+    out = C.c_size_t(0)
+    assert hq.lib.hq_layer_workspace_size(None, a_bits, 0, rows, 1, C.byref(out)) == 1
+    assert hq.lib.hq_layer_workspace_size(C.byref(pw.desc), 5, 0, rows, 1, C.byref(out)) == 1
+    assert hq.lib.hq_layer_workspace_size(C.byref(pw.desc), a_bits, 0, -1, 1, C.byref(out)) == 2
+    assert hq.lib.hq_layer_workspace_size(C.byref(pw.desc), a_bits, 0, rows, 3, C.byref(out)) == 3

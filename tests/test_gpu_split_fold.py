@@ -145,3 +145,22 @@ def test_convolution_on_one_limb_is_the_convolution_on_two(Nb, H, W, C, Cout, R,
     hq.hq_check_status(status)
     assert torch.equal(y1, y2)
     assert not bool((z == 0x11).all()), "the layer was meant to run on one limb"
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [3400, 7000, 7400])                  # 3.8, 7.7 and 8.2 MiB of codes and scales
+@pytest.mark.parametrize("container", [0, 1])
+def test_a_workspace_of_the_layer_query_takes_the_one_limb_route_at_any_size(M, container):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    K, N = 1152, 4608
+    x = torch.randn((M, K), generator=torch.Generator(device="cuda").manual_seed(M), device="cuda").to(torch.bfloat16)
+    pw = hq.hq_weight_prepare(inputs.weights((N, K), seed=1), 4, 128, hq.HQ_W_FOLDED, container).to_device()
+    base, full = _codes_bytes(M, K, container), hq.hq_layer_workspace_size(pw, 4, M)
+    assert full > base
+    y = []
+    for ws in (torch.full((full,), 0x11, dtype=torch.uint8, device="cuda"), torch.zeros((base,), dtype=torch.uint8, device="cuda")):
+        y.append(torch.zeros((M, N), dtype=torch.bfloat16, device="cuda"))
+        hq.hq_qlinear(x, pw, None, 4, y[-1], ws)
+        assert ws.numel() == base or not bool((ws[(base + 255) // 256 * 256:] == 0x11).all())
+    assert torch.equal(y[0], y[1])
