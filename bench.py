@@ -68,7 +68,16 @@ def ws_views(torch, ws, rows, cols):
     return ws[: rows * pitch].view(rows, pitch), ws[off: off + rows * 4].view(torch.float32)
 
 
-STEP_KERNEL_SOURCES = ("hq_common.cuh", "hq_fwht.cuh", "hq_quant.cu", "hq_gemm_kernel.cuh", "hq_gemm.cu", "hq_gemm_pair.cu", "hq_api.cu",
+def limbs_run(hq, pw, a_bits, rows, ws, static=False, stride=1):
+    """Weight limbs a fused call of this layer runs on in this workspace: one where it takes the split fold (the query asks
+    for the room its codes need; 8-bit codes never fold, so theirs is codes and scales alone), else the descriptor's."""
+    alone = hq.hq_layer_workspace_size(pw, 8, rows, static, stride)
+    need = hq.hq_layer_workspace_size(pw, a_bits, rows, static, stride)
+    return 1 if alone < need <= ws.nbytes else pw.desc.limbs
+
+
+STEP_KERNEL_SOURCES = ("hq_common.cuh", "hq_cluster.cuh", "hq_fwht.cuh", "hq_quant.cu", "hq_gemm_kernel.cuh", "hq_gemm.cu",
+                       "hq_gemm_pair.cu", "hq_gemm_splitk.cu", "hq_api.cu",
                        "hq_gemm_inst_i8_gemm.cu", "hq_gemm_inst_i8_conv.cu", "hq_gemm_inst_nibble_gemm.cu",
                        "hq_gemm_inst_nibble_conv.cu")
 
@@ -188,7 +197,6 @@ def build_layers(torch, hq, device, seed, cont=None, share=None, weight_mode=Non
         w, b = cfg["w"], cfg["bias"]
         pw = hq.hq_weight_prepare(w, W_BITS, L["had_block"], mode, cont).to_device(device)
         L["pw"] = pw
-        L["limbs"] = pw.desc.limbs
         rows, cols = (L["M"], L["K"]) if L["kind"] == "linear" else (L["M"], CONV["C"])
         L["rows"], L["cols"] = rows, cols
         oshape = (L["M"], L["N"]) if L["kind"] == "linear" else (CONV["Nb"], CONV["H"], CONV["W"], CONV["Cout"])
@@ -204,11 +212,14 @@ def build_layers(torch, hq, device, seed, cont=None, share=None, weight_mode=Non
             L["static_scale"] = None
         L["cont"] = cont
         L["ws"] = torch.empty((hq.hq_workspace_size(rows, cols, cont),), dtype=torch.uint8, device=device)
+        # what the fused call issues: its weight limbs, and one byte per code where it reads the split-fold codes
+        L["limbs"] = limbs_run(hq, pw, A_BITS, rows, L["ws"], static=L["kind"] == "conv")
+        L["split"] = L["limbs"] < pw.desc.limbs
         L["ops"] = 2.0 * L["M"] * L["N"] * L["K"] * L["limbs"]
         L["ops_1limb"] = 2.0 * L["M"] * L["N"] * L["K"]
         # algorithmic HBM bytes of the two kernels (fp32 in, codes out + scales; codes + weights in, bf16 out)
         L["quant_bytes"] = rows * cols * 4.0 + rows * cols * cb + rows * 4.0
-        L["gemm_bytes"] = rows * cols * cb + L["N"] * L["K"] * L["limbs"] + L["M"] * L["N"] * 2.0 + 4.0 * L["M"] + 8.0 * L["N"]
+        L["gemm_bytes"] = rows * cols * (1.0 if L["split"] else cb) + L["N"] * L["K"] * L["limbs"] + L["M"] * L["N"] * 2.0 + 4.0 * L["M"] + 8.0 * L["N"]
     torch.cuda.synchronize()
     # The conv uses one static activation scale (the paper's learned per-tensor scale): calibrate it once with the
     # library's own dynamic pass: S = max over pixels of the per-pixel scale.
@@ -244,32 +255,50 @@ def split_views(torch, L):
     return codes, L["ws"][off: off + rows * 4].view(torch.float32)
 
 
+def fused_layer(hq, L, status, stream=None):
+    if L["kind"] == "linear":
+        hq.hq_qlinear(L["x"], L["pw"], L["bias"], A_BITS, L["y"], L["ws"], dev_status=status, stream=stream)
+    else:
+        c = CONV
+        hq.hq_qconv(L["x"], L["pw"], c["R"], c["S"], c["stride"], c["pad"], L["bias"], A_BITS, L["y"], L["ws"],
+                    static_scale=L["static_scale"], dev_status=status, stream=stream)
+
+
 def run_step_split(torch, hq, layers, status, evs, gemm_only=False):
-    """Same kernels as run_step, launched through the unfused entry points with an event between them."""
+    """The kernels of run_step through the unfused entry points, with an event between the two of a layer.  A layer on the split
+    fold has no unfused product on one limb: there the transform alone is followed by the whole fused layer, and the product's
+    time is the difference (kernel_ms), the write of the split-fold codes included."""
     stream = torch.cuda.current_stream()
     for L in layers:
         rows, cols, cont = L["rows"], L["cols"], L["cont"]
         codes, scales = split_views(torch, L)
         x2d = L["x"].view(rows, cols)
+        static = L["static_scale"] if L["kind"] == "conv" else None
+        split = L["split"] and not gemm_only
         e0, e1, e2 = (torch.cuda.Event(enable_timing=True) for _ in range(3))
         e0.record(stream)
-        if L["kind"] == "linear":
-            if not gemm_only:
-                hq.hq_hadamard_quant(x2d, L["had_block"], A_BITS, codes, cont, scales=scales)
-            e1.record(stream)
+        if not gemm_only:
+            hq.hq_hadamard_quant(x2d, L["had_block"], A_BITS, codes, cont, scales=scales if static is None else scales[:1],
+                                 static_scale=static)
+        e1.record(stream)
+        if split:
+            fused_layer(hq, L, status)
+        elif L["kind"] == "linear":
             hq.hq_qgemm(codes, cont, A_BITS, L["K"], L["pw"], scale_a=scales, bias=L["bias"],
                         alpha=L["pw"].alpha, y=L["y"], dev_status=status)
         else:
             c = CONV
-            if not gemm_only:
-                hq.hq_hadamard_quant(x2d, L["had_block"], A_BITS, codes, cont, scales=scales[:1],
-                                     static_scale=L["static_scale"])
-            e1.record(stream)
             hq.hq_qconv2d(codes, cont, A_BITS, c["Nb"], c["H"], c["W"], c["C"], L["pw"], c["R"], c["S"],
-                          c["stride"], c["pad"], scale_a=L["static_scale"], bias=L["bias"], alpha=L["pw"].alpha,
+                          c["stride"], c["pad"], scale_a=static, bias=L["bias"], alpha=L["pw"].alpha,
                           y=L["y"], dev_status=status)
         e2.record(stream)
         evs.append((L, e0, e1, e2))
+
+
+def kernel_ms(L, e0, e1, e2):
+    """Milliseconds of the transform and of the product from a layer's events (see run_step_split)."""
+    q, g = e0.elapsed_time(e1), e1.elapsed_time(e2)
+    return q, g - q if L["split"] else g
 
 
 def measure_variants(torch, hq, device, layers, status, stream, rank):
@@ -297,8 +326,9 @@ def measure_variants(torch, hq, device, layers, status, stream, rank):
     per = {}
     for L, a, b, c in evs:
         d = per.setdefault(L["name"], dict(q=[], g=[], L=L))
-        d["q"].append(a.elapsed_time(b))
-        d["g"].append(b.elapsed_time(c))
+        q, g = kernel_ms(L, a, b, c)
+        d["q"].append(q)
+        d["g"].append(g)
     out["nibble_container" if other == 0 else "int8_container"] = dict(
         ms_per_pass=ms_alt, tops=ops1 / (ms_alt * 1e-3) / 1e12,
         per_layer={k: dict(quant_ms=float(np.median(d["q"])), gemm_ms=float(np.median(d["g"])),
@@ -539,8 +569,14 @@ def main_layer_list(args, which):
         evs[i + 1].record()
     torch.cuda.synchronize()
     per_shape = {}
+
+    def limbs_of(L):
+        r = L["res"]
+        rows = L["Nb"] * L["H"] * L["W"] if L["kind"] == "conv" else L["M"]
+        return limbs_run(hq, r["pw"], A_BITS, rows, r["ws"], r["static"] is not None, L.get("stride", 1))
+
     for i, L in enumerate(layers):
-        d = per_shape.setdefault(str(key(L)), dict(count=0, ms=0.0, macs=L["macs"], limbs=L["res"]["pw"].desc.limbs))
+        d = per_shape.setdefault(str(key(L)), dict(count=0, ms=0.0, macs=L["macs"], limbs=limbs_of(L)))
         d["count"] += 1
         d["ms"] += evs[i].elapsed_time(evs[i + 1])
     for d in per_shape.values():
@@ -602,11 +638,11 @@ def main_layer_list(args, which):
                         ln_quant_us=ln_us, plain_quant_us=pl_us,
                         note="LayerNorm + per-sample modulation fused in front of the QKV and FC1 linears (hq_ln_qlinear)")
     macs = sum(L["macs"] for L in layers)
-    ops_limbs = sum(2.0 * L["macs"] * L["res"]["pw"].desc.limbs for L in layers)
+    ops_limbs = sum(2.0 * L["macs"] * limbs_of(L) for L in layers)
     print(json.dumps(dict(metric="forwards/s of " + label,
                           value=1e3 / ms, unit="forwards/s", n_gpus=1, steps=steps, warmup=warmup, ms_per_step=ms,
                           higher_is_better=True, scaling="weak", vs_baseline=None, dtype="int8", data="synthetic",
-                          config=dict(workload=wl + f", bf16 in/out, W4A{A_BITS} folded two-limb weights, " + codes_name() + " codes",
+                          config=dict(workload=wl + f", bf16 in/out, W4A{A_BITS} folded weights, " + codes_name() + " codes",
                                       layers=len(layers),
                                       layers_per_s=len(layers) * 1e3 / ms, tops_limbs=ops_limbs / ms / 1e9,
                                       tops_1limb_equiv=2.0 * macs / ms / 1e9,
@@ -784,7 +820,7 @@ def main_sweep(args):
     print(json.dumps(dict(metric="shape sweep: int TOPS of the GEMM and GB/s of transform+quantize per point", value=best["gemm_tops_limbs"],
                           unit="TOPS issued (best point)", n_gpus=1, steps=reps, warmup=10, higher_is_better=True, dtype="int8",
                           data="synthetic", vs_baseline=None,
-                          config=dict(workload="configs[4] shape sweep, " + codes_name() + " codes for W4A4",
+                          config=dict(workload="shape sweep, " + codes_name() + " codes for W4A4",
                                       int8_peak_tops=int8_peak, int8_peak_source="kind::i8 issue-rate probe of this run",
                                       probe_sm_mhz=probe["sm_mhz"], hbm_gbs=pk["hbm_gbs"], peak_source=pk["source"],
                                       l2=f"buffers of a point rotate through at least {ROTATE_BYTES / 1e6:.0f} MB"),
@@ -1038,8 +1074,9 @@ def main():
     per = {}
     for L, a, b, c in evs:
         d = per.setdefault(L["name"], dict(quant=[], gemm=[], L=L))
-        d["quant"].append(a.elapsed_time(b))
-        d["gemm"].append(b.elapsed_time(c))
+        q, g = kernel_ms(L, a, b, c)
+        d["quant"].append(q)
+        d["gemm"].append(g)
     for d in per.values():
         d["quant_ms"], d["gemm_ms"] = float(np.median(d["quant"])), float(np.median(d["gemm"]))
         d["quant_best"], d["gemm_best"] = float(np.min(d["quant"])), float(np.min(d["gemm"]))
@@ -1134,6 +1171,7 @@ def main():
                                                 f"limbs={L['limbs']})",
                         achieved=ach, peak=int8_peak, unit="TOPS", frac=ach / int8_peak,
                         achieved_counts="2*M*N*K*limbs (the tensor work issued; the layer's own 2*M*N*K is achieved/limbs)",
+                        launch_ms_is=("the fused layer less the transform alone" if L["split"] else "the product kernel"),
                         traffic=(traffic.get("gemm") or {}).get(L["name"]),
                         algorithmic_bytes=L["gemm_bytes"], peak_source=peak_source,
                         peak_probe_tops=None if probe is None else probe["tops"],
