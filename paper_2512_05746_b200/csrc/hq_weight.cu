@@ -137,9 +137,9 @@ extern "C" hq_status hq_weight_prepare(const float* w, int64_t N, int32_t RS, in
             for (int64_t b = 0; b < KK / n; ++b) fwht_bits_inplace(B1.data() + b * n, n, weight_mask);
             for (int t = 0; t < RS; ++t)
                 for (int64_t c = 0; c < C; ++c) {
-                    const int32_t v = B1[t * C + c];                // at most 7 * 16: Q(W) of an absmax scale has no -8
-                    if (v < -128 || v > 127) return HQ_ERR_OVERFLOW_RISK;
-                    out[base + o * Kp + int64_t(t) * C_pad + c] = int8_t(v);
+                    // 16 integers of -8 .. 7 (-8 only where the scale is subnormal or a weight no number) under the signs of
+                    // a Hadamard row: all of one sign, at least 16 * -8 and at most 16 * 7, or eight of each, at most 8 * 8 + 8 * 7
+                    out[base + o * Kp + int64_t(t) * C_pad + c] = int8_t(B1[t * C + c]);
                 }
         }
         if (mode == HQ_W_FOLDED && n > 1)

@@ -199,3 +199,27 @@ def test_layer_workspace_asks_for_what_the_layer_uses(hq, rows, cols, n, mode, w
     assert hq.lib.hq_layer_workspace_size(C.byref(pw.desc), 5, 0, rows, 1, C.byref(out)) == 1
     assert hq.lib.hq_layer_workspace_size(C.byref(pw.desc), a_bits, 0, -1, 1, C.byref(out)) == 2
     assert hq.lib.hq_layer_workspace_size(C.byref(pw.desc), a_bits, 0, rows, 3, C.byref(out)) == 3
+
+
+@pytest.mark.parametrize("n", [32, 512])
+@pytest.mark.parametrize("kind", ["subnormal", "not a number", "all not a number"])
+def test_split_section_holds_the_extreme_integers(hq, n, kind):
+    """-8 in the quantized weights: the scale of the largest of them is rounded to a subnormal, or they are no numbers."""
+    N, rng = 64, np.random.default_rng(n)
+    w = rng.choice([-1.0, 1.0], size=(N, n)).astype(np.float32)
+    if kind == "subnormal":                 # the absolute maximum, 11 units, over a scale of one and a half, rounded to one or two
+        w = (np.where(rng.random((N, n)) < 0.5, -11.0, 7.0) * 2.0 ** -149).astype(np.float32)
+    elif kind == "not a number":
+        w[rng.random((N, n)) < 0.5] = np.nan
+    else:
+        w[:] = np.nan
+    pw = hq.hq_weight_prepare(w, 4, n, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8)
+    d = pw.desc
+    assert d.reserved == 1
+    B1 = pw.blob[d.N_pad * 2 * d.C_pad:].reshape(d.N_pad, d.C_pad)[:N, :n].astype(np.int64)
+    B = decode_blob(pw).reshape(N, n).astype(np.int64)
+    # the remaining factors of the folded weights, index bits 2, 3, 4, 1, 0 in this order
+    for bit in [2, 3, 4, 1, 0][: n.bit_length() - 5]:
+        v = B1.reshape(N, -1, 2, 1 << bit)
+        B1 = np.stack([v[:, :, 0] + v[:, :, 1], v[:, :, 0] - v[:, :, 1]], axis=2).reshape(N, n)
+    assert np.array_equal(B1, B)
