@@ -139,6 +139,7 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     const int ew = warp - 2, q = warp & 3, chalf = ew >> 2;     // epilogue warps: tensor-memory lane quarter, half of the columns
     float sa_eff = 0.f;                                         // of the row this thread finishes
     bool ok = true;
+    int armed = 0;                                              // K blocks requested (the producing thread's)
     if (warp != 0) cluster_wait();
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -172,16 +173,13 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
             for (int i = 0; i < first; ++i) load_b(i);
             if (p.pdl) griddep_wait();                 // the codes come from the kernel before this one
             for (int i = 0; i < first; ++i) load_a(i);
-            int armed = first;
+            armed = first;
             for (int i = first; i < count; ++i) {
                 if (!wait_splitk<false>(&ctl->empty[i % STAGES], uint32_t(i / STAGES - 1) & 1u, ctl, p.dev_status, kStatusEmptyWait)) { ok = false; break; }
                 load_b(i);
                 load_a(i);
                 ++armed;
             }
-            if (!ok || ctl->abort_flag)                // the copies in flight must land before the ring is given up
-                for (int i = armed > STAGES ? armed - STAGES : 0; i < armed; ++i)
-                    mbar_wait(&ctl->full[i % STAGES], uint32_t(i / STAGES) & 1u, nullptr, 0);
         }
         __syncwarp();
         cluster_wait();
@@ -281,6 +279,9 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     __syncwarp();
     cluster_arrive_relaxed();
     __syncthreads();
+    if (threadIdx.x == 0 && ctl->abort_flag)                    // the copies in flight must land before the ring is given up
+        for (int i = armed > STAGES ? armed - STAGES : 0; i < armed; ++i)
+            mbar_wait(&ctl->full[i % STAGES], uint32_t(i / STAGES) & 1u, nullptr, 0);
     if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, kSkCols * LIMBS); }
     cluster_wait();                        // nobody leaves while another CTA may still write or arrive here
 }
