@@ -86,7 +86,8 @@ typedef struct {
     int64_t N_pad;      /* N rounded up to 128; padding rows are zero */
     int64_t bytes;      /* size of the blob */
     int32_t max_abs_b;  /* largest |B| entry, for the accumulator-range check */
-    int32_t reserved;   /* 1: the one-limb section of the split fold follows (see hq_weight_prepare); 0: it does not */
+    int32_t reserved;   /* 1: the one-limb section of the split fold follows (see hq_weight_prepare); 0: it does not (blocks above
+                           512: see bytes) */
 } hq_weight_desc;
 
 int hq_version(void);
@@ -116,8 +117,10 @@ hq_status hq_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t c
  * desc       filled on success.
  * FOLDED 4-bit weights with blocks of 32 .. 512 channels get a second section of half the first one's size: one-limb
  *   weights with four of the log2(had_block) factors of H_raw applied, for the fused layer calls, which give the other
- *   factors to the codes (same integers, half the tensor work).  A blob_bytes that holds only the first section is taken
- *   as well; the layer then always runs on two limbs.
+ *   factors to the codes (same integers, half the tensor work).  Blocks of 1024 .. 4096 channels get one too (four factors to
+ *   the codes, the rest applied here) where the integers of these weights fit a byte, or, for linear layers of one block of
+ *   2048 or 4096, where they do when halved; desc->bytes says which (hq_weight_blob_bytes is the most it may be).  A blob_bytes
+ *   that holds only the first section is taken as well; the layer then always runs on two limbs.
  * Errors: FOLDED/DOUBLE with C % had_block != 0; FOLDED whose integers need more than 2 limbs -> HQ_ERR_OVERFLOW_RISK. */
 int64_t hq_weight_blob_bytes(int64_t N, int32_t RS, int64_t C, int32_t w_bits, int32_t had_block,
                              hq_weight_mode mode);
@@ -161,7 +164,9 @@ hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t
  *    hq_qlinear_noalloc takes a layer).
  *  hq_layer_workspace_size knows the layer (weights, width of the codes, one static scale or one per row, stride; rows of
  *    its input: M or Nb * H * W) and asks for the room at any size, and only where the layer then uses it.  On the current
- *    device: the choice depends on its number of SMs.
+ *    device: the choice depends on its number of SMs.  It never asks for the room of blocks above 512 or of one scale per pixel
+ *    under a window, which such layers use where they are given it (hq_workspace_size's figure has it, with 128 bytes a row
+ *    more at 2048 and 4096 columns for the further columns of halved weights).
  * alpha is derived from the descriptor.  y pitch ldy elements.
  * The product kernel is launched so that it may begin (set-up, first weight tile) while the transform kernel is still
  * running; it waits for the transform before it touches codes or activation scales.  Work enqueued on the stream before

@@ -16,7 +16,9 @@ hq_status launch_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows, int64
 hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64_t M, int64_t K, int64_t lda,
                        const hq_weight_desc* desc, const void* w_dev, const float* scale_a, int scale_a_is_scalar,
                        const float* scale_w, const float* bias, float alpha, int32_t* acc_out, void* y,
-                       hq_dtype ydt, int64_t ldy, int32_t* dev_status, cudaStream_t st, bool after_quant);
+                       hq_dtype ydt, int64_t ldy, int32_t* dev_status, cudaStream_t st, bool after_quant,
+                       const HalvedParity* halved = nullptr);
+bool halved_product_covers(int64_t M, const void* y, hq_dtype ydt, int64_t ldy);      // hq_gemm.cu
 hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t Nb, int64_t H, int64_t W,
                          int64_t C, const hq_weight_desc* desc, const void* w_dev, int R, int S, int stride, int pad,
                          const float* scale_a, int scale_a_is_scalar, const float* scale_w, const float* bias,
@@ -61,6 +63,9 @@ int64_t split_offset(int64_t rows, int64_t cols, hq_container cont) { return (co
 int64_t split_bytes(int64_t rows, int64_t cols, hq_container cont) {
     return split_offset(rows, cols, cont) + rows * code_pitch(cols, HQ_CODES_INT8);
 }
+int64_t halved_bytes(int64_t rows, int64_t cols, hq_container cont) {
+    return split_offset(rows, cols, cont) + rows * (cols + kHalvedCols);
+}
 
 // What a fused layer call cannot do without: its codes and scales.
 hq_status layer_bytes(int64_t rows, int64_t cols, hq_container cont, size_t* bytes) {
@@ -81,39 +86,61 @@ struct LayerCodes {
     hq_weight_desc split_desc;
     const void* split_w;
 
+    HalvedParity parity;
+
     // rows x cols codes.  The caller has refused a null w_dev: split_w is never null, so the product's own check no longer
-    // sees one.
+    // sees one.  halved_ok: the product is one that halved weights are read by (halved_product_covers).
     LayerCodes(const hq_weight_desc* desc, const void* w_dev, int a_bits, hq_scale_mode mode, int64_t rows, int64_t cols, int stride,
-               hq_container cont, void* workspace, size_t ws_bytes)
+               hq_container cont, void* workspace, size_t ws_bytes, bool halved_ok)
         : codes(static_cast<unsigned char*>(workspace)),
           scales(reinterpret_cast<float*>(codes + scales_offset(rows, cols, cont))), ld(code_pitch(cols, cont)) {
-        if (ws_bytes >= size_t(split_bytes(rows, cols, cont)) && split_taken(desc, a_bits, mode, rows, cols, stride)) {
-            z.z = codes + split_offset(rows, cols, cont);
-            z.ld = code_pitch(cols, HQ_CODES_INT8);
-            split_desc = *desc;
-            split_desc.limbs = 1;
-            split_desc.container = HQ_CODES_INT8;
-            split_w = static_cast<const unsigned char*>(w_dev) + desc->N_pad * 2 * desc->RS * desc->C_pad;
+        const Section sec = section(desc, a_bits, cols);
+        if (sec == kNone || (sec == kHalved && !halved_ok)) return;
+        const int64_t room = sec == kHalved ? halved_bytes(rows, cols, cont) : split_bytes(rows, cols, cont);
+        if (ws_bytes < size_t(room) || !split_taken(desc, a_bits, mode, rows, cols, stride)) return;
+        z.z = codes + split_offset(rows, cols, cont);
+        z.ld = sec == kHalved ? cols + kHalvedCols : code_pitch(cols, HQ_CODES_INT8);
+        z.halved = sec == kHalved;
+        split_desc = *desc;
+        split_desc.limbs = 1;
+        split_desc.container = HQ_CODES_INT8;
+        split_w = static_cast<const unsigned char*>(w_dev) + desc->N_pad * 2 * desc->RS * desc->C_pad;
+        if (z.halved) {
+            split_desc.C += kHalvedCols;
+            split_desc.C_pad += kHalvedCols;
+            parity = HalvedParity{z.z + cols + kHalvedQ, z.ld, static_cast<const uint8_t*>(split_w) + desc->N_pad * split_desc.C_pad};
         }
+    }
+    // The one-limb section behind the two-limb weights, and whether codes of a_bits bits can be multiplied with it.
+    enum Section { kNone, kBytes, kHalved };
+    static Section section(const hq_weight_desc* desc, int a_bits, int64_t cols) {
+        if (desc->limbs != 2 || desc->C != cols || cols >= 131072) return kNone;
+        const int klog = ilog2(desc->had_block);
+        if (!split_fits(klog, a_bits)) return kNone;
+        if (split_block_ok(klog)) return desc->reserved == kBlobHasSplit ? kBytes : kNone;
+        if (!split_wide(klog) || desc->mode != HQ_W_FOLDED) return kNone;
+        const int64_t more = desc->bytes - desc->N_pad * 2 * desc->RS * desc->C_pad;      // what the preparation put there
+        return more == desc->N_pad * desc->RS * desc->C_pad ? kBytes
+             : more == desc->N_pad * (desc->C_pad + kHalvedCols + 1) ? kHalved : kNone;
     }
     // Per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb.
     static bool split_taken(const hq_weight_desc* desc, int a_bits, hq_scale_mode mode, int64_t rows, int64_t cols, int stride) {
-        return (mode == HQ_SCALE_STATIC || desc->RS == 1) && split_applies(desc, a_bits, cols) &&
-               split_pays(desc, rows, cols, rows / (stride == 2 ? 4 : 1));
-    }
-    static bool split_applies(const hq_weight_desc* desc, int a_bits, int64_t cols) {
-        if (desc->reserved != kBlobHasSplit || desc->limbs != 2 || desc->C != cols) return false;
-        const int klog = ilog2(desc->had_block);
-        return split_block_ok(klog) && split_fits(klog, a_bits) && cols < 131072;
+        const Section sec = section(desc, a_bits, cols);
+        return (mode == HQ_SCALE_STATIC || desc->RS == 1) && sec != kNone &&
+               split_pays(desc, rows, cols, rows / (stride == 2 ? 4 : 1), sec == kHalved ? kHalvedCols / 128 : 0);
     }
     // One limb halves the column tiles (or the weights a CTA of the split kernel streams), and the transform kernel computes
     // and writes a second byte per code, which costs 0.7 us plus its traffic at about 5.2 TB/s.  Measured (two limbs / one):
     // 8192 x 1152 -> 4608 57.9 / 44.2 us, 64 x 32 x 32 x 512 3x3 176 / 117 us, 2 x 16 x 16 x 768 3x3 13.1 / 11.8 us; where
     // no round of tiles is saved it only costs: 256 x 256 -> 256 6.1 / 6.8 us, 8 x 64 x 64 x 256 3x3 stride 2 16.5 / 17.6.
-    static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows) {
+    // Blocks above 512, the same rule: 65536 x 4096 -> 4096 1657 / 1127 us (the second byte costs the transform 84 of its 341 us),
+    // 65536 x 4096 -> 1024 536 / 487, 32768 x 2048 -> 2048 195 / 161, 65536 x 1024 -> 1024 125 / 113, 32768 x 2048 -> 512 with two
+    // codes per byte 113 / 111; not taken: the same with one code per byte, 101 / 104.
+    static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows, int more_kb) {
         const int num_kb = int(desc->RS * desc->C_pad / 128), tile_rows = out_rows < 128 ? int(out_rows > 0 ? out_rows : 1) : 128;
-        const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us;
-        const double one = plan_product(1, out_rows, tile_rows, desc->N_pad, num_kb).us;
+        // with two codes per byte the two-limb product unpacks them on one SM a tile (32768 x 2048 -> 512 52 us against 45)
+        const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us * (desc->container == HQ_CODES_NIBBLE ? 1.15 : 1.0);
+        const double one = plan_product(1, out_rows, tile_rows, desc->N_pad, num_kb + more_kb).us;
         return two - one > 0.7 + double(rows) * double(cols) / 5.2e6;
     }
     const void* a() const { return z.written ? z.z : codes; }
@@ -121,6 +148,8 @@ struct LayerCodes {
     hq_container container(hq_container cont) const { return z.written ? HQ_CODES_INT8 : cont; }
     const hq_weight_desc* desc(const hq_weight_desc* d) const { return z.written ? &split_desc : d; }
     const void* w(const void* w_dev) const { return z.written ? split_w : w_dev; }
+    int64_t k(int64_t K) const { return z.written && z.halved ? K + kHalvedCols : K; }
+    const HalvedParity* halved() const { return z.written && z.halved ? &parity : nullptr; }
 };
 }  // namespace
 }  // namespace hq
@@ -156,7 +185,8 @@ extern "C" hq_status hq_workspace_size(int64_t rows, int64_t cols, hq_container 
     // whether the layer has a use for it.  Smaller layers gain from it as well (4096 x 1152 -> 4608 30.7 / 24.5 us), but for
     // them this is the size at which the no-allocation entry point takes a layer: they ask hq_layer_workspace_size.
     *bytes = size_t(hq::codes_bytes(rows, cols, cont));
-    if (*bytes > size_t(HQ_NOALLOC_SCRATCH_BYTES)) *bytes = size_t(hq::split_bytes(rows, cols, cont));
+    if (*bytes > size_t(HQ_NOALLOC_SCRATCH_BYTES))
+        *bytes = size_t(cols == 2048 || cols == 4096 ? hq::halved_bytes(rows, cols, cont) : hq::split_bytes(rows, cols, cont));
     return HQ_OK;
 }
 
@@ -172,7 +202,7 @@ extern "C" hq_status hq_layer_workspace_size(const hq_weight_desc* desc, int a_b
     const hq_container cont = hq_container(desc->container);
     const hq_status s = layer_bytes(rows, desc->C, cont, bytes);
     if (s != HQ_OK) return s;
-    if (LayerCodes::split_taken(desc, a_bits, mode, rows, desc->C, stride)) *bytes = size_t(split_bytes(rows, desc->C, cont));
+    if (desc->had_block <= 512 && LayerCodes::split_taken(desc, a_bits, mode, rows, desc->C, stride)) *bytes = size_t(split_bytes(rows, desc->C, cont));
     return HQ_OK;
 }
 
@@ -190,12 +220,12 @@ extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t 
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, workspace, ws_bytes, halved_product_covers(M, y, ydt, ldy));
     s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
                               &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, K, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
-                        hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true);
+    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, lc.k(K), lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
+                        hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true, lc.halved());
 }
 
 extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const float* ln_weight,
@@ -212,7 +242,7 @@ extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, K, 1, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, K, 1, cont, workspace, ws_bytes, false);
     s = launch_ln_quant(x, xdt, M, K, ldx, ln_weight, ln_bias, rows_per_group, eps, desc->had_block, a_bits, HQ_SCALE_PER_ROW,
                         nullptr, lc.codes, cont, lc.ld, lc.scales, st, &lc.z);
     if (s != HQ_OK) return s;
@@ -240,7 +270,7 @@ static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes, false);
     s = launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, desc->had_block, a_bits, mode, static_scale,
                              lc.codes, cont, ldc, lc.scales, scratch, scratch_bytes, st, 1, pre_bias, x2, split, &lc.z);
     if (s != HQ_OK) return s;
@@ -292,7 +322,7 @@ extern "C" hq_status hq_gn_qlinear(const void* x, hq_dtype xdt, int64_t Nb, int6
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, C, 1, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, C, 1, cont, workspace, ws_bytes, false);
     s = launch_gn_silu_quant(x, xdt, Nb, rows_per_sample, 1, C, groups, gamma, beta, eps, desc->had_block, a_bits,
                              HQ_SCALE_PER_ROW, nullptr, lc.codes, cont, lc.ld, lc.scales, scratch, scratch_bytes, st,
                              silu != 0, nullptr, nullptr, 0, &lc.z);
@@ -319,7 +349,7 @@ static hq_status qconv_impl(const void* x, const void* x2, int64_t split, hq_dty
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes);
+    LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes, false);
     if (x2 != nullptr)
         s = launch_hadamard_quant_cat(x, split, x2, C - split, split, xdt, rows, C, desc->had_block, a_bits, mode, static_scale,
                                       lc.codes, cont, ldc, lc.scales, st, &lc.z);
@@ -437,10 +467,10 @@ extern "C" hq_status hq_qlinear_noalloc(const void* x, hq_dtype xdt, int64_t M, 
     s = noalloc_scratch_address(&codes);
     if (s != HQ_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, codes, HQ_NOALLOC_SCRATCH_BYTES);
+    LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, codes, HQ_NOALLOC_SCRATCH_BYTES, halved_product_covers(M, y, ydt, ldy));
     s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
                               &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, K, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
-                        hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true);
+    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, lc.k(K), lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
+                        hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true, lc.halved());
 }

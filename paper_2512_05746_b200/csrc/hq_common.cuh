@@ -25,10 +25,13 @@ enum : int32_t {
     kStatusUnpackWait = 0x500,   // unpack warps / MMA issuer waited on the staging ring
 };
 
-// Where the transform kernel may leave the codes' share of the split fold (split_codes in hq_fwht.cuh) beside the codes;
-// `written`: it did.
+// Where the transform kernel may leave the codes' share of the split fold (split_codes in hq_fwht.cuh) beside the codes, with the
+// further columns of halved weights behind each row (`halved`) or without; `written`: it did.
 constexpr int32_t kBlobHasSplit = 1;      // hq_weight_desc::reserved: the one-limb section follows the two-limb one
-struct SplitOut { uint8_t* z; int64_t ld; bool written; };
+struct SplitOut { uint8_t* z; int64_t ld; bool written; bool halved; };
+// What a product on halved weights (hq_fwht.cuh) adds to twice its sums: 1 where the parity byte of the row (every `pitch`
+// bytes) and that of the output channel are both 1.
+struct HalvedParity { const uint8_t* row; int64_t pitch; const uint8_t* col; };
 
 // hq_gemm_splitk.cu: CTAs a tile's reduction is divided over (0: persistent kernels) and the estimated time of a product.
 struct ProductPlan { int ways; double us; };
@@ -120,6 +123,11 @@ __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.
 __device__ __forceinline__ float ld_dependent(const float* p) {
     float v;
     asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_dependent_u8(const uint8_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 __device__ __forceinline__ float2 ld_dependent2(const float2* p) {

@@ -181,9 +181,28 @@ __device__ __forceinline__ void pack_codes(const f32x2 (&v)[E / 2], float inv, i
 // that a thread's 32 consecutive codes, four to a word, hold between words and then inside a word.
 constexpr int kSplitWeightBits = 4;                    // index bits whose factors stay with the weights
 __host__ __device__ constexpr bool split_block_ok(int klog) { return klog >= 5 && klog <= 9; }
+// Blocks of 1024 .. 4096: four bits go to the codes, whatever their width, and the other k - 4 stay with the weights, whose
+// integers then fit a byte (or, halved, nine bits) or not: the weight preparation looks (hq_weight.cu).
+constexpr int kSplitWideCodeBits = 4;
+__host__ __device__ constexpr bool split_wide(int klog) { return klog >= 10 && klog <= 12; }
+__host__ __device__ constexpr int split_code_bits(int klog) { return klog <= 9 ? klog - kSplitWeightBits : kSplitWideCodeBits; }
 __host__ __device__ constexpr int split_code_bit(int i) { return i < 3 ? 2 + i : 4 - i; }       // 2, 3, 4, 1, 0
 // Whether z fits a signed byte for codes of a_bits bits (every row of H_raw but the first has as many -1 as +1).
-__host__ __device__ constexpr bool split_fits(int klog, int a_bits) { return a_bits - 1 + klog - kSplitWeightBits <= 7; }
+__host__ __device__ constexpr bool split_fits(int klog, int a_bits) { return a_bits - 1 + split_code_bits(klog) <= 7; }
+
+// Halved weights.  With k - 4 = 7 or 8 factors B' no longer fits a byte, but its entries have a common parity over the
+// index bits that stay with the weights: that of their sum.  So with a the four code bits of a channel (bits 1 .. 4) and r the
+// others, B'(a, r) = 2 B''(a, r) + w(a), w(a) = -1 or 0, and B'' is a byte again.  The product is
+//   z . B' = 2 (z . B'') + sum_a w(a) sum_r z(a, r) = 2 (z . B'') + sum_p u(p) v(p),
+// u(p) = sum_r q(p, r) the sums of the row's codes over r and v(p) = sum_a H(a, p) w(a).  All v(p) of a channel have one
+// parity e, v = 2 v' + e, and with U = sum_p u(p) = 2 U' + Q the integer is
+//   2 (z . B'' + sum_p u(p) v'(p) + e U') + e Q:
+// the bracket is one product with 35 further columns on the reduction (one K block), e Q is added as the accumulator is read.
+// Columns of that block, activations x weights: u(p) = 16 h + l as (h, 16 v') and (l, v'), U' = 128 c1 + c0 as (c1, 64 e) twice
+// and (c0, e); the next byte of the activations' row holds Q, against a zero weight.
+constexpr int kHalvedCols = 128;                       // bytes the further columns take in a row of either operand
+constexpr int kHalvedH = 0, kHalvedL = 16, kHalvedC1 = 32, kHalvedC0 = 34, kHalvedQ = 35;
+__host__ __device__ constexpr bool split_halved(int klog) { return klog == 11 || klog == 12; }
 
 // u: 32 consecutive codes as bytes, biased by 128 >> A so that every sum below stays in its byte; on return z as signed
 // bytes.  A byte-wise butterfly is two additions per word pair: a + b, and a - b + (the bias to come); inside a word the
@@ -221,7 +240,7 @@ __device__ __forceinline__ void split_butterflies(uint32_t (&u)[8]) {
 // z of the 32 codes in w (8 words of bytes, or 4 words of nibbles, element 2j in the low one).
 template <int KLOG, bool INT8_IN>
 __device__ __forceinline__ void split_codes(const uint32_t (&w)[INT8_IN ? 8 : 4], uint32_t (&z)[8]) {
-    constexpr int A = KLOG - kSplitWeightBits;
+    constexpr int A = split_code_bits(KLOG);
     constexpr uint32_t kOnes = 0x01010101u, off = 128u >> A;
     if (INT8_IN) {
 #pragma unroll
@@ -236,6 +255,57 @@ __device__ __forceinline__ void split_codes(const uint32_t (&w)[INT8_IN ? 8 : 4]
         }
     }
     split_butterflies<A>(z);
+}
+
+// The further columns of a row against halved weights.  w: the 64 consecutive codes of a thread; part: shared scratch of eight
+// words per warp of the row when it has two (a row of 2^KLOG channels belongs to 2^(KLOG-6) threads, tb = 0 ..; every thread of
+// the CTA calls).  Thread tb < 8 gets its 16 of the 128 bytes.
+template <int KLOG, bool INT8_IN>
+__device__ __forceinline__ uint4 halved_columns(const uint32_t (&w)[INT8_IN ? 16 : 8], uint32_t* part, int tb) {
+    constexpr uint32_t kOnes = 0x01010101u;
+    constexpr int kBias = (1 << KLOG) / 2;             // the codes are summed as code + 8, 2^KLOG / 16 to a sum
+    uint32_t s[8];                                     // channel bits 2-4; the 16-bit fields are bit 1
+    if (INT8_IN) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t t = ((w[i] ^ 0x80808080u) - 120u * kOnes) + ((w[i + 8] ^ 0x80808080u) - 120u * kOnes);
+            s[i] = (t & 0x00FF00FFu) + ((t >> 8) & 0x00FF00FFu);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t n0 = w[i] ^ 0x88888888u, n1 = w[i + 4] ^ 0x88888888u;
+            const uint32_t t = (n0 & 0x0F0F0F0Fu) + ((n0 >> 4) & 0x0F0F0F0Fu) + (n1 & 0x0F0F0F0Fu) + ((n1 >> 4) & 0x0F0F0F0Fu);
+            s[2 * i] = __byte_perm(t, 0u, 0x4140);
+            s[2 * i + 1] = __byte_perm(t, 0u, 0x4342);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] = __reduce_add_sync(0xffffffffu, s[i]);     // at most 32 * 60 a field
+    if (KLOG == 12) {
+        __syncthreads();
+        if ((tb & 31) == 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) part[(tb >> 5) * 8 + i] = s[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] += part[((tb >> 5) ^ 1) * 8 + i];
+    }
+    uint32_t hw[4], lw[4], tot = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t a = s[2 * i] + 0x00080008u, b = s[2 * i + 1] + 0x00080008u;
+        tot += s[2 * i] + s[2 * i + 1];
+        hw[i] = (__byte_perm(a >> 4, b >> 4, 0x6420) + uint32_t(128 - kBias / 16) * kOnes) ^ 0x80808080u;
+        lw[i] = (__byte_perm(a & 0x000F000Fu, b & 0x000F000Fu, 0x6420) + 120u * kOnes) ^ 0x80808080u;
+    }
+    const int U = int(tot & 0xFFFFu) + int(tot >> 16) - 16 * kBias;
+    const int half = U >> 1, c1 = (half + 64) >> 7, c0 = half - 128 * c1;
+    const uint32_t c = uint32_t(c1 & 0xFF) * 0x0101u | uint32_t(c0 & 0xFF) << 16 | uint32_t(U & 1) << 24;
+    if (tb == 0) return make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    if (tb == 1) return make_uint4(lw[0], lw[1], lw[2], lw[3]);
+    return make_uint4(tb == 2 ? c : 0u, 0u, 0u, 0u);
 }
 
 }  // namespace hq

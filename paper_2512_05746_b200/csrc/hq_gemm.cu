@@ -34,7 +34,7 @@ bool pair_stream_covers_conv(hq_container cont, const gemm::GemmParams& g);
 hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, int64_t lda, const hq_weight_desc* desc,
                                    const void* w_dev, const float* scale_a, int scale_a_is_scalar, const float* scale_w,
                                    const float* bias, float alpha, void* y, int64_t ldy, int32_t* dev_status, cudaStream_t st,
-                                   bool after_quant);
+                                   bool after_quant, const HalvedParity* halved = nullptr);
 hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, const CUtensorMap& tmY,
                             const hq_weight_desc* desc, const void* w_dev, cudaStream_t st);
 // hq_gemm_splitk.cu: the same product with a tile's reduction divided over a cluster, for problems of few tiles
@@ -276,10 +276,17 @@ hq_status check_common(const void* a_codes, hq_container cont, int a_bits, const
 
 }  // namespace
 
+// Products on halved weights run on the streamed pair kernel alone: what it covers, the reduction being 2048 or more and the
+// 2^30 by which the sums are bounded there (2^12 codes of -8 against integers of 2^15) never in question.
+bool halved_product_covers(int64_t M, const void* y, hq_dtype ydt, int64_t ldy) {
+    return g_pair_gemm != 0 && M >= 256 && y != nullptr && ydt == HQ_BF16 && aligned16(y) && (ldy * 2) % 16 == 0;
+}
+
 hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64_t M, int64_t K, int64_t lda,
                        const hq_weight_desc* desc, const void* w_dev, const float* scale_a, int scale_a_is_scalar,
                        const float* scale_w, const float* bias, float alpha, int32_t* acc_out, void* y,
-                       hq_dtype ydt, int64_t ldy, int32_t* dev_status, cudaStream_t st, bool after_quant) {
+                       hq_dtype ydt, int64_t ldy, int32_t* dev_status, cudaStream_t st, bool after_quant,
+                       const HalvedParity* halved) {
     hq_status s = check_common(a_codes, cont, a_bits, desc, w_dev, scale_a, scale_w, acc_out, y, ydt, K);
     if (s != HQ_OK) return s;
     if (desc->RS != 1 || desc->C != K) return HQ_ERR_SHAPE;
@@ -302,6 +309,9 @@ hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64
     fill_epilogue(p, cont, a_bits, desc, K, scale_a, scale_a_is_scalar, scale_w, bias, alpha, acc_out, y, ydt, ldy,
                   dev_status);
 
+    if (halved != nullptr)                             // the caller has asked halved_product_covers
+        return launch_qgemm_pair_stream(a_codes, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias, alpha, y,
+                                        ldy, dev_status, st, after_quant, halved);
     if (const int ways = g_pair_gemm == 2 ? splitk_ways(cont, p, M, kBM, desc->N_pad) : 0) {
         CUtensorMap tmA;
         if (!encode_2d(&tmA, a_codes, uint64_t(row_bytes), uint64_t(M), uint64_t(lda), kBK, kBM, true)) return HQ_ERR_CUDA;
@@ -413,7 +423,7 @@ extern "C" hq_status hq_qgemm(const void* a_codes, hq_container cont, int a_bits
                               int32_t* acc_out, void* y, hq_dtype ydt, int64_t ldy, int32_t* dev_status,
                               void* stream) {
     return hq::launch_qgemm(a_codes, cont, a_bits, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias,
-                            alpha, acc_out, y, ydt, ldy, dev_status, static_cast<cudaStream_t>(stream), false);
+                            alpha, acc_out, y, ydt, ldy, dev_status, static_cast<cudaStream_t>(stream), false, nullptr);
 }
 
 extern "C" hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t Nb, int64_t H, int64_t W,

@@ -151,11 +151,15 @@ __device__ __forceinline__ bool wait_pair(uint64_t* bar, uint32_t parity, PairCt
 // tile) and takes the staging stores and the bulk stores' reads (520): together more than the 2144 cycles of a tile's MMAs.
 // NBUF: the warp's staging buffers (two used in turn, or one).
 // BN: operand-B rows (accumulator columns) of the tile.
-template <int LIMBS, int PREG = 0, int NBUF = 2, int BN = kBN>
+// HALVED (halved weights, hq_fwht.cuh): the integer is twice the accumulator plus the column's bit in `odd` (the column parities
+// of the warp, 32 to a word, zero for a row of parity 0).
+template <int LIMBS, int PREG = 0, int NBUF = 2, int BN = kBN, bool HALVED = false>
 __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg, int lane, const float* prm_sw,
                                               const float* prm_b, float sa_eff, const CUtensorMap* tmY, int col0, int row0,
                                               uint32_t tempty_leader, const float (&rsw)[PREG > 0 ? PREG * 16 : 1] = {0.f},
-                                              const float (&rb)[PREG > 0 ? PREG * 16 : 1] = {0.f}) {
+                                              const float (&rb)[PREG > 0 ? PREG * 16 : 1] = {0.f},
+                                              const uint32_t (&odd)[HALVED ? BN / 64 : 1] = {0u}) {
+    static_assert(!HALVED || LIMBS == 1, "halved weights are one limb");
     static_assert(LIMBS == 1 || BN == kBN, "narrower tiles exist with one limb");
     constexpr int NSTEPS = LIMBS == 2 ? kBN / 2 / 2 / 16 : BN / 2 / 16;
     const uint32_t wsw = (lane >> 1) & 3;
@@ -172,7 +176,8 @@ __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg
             for (int j = 0; j < 16; ++j) w[j] = int32_t(hi[j]) * 256 + int32_t(lo[j]);
         } else {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) w[j] = int32_t(hi[j]);
+            for (int j = 0; j < 16; ++j)
+                w[j] = HALVED ? int32_t(2u * hi[j] + ((odd[HALVED ? st >> 1 : 0] >> (16 * (st & 1) + j)) & 1u)) : int32_t(hi[j]);
         }
         if (st + 1 < NSTEPS) {
             tmem_ld_32x16(t_row + uint32_t((st + 1) * 16), hi);
@@ -487,6 +492,7 @@ struct PairStreamParams {
     const float* scale_w; const float* bias; float alpha;
     int pdl;
     int32_t* dev_status;
+    HalvedParity parity;               // HALVED instantiations
     // convolution geometry (CONV instantiations)
     int kb_per_tap, S, stride, pad, bw, bh, bn, tiles_w, tiles_h;
 };
@@ -518,7 +524,9 @@ __device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const void* tma
 // rounds halve (a wait, a fence, eight MMAs and a commit per 64 KB stage); three stages fit.
 // BN: operand-B rows per tile, 256, or with one limb also 192 or 128 (the host takes the width whose rounds of tiles cost
 // least, see stream_width); a narrower tile's weight half fills only part of its place in the stage.
-template <int LIMBS, bool CONV, int KPS, int BN>
+// HALVED: halved weights (hq_fwht.cuh); the further columns are the last K block of both operands.  65536 x 4096 -> 4096 1195 us
+// on two limbs, 653 so (the whole layer 1657 / 1127; tensor pipe 88 % active, 92 on two limbs).
+template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED>
 __global__ void __launch_bounds__(kPairThreads, 1)
 qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmY, const PairStreamParams p) {
@@ -646,6 +654,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         const uint32_t tempty_leader[2] = {map_to_cta(&ctl->tempty[0], 0), map_to_cta(&ctl->tempty[1], 0)};
         int last_n = -1;
         bool ok = true;
+        uint32_t col_odd[HALVED ? BN / 64 : 1] = {0u};
         if (p.pdl) griddep_wait();                    // scale_a comes from the kernel before this one
         for (int i = 0; i < count && ok; ++i) {
             const int u = c + i * G;
@@ -660,16 +669,30 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
                     prm_sw[cc] = col < p.N ? __ldg(p.scale_w + col) : 0.f;
                     prm_b[cc] = (p.bias != nullptr && col < p.N) ? __ldg(p.bias + col) : 0.f;
                 }
+                if constexpr (HALVED) {
+#pragma unroll
+                    for (int j = 0; j < BN / 64; ++j) {
+                        const int col = col_base + wc0 + 32 * j + lane;
+                        col_odd[j] = __ballot_sync(0xffffffffu, col < p.N && __ldg(p.parity.col + col) != 0);
+                    }
+                }
                 __syncwarp();
             }
             const int64_t my_row = int64_t(m2) * 256 + int(rank) * 128 + q * 32 + lane;
             const float sa = p.sa_scalar ? ld_dependent(p.scale_a) : (my_row < p.M ? ld_dependent(p.scale_a + my_row) : 0.f);
+            uint32_t odd[HALVED ? BN / 64 : 1] = {0u};
+            if constexpr (HALVED) {
+                const bool row_odd = my_row < p.M && ld_dependent_u8(p.parity.row + my_row * p.parity.pitch) != 0;
+#pragma unroll
+                for (int j = 0; j < BN / 64; ++j) odd[j] = row_odd ? col_odd[j] : 0u;
+            }
             if (!wait_pair(&ctl->tfull[as], uint32_t(i >> 1) & 1u, ctl, p.dev_status, kStatusAccumWait)) { ok = false; break; }
             tc_fence_after();
             const float sa_eff = p.alpha * sa;
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
             const uint32_t t_fast = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as * kBN + wc0);
-            epilogue_pair<LIMBS, 0, NBUF, BN>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as]);
+            epilogue_pair<LIMBS, 0, NBUF, BN, HALVED>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as],
+                                                      {0.f}, {0.f}, odd);
         }
         if (lane == 0) bulk_wait_read_all();           // shared memory must outlive the copy engine's reads
     }
@@ -760,10 +783,10 @@ int max_pairs(size_t smem) {
     return slot;
 }
 
-template <int LIMBS, bool CONV, int KPS, int BN>
+template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED = false>
 cudaError_t launch_pair_stream(int pairs_wanted, size_t smem, cudaStream_t st, const CUtensorMap& tmA, const CUtensorMap& tmB,
                                const CUtensorMap& tmY, const PairStreamParams& p) {
-    auto kern = qgemm_pair_stream_kernel<LIMBS, CONV, KPS, BN>;
+    auto kern = qgemm_pair_stream_kernel<LIMBS, CONV, KPS, BN, HALVED>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -852,12 +875,13 @@ bool pair_stream_covers_conv(hq_container cont, const gemm::GemmParams& g) {
 hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, int64_t lda, const hq_weight_desc* desc,
                                    const void* w_dev, const float* scale_a, int scale_a_is_scalar, const float* scale_w,
                                    const float* bias, float alpha, void* y, int64_t ldy, int32_t* dev_status, cudaStream_t st,
-                                   bool after_quant) {
+                                   bool after_quant, const HalvedParity* halved) {
     PairStreamParams p{};
+    if (halved != nullptr) p.parity = *halved;
     p.M = M; p.N = int(desc->N); p.limbs = desc->limbs;
     p.num_kb = int(desc->C_pad / kBK);
     p.tiles_m2 = int((M + 255) / 256);
-    const int bn = desc->limbs == 2 ? kBN : stream_width(p.tiles_m2, desc->N);
+    const int bn = desc->limbs == 2 || halved != nullptr ? kBN : stream_width(p.tiles_m2, desc->N);
     p.tiles_n = int(desc->limbs == 2 ? desc->N_pad / 128 : (desc->N + bn - 1) / bn);
     p.scale_a = scale_a; p.sa_scalar = scale_a_is_scalar; p.scale_w = scale_w; p.bias = bias; p.alpha = alpha;
     p.pdl = after_quant ? 1 : 0; p.dev_status = dev_status;
@@ -874,6 +898,7 @@ hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, in
     const int tiles = p.tiles_m2 * p.tiles_n;
     cudaError_t e;
     if (desc->limbs == 2) e = launch_pair_stream<2, false, 1, kBN>(tiles, smem, st, tmA, tmB, tmY, p);
+    else if (halved != nullptr) e = launch_pair_stream<1, false, 1, kBN, true>(tiles, smem, st, tmA, tmB, tmY, p);
     else if (kps == 2) e = bn == 192 ? launch_pair_stream<1, false, 2, 192>(tiles, smem, st, tmA, tmB, tmY, p)
                                      : launch_pair_stream<1, false, 2, 128>(tiles, smem, st, tmA, tmB, tmY, p);
     else e = launch_pair_stream_bn<1, false, 1>(bn, tiles, smem, st, tmA, tmB, tmY, p);

@@ -39,8 +39,9 @@ struct QuantParams {
     uint8_t* codes;
     int64_t ld_codes;
     float* scales;
-    uint8_t* z;          // optional second output: the codes with the k - 4 factors of H_raw that the weights leave to them
-    int64_t ld_z;        // (split_codes), one signed byte each, for the one-limb product
+    uint8_t* z;          // optional second output: the codes with the factors of H_raw that the weights leave to them
+    int64_t ld_z;        // (split_codes), one signed byte each, for the one-limb product; z_halved: and behind each row the
+    int z_halved;        // further columns of halved weights (halved_columns)
     // optional GroupNorm + SiLU applied to the values as they are loaded (gn_stats == nullptr: off)
     const float* gn_stats;   // [samples][groups][2]: mean, 1/sqrt(var + eps)
     const float* gn_gamma;   // [cols]
@@ -326,14 +327,25 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
             if (!STATIC) { if (tr == 0) p.scales[row] = scale; }
             else if (row == 0 && tr == 0) p.scales[0] = scale;
         }
-        if constexpr (split_block_ok(KLOG)) {              // E = 32 here: the thread's codes are 32 consecutive channels
+        if constexpr (split_block_ok(KLOG) || (split_wide(KLOG) && PRO == 0)) {      // the thread's codes are E consecutive channels
             if (p.z != nullptr) {
-                uint32_t zw[8];
-                split_codes<KLOG, INT8_OUT>(w, zw);
                 uint4* zd = reinterpret_cast<uint4*>(p.z + row * p.ld_z + int64_t(blk) * N + E * tb);
-                zd[0] = make_uint4(zw[0], zw[1], zw[2], zw[3]);
-                zd[1] = make_uint4(zw[4], zw[5], zw[6], zw[7]);
+#pragma unroll
+                for (int h = 0; h < E / 32; ++h) {
+                    uint32_t c[INT8_OUT ? 8 : 4], zw[8];
+#pragma unroll
+                    for (int i = 0; i < (INT8_OUT ? 8 : 4); ++i) c[i] = w[h * (INT8_OUT ? 8 : 4) + i];
+                    split_codes<KLOG, INT8_OUT>(c, zw);
+                    zd[2 * h] = make_uint4(zw[0], zw[1], zw[2], zw[3]);
+                    zd[2 * h + 1] = make_uint4(zw[4], zw[5], zw[6], zw[7]);
+                }
             }
+        }
+    }
+    if constexpr (split_halved(KLOG) && PRO == 0) {        // a row is one Hadamard block here (m = 1)
+        if (p.z_halved) {
+            const uint4 c = halved_columns<KLOG, INT8_OUT>(w, reinterpret_cast<uint32_t*>(smem_raw) + row_in_cta * 16, tb);
+            if (valid && tb < kHalvedCols / 16) *reinterpret_cast<uint4*>(p.z + row * p.ld_z + N + 16 * tb) = c;
         }
     }
 }
@@ -1004,8 +1016,9 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
             p.ln_table = ln_table(*ln, grid, threads, E, smem + table);
             if (p.ln_table) smem += table;
         }
-        if (zo != nullptr && zo->z != nullptr && split_block_ok(klog) && split_fits(klog, bits)) {
-            p.z = zo->z; p.ld_z = zo->ld;
+        if (zo != nullptr && zo->z != nullptr && (split_block_ok(klog) || (split_wide(klog) && gn == nullptr && ln == nullptr)) && split_fits(klog, bits) &&
+            (!zo->halved || (split_halved(klog) && p.m == 1))) {
+            p.z = zo->z; p.ld_z = zo->ld; p.z_halved = zo->halved;
             zo->written = true;
         }
         cudaError_t e = xdt == HQ_F32
