@@ -97,6 +97,25 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
     return f;
 }
 
+// Every lane's four 16-byte pieces to 64 contiguous bytes at its `dst` (nullptr: nowhere).  Stored by the lanes that hold them, each
+// store instruction of a warp would fill half sectors only; so they change lanes through `stage` (the warp's, five slots a lane)
+// and a lane stores pieces of others, whose addresses it asks them for.  Taken at 4096-channel blocks, whose transform waits for
+// its two-warp barriers and has issue slots to spare (65536 x 4096 fp32 248 -> 232 us, bf16 208 -> 201); one-warp blocks of 32
+// values a thread lose by it (65536 x 1152 bf16 55 -> 64 us, 65536 x 256 12.6 -> 13.3), 1024 and 2048 are level.
+__host__ __device__ constexpr bool staged_stores(int klog, bool int8_out) { return klog == 12 && int8_out; }
+__device__ __forceinline__ void store_staged(const uint4 (&w)[4], uint4* stage, uint8_t* dst) {
+    const int lane = threadIdx.x & 31, part = lane & 3;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) stage[lane * 5 + i] = w[i];
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int from = 8 * i + lane / 4;
+        uint8_t* d = reinterpret_cast<uint8_t*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(dst), from));
+        if (d != nullptr) reinterpret_cast<uint4*>(d)[part] = stage[from * 5 + part];
+    }
+}
+
 // Fast path.  A Hadamard block of n = 2^KLOG channels is owned by TB = n / E threads that hold E values each, as
 // E/2 two-wide registers (butterflies between pairs are one instruction per two values).
 //   phase A  thread t holds the float4s {t + TB i}: coalesced 16-byte loads; the E-point in-register transform
@@ -318,16 +337,43 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     constexpr int NW = INT8_OUT ? E / 4 : E / 8;       // packed words per thread
     uint32_t w[NW];
     pack_codes<KLOG, E, INT8_OUT, STATIC>(v, inv, p.bits, tb, w);
-    if (valid) {
-        uint8_t* dst = p.codes + row * p.ld_codes + (int64_t(blk) * N + E * tb) / (INT8_OUT ? 1 : 2);
+    constexpr bool STAGED = staged_stores(KLOG, INT8_OUT);
+    // the warp's half of its block's exchange buffer, whose values both warps have read (dynamic scales: at the row maximum)
+    uint4* stage = reinterpret_cast<uint4*>(smem_raw + (STAGED ? size_t(tid >> 5) * (GS * 8) : 0));
+    if constexpr (STAGED) {
+        if (STATIC) __syncthreads();
+        uint4 c4[4];
 #pragma unroll
-        for (int i = 0; i < NW / 4; ++i)
-            reinterpret_cast<uint4*>(dst)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+        for (int i = 0; i < 4; ++i) c4[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+        store_staged(c4, stage, valid ? p.codes + row * p.ld_codes + int64_t(blk) * N + E * tb : nullptr);
+        if constexpr (PRO == 0) {
+            if (p.z != nullptr) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t c[8], zw[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) c[i] = w[8 * h + i];
+                    split_codes<KLOG, true>(c, zw);
+                    c4[2 * h] = make_uint4(zw[0], zw[1], zw[2], zw[3]);
+                    c4[2 * h + 1] = make_uint4(zw[4], zw[5], zw[6], zw[7]);
+                }
+                __syncwarp();
+                store_staged(c4, stage, valid ? p.z + row * p.ld_z + int64_t(blk) * N + E * tb : nullptr);
+            }
+        }
+    }
+    if (valid) {
+        if constexpr (!STAGED) {
+            uint8_t* dst = p.codes + row * p.ld_codes + (int64_t(blk) * N + E * tb) / (INT8_OUT ? 1 : 2);
+#pragma unroll
+            for (int i = 0; i < NW / 4; ++i)
+                reinterpret_cast<uint4*>(dst)[i] = make_uint4(w[4 * i], w[4 * i + 1], w[4 * i + 2], w[4 * i + 3]);
+        }
         if (p.scales != nullptr) {
             if (!STATIC) { if (tr == 0) p.scales[row] = scale; }
             else if (row == 0 && tr == 0) p.scales[0] = scale;
         }
-        if constexpr (split_block_ok(KLOG) || (split_wide(KLOG) && PRO == 0)) {      // the thread's codes are E consecutive channels
+        if constexpr (!STAGED && (split_block_ok(KLOG) || (split_wide(KLOG) && PRO == 0))) {      // the thread's codes are E consecutive channels
             if (p.z != nullptr) {
                 uint4* zd = reinterpret_cast<uint4*>(p.z + row * p.ld_z + int64_t(blk) * N + E * tb);
 #pragma unroll
