@@ -123,10 +123,9 @@ struct LayerCodes {
         return more == desc->N_pad * desc->RS * desc->C_pad ? kBytes
              : more == desc->N_pad * (desc->C_pad + kHalvedCols + 1) ? kHalved : kNone;
     }
-    // Per-pixel scales under a window drain the accumulator per tap, 64 columns a warp: nothing to gain from one limb.
     static bool split_taken(const hq_weight_desc* desc, int a_bits, hq_scale_mode mode, int64_t rows, int64_t cols, int stride) {
         const Section sec = section(desc, a_bits, cols);
-        return (mode == HQ_SCALE_STATIC || desc->RS == 1) && sec != kNone &&
+        return sec != kNone &&
                split_pays(desc, rows, cols, rows / (stride == 2 ? 4 : 1), sec == kHalved ? kHalvedCols / 128 : 0);
     }
     // One limb halves the column tiles (or the weights a CTA of the split kernel streams), and the transform kernel computes
@@ -202,7 +201,9 @@ extern "C" hq_status hq_layer_workspace_size(const hq_weight_desc* desc, int a_b
     const hq_container cont = hq_container(desc->container);
     const hq_status s = layer_bytes(rows, desc->C, cont, bytes);
     if (s != HQ_OK) return s;
-    if (desc->had_block <= 512 && LayerCodes::split_taken(desc, a_bits, mode, rows, desc->C, stride)) *bytes = size_t(split_bytes(rows, desc->C, cont));
+    if (desc->had_block <= 512 && (mode == HQ_SCALE_STATIC || desc->RS == 1) &&
+        LayerCodes::split_taken(desc, a_bits, mode, rows, desc->C, stride))
+        *bytes = size_t(split_bytes(rows, desc->C, cont));
     return HQ_OK;
 }
 

@@ -213,9 +213,10 @@ namespace {
 // Ring depth and weight residency for a problem; fills p.stages / p.b_resident and returns the shared-memory size.
 size_t plan_smem(GemmParams& p, bool frag) {
     const int num_kb = p.kb_per_tap * p.taps;
-    p.b_resident = num_kb <= kResidentKb ? 1 : 0;
+    p.b_resident = num_kb <= kResidentKb && !p.per_tap ? 1 : 0;
+    const int b_bytes = (p.per_tap ? per_tap_rows(p.limbs) : kBN) * kBK;
     for (int stages = kMaxStages; stages >= 2; --stages) {
-        const SmemLayout L = smem_layout(stages, p.b_resident != 0, num_kb, frag);
+        const SmemLayout L = smem_layout(stages, p.b_resident != 0, num_kb, frag, b_bytes);
         if (L.total <= kSmemLimit) { p.stages = stages; return size_t(L.total); }
     }
     return 0;
@@ -368,7 +369,7 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     GemmParams p{};
     p.N = int(desc->N); p.limbs = desc->limbs;
     p.kb_per_tap = int(desc->C_pad / kBK); p.taps = R * S;
-    p.pdl = (after_quant && !per_tap) ? 1 : 0;       // a per-tap layer may take several launches: keep those plain
+    p.pdl = after_quant ? 1 : 0;
     p.conv = 1; p.Nb = int(Nb); p.H = int(H); p.W = int(W); p.Ho = int(Ho); p.Wo = int(Wo);
     p.R = R; p.S = S; p.stride = stride; p.pad = pad;
     p.bw = int(Wo < kBM ? Wo : kBM);
@@ -381,7 +382,7 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     p.tiles_h = int((Ho + p.bh - 1) / p.bh);
     const int tiles_nb = int((Nb + p.bn - 1) / p.bn);
     p.tiles_m = p.tiles_w * p.tiles_h * tiles_nb;
-    p.tiles_n = int(desc->limbs == 2 ? desc->N_pad / 128 : (desc->N_pad + 255) / 256);
+    p.tiles_n = int(desc->limbs == 2 || per_tap ? desc->N_pad / 128 : (desc->N_pad + 255) / 256);
     const bool nib = cont == HQ_CODES_NIBBLE;
     const int box_rows = p.bw * p.bh * p.bn;
     p.a_box_bytes = uint32_t(box_rows) * (nib ? kBK / 2 : kBK);
@@ -405,14 +406,10 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     if (!encode_4d(&tmA, a_codes, dims, box, estr, !nib)) return HQ_ERR_CUDA;
     if (ways > 0) return launch_qgemm_splitk(p, ways, box_rows, Nb * Ho * Wo, tmA, desc, w_dev, st);
     const uint64_t Kp = uint64_t(desc->C_pad) * desc->RS;
-    if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, kBN, true)) return HQ_ERR_CUDA;
+    if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, uint32_t(per_tap ? per_tap_rows(desc->limbs) : kBN), true))
+        return HQ_ERR_CUDA;
     if (g_pair_gemm && pair_stream_covers_conv(cont, p)) return launch_qconv_pair(p, tmA, tmY, desc, w_dev, st);
-    s = launch(nib, tmA, tmB, tmY, p, st);
-    if (s == HQ_OK && per_tap && desc->limbs == 1) {      // the other 64 of every warp's 128 columns
-        p.col_pass = 1;
-        s = launch(nib, tmA, tmB, tmY, p, st);
-    }
-    return s;
+    return launch(nib, tmA, tmB, tmY, p, st);
 }
 
 }  // namespace hq

@@ -55,12 +55,16 @@ struct GemmParams {
     int32_t* acc_out; void* y; int y_bf16; int64_t ldy;
     int y_vec_ok, acc_vec_ok;
     int per_tap;          // convolution with one activation scale per input pixel: the accumulator is drained per filter tap
-    int col_pass;         // per_tap with one weight limb: which 64 of a warp's 128 columns this launch produces
     int pdl;              // launched ahead of the completion of the kernel that produces the codes and scale_a
     int frag;             // fragment-layout epilogue + second MMA issuer (see use_frag)
     int tma_store;        // bf16 output goes out through bulk tensor stores (rows of a tile are consecutive output rows)
     int32_t* dev_status;
 };
+
+// Operand-B rows of a tile that is drained per filter tap: 128 output channels, 64 a warp, are what the running sums' registers
+// hold, whatever the limbs.  One limb in one launch of such tiles / in two of 256 rows (64 columns a warp each): 8 x 32 x 32 x 256
+// 3x3 15.4 / 31.6 us, 64 x 32 x 32 x 512 212 / 242.
+__host__ __device__ constexpr int per_tap_rows(int limbs) { return limbs == 1 ? kBN / 2 : kBN; }
 
 struct SharedCtl {
     uint64_t full[kMaxStages];
@@ -79,10 +83,11 @@ struct SharedCtl {
 // Shared-memory carve-up (all offsets from a 1024-byte aligned base).
 struct SmemLayout { int b_off, a_off, staging_off, param_off, ctl_off, total; };
 // `frag`: the fragment-layout fast epilogue (two staging buffers per warp, column parameters in registers).
-__host__ __device__ inline SmemLayout smem_layout(int stages, bool resident, int num_kb, bool frag) {
+// `b_bytes`: a weight K block (see per_tap_rows).
+__host__ __device__ inline SmemLayout smem_layout(int stages, bool resident, int num_kb, bool frag, int b_bytes) {
     SmemLayout L;
     L.b_off = 0;
-    L.a_off = (resident ? num_kb : stages) * kBBytes;
+    L.a_off = (resident ? num_kb : stages) * b_bytes;
     L.staging_off = L.a_off + stages * kABytes;
     L.param_off = L.staging_off + kEpiWarps * kStagingBytes * (frag ? 2 : 1);
     L.ctl_off = L.param_off + (frag ? 0 : kParamBytes);
@@ -515,6 +520,8 @@ __global__ void __launch_bounds__(cta_threads(NIBBLE, FRAG), 1)
 qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const __grid_constant__ CUtensorMap tmY, const GemmParams p) {
     constexpr bool PERTAP = MODE == kModePerTap;
+    static_assert(!PERTAP || LIMBS_T != 0, "the per-tap drain is compiled per number of limbs");
+    constexpr int BN = PERTAP ? per_tap_rows(LIMBS_T) : kBN, kBBlock = BN * kBK;      // operand-B rows of a tile, bytes of a K block
     static_assert(!FRAG || (MODE == kModeFast && !NIBBLE), "the fragment-layout epilogue exists for the fast mode with one code per byte");
     // MMA-issuing warps: two (warp 1 and the CTA's last warp) together with the fragment-layout epilogue, else one
     constexpr int ISSUERS = FRAG ? 2 : 1;
@@ -524,7 +531,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int num_kb = p.kb_per_tap * p.taps;
-    const SmemLayout L = smem_layout(p.stages, resident, num_kb, FRAG);
+    const SmemLayout L = smem_layout(p.stages, resident, num_kb, FRAG, kBBlock);
     unsigned char* sB = smem + L.b_off;
     unsigned char* sA = smem + L.a_off;
     unsigned char* sStage = smem + L.staging_off;
@@ -575,8 +582,8 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     if (reloads > 0 &&
                         !wait_or_abort(&ctl->bfree, uint32_t(reloads - 1) & 1u, ctl, p.dev_status, kStatusEmptyWait)) { ok = false; break; }
                     for (int kb = 0; kb < num_kb; ++kb) {
-                        mbar_expect_tx(&ctl->bfull[kb], kBBytes);
-                        tma_load_2d(sB + kb * kBBytes, &tmB, &ctl->bfull[kb], kb * kBK, tc.n_tile * kBN);
+                        mbar_expect_tx(&ctl->bfull[kb], kBBlock);
+                        tma_load_2d(sB + kb * kBBlock, &tmB, &ctl->bfull[kb], kb * kBK, tc.n_tile * BN);
                     }
                     cur_n = tc.n_tile; ++reloads;
                 }
@@ -589,7 +596,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     uint64_t* fbar = (ISSUERS == 2 && (i & 1)) ? &ctl->full2[stage] : &ctl->full[stage];
                     if (ISSUERS == 2 && (i & 1)) { last_fill |= 1u << stage; par_b ^= 1u << stage; }
                     else { last_fill &= ~(1u << stage); par_a ^= 1u << stage; }
-                    mbar_expect_tx(fbar, p.a_box_bytes + (resident ? 0u : uint32_t(kBBytes)));
+                    mbar_expect_tx(fbar, p.a_box_bytes + (resident ? 0u : uint32_t(kBBlock)));
                     unsigned char* a_dst = sA + stage * kABytes + (NIBBLE ? kABytes - kRawBytes : 0);
                     const int a_k = (NIBBLE ? kBK / 2 : kBK);
                     if (CONV) {
@@ -600,7 +607,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     } else {
                         tma_load_2d(a_dst, &tmA, fbar, kb * a_k, tc.m_tile * kBM);
                     }
-                    if (!resident) tma_load_2d(sB + stage * kBBytes, &tmB, fbar, kb * kBK, tc.n_tile * kBN);
+                    if (!resident) tma_load_2d(sB + stage * kBBlock, &tmB, fbar, kb * kBK, tc.n_tile * BN);
                     ++armed;
                     if (++stage == nstages) { stage = 0; phase ^= 1; }
                 }
@@ -628,7 +635,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         if (lane == 0) {
             const int me = warp == 1 ? 0 : 1;
             uint64_t* fullbar = me ? ctl->full2 : ctl->full;
-            const uint32_t idesc = make_idesc_i8(kBM, kBN);
+            const uint32_t idesc = make_idesc_i8(kBM, BN);
             int stage = 0; uint32_t phase = 0;            // position in the ring (phase: the unpack barriers' parity)
             uint32_t par = 0;                             // per stage: parity of the next phase of this issuer's barrier
             int cur_n = -1, reloads = 0;
@@ -671,7 +678,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                             }
                             tc_fence_after();
                             const uint64_t a_desc = make_sw128_kmajor_desc(smem_u32(sA + stage * kABytes));
-                            const uint64_t b_desc = make_sw128_kmajor_desc(smem_u32(sB + (resident ? kb : stage) * kBBytes));
+                            const uint64_t b_desc = make_sw128_kmajor_desc(smem_u32(sB + (resident ? kb : stage) * kBBlock));
 #pragma unroll
                             for (int k = 0; k < kBK / 32; ++k)
                                 mma_i8(d_tmem, a_desc + uint64_t(k * 2), b_desc + uint64_t(k * 2), idesc, (kk | k) != 0 ? 1u : 0u);
@@ -699,7 +706,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
         unsigned char* stg = sStage + (warp - 2) * kStagingBytes;
         float* prm_sw = sParam + (warp - 2) * 2 * (kBN / 2);
         float* prm_b = prm_sw + kBN / 2;
-        const int cols_per_tile = limbs == 2 ? kBN / 2 : kBN;
+        const int cols_per_tile = limbs == 2 ? kBN / 2 : BN;
         const int cols_per_warp = cols_per_tile / 2;
         const bool want_y = MODE == kModeFast ? true : p.y != nullptr;
         const bool want_acc = MODE == kModeFast ? false : p.acc_out != nullptr;
@@ -729,8 +736,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
             if (PERTAP) {
                 // One scale per INPUT pixel: every filter tap's integer sum is drained on its own, multiplied by the
                 // scale of the pixel that tap read for this output pixel, and added up in fp32 registers (64 columns
-                // per warp and launch).  y = alpha * S_w[o] * sum_taps S_a[pix(tap)] * acc_tap + bias[o].
-                const int pc0 = limbs == 2 ? wc0 : wc0 + p.col_pass * 64;   // first column (in the tile) handled here
+                // per warp).  y = alpha * S_w[o] * sum_taps S_a[pix(tap)] * acc_tap + bias[o].
                 const int r_tile = q * 32 + lane;
                 const int iw = r_tile % p.bw, ih = (r_tile / p.bw) % p.bh, in_ = r_tile / (p.bw * p.bh);
                 const int n = tc.n0 + in_, ho = tc.h0 + ih, wo = tc.w0 + iw;
@@ -740,7 +746,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     const int r = g / p.S, sx = g - r * p.S;
                     const int hi_ = ho * p.stride + r - p.pad, wi_ = wo * p.stride + sx - p.pad;
                     if (!row_ok || hi_ < 0 || hi_ >= p.H || wi_ < 0 || wi_ >= p.W) return 0.f;
-                    return __ldg(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);      // never a dependent launch (pdl = 0)
+                    return ld_dependent(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);
                 };
                 float run[64];
 #pragma unroll
@@ -753,7 +759,7 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                     if (g + 1 < p.taps) s_next = tap_scale(g + 1);
                     if (!wait_or_abort(&ctl->tfull[as2], uint32_t(seq >> 1) & 1u, ctl, p.dev_status, kStatusAccumWait)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t t_tap = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as2 * kBN + pc0);
+                    const uint32_t t_tap = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as2 * kBN + wc0);
                     uint32_t hi[16], lo[16];
                     tmem_ld_32x16(t_tap, hi);
                     if (limbs == 2) tmem_ld_32x16(t_tap + uint32_t(kBN / 2), lo);
@@ -790,15 +796,14 @@ qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
                 if (!ok) break;
                 if (my_out >= 0) {
                     const float a_eff = p.combine_fast ? p.alpha / float(1 << p.a_shift) : p.alpha;
-                    const int prm0 = pc0 - wc0;                    // offset into the warp's staged column parameters
                     unsigned char* y_row = static_cast<unsigned char*>(p.y) + int64_t(my_out) * p.ldy * (p.y_bf16 ? 2 : 4);
 #pragma unroll
                     for (int st = 0; st < 4; ++st) {
                         uint32_t f[16];
 #pragma unroll
                         for (int j = 0; j < 16; ++j)
-                            f[j] = __float_as_uint(fmaf(run[st * 16 + j] * prm_sw[prm0 + st * 16 + j], a_eff, prm_b[prm0 + st * 16 + j]));
-                        const int col = col_base + pc0 + st * 16;
+                            f[j] = __float_as_uint(fmaf(run[st * 16 + j] * prm_sw[st * 16 + j], a_eff, prm_b[st * 16 + j]));
+                        const int col = col_base + wc0 + st * 16;
                         if (col < p.N) {
                             if (p.y_bf16) store_row16<2>(y_row, f, col, p.N, p.y_vec_ok != 0);
                             else store_row16<4>(y_row, f, col, p.N, p.y_vec_ok != 0);
@@ -1018,7 +1023,9 @@ cudaError_t dispatch(int mode, int grid, size_t smem, cudaStream_t st, const CUt
                             : launch_one<NIBBLE, kModeFast, CONV, 1, 0>(grid, smem, st, tmA, tmB, tmY, p);
     }
     if (mode == kModePerTap) {
-        if constexpr (CONV) return launch_one<NIBBLE, kModePerTap, true, 0, -1>(grid, smem, st, tmA, tmB, tmY, p);
+        if constexpr (CONV)
+            return p.limbs == 1 ? launch_one<NIBBLE, kModePerTap, true, 1, 0>(grid, smem, st, tmA, tmB, tmY, p)
+                                : launch_one<NIBBLE, kModePerTap, true, 2, 0>(grid, smem, st, tmA, tmB, tmY, p);
         else return cudaErrorInvalidValue;
     }
     return launch_one<NIBBLE, kModeGeneric, CONV, 0, -1>(grid, smem, st, tmA, tmB, tmY, p);
