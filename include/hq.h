@@ -302,6 +302,20 @@ hq_status hq_qconv_cat(const void* x, const void* x2, int64_t C1, hq_dtype xdt, 
                        const hq_weight_desc* desc, const void* w_dev, int R, int S, int stride, int pad,
                        const float* scale_w, const float* bias, int a_bits, hq_scale_mode mode, const float* static_scale,
                        void* y, hq_dtype ydt, void* workspace, size_t ws_bytes, int32_t* dev_status, void* stream);
+/* ---- Fused layers with a residual connection: y = bf16(bf16(layer) + residual), the same bits as hq_add on the stored output.
+ * residual: device, bf16, the shape of y (dense), not y itself; N a multiple of 8, both 16-byte aligned.  The product kernel adds it
+ * as it stores; where the product runs on a kernel that does not, hq_add is launched behind it.  One scale per row (linear);
+ * bf16 output.  pre_bias may have a pitch of its own: ld_pre_bias elements (a multiple of 4, at least C) between samples. */
+hq_status hq_qlinear_add(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc,
+                         const void* w_dev, const float* scale_w, const float* bias, int a_bits, const void* residual, void* y,
+                         void* workspace, size_t ws_bytes, int32_t* dev_status, void* stream);
+hq_status hq_gn_silu_qconv_add(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C, int groups,
+                               const float* gamma, const float* beta, const void* pre_bias, int64_t ld_pre_bias, float eps, const hq_weight_desc* desc,
+                               const void* w_dev, int R, int S, int stride, int pad, const float* scale_w, const float* bias,
+                               int a_bits, hq_scale_mode mode, const float* static_scale, const void* residual, void* y,
+                               void* workspace, size_t ws_bytes, void* scratch, size_t scratch_bytes, int32_t* dev_status,
+                               void* stream);
+
 
 /* ---- Fused linear layer with GroupNorm (optionally + SiLU) in front, on the pixels of an NHWC tensor: the QKV
  * projection of an attention block (no counterpart in the paper's equations; the paper quantizes the projection, the

@@ -28,7 +28,8 @@ EXPORTS = ["hq_version", "hq_status_string", "hq_check_status", "hq_hadamard_qua
            "hq_ln_quant", "hq_ln_qlinear", "hq_gn_silu_qconv", "hq_gn_qlinear", "hq_silu", "hq_add", "hq_add_rows_bcast",
            "hq_class_embed_add", "hq_timestep_embedding", "hq_upsample_nearest2x", "hq_concat_channels", "hq_groupnorm_act",
            "hq_conv2d_direct", "hq_attention", "hq_hadamard_quant_width2", "hq_qlinear_fused", "hq_set_pair_gemm", "hq_mma_i8_probe_pair",
-           "hq_hadamard_quant_cat", "hq_gn_silu_quant_cat", "hq_gn_silu_qconv_cat", "hq_qconv_cat"]
+           "hq_hadamard_quant_cat", "hq_gn_silu_quant_cat", "hq_gn_silu_qconv_cat", "hq_qconv_cat",
+           "hq_qlinear_add", "hq_gn_silu_qconv_add"]
 HQ_NOALLOC_SCRATCH_BYTES = 8 * 1024 * 1024
 
 
@@ -92,6 +93,9 @@ def _load():
                                    i32, p, p, i32, i32, p, p, i32, p, C.c_size_t, p, C.c_size_t, p, p]
     L.hq_gn_qlinear.argtypes = [p, i32, i64, i64, i64, i32, p, p, C.c_float, i32, C.POINTER(WeightDesc), p, p, p, i32, p, i32,
                                 i64, p, C.c_size_t, p, C.c_size_t, p, p]
+    L.hq_qlinear_add.argtypes = [p, i32, i64, i64, i64, C.POINTER(WeightDesc), p, p, p, i32, p, p, p, C.c_size_t, p, p]
+    L.hq_gn_silu_qconv_add.argtypes = [p, i32, i64, i64, i64, i64, i32, p, p, p, i64, C.c_float, C.POINTER(WeightDesc), p, i32, i32, i32,
+                                       i32, p, p, i32, i32, p, p, p, p, C.c_size_t, p, C.c_size_t, p, p]
     L.hq_silu.argtypes = [p, i64, p, p]
     L.hq_add.argtypes = [p, p, i64, p, p]
     L.hq_add_rows_bcast.argtypes = [p, p, i64, i64, i64, p]
@@ -117,7 +121,8 @@ def _load():
                  "hq_hadamard_quant_width", "hq_qconv_width", "hq_gn_silu_quant", "hq_ln_quant", "hq_ln_qlinear", "hq_gn_silu_qconv",
                  "hq_gn_qlinear", "hq_silu", "hq_add", "hq_add_rows_bcast", "hq_class_embed_add", "hq_timestep_embedding",
                  "hq_upsample_nearest2x", "hq_concat_channels", "hq_groupnorm_act", "hq_conv2d_direct", "hq_attention",
-                 "hq_hadamard_quant_cat", "hq_gn_silu_quant_cat", "hq_gn_silu_qconv_cat", "hq_qconv_cat"):
+                 "hq_hadamard_quant_cat", "hq_gn_silu_quant_cat", "hq_gn_silu_qconv_cat", "hq_qconv_cat",
+                 "hq_qlinear_add", "hq_gn_silu_qconv_add"):
         getattr(L, name).restype = C.c_int
     return L
 
@@ -268,8 +273,17 @@ def hq_layer_workspace_size(pw: PreparedWeight, a_bits: int, rows: int, static: 
 
 
 def hq_qlinear(x, pw: PreparedWeight, bias, a_bits: int, y, workspace, static_scale=None, dev_status=None,
-               stream=None) -> None:
+               stream=None, residual=None) -> None:
+    """residual: bf16 tensor of y's shape added to the rounded output (y bf16 and dense, one scale per row), or None."""
     M, K = x.shape
+    if residual is not None:
+        if static_scale is not None or y.element_size() != 2 or not (y.is_contiguous() and residual.is_contiguous()) or \
+                residual.shape != y.shape or residual.dtype != y.dtype:
+            raise ValueError("hq_qlinear: a residual goes with a dense bf16 output of its shape and one scale per row")
+        _check(lib.hq_qlinear_add(_dptr(x), _dtype_code(x), M, K, x.stride(0), C.byref(pw.desc), _dptr(pw.blob_dev),
+                                  _dptr(pw.s_w_dev), _dptr(bias), a_bits, _dptr(residual), _dptr(y), _dptr(workspace),
+                                  workspace.nbytes, _dptr(dev_status), _stream(stream)), "hq_qlinear_add")
+        return
     mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
     _check(lib.hq_qlinear(_dptr(x), _dtype_code(x), M, K, x.stride(0), C.byref(pw.desc), _dptr(pw.blob_dev),
                           _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode, _dptr(static_scale), _dptr(y), _dtype_code(y),
@@ -328,11 +342,22 @@ def hq_gn_silu_quant(x, groups: int, gamma, beta, eps: float, had_block: int, bi
 
 def hq_gn_silu_qconv(x, groups: int, gamma, beta, eps: float, pw: PreparedWeight, R: int, S: int, stride: int, pad: int,
                      bias, a_bits: int, y, workspace, scratch, static_scale=None, dev_status=None, stream=None,
-                     pre_bias=None, x2=None) -> None:
+                     pre_bias=None, x2=None, residual=None) -> None:
     """The fused convolution layer with GroupNorm + SiLU in front (x NHWC; pre_bias: bf16 [Nb, C] added to x before the
-    normalisation, or None; x2: the input is the channel concatenation [x | x2], read in place)."""
+    normalisation, or None; x2: the input is the channel concatenation [x | x2], read in place; residual: bf16 tensor of y's
+    shape added to the rounded output, or None -- with it y is bf16 and x2 None)."""
     Nb, H, W, Cin = x.shape
     mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
+    if residual is not None:
+        if x2 is not None or y.element_size() != 2 or not (y.is_contiguous() and residual.is_contiguous()) or \
+                residual.shape != y.shape or residual.dtype != y.dtype:
+            raise ValueError("hq_gn_silu_qconv: a residual goes with a dense bf16 output of its shape and a single input")
+        _check(lib.hq_gn_silu_qconv_add(_dptr(x), _dtype_code(x), Nb, H, W, Cin, groups, _dptr(gamma), _dptr(beta), _dptr(pre_bias),
+                                        Cin if pre_bias is None else pre_bias.stride(0), eps, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias),
+                                        a_bits, mode, _dptr(static_scale), _dptr(residual), _dptr(y), _dptr(workspace),
+                                        workspace.nbytes, _dptr(scratch), scratch.nbytes, _dptr(dev_status), _stream(stream)),
+               "hq_gn_silu_qconv_add")
+        return
     if x2 is not None:
         _check(lib.hq_gn_silu_qconv_cat(_dptr(x), _dptr(x2), Cin, _dtype_code(x), Nb, H, W, Cin + x2.shape[3], groups,
                                         _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps, C.byref(pw.desc), _dptr(pw.blob_dev),

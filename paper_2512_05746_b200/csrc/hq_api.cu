@@ -17,19 +17,19 @@ hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64
                        const hq_weight_desc* desc, const void* w_dev, const float* scale_a, int scale_a_is_scalar,
                        const float* scale_w, const float* bias, float alpha, int32_t* acc_out, void* y,
                        hq_dtype ydt, int64_t ldy, int32_t* dev_status, cudaStream_t st, bool after_quant,
-                       const HalvedParity* halved = nullptr);
+                       const HalvedParity* halved = nullptr, ResidualAdd* res = nullptr);
 bool halved_product_covers(int64_t M, const void* y, hq_dtype ydt, int64_t ldy);      // hq_gemm.cu
 hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t Nb, int64_t H, int64_t W,
                          int64_t C, const hq_weight_desc* desc, const void* w_dev, int R, int S, int stride, int pad,
                          const float* scale_a, int scale_a_is_scalar, const float* scale_w, const float* bias,
                          float alpha, int32_t* acc_out, void* y, hq_dtype ydt, int32_t* dev_status, cudaStream_t st,
-                         bool after_quant);
+                         bool after_quant, ResidualAdd* res = nullptr);
 
 hq_status launch_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C, int groups,
                                const float* gamma, const float* beta, float eps, int had_block, int bits,
                                hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont,
                                int64_t ld_codes, float* scales, void* scratch, size_t scratch_bytes, cudaStream_t st,
-                               int silu, const void* pre_bias, const void* x2, int64_t split, SplitOut* zo = nullptr);
+                               int silu, const void* pre_bias, int64_t pre_ld, const void* x2, int64_t split, SplitOut* zo = nullptr);
 hq_status launch_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, int64_t ldx2, int64_t split, hq_dtype xdt,
                                     int64_t rows, int64_t cols, int had_block, int bits, hq_scale_mode mode,
                                     const float* static_scale, void* codes, hq_container cont, int64_t ld_codes,
@@ -150,6 +150,19 @@ struct LayerCodes {
     int64_t k(int64_t K) const { return z.written && z.halved ? K + kHalvedCols : K; }
     const HalvedParity* halved() const { return z.written && z.halved ? &parity : nullptr; }
 };
+
+// A residual that a fused layer call adds to its bf16 output: checked before anything is launched, added by the product kernel
+// where that takes it and by a launch of its own where not (other kernels, and halved weights).
+hq_status check_residual(const void* residual, const void* y, hq_dtype ydt, int64_t N, int64_t ldy) {
+    if (residual == nullptr) return HQ_OK;
+    if (residual == y || ydt != HQ_BF16) return HQ_ERR_INVALID_ARG;
+    if (N % 8 != 0 || ldy != N) return HQ_ERR_SHAPE;
+    return aligned16(residual) && aligned16(y) ? HQ_OK : HQ_ERR_ALIGNMENT;
+}
+hq_status finish_residual(hq_status s, const ResidualAdd& res, void* y, int64_t count, void* stream) {
+    if (s != HQ_OK || res.r == nullptr || res.done) return s;
+    return hq_add(y, res.r, count, y, stream);
+}
 }  // namespace
 }  // namespace hq
 
@@ -207,11 +220,10 @@ extern "C" hq_status hq_layer_workspace_size(const hq_weight_desc* desc, int a_b
     return HQ_OK;
 }
 
-extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx,
-                                const hq_weight_desc* desc, const void* w_dev, const float* scale_w,
-                                const float* bias, int a_bits, hq_scale_mode mode, const float* static_scale, void* y,
-                                hq_dtype ydt, int64_t ldy, void* workspace, size_t ws_bytes, int32_t* dev_status,
-                                void* stream) {
+static hq_status qlinear_impl(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc,
+                              const void* w_dev, const float* scale_w, const float* bias, int a_bits, hq_scale_mode mode,
+                              const float* static_scale, void* y, hq_dtype ydt, int64_t ldy, const void* residual, void* workspace,
+                              size_t ws_bytes, int32_t* dev_status, void* stream) {
     using namespace hq;
     if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
@@ -220,13 +232,35 @@ extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t 
     hq_status s = layer_bytes(M, K, cont, &need);
     if (s != HQ_OK) return s;
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
+    s = check_residual(residual, y, ydt, desc->N, ldy);
+    if (s != HQ_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    ResidualAdd res{static_cast<const __nv_bfloat16*>(residual), false};
     LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, workspace, ws_bytes, halved_product_covers(M, y, ydt, ldy));
     s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
                               &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, lc.k(K), lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
-                        hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true, lc.halved());
+    s = launch_qgemm(lc.a(), lc.container(cont), a_bits, M, lc.k(K), lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, mode == HQ_SCALE_STATIC, scale_w, bias,
+                     hq_alpha_for(desc), nullptr, y, ydt, ldy, dev_status, st, true, lc.halved(), residual != nullptr ? &res : nullptr);
+    return finish_residual(s, res, y, M * desc->N, stream);
+}
+
+extern "C" hq_status hq_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx,
+                                const hq_weight_desc* desc, const void* w_dev, const float* scale_w,
+                                const float* bias, int a_bits, hq_scale_mode mode, const float* static_scale, void* y,
+                                hq_dtype ydt, int64_t ldy, void* workspace, size_t ws_bytes, int32_t* dev_status,
+                                void* stream) {
+    return qlinear_impl(x, xdt, M, K, ldx, desc, w_dev, scale_w, bias, a_bits, mode, static_scale, y, ydt, ldy, nullptr, workspace,
+                        ws_bytes, dev_status, stream);
+}
+
+// The linear layer with a residual added to its rounded output (the output projection of an attention block).
+extern "C" hq_status hq_qlinear_add(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc,
+                                    const void* w_dev, const float* scale_w, const float* bias, int a_bits, const void* residual,
+                                    void* y, void* workspace, size_t ws_bytes, int32_t* dev_status, void* stream) {
+    if (residual == nullptr || desc == nullptr) return HQ_ERR_INVALID_ARG;
+    return qlinear_impl(x, xdt, M, K, ldx, desc, w_dev, scale_w, bias, a_bits, HQ_SCALE_PER_ROW, nullptr, y, HQ_BF16, desc->N,
+                        residual, workspace, ws_bytes, dev_status, stream);
 }
 
 extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const float* ln_weight,
@@ -253,12 +287,12 @@ extern "C" hq_status hq_ln_qlinear(const void* x, hq_dtype xdt, int64_t M, int64
 
 static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split, hq_dtype xdt, int64_t Nb, int64_t H,
                                     int64_t W, int64_t C, int groups,
-                                      const float* gamma, const float* beta, const void* pre_bias, float eps,
+                                      const float* gamma, const float* beta, const void* pre_bias, int64_t pre_ld, float eps,
                                       const hq_weight_desc* desc,
                                       const void* w_dev, int R, int S, int stride, int pad, const float* scale_w,
                                       const float* bias, int a_bits, hq_scale_mode mode, const float* static_scale, void* y,
-                                      hq_dtype ydt, void* workspace, size_t ws_bytes, void* scratch, size_t scratch_bytes,
-                                      int32_t* dev_status, void* stream) {
+                                      hq_dtype ydt, const void* residual, void* workspace, size_t ws_bytes, void* scratch,
+                                      size_t scratch_bytes, int32_t* dev_status, void* stream) {
     using namespace hq;
     if (desc == nullptr || w_dev == nullptr || workspace == nullptr || y == nullptr) return HQ_ERR_INVALID_ARG;
     if (!aligned16(workspace)) return HQ_ERR_ALIGNMENT;
@@ -270,13 +304,19 @@ static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split
     if (ws_bytes < need) return HQ_ERR_WORKSPACE;
     const int64_t ldc = code_pitch(C, cont);
     if (ldc != (cont == HQ_CODES_NIBBLE ? C / 2 : C)) return HQ_ERR_ALIGNMENT;   // conv needs densely packed pixels
+    s = check_residual(residual, y, ydt, desc->N, desc->N);
+    if (s != HQ_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    ResidualAdd res{static_cast<const __nv_bfloat16*>(residual), false};
     LayerCodes lc(desc, w_dev, a_bits, mode, rows, C, stride, cont, workspace, ws_bytes, false);
     s = launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, desc->had_block, a_bits, mode, static_scale,
-                             lc.codes, cont, ldc, lc.scales, scratch, scratch_bytes, st, 1, pre_bias, x2, split, &lc.z);
+                             lc.codes, cont, ldc, lc.scales, scratch, scratch_bytes, st, 1, pre_bias, pre_ld, x2, split, &lc.z);
     if (s != HQ_OK) return s;
-    return launch_qconv2d(lc.a(), lc.container(cont), a_bits, Nb, H, W, C, lc.desc(desc), lc.w(w_dev), R, S, stride, pad, lc.scales,
-                          mode == HQ_SCALE_STATIC, scale_w, bias, hq_alpha_for(desc), nullptr, y, ydt, dev_status, st, true);
+    s = launch_qconv2d(lc.a(), lc.container(cont), a_bits, Nb, H, W, C, lc.desc(desc), lc.w(w_dev), R, S, stride, pad, lc.scales,
+                       mode == HQ_SCALE_STATIC, scale_w, bias, hq_alpha_for(desc), nullptr, y, ydt, dev_status, st, true,
+                       residual != nullptr ? &res : nullptr);
+    const int64_t Ho = (H + 2 * pad - R) / stride + 1, Wo = (W + 2 * pad - S) / stride + 1;
+    return finish_residual(s, res, y, Nb * Ho * Wo * desc->N, stream);
 }
 
 extern "C" hq_status hq_gn_silu_qconv(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C, int groups,
@@ -285,8 +325,21 @@ extern "C" hq_status hq_gn_silu_qconv(const void* x, hq_dtype xdt, int64_t Nb, i
                                       const float* scale_w, const float* bias, int a_bits, hq_scale_mode mode,
                                       const float* static_scale, void* y, hq_dtype ydt, void* workspace, size_t ws_bytes,
                                       void* scratch, size_t scratch_bytes, int32_t* dev_status, void* stream) {
-    return gn_silu_qconv_impl(x, nullptr, 0, xdt, Nb, H, W, C, groups, gamma, beta, pre_bias, eps, desc, w_dev, R, S, stride,
-                              pad, scale_w, bias, a_bits, mode, static_scale, y, ydt, workspace, ws_bytes, scratch,
+    return gn_silu_qconv_impl(x, nullptr, 0, xdt, Nb, H, W, C, groups, gamma, beta, pre_bias, C, eps, desc, w_dev, R, S, stride,
+                              pad, scale_w, bias, a_bits, mode, static_scale, y, ydt, nullptr, workspace, ws_bytes, scratch,
+                              scratch_bytes, dev_status, stream);
+}
+
+// The same layer with a residual added to its rounded output (the second convolution of a residual block).
+extern "C" hq_status hq_gn_silu_qconv_add(const void* x, hq_dtype xdt, int64_t Nb, int64_t H, int64_t W, int64_t C, int groups,
+                                          const float* gamma, const float* beta, const void* pre_bias, int64_t ld_pre_bias, float eps,
+                                          const hq_weight_desc* desc, const void* w_dev, int R, int S, int stride, int pad,
+                                          const float* scale_w, const float* bias, int a_bits, hq_scale_mode mode,
+                                          const float* static_scale, const void* residual, void* y, void* workspace,
+                                          size_t ws_bytes, void* scratch, size_t scratch_bytes, int32_t* dev_status, void* stream) {
+    if (residual == nullptr) return HQ_ERR_INVALID_ARG;
+    return gn_silu_qconv_impl(x, nullptr, 0, xdt, Nb, H, W, C, groups, gamma, beta, pre_bias, ld_pre_bias, eps, desc, w_dev, R, S, stride,
+                              pad, scale_w, bias, a_bits, mode, static_scale, y, HQ_BF16, residual, workspace, ws_bytes, scratch,
                               scratch_bytes, dev_status, stream);
 }
 
@@ -300,8 +353,8 @@ extern "C" hq_status hq_gn_silu_qconv_cat(const void* x, const void* x2, int64_t
                                           void* workspace, size_t ws_bytes, void* scratch, size_t scratch_bytes,
                                           int32_t* dev_status, void* stream) {
     if (x2 == nullptr) return HQ_ERR_INVALID_ARG;
-    return gn_silu_qconv_impl(x, x2, C1, xdt, Nb, H, W, C, groups, gamma, beta, pre_bias, eps, desc, w_dev, R, S, stride, pad,
-                              scale_w, bias, a_bits, mode, static_scale, y, ydt, workspace, ws_bytes, scratch, scratch_bytes,
+    return gn_silu_qconv_impl(x, x2, C1, xdt, Nb, H, W, C, groups, gamma, beta, pre_bias, C, eps, desc, w_dev, R, S, stride, pad,
+                              scale_w, bias, a_bits, mode, static_scale, y, ydt, nullptr, workspace, ws_bytes, scratch, scratch_bytes,
                               dev_status, stream);
 }
 
@@ -326,7 +379,7 @@ extern "C" hq_status hq_gn_qlinear(const void* x, hq_dtype xdt, int64_t Nb, int6
     LayerCodes lc(desc, w_dev, a_bits, HQ_SCALE_PER_ROW, M, C, 1, cont, workspace, ws_bytes, false);
     s = launch_gn_silu_quant(x, xdt, Nb, rows_per_sample, 1, C, groups, gamma, beta, eps, desc->had_block, a_bits,
                              HQ_SCALE_PER_ROW, nullptr, lc.codes, cont, lc.ld, lc.scales, scratch, scratch_bytes, st,
-                             silu != 0, nullptr, nullptr, 0, &lc.z);
+                             silu != 0, nullptr, 0, nullptr, 0, &lc.z);
     if (s != HQ_OK) return s;
     return launch_qgemm(lc.a(), lc.container(cont), a_bits, M, C, lc.lda(), lc.desc(desc), lc.w(w_dev), lc.scales, 0, scale_w, bias, hq_alpha_for(desc), nullptr,
                         y, ydt, ldy, dev_status, st, true);

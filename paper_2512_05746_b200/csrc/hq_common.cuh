@@ -33,6 +33,10 @@ struct SplitOut { uint8_t* z; int64_t ld; bool written; bool halved; };
 // bytes) and that of the output channel are both 1.
 struct HalvedParity { const uint8_t* row; int64_t pitch; const uint8_t* col; };
 
+// A bf16 tensor of the output's shape and pitch that is added to the rounded output of a product (a residual connection);
+// `done`: the product kernel has added it.
+struct ResidualAdd { const __nv_bfloat16* r; bool done; };
+
 // hq_gemm_splitk.cu: CTAs a tile's reduction is divided over (0: persistent kernels) and the estimated time of a product.
 struct ProductPlan { int ways; double us; };
 ProductPlan plan_product(int limbs, int64_t out_rows, int tile_rows, int64_t n_pad, int num_kb);
@@ -43,6 +47,14 @@ ProductPlan plan_product(int limbs, int64_t out_rows, int tile_rows, int64_t n_p
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
+}
+
+// bf16(y) + r for two packed pairs of values, rounded again: what an addition of the stored output gives.
+__device__ __forceinline__ uint32_t add_bf16x2(uint32_t y, uint32_t r) {
+    const float lo = __uint_as_float(y << 16) + __uint_as_float(r << 16);
+    const float hi = __uint_as_float(y & 0xFFFF0000u) + __uint_as_float(r & 0xFFFF0000u);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // ---- mbarrier -------------------------------------------------------------------------------

@@ -34,7 +34,7 @@ bool pair_stream_covers_conv(hq_container cont, const gemm::GemmParams& g);
 hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, int64_t lda, const hq_weight_desc* desc,
                                    const void* w_dev, const float* scale_a, int scale_a_is_scalar, const float* scale_w,
                                    const float* bias, float alpha, void* y, int64_t ldy, int32_t* dev_status, cudaStream_t st,
-                                   bool after_quant, const HalvedParity* halved = nullptr);
+                                   bool after_quant, const HalvedParity* halved, const __nv_bfloat16* res);
 hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, const CUtensorMap& tmY,
                             const hq_weight_desc* desc, const void* w_dev, cudaStream_t st);
 // hq_gemm_splitk.cu: the same product with a tile's reduction divided over a cluster, for problems of few tiles
@@ -287,7 +287,8 @@ hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64
                        const hq_weight_desc* desc, const void* w_dev, const float* scale_a, int scale_a_is_scalar,
                        const float* scale_w, const float* bias, float alpha, int32_t* acc_out, void* y,
                        hq_dtype ydt, int64_t ldy, int32_t* dev_status, cudaStream_t st, bool after_quant,
-                       const HalvedParity* halved) {
+                       const HalvedParity* halved, ResidualAdd* res) {
+    if (res != nullptr) res->done = false;
     hq_status s = check_common(a_codes, cont, a_bits, desc, w_dev, scale_a, scale_w, acc_out, y, ydt, K);
     if (s != HQ_OK) return s;
     if (desc->RS != 1 || desc->C != K) return HQ_ERR_SHAPE;
@@ -312,19 +313,22 @@ hq_status launch_qgemm(const void* a_codes, hq_container cont, int a_bits, int64
 
     if (halved != nullptr)                             // the caller has asked halved_product_covers
         return launch_qgemm_pair_stream(a_codes, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias, alpha, y,
-                                        ldy, dev_status, st, after_quant, halved);
+                                        ldy, dev_status, st, after_quant, halved, nullptr);
     if (const int ways = g_pair_gemm == 2 ? splitk_ways(cont, p, M, kBM, desc->N_pad) : 0) {
         CUtensorMap tmA;
         if (!encode_2d(&tmA, a_codes, uint64_t(row_bytes), uint64_t(M), uint64_t(lda), kBK, kBM, true)) return HQ_ERR_CUDA;
+        if (res != nullptr) { p.res = res->r; res->done = true; }
         return launch_qgemm_splitk(p, ways, kBM, M, tmA, desc, w_dev, st);
     }
     if (g_pair_gemm && pair_kernel_covers(cont, desc, M, y, ydt, ldy, acc_out, p.combine_fast != 0) &&
         (g_pair_gemm == 1 || pair_kernel_pays(desc, M)))
         return launch_qgemm_pair(a_codes, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias, alpha, y, ldy,
                                  dev_status, st, after_quant);
-    if (g_pair_gemm && pair_stream_covers_gemm(cont, desc, M, y, ydt, ldy, acc_out, p.combine_fast != 0))
+    if (g_pair_gemm && pair_stream_covers_gemm(cont, desc, M, y, ydt, ldy, acc_out, p.combine_fast != 0)) {
+        if (res != nullptr) res->done = true;
         return launch_qgemm_pair_stream(a_codes, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias, alpha, y,
-                                        ldy, dev_status, st, after_quant);
+                                        ldy, dev_status, st, after_quant, nullptr, res != nullptr ? res->r : nullptr);
+    }
 
     CUtensorMap tmA, tmB, tmY{};
     const bool nib = cont == HQ_CODES_NIBBLE;
@@ -342,7 +346,8 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
                          int64_t C, const hq_weight_desc* desc, const void* w_dev, int R, int S, int stride, int pad,
                          const float* scale_a, int scale_a_is_scalar, const float* scale_w, const float* bias,
                          float alpha, int32_t* acc_out, void* y, hq_dtype ydt, int32_t* dev_status, cudaStream_t st,
-                         bool after_quant) {
+                         bool after_quant, ResidualAdd* res) {
+    if (res != nullptr) res->done = false;
     hq_status s = check_common(a_codes, cont, a_bits, desc, w_dev, scale_a, scale_w, acc_out, y, ydt,
                                int64_t(R) * S * C);
     if (s != HQ_OK) return s;
@@ -361,7 +366,7 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     if (per_tap && acc_out != nullptr) {
         // the whole-window integer sums never exist in that mode: produce them with a launch of their own
         s = launch_qconv2d(a_codes, cont, a_bits, Nb, H, W, C, desc, w_dev, R, S, stride, pad, nullptr, 1, nullptr,
-                           nullptr, 1.0f, acc_out, nullptr, ydt, dev_status, st, after_quant);
+                           nullptr, 1.0f, acc_out, nullptr, ydt, dev_status, st, after_quant, nullptr);
         if (s != HQ_OK) return s;
         acc_out = nullptr;
     }
@@ -404,11 +409,17 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     const uint32_t box[4] = {uint32_t(nib ? kBK / 2 : kBK), uint32_t(p.bw * stride), uint32_t(p.bh * stride), uint32_t(p.bn)};
     const uint32_t estr[4] = {1, uint32_t(stride), uint32_t(stride), 1};
     if (!encode_4d(&tmA, a_codes, dims, box, estr, !nib)) return HQ_ERR_CUDA;
-    if (ways > 0) return launch_qgemm_splitk(p, ways, box_rows, Nb * Ho * Wo, tmA, desc, w_dev, st);
+    if (ways > 0) {
+        if (res != nullptr) { p.res = res->r; res->done = true; }
+        return launch_qgemm_splitk(p, ways, box_rows, Nb * Ho * Wo, tmA, desc, w_dev, st);
+    }
     const uint64_t Kp = uint64_t(desc->C_pad) * desc->RS;
     if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, uint32_t(per_tap ? per_tap_rows(desc->limbs) : kBN), true))
         return HQ_ERR_CUDA;
-    if (g_pair_gemm && pair_stream_covers_conv(cont, p)) return launch_qconv_pair(p, tmA, tmY, desc, w_dev, st);
+    if (g_pair_gemm && pair_stream_covers_conv(cont, p)) {
+        if (res != nullptr) { p.res = res->r; res->done = true; }
+        return launch_qconv_pair(p, tmA, tmY, desc, w_dev, st);
+    }
     return launch(nib, tmA, tmB, tmY, p, st);
 }
 
@@ -420,7 +431,7 @@ extern "C" hq_status hq_qgemm(const void* a_codes, hq_container cont, int a_bits
                               int32_t* acc_out, void* y, hq_dtype ydt, int64_t ldy, int32_t* dev_status,
                               void* stream) {
     return hq::launch_qgemm(a_codes, cont, a_bits, M, K, lda, desc, w_dev, scale_a, scale_a_is_scalar, scale_w, bias,
-                            alpha, acc_out, y, ydt, ldy, dev_status, static_cast<cudaStream_t>(stream), false, nullptr);
+                            alpha, acc_out, y, ydt, ldy, dev_status, static_cast<cudaStream_t>(stream), false, nullptr, nullptr);
 }
 
 extern "C" hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t Nb, int64_t H, int64_t W,
@@ -430,7 +441,7 @@ extern "C" hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bi
                                 int32_t* dev_status, void* stream) {
     return hq::launch_qconv2d(a_codes, cont, a_bits, Nb, H, W, C, desc, w_dev, R, S, stride, pad, scale_a,
                               scale_a_is_scalar, scale_w, bias, alpha, acc_out, y, ydt, dev_status,
-                              static_cast<cudaStream_t>(stream), false);
+                              static_cast<cudaStream_t>(stream), false, nullptr);
 }
 
 extern "C" int hq_set_pair_gemm(int mode) {

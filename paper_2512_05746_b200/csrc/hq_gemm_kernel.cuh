@@ -58,6 +58,7 @@ struct GemmParams {
     int pdl;              // launched ahead of the completion of the kernel that produces the codes and scale_a
     int frag;             // fragment-layout epilogue + second MMA issuer (see use_frag)
     int tma_store;        // bf16 output goes out through bulk tensor stores (rows of a tile are consecutive output rows)
+    const __nv_bfloat16* res;   // added to the rounded output by the kernels that take it (split reductions, streamed pairs)
     int32_t* dev_status;
 };
 

@@ -153,12 +153,15 @@ __device__ __forceinline__ bool wait_pair(uint64_t* bar, uint32_t parity, PairCt
 // BN: operand-B rows (accumulator columns) of the tile.
 // HALVED (halved weights, hq_fwht.cuh): the integer is twice the accumulator plus the column's bit in `odd` (the column parities
 // of the warp, 32 to a word, zero for a row of parity 0).
-template <int LIMBS, int PREG = 0, int NBUF = 2, int BN = kBN, bool HALVED = false>
+// RES: `res` points to this lane's row of a residual (nullptr: a row past the end) at column col0, `ncols` of its columns exist;
+// 32 bytes a lane and step, requested one step ahead, are added to the rounded output.
+template <int LIMBS, int PREG = 0, int NBUF = 2, int BN = kBN, bool HALVED = false, bool RES = false>
 __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg, int lane, const float* prm_sw,
                                               const float* prm_b, float sa_eff, const CUtensorMap* tmY, int col0, int row0,
                                               uint32_t tempty_leader, const float (&rsw)[PREG > 0 ? PREG * 16 : 1] = {0.f},
                                               const float (&rb)[PREG > 0 ? PREG * 16 : 1] = {0.f},
-                                              const uint32_t (&odd)[HALVED ? BN / 64 : 1] = {0u}) {
+                                              const uint32_t (&odd)[HALVED ? BN / 64 : 1] = {0u},
+                                              const __nv_bfloat16* res = nullptr, int ncols = 0) {
     static_assert(!HALVED || LIMBS == 1, "halved weights are one limb");
     static_assert(LIMBS == 1 || BN == kBN, "narrower tiles exist with one limb");
     constexpr int NSTEPS = LIMBS == 2 ? kBN / 2 / 2 / 16 : BN / 2 / 16;
@@ -166,8 +169,21 @@ __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg
     uint32_t hi[16], lo[16];
     tmem_ld_32x16(t_row, hi);
     if (LIMBS == 2) tmem_ld_32x16(t_row + uint32_t(kBN / 2), lo);
+    uint4 rn[RES ? 2 : 1];
+    auto request = [&](int st) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            rn[RES ? j : 0] = res != nullptr && st * 16 + 8 * j < ncols ? __ldcs(reinterpret_cast<const uint4*>(res + st * 16 + 8 * j))
+                                                                        : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if constexpr (RES) request(0);
 #pragma unroll
     for (int st = 0; st < NSTEPS; ++st) {
+        uint4 rc[RES ? 2 : 1];
+        if constexpr (RES) {
+            rc[0] = rn[0]; rc[1] = rn[1];
+            if (st + 1 < NSTEPS) request(st + 1);
+        }
         int32_t w[16];
         tmem_ld_wait_16(hi);
         if (LIMBS == 2) {
@@ -211,6 +227,8 @@ __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg
             o.y = pack_bf16x2(fmaf(float(w[8 * j + 2]) * s0.z, sa_eff, c0.z), fmaf(float(w[8 * j + 3]) * s0.w, sa_eff, c0.w));
             o.z = pack_bf16x2(fmaf(float(w[8 * j + 4]) * s1.x, sa_eff, c1.x), fmaf(float(w[8 * j + 5]) * s1.y, sa_eff, c1.y));
             o.w = pack_bf16x2(fmaf(float(w[8 * j + 6]) * s1.z, sa_eff, c1.z), fmaf(float(w[8 * j + 7]) * s1.w, sa_eff, c1.w));
+            if constexpr (RES)
+                o = make_uint4(add_bf16x2(o.x, rc[j].x), add_bf16x2(o.y, rc[j].y), add_bf16x2(o.z, rc[j].z), add_bf16x2(o.w, rc[j].w));
             *reinterpret_cast<uint4*>(wr + (((2 * (st & 1) + j) ^ wsw) << 4)) = o;
         }
         if (st & 1) {
@@ -493,6 +511,8 @@ struct PairStreamParams {
     int pdl;
     int32_t* dev_status;
     HalvedParity parity;               // HALVED instantiations
+    const __nv_bfloat16* res;          // added to the rounded output (pitch ldr, N a multiple of 8), or nullptr
+    int64_t ldr;
     // convolution geometry (CONV instantiations)
     int kb_per_tap, S, stride, pad, bw, bh, bn, tiles_w, tiles_h;
 };
@@ -691,8 +711,13 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             const float sa_eff = p.alpha * sa;
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
             const uint32_t t_fast = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as * kBN + wc0);
-            epilogue_pair<LIMBS, 0, NBUF, BN, HALVED>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as],
-                                                      {0.f}, {0.f}, odd);
+            if (!HALVED && p.res != nullptr)
+                epilogue_pair<LIMBS, 0, NBUF, BN, HALVED, true>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as],
+                                                                {0.f}, {0.f}, odd,
+                                                                my_row < p.M ? p.res + my_row * p.ldr + col_base + wc0 : nullptr, p.N - col_base - wc0);
+            else
+                epilogue_pair<LIMBS, 0, NBUF, BN, HALVED>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as],
+                                                          {0.f}, {0.f}, odd);
         }
         if (lane == 0) bulk_wait_read_all();           // shared memory must outlive the copy engine's reads
     }
@@ -875,9 +900,10 @@ bool pair_stream_covers_conv(hq_container cont, const gemm::GemmParams& g) {
 hq_status launch_qgemm_pair_stream(const void* a_codes, int64_t M, int64_t K, int64_t lda, const hq_weight_desc* desc,
                                    const void* w_dev, const float* scale_a, int scale_a_is_scalar, const float* scale_w,
                                    const float* bias, float alpha, void* y, int64_t ldy, int32_t* dev_status, cudaStream_t st,
-                                   bool after_quant, const HalvedParity* halved) {
+                                   bool after_quant, const HalvedParity* halved, const __nv_bfloat16* res) {
     PairStreamParams p{};
     if (halved != nullptr) p.parity = *halved;
+    p.res = res; p.ldr = ldy;
     p.M = M; p.N = int(desc->N); p.limbs = desc->limbs;
     p.num_kb = int(desc->C_pad / kBK);
     p.tiles_m2 = int((M + 255) / 256);
@@ -911,6 +937,7 @@ hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, c
                             const hq_weight_desc* desc, const void* w_dev, cudaStream_t st) {
     PairStreamParams p{};
     p.M = int64_t(g.Nb) * g.Ho * g.Wo; p.N = g.N; p.limbs = g.limbs;
+    p.res = g.res; p.ldr = g.ldy;
     p.num_kb = g.kb_per_tap * g.taps;
     p.tiles_m2 = (g.tiles_m + 1) / 2;
     const int bn = g.limbs == 2 ? kBN : stream_width(p.tiles_m2, g.N);

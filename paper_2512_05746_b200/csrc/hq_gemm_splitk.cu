@@ -39,6 +39,7 @@ struct SplitKParams {
     const float* scale_a; int sa_scalar;
     const float* scale_w; const float* bias; float alpha;
     __nv_bfloat16* y; int y_vec_ok;
+    const __nv_bfloat16* res;                     // added to the rounded output (same pitch, N a multiple of 8), or nullptr
     int pdl;
     int32_t* dev_status;
     int kb_per_tap, S, stride, pad, bw, bh, bn, tiles_w, tiles_h;       // convolution geometry
@@ -211,6 +212,15 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (p.pdl) griddep_wait();                     // scale_a comes from the kernel before this one
         if ((e & 127) < rows) sa_eff = p.alpha * ld_dependent(p.scale_a + (p.sa_scalar ? 0 : row0 + (e & 127)));
         // from here on every CTA's ring is its receive buffer: [from CTA][4-column group][row] of 16-byte pieces
+        uint4 resid[4];                                // the residual's share, 8 columns each (cw <= 64), requested ahead
+        if (p.res != nullptr) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int g = (e >> 7) + 2 * i, col0 = n_tile * kSkCols + rank * cw + g * 8;
+                resid[i] = g < cw / 8 && col0 < p.N && (e & 127) < rows
+                               ? __ldg(reinterpret_cast<const uint4*>(p.res + (row0 + (e & 127)) * p.ldy + col0)) : make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
         ok = wait_splitk<true>(&ctl->ready, 0, ctl, p.dev_status, kStatusAccumWait);
         tc_fence_after();
         const int row = q * 32 + lane;
@@ -251,7 +261,10 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         ok = ok && wait_splitk<true>(&ctl->recv, 0, ctl, p.dev_status, kStatusAccumWait);
         if (ok && (e & 127) < rows) {
             const int row = e & 127;
-            for (int g = e >> 7; g < cw / 8; g += 2) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int g = (e >> 7) + 2 * i;
+                if (g >= cw / 8) break;
                 const int col0 = n_tile * kSkCols + rank * cw + g * 8;
                 if (col0 >= p.N) break;
                 int32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -267,8 +280,11 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                 for (int j = 0; j < 8; ++j) f[j] = fmaf(float(w[j]) * ctl->sw[g * 8 + j], sa_eff, ctl->bias[g * 8 + j]);
                 __nv_bfloat16* dst = p.y + (row0 + row) * p.ldy + col0;
                 if (p.y_vec_ok && col0 + 8 <= p.N) {
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]),
-                                                                pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+                    uint4 o = make_uint4(pack_bf16x2(f[0], f[1]), pack_bf16x2(f[2], f[3]), pack_bf16x2(f[4], f[5]), pack_bf16x2(f[6], f[7]));
+                    if (p.res != nullptr)
+                        o = make_uint4(add_bf16x2(o.x, resid[i].x), add_bf16x2(o.y, resid[i].y), add_bf16x2(o.z, resid[i].z),
+                                       add_bf16x2(o.w, resid[i].w));
+                    *reinterpret_cast<uint4*>(dst) = o;
                 } else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j) if (col0 + j < p.N) dst[j] = __float2bfloat16_rn(f[j]);
@@ -377,7 +393,7 @@ hq_status launch_qgemm_splitk(const gemm::GemmParams& g, int ways, int tile_rows
     p.tiles_n = (g.N + kSkCols - 1) / kSkCols; p.split = ways; p.tile_rows = tile_rows;
     p.a_bytes = g.a_box_bytes;
     p.scale_a = g.scale_a; p.sa_scalar = g.sa_scalar; p.scale_w = g.scale_w; p.bias = g.bias; p.alpha = g.alpha;
-    p.y = static_cast<__nv_bfloat16*>(g.y); p.y_vec_ok = g.y_vec_ok; p.pdl = g.pdl; p.dev_status = g.dev_status;
+    p.y = static_cast<__nv_bfloat16*>(g.y); p.y_vec_ok = g.y_vec_ok; p.res = g.res; p.pdl = g.pdl; p.dev_status = g.dev_status;
     p.kb_per_tap = g.kb_per_tap; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
     p.bw = g.bw; p.bh = g.bh; p.bn = g.bn; p.tiles_w = g.tiles_w; p.tiles_h = g.tiles_h;
     CUtensorMap tmB;

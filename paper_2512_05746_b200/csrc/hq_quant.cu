@@ -48,7 +48,8 @@ struct QuantParams {
     const float* gn_beta;    // [cols]
     int gn_groups;
     int gn_silu;             // 1: SiLU after the normalisation, 0: none
-    const __nv_bfloat16* gn_pre_bias;   // [samples][cols] added to x before the normalisation, or nullptr
+    const __nv_bfloat16* gn_pre_bias;   // [samples][cols], pitch gn_pre_ld, added to x before the normalisation, or nullptr
+    int gn_pre_ld;
     int gn_sets_per_sample;  // CTAs per sample (a CTA never straddles two samples)
     int gn_cg;               // channels per group, and its log2 when it is a power of two (else -1)
     int gn_cg_shift;
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
             // (x + e - mean) a + beta = x a + (beta + (e - mean) a): the per-sample addend e costs nothing per element
             float4 sh = make_float4(-ms.x, -ms.x, -ms.x, -ms.x);
             if (p.gn_pre_bias != nullptr) {
-                const uint2 er = __ldg(reinterpret_cast<const uint2*>(p.gn_pre_bias + size_t(sample) * p.cols + c));
+                const uint2 er = __ldg(reinterpret_cast<const uint2*>(p.gn_pre_bias + size_t(sample) * unsigned(p.gn_pre_ld) + c));
                 sh.x += __uint_as_float(er.x << 16); sh.y += __uint_as_float(er.x & 0xFFFF0000u);
                 sh.z += __uint_as_float(er.y << 16); sh.w += __uint_as_float(er.y & 0xFFFF0000u);
             }
@@ -665,7 +666,7 @@ __device__ __forceinline__ void gn_quad(const GnPiece<8>& r, int q, f32x2& lo, f
 
 template <typename InT, int VEC>
 __global__ void __launch_bounds__(256, 4) gn_stats_kernel(const InT* x, const InT* x2, int split,
-                                                          const __nv_bfloat16* pre_bias, int64_t hw, int64_t total_px,
+                                                          const __nv_bfloat16* pre_bias, int64_t pre_ld, int64_t hw, int64_t total_px,
                                                           int64_t span, int C, int groups, double* sums, float* stats,
                                                           double inv_count, double eps) {
     constexpr int Q = VEC / 4;                         // channel quads per piece
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_kernel(const InT* x, const In
                 if (pre_bias != nullptr) {
 #pragma unroll
                     for (int q = 0; q < Q; ++q) {
-                        const uint2 er = __ldg(reinterpret_cast<const uint2*>(pre_bias + sample * C + int64_t(col) * VEC + 4 * q));
+                        const uint2 er = __ldg(reinterpret_cast<const uint2*>(pre_bias + sample * pre_ld + int64_t(col) * VEC + 4 * q));
                         e_lo[q] = pk2(__uint_as_float(er.x << 16), __uint_as_float(er.x & 0xFFFF0000u));
                         e_hi[q] = pk2(__uint_as_float(er.y << 16), __uint_as_float(er.y & 0xFFFF0000u));
                     }
@@ -798,7 +799,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_kernel(const InT* x, const In
 // in fp32 (eight pixels `ppl` apart), so the fp32 partial sums are the same; only the fp64 sums over them run in another
 // order.  The CTA reads `pieces` * 16 contiguous bytes of every pixel, its neighbours in the grid the rest.
 template <typename InT, int VEC>
-__global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, const InT* x2, int split, const __nv_bfloat16* pre_bias,
+__global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, const InT* x2, int split, const __nv_bfloat16* pre_bias, int64_t pre_ld,
                                                                int hw, int C, int groups, int run, int ppl, float* stats,
                                                                double inv_count, double eps) {
     constexpr int Q = VEC / 4, U = 8;
@@ -819,7 +820,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
         if (pre_bias != nullptr) {
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
-                const uint2 er = __ldg(reinterpret_cast<const uint2*>(pre_bias + int64_t(sample) * C + ch + 4 * q));
+                const uint2 er = __ldg(reinterpret_cast<const uint2*>(pre_bias + sample * pre_ld + ch + 4 * q));
                 e_lo[q] = pk2(__uint_as_float(er.x << 16), __uint_as_float(er.x & 0xFFFF0000u));
                 e_hi[q] = pk2(__uint_as_float(er.y << 16), __uint_as_float(er.y & 0xFFFF0000u));
             }
@@ -962,7 +963,7 @@ cudaError_t dispatch_fast(int klog, const QuantParams& p, bool int8_out, int gri
 
 // Launches the transform+quantize kernel; shared by the public entry point and the fused layer calls.
 struct GnArgs { const float* stats; const float* gamma; const float* beta; int groups; int64_t rows_per_sample; int silu;
-                const __nv_bfloat16* pre_bias; };
+                const __nv_bfloat16* pre_bias; int64_t pre_ld; };
 struct LnArgs { const float* w; const float* b; int64_t rows_per_group; float eps; };
 
 struct SplitArgs { const void* x2; int64_t split, ldx2; };
@@ -1021,6 +1022,7 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         p.gn_stats = gn->stats; p.gn_gamma = gn->gamma; p.gn_beta = gn->beta; p.gn_groups = gn->groups;
         p.gn_silu = gn->silu;
         p.gn_pre_bias = gn->pre_bias;
+        p.gn_pre_ld = int(gn->pre_ld);
         p.gn_cg = int(cols / gn->groups);
         p.gn_cg_shift = is_pow2(p.gn_cg) ? ilog2(p.gn_cg) : -1;
     }
@@ -1153,7 +1155,7 @@ static int gn_slab_run(int64_t Nb, int64_t hw, int64_t C, int groups, int elt, i
 // here), then mean and 1/sqrt(var + eps) as floats behind them.  scratch: Nb * groups * (2 doubles + 2 floats).
 hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, int64_t C, int groups, float eps,
                           void* scratch, size_t scratch_bytes, const float** stats_out, cudaStream_t st,
-                          const void* pre_bias, const void* x2, int64_t split) {
+                          const void* pre_bias, int64_t pre_ld, const void* x2, int64_t split) {
     if (x == nullptr || scratch == nullptr) return HQ_ERR_INVALID_ARG;
     if (xdt != HQ_F32 && xdt != HQ_BF16) return HQ_ERR_INVALID_ARG;
     if (Nb <= 0 || hw <= 0 || C <= 0 || groups <= 0) return HQ_ERR_SHAPE;
@@ -1164,7 +1166,8 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     if (reinterpret_cast<uintptr_t>(scratch) % 16 != 0) return HQ_ERR_ALIGNMENT;
     const int elt = xdt == HQ_F32 ? 4 : 2;
     if (reinterpret_cast<uintptr_t>(x) % (4 * elt) != 0) return HQ_ERR_ALIGNMENT;
-    if (pre_bias != nullptr && reinterpret_cast<uintptr_t>(pre_bias) % 8 != 0) return HQ_ERR_ALIGNMENT;
+    if (pre_bias != nullptr && (reinterpret_cast<uintptr_t>(pre_bias) % 8 != 0 || pre_ld % 4 != 0)) return HQ_ERR_ALIGNMENT;
+    if (pre_bias != nullptr && (pre_ld < C || pre_ld > 0x7fffffff)) return HQ_ERR_SHAPE;
     const __nv_bfloat16* pre = static_cast<const __nv_bfloat16*>(pre_bias);
     double* sums = static_cast<double*>(scratch);
     float* stats = reinterpret_cast<float*>(sums + size_t(Nb) * groups * 2);
@@ -1180,7 +1183,7 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     const double inv_count = 1.0 / (double(hw) * double(C / groups));
     if (const int run = gn_slab_run(Nb, hw, C, groups, elt, wide ? 8 : 4)) {
         const unsigned slabs = unsigned(Nb * (groups / run));
-#define HQ_SLAB(T, V) gn_stats_slab_kernel<T, V><<<slabs, 256, 0, st>>>(static_cast<const T*>(x), static_cast<const T*>(x2), int(split), pre, int(hw), \
+#define HQ_SLAB(T, V) gn_stats_slab_kernel<T, V><<<slabs, 256, 0, st>>>(static_cast<const T*>(x), static_cast<const T*>(x2), int(split), pre, pre_ld, int(hw), \
                                                                         int(C), groups, run, int(ppl), stats, inv_count, double(eps))
         if (xdt == HQ_F32) HQ_SLAB(float, 4);
         else if (wide) HQ_SLAB(__nv_bfloat16, 8);
@@ -1194,13 +1197,13 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     const int64_t total_px = Nb * hw, span = gn_wave_span(Nb, hw, C, wide ? 8 : 4);
     const unsigned grid = unsigned(gn_wave_ctas(Nb, hw, C, wide ? 8 : 4));
     if (xdt == HQ_F32)
-        gn_stats_kernel<float, 4><<<grid, 256, 0, st>>>(static_cast<const float*>(x), static_cast<const float*>(x2), int(split), pre, hw, total_px, span, int(C), groups, sums,
+        gn_stats_kernel<float, 4><<<grid, 256, 0, st>>>(static_cast<const float*>(x), static_cast<const float*>(x2), int(split), pre, pre_ld, hw, total_px, span, int(C), groups, sums,
                                                        stats, inv_count, double(eps));
     else if (wide)
-        gn_stats_kernel<__nv_bfloat16, 8><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(x2), int(split), pre, hw, total_px, span, int(C),
+        gn_stats_kernel<__nv_bfloat16, 8><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(x2), int(split), pre, pre_ld, hw, total_px, span, int(C),
                                                                groups, sums, stats, inv_count, double(eps));
     else
-        gn_stats_kernel<__nv_bfloat16, 4><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(x2), int(split), pre, hw, total_px, span, int(C),
+        gn_stats_kernel<__nv_bfloat16, 4><<<grid, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(x2), int(split), pre, pre_ld, hw, total_px, span, int(C),
                                                                groups, sums, stats, inv_count, double(eps));
     if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
     *stats_out = stats;
@@ -1213,14 +1216,14 @@ hq_status launch_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, int64_t 
                                const float* gamma, const float* beta, float eps, int had_block, int bits,
                                hq_scale_mode mode, const float* static_scale, void* codes, hq_container cont,
                                int64_t ld_codes, float* scales, void* scratch, size_t scratch_bytes, cudaStream_t st,
-                               int silu, const void* pre_bias, const void* x2, int64_t split, SplitOut* zo) {
+                               int silu, const void* pre_bias, int64_t pre_ld, const void* x2, int64_t split, SplitOut* zo) {
     if (gamma == nullptr || beta == nullptr) return HQ_ERR_INVALID_ARG;
     if (H <= 0 || W <= 0) return HQ_ERR_SHAPE;
     const int64_t hw = H * W;
     const float* stats = nullptr;
-    hq_status s = launch_gn_stats(x, xdt, Nb, hw, C, groups, eps, scratch, scratch_bytes, &stats, st, pre_bias, x2, split);
+    hq_status s = launch_gn_stats(x, xdt, Nb, hw, C, groups, eps, scratch, scratch_bytes, &stats, st, pre_bias, pre_ld, x2, split);
     if (s != HQ_OK) return s;
-    const GnArgs gn{stats, gamma, beta, groups, hw, silu, static_cast<const __nv_bfloat16*>(pre_bias)};
+    const GnArgs gn{stats, gamma, beta, groups, hw, silu, static_cast<const __nv_bfloat16*>(pre_bias), pre_ld};
     if (x2 != nullptr) {
         const SplitArgs sp{x2, split, C - split};
         return launch_quant_impl(x, xdt, Nb * hw, C, split, had_block, bits, mode, static_scale, codes, cont, ld_codes, scales,
@@ -1336,7 +1339,7 @@ extern "C" hq_status hq_gn_silu_quant(const void* x, hq_dtype xdt, int64_t Nb, i
                                       size_t scratch_bytes, void* stream) {
     return hq::launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, had_block, bits, mode, static_scale, codes,
                                     cont, ld_codes, scales, scratch, scratch_bytes, static_cast<cudaStream_t>(stream), 1,
-                                    pre_bias, nullptr, 0, nullptr);
+                                    pre_bias, C, nullptr, 0, nullptr);
 }
 
 extern "C" hq_status hq_gn_silu_quant_cat(const void* x, const void* x2, int64_t C1, hq_dtype xdt, int64_t Nb, int64_t H,
@@ -1347,7 +1350,7 @@ extern "C" hq_status hq_gn_silu_quant_cat(const void* x, const void* x2, int64_t
     if (x2 == nullptr) return HQ_ERR_INVALID_ARG;
     return hq::launch_gn_silu_quant(x, xdt, Nb, H, W, C, groups, gamma, beta, eps, had_block, bits, mode, static_scale, codes,
                                     cont, ld_codes, scales, scratch, scratch_bytes, static_cast<cudaStream_t>(stream), 1,
-                                    pre_bias, x2, C1, nullptr);
+                                    pre_bias, C, x2, C1, nullptr);
 }
 
 extern "C" hq_status hq_hadamard_quant_cat(const void* x, int64_t ldx, const void* x2, int64_t ldx2, int64_t cols1,

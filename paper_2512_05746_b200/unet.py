@@ -133,6 +133,44 @@ class UNet:
         self.calibrating = False
         self.recording = None
         self.graph, self.graph_key = None, None
+        self._group_embeddings()
+
+    def _group_embeddings(self):
+        """The projections of the step embedding, one per residual block and all of the same input, laid out as one layer: their
+        weights, weight scales and biases become views of tensors that hold all of them, so that a forward projects once."""
+        self.emb = None
+        names = [n for n in self.pw if n.endswith(".emb")]
+        shape = lambda d: (d.C, d.C_pad, d.RS, d.w_bits, d.had_block, d.mode, d.limbs, d.container)
+        descs = [self.pw[n].desc for n in names]
+        if len(names) < 2 or len({shape(d) for d in descs}) > 1 or any(d.N % 128 for d in descs):
+            return
+        rows = [d.N * d.limbs * d.C_pad for d in descs]                 # whole 128-row groups follow one another in a blob
+        cat = self.torch.cat
+        whole = self.hq.PreparedWeight(type(descs[0]).from_buffer_copy(descs[0]), None, None)
+        whole.blob_dev = cat([self.pw[n].blob_dev[:r] for n, r in zip(names, rows)])
+        whole.s_w_dev = cat([self.pw[n].s_w_dev for n in names])
+        bias = cat([self.f32[n + ".b"] for n in names])
+        whole.desc.N = whole.desc.N_pad = sum(d.N for d in descs)
+        whole.desc.bytes, whole.desc.reserved = sum(rows), 0            # without the one-limb section: Nb rows never use it
+        whole.desc.max_abs_b = max(d.max_abs_b for d in descs)
+        at, byte, start = 0, 0, {}
+        for n, d, r in zip(names, descs, rows):
+            pw = self.pw[n]
+            pw.blob_dev, pw.s_w_dev, self.f32[n + ".b"] = whole.blob_dev[byte:byte + r], whole.s_w_dev[at:at + d.N], bias[at:at + d.N]
+            d.bytes, d.reserved = r, 0
+            start[n] = at
+            at, byte = at + d.N, byte + r
+        self.emb = (whole, bias, start)
+        self.emb_key = self._emb_operands()
+
+    def _emb_operands(self):
+        return [(pw.blob_dev.data_ptr(), pw.s_w_dev.data_ptr(), self.f32[n + ".b"].data_ptr(), bytes(pw.desc))
+                for n, pw in ((n, self.pw[n]) for n in self.emb[2])]
+
+    def _emb_together(self):
+        """Whether this run projects the step embedding for all blocks at once: not while calls are recorded or calibrated one by
+        one, and not once a block has been given operands elsewhere."""
+        return self.recording is None and not self.calibrating and self._emb_operands() == self.emb_key
 
     # ------------------------------------------------------------------ recording helpers
     def _emit(self, tag, name, fn, rec=None):
@@ -158,18 +196,20 @@ class UNet:
         return self.ws[: rows * pitch].view(rows, pitch), self.ws[off: off + rows * 4].view(self.torch.float32)
 
     # ------------------------------------------------------------------ layers
-    def _conv3(self, name, x, norm=None, stride=1, pre_bias=None, x2=None):
-        """x2: the layer's input is the channel concatenation [x | x2], which is read in place and never written."""
+    def _conv3(self, name, x, norm=None, stride=1, pre_bias=None, x2=None, residual=None):
+        """x2: the layer's input is the channel concatenation [x | x2], which is read in place and never written.  pre_bias: a
+        function that gives the addend in front of the normalisation.  residual: added to the output as it is stored; a recorded forward leaves the addition to `_residual`."""
         hq, t = self.hq, self.torch
         Nb, H, W, Cin = x.shape
         Cin += x2.shape[3] if x2 is not None else 0
         pw = self.pw[name]
         self._need_ws(pw, Nb * H * W, static=True, stride=stride)
-        y = self._new((Nb, H // stride, W // stride, pw.desc.N))
+        y, plain = self._output((Nb, H // stride, W // stride, pw.desc.N), residual)
         bias = self.f32[name + ".b"]
         ss = self.static.setdefault(name, t.ones((1,), dtype=t.float32, device=self.dev))
         g = (self.f32[norm + ".gamma"], self.f32[norm + ".beta"]) if norm else None
         G = self.cfg["groups"]
+        addend = pre_bias or (lambda: None)
 
         def calibrate():
             if not self.calibrating:
@@ -177,7 +217,7 @@ class UNet:
             codes, sc = self._ws_views(Nb * H * W, Cin)
             if g:
                 hq.hq_gn_silu_quant(x, G, g[0], g[1], self.EPS, pw.desc.had_block, self.a_bits, codes, self.cont, self.scratch,
-                                    scales=sc, pre_bias=pre_bias, x2=x2)
+                                    scales=sc, pre_bias=addend(), x2=x2)
             else:
                 hq.hq_hadamard_quant(x.view(-1, x.shape[3]), pw.desc.had_block, self.a_bits, codes, self.cont, scales=sc,
                                      x2=None if x2 is None else x2.view(-1, x2.shape[3]))
@@ -186,15 +226,17 @@ class UNet:
         def run():
             calibrate()
             if g:
-                hq.hq_gn_silu_qconv(x, G, g[0], g[1], self.EPS, pw, 3, 3, stride, 1, bias, self.a_bits, y, self.ws, self.scratch,
-                                    static_scale=ss, dev_status=self.status, pre_bias=pre_bias, x2=x2)
+                fused = residual is not None and self.recording is None
+                hq.hq_gn_silu_qconv(x, G, g[0], g[1], self.EPS, pw, 3, 3, stride, 1, bias, self.a_bits, y if fused else plain(), self.ws,
+                                    self.scratch, static_scale=ss, dev_status=self.status, pre_bias=addend(), x2=x2,
+                                    residual=residual if fused else None)
             else:
-                hq.hq_qconv(x, pw, 3, 3, stride, 1, bias, self.a_bits, y, self.ws, static_scale=ss, dev_status=self.status,
+                hq.hq_qconv(x, pw, 3, 3, stride, 1, bias, self.a_bits, plain(), self.ws, static_scale=ss, dev_status=self.status,
                             x2=x2)
 
-        self._emit("q", name, run, lambda: dict(op="conv3", x=x, x2=x2, y=y, norm=norm, stride=stride, static=ss, pre_bias=pre_bias,
+        self._emit("q", name, run, lambda: dict(op="conv3", x=x, x2=x2, y=plain(), norm=norm, stride=stride, static=ss, pre_bias=addend(),
                                                 codes=self._ws_views(Nb * H * W, Cin)[0]))
-        return y
+        return y if residual is None else (y, plain)
 
     def _conv1(self, name, x, x2=None):
         hq = self.hq
@@ -210,22 +252,78 @@ class UNet:
                                 scales=self._ws_views(Nb * H * W, Cin)[1]))
         return y
 
-    def _linear(self, name, x, norm=None, Nb=None):
+    def _linear(self, name, x, norm=None, Nb=None, residual=None):
         hq = self.hq
         M, K = x.shape
         pw = self.pw[name]
         self._need_ws(pw, M)
-        y = self._new((M, pw.desc.N))
+        y, plain = self._output((M, pw.desc.N), residual)
         bias = self.f32[name + ".b"]
         if norm:
             gm, bt = self.f32[norm + ".gamma"], self.f32[norm + ".beta"]
             fn = lambda: hq.hq_gn_qlinear(x, Nb, self.cfg["groups"], gm, bt, self.EPS, False, pw, bias, self.a_bits, y, self.ws,
                                           self.scratch, dev_status=self.status)
         else:
-            fn = lambda: hq.hq_qlinear(x, pw, bias, self.a_bits, y, self.ws, dev_status=self.status)
-        self._emit("q", name, fn, lambda: dict(op="linear", x=x, y=y, norm=norm, Nb=Nb, codes=self._ws_views(M, K)[0],
+            def fn():
+                fused = residual is not None and self.recording is None
+                hq.hq_qlinear(x, pw, bias, self.a_bits, y if fused else plain(), self.ws, dev_status=self.status,
+                              residual=residual if fused else None)
+        self._emit("q", name, fn, lambda: dict(op="linear", x=x, y=plain(), norm=norm, Nb=Nb, codes=self._ws_views(M, K)[0],
                                                scales=self._ws_views(M, K)[1]))
-        return y
+        return y if residual is None else (y, plain)
+
+    def _embedding(self, name, x):
+        """A block's projection of the step embedding; returns a function that gives its [Nb, C] (rows of a wider tensor where all
+        blocks' projections are made at once, by the first of them)."""
+        hq = self.hq
+        if self.emb is None:
+            e = self._linear(name, x)
+            return lambda: e
+        (whole, bias_all, start), pw, bias = self.emb, self.pw[name], self.f32[name + ".b"]
+        M, K = x.shape
+        self._need_ws(pw, M)
+        first = self.emb_out is None
+        if first:
+            self._need_ws(whole, M)
+            self.emb_out = self._new((M, whole.desc.N))
+        out, rows = self.emb_out, self.emb_out[:, start[name]:start[name] + pw.desc.N]
+        apart = self._later((M, pw.desc.N))
+
+        def fn():
+            if first:                                                   # once for all blocks of a run
+                self.emb_joined = self._emb_together()
+            if not self.emb_joined:
+                hq.hq_qlinear(x, pw, bias, self.a_bits, apart(), self.ws, dev_status=self.status)
+            elif first:
+                hq.hq_qlinear(x, whole, bias_all, self.a_bits, out, self.ws, dev_status=self.status)
+        self._emit("q", name, fn, lambda: dict(op="linear", x=x, y=apart(), norm=None, Nb=None, codes=self._ws_views(M, K)[0],
+                                               scales=self._ws_views(M, K)[1]))
+        return lambda: rows if self.emb_joined else apart()
+
+    def _output(self, shape, residual):
+        """A layer's output, and a function that gives the buffer of its output before the residual is added: the output itself
+        without one, else a buffer that only a recorded forward, which takes the two steps apart, makes."""
+        y = self._new(shape)
+        return y, (lambda: y) if residual is None else self._later(shape)
+
+    def _later(self, shape):
+        """A function that gives a buffer and makes it when it is first asked for."""
+        made = []
+
+        def buffer():
+            if not made:
+                made.append(self._new(shape))
+            return made[0]
+        return buffer
+
+    def _residual(self, name, a, out, plain):
+        """The addition out = a + plain(), which the layer that produces the sum has done except in a recorded forward."""
+        hq = self.hq
+
+        def fn():
+            if self.recording is not None:
+                hq.hq_add(a, plain(), out)
+        self._emit("g", name, fn, lambda: dict(op="add", a=a, b=plain(), out=out))
 
     def _glue(self, name, op, fn, **tensors):
         self._emit("g", name, fn, lambda: dict(op=op, **tensors))
@@ -233,16 +331,15 @@ class UNet:
     def _resblock(self, name, x, semb, x2=None):
         """x2: the block's input is the channel concatenation [x | x2] (a skip connection joining the up-sampling path);
         its two consumers, the first convolution and the 1x1 skip convolution, read the two tensors in place."""
-        hq = self.hq
         cin, cout = x.shape[-1] + (x2.shape[-1] if x2 is not None else 0), self.pw[name + ".conv1"].desc.N
         h = self._conv3(name + ".conv1", x, norm=name + ".norm1", x2=x2)
-        e = self._linear(name + ".emb", semb)
-        # h + e is never stored: the second convolution's normalisation takes the embedding as a per-sample addend
-        h2 = self._conv3(name + ".conv2", h, norm=name + ".norm2", pre_bias=e)
+        e = self._embedding(name + ".emb", semb)
         assert x2 is None or cin != cout       # a concatenated input always changes the channel count here
         xs = x if cin == cout else self._conv1(name + ".skip", x, x2=x2)
-        out = self._new(h2.shape)
-        self._glue(name + ".residual", "add", lambda: hq.hq_add(xs, h2, out), a=xs, b=h2, out=out)
+        # h + e is never stored: the second convolution's normalisation takes the embedding as a per-sample addend; nor is its own
+        # output, to which the block's input (or its 1x1 convolution) is added as it is stored
+        out, plain = self._conv3(name + ".conv2", h, norm=name + ".norm2", pre_bias=e, residual=xs)
+        self._residual(name + ".residual", xs, out, plain)
         return out
 
     def _attention(self, name, x):
@@ -255,10 +352,9 @@ class UNet:
         self.attn_flops += 4.0 * Nb * float(H * W) ** 2 * ch
         self._glue(name + ".core", "attention", lambda: hq.hq_attention(qkv, Nb, heads, a, dev_status=self.status),
                    qkv=qkv, out=a, Nb=Nb, heads=heads)
-        pr = self._linear(name + ".proj", a)
-        out = self._new(x.shape)
-        self._glue(name + ".residual", "add", lambda: hq.hq_add(x2, pr, out), a=x2, b=pr, out=out)
-        return out
+        out, plain = self._linear(name + ".proj", a, residual=x2)
+        self._residual(name + ".residual", x2, out, plain)
+        return out.view(x.shape)
 
     # ------------------------------------------------------------------ the network
     def build(self, Nb: int):
@@ -269,6 +365,8 @@ class UNet:
         self.tape = []
         self.graph, self.graph_key = None, None
         self.Nb = Nb
+        self.emb_out = None            # [Nb, channels of all blocks]: the projections of the step embedding,
+        self.emb_joined = False        # where the running pass made them at once
         self.attn_flops = 0.0          # 4 L^2 C per sample and attention block (QK^T and PV)
         self._ws_need = 256
         self.scratch = t.empty((Nb * cfg["groups"] * 24,), dtype=t.uint8, device=self.dev)

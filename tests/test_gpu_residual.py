@@ -1,0 +1,97 @@
+"""Fused layers with a residual connection: the sum is bit for bit that of hq_add on the layer's own output, whichever kernel runs
+the product (a reduction divided over a cluster, streamed weights on pairs of SMs, and those that leave the addition to a launch
+of its own)."""
+import ctypes as C
+
+import pytest
+
+from paper_2512_05746_b200 import inputs
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K,N,n,room", [
+    (2, 1024, 1024, 256, False),        # divided eight ways, 16 columns a CTA; two rows of a tile
+    (130, 768, 264, 256, False),        # ragged rows and columns, divided
+    (200, 1024, 512, 256, False),       # two rows of tiles
+    (4096, 1024, 1024, 256, True),      # pairs of SMs, one limb
+    (1001, 2304, 1160, 256, True),      # ... rows of the last tile missing, a column tile cut off inside a 32-column store
+    (16385, 768, 200, 256, True),       # ... narrower column tiles
+    (5000, 1024, 776, 256, False),      # ... two limbs
+    (4096, 512, 512, 256, True),        # resident weights: a launch of its own
+    (8200, 2048, 520, 2048, True),      # halved weights: likewise
+])
+def test_linear_with_a_residual_is_the_linear_and_an_addition(M, K, N, n, room):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    gen = torch.Generator(device="cuda").manual_seed(M + K + N)
+    x = torch.randn((M, K), generator=gen, device="cuda").to(torch.bfloat16)
+    r = (3 * torch.randn((M, N), generator=gen, device="cuda")).to(torch.bfloat16)
+    pw = hq.hq_weight_prepare(inputs.weights((N, K), seed=N), 4, n, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device()
+    b = torch.from_numpy(inputs.bias(N, seed=3)).cuda()
+    codes = (M * K + 255) // 256 * 256 + 4 * M
+    ws = torch.zeros((max(codes, hq.hq_layer_workspace_size(pw, 4, M), hq.hq_workspace_size(M, K, 1)) if room else codes,),
+                     dtype=torch.uint8, device="cuda")
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    y, want = (torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    guard = torch.full((M * N + 1024,), 7.0, dtype=torch.bfloat16, device="cuda")
+    got = guard[512: 512 + M * N].view(M, N)
+    hq.hq_qlinear(x, pw, b, 4, y, ws, dev_status=status)
+    hq.hq_add(y.view(-1), r.view(-1), want.view(-1))
+    hq.hq_qlinear(x, pw, b, 4, got, ws, dev_status=status, residual=r)
+    torch.cuda.synchronize()
+    hq.hq_check_status(status)
+    assert torch.equal(got, want)
+    assert bool((guard[:512] == 7).all()) and bool((guard[512 + M * N:] == 7).all())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("Nb,H,W,Cin,Cout,stride,static", [
+    (2, 8, 8, 2048, 1024, 1, True),     # divided eight ways
+    (3, 16, 16, 768, 776, 1, True),
+    (5, 32, 32, 512, 512, 1, True),     # pairs of SMs; an odd number of row tiles
+    (40, 32, 32, 256, 264, 1, True),
+    (7, 64, 64, 256, 256, 2, True),
+    (2, 20, 24, 256, 520, 1, True),     # rows of a tile are not consecutive output rows: a launch of its own
+    (2, 16, 16, 256, 256, 1, False),    # one scale per pixel under the window: likewise
+])
+def test_convolution_with_a_residual_is_the_convolution_and_an_addition(Nb, H, W, Cin, Cout, stride, static):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    gen = torch.Generator(device="cuda").manual_seed(Cin + Nb)
+    x = torch.randn((Nb, H, W, Cin), generator=gen, device="cuda").to(torch.bfloat16)
+    pw = hq.hq_weight_prepare(inputs.weights((Cout, 3, 3, Cin), seed=Cin), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device()
+    b = torch.from_numpy(inputs.bias(Cout, seed=3)).cuda()
+    g, bt = torch.ones(Cin, device="cuda"), torch.zeros(Cin, device="cuda")
+    shape = (Nb, H // stride, W // stride, Cout)
+    r = (3 * torch.randn(shape, generator=gen, device="cuda")).to(torch.bfloat16)
+    ws = torch.zeros((max(hq.hq_layer_workspace_size(pw, 4, Nb * H * W, static, stride), hq.hq_workspace_size(Nb * H * W, Cin, 1)),),
+                     dtype=torch.uint8, device="cuda")
+    scr = torch.zeros((Nb * 32 * 24,), dtype=torch.uint8, device="cuda")
+    ss = torch.tensor([0.3], device="cuda") if static else None
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    y, got = (torch.empty(shape, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    args = (x, 32, g, bt, 1e-5, pw, 3, 3, stride, 1, b, 4)
+    hq.hq_gn_silu_qconv(*args, y, ws, scr, static_scale=ss, dev_status=status)
+    want = torch.empty_like(y)
+    hq.hq_add(y.view(-1), r.view(-1), want.view(-1))
+    hq.hq_gn_silu_qconv(*args, got, ws, scr, static_scale=ss, dev_status=status, residual=r)
+    torch.cuda.synchronize()
+    hq.hq_check_status(status)
+    assert torch.equal(got, want)
+
+
+def test_residuals_that_cannot_be_added_are_refused_before_a_launch():
+    from paper_2512_05746_b200 import binding as hq
+    L, big = hq.lib, 1 << 30
+    p = lambda v: C.c_void_p(v)
+    odd = hq.hq_weight_prepare(inputs.weights((36, 256), seed=1), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8)
+    lin = hq.hq_weight_prepare(inputs.weights((64, 256), seed=1), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8)
+
+    def call(pw, residual, y):
+        return L.hq_qlinear_add(p(0x1000), 1, 64, 256, 256, C.byref(pw.desc), p(0x1000), p(0x1000), None, 4, residual, y, p(0x1000),
+                                big, None, None)
+    assert call(lin, None, p(0x2000)) == 1
+    assert call(lin, p(0x2000), p(0x2000)) == 1                       # the output itself
+    assert call(odd, p(0x3000), p(0x2000)) == 2                       # 36 columns
+    assert call(lin, p(0x3008), p(0x2000)) == 4
+    assert call(lin, p(0x3000), p(0x2008)) == 4
