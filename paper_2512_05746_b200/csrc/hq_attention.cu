@@ -327,9 +327,16 @@ __device__ __forceinline__ uint64_t make_sw128_mnmajor_desc(uint32_t smem_addr, 
     return d;
 }
 
+// Warps 0-3 do the softmax, thread t the row t of the tile; one lane of warp 4 issues every load and product, so that no softmax
+// warp waits for its own instruction issue.  The S columns are free as soon as the four warps hold block j's scores in registers:
+// S of block j + 1 is computed during the softmax of block j (bar_read), O += P(j) V(j) once P(j) is stored (bar_p), the K buffer
+// is refilled when S(j) is complete and the V buffer when the product before has read it.  With thread 0 of the softmax issuing
+// (S of the next block in one batch with O += P V) / so: 64 x 1024 tokens, 8 heads of 64 242.6 / 204.2 us, 2 x 1024 26.9 / 18.4,
+// 64 x 256, 8 of 96 49.5 / 43.6, 8 x 512, 16 of 128 40.4 / 30.2; of the first figure 9 us are the elected lane's alone.
 // LAZY: that rule; otherwise the maximum moves with every block.
+constexpr int kAttnTmaThreads = 160;
 template <int DH, bool LAZY>
-__global__ void __launch_bounds__(128, (DH <= 64 ? 4 : 2))
+__global__ void __launch_bounds__(kAttnTmaThreads, (DH <= 64 ? 4 : 2))
 attention_tma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmKV, const AttnParams p) {
     extern __shared__ __align__(1024) unsigned char smem_attn_tma[];
     constexpr int KB = kKeyBlock, NH = (DH + 63) / 64;         // 64-channel parts per tile (the last may reach into the next
@@ -340,17 +347,20 @@ attention_tma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     unsigned char* sK = sQ + NH * kQHalf;
     unsigned char* sV = sK + NH * kKVHalf;
     unsigned char* sP = sV + NH * kKVHalf;                     // 128 x KB bf16, unswizzled core matrices
-    __shared__ uint64_t bar_mma, bar_q, bar_k, bar_v;
+    __shared__ uint64_t bar_q, bar_k, bar_v;                   // loads have landed
+    __shared__ uint64_t bar_s, bar_o;                          // S of a block / O with a block's P V is complete
+    __shared__ uint64_t bar_read, bar_p;                       // the softmax warps hold S in registers / have stored P
     __shared__ uint32_t tmem_slot;
 
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int q0 = blockIdx.x * kQTile, head = blockIdx.y, n = blockIdx.z;
     const int L = p.L, C = p.C;
     const int row0 = n * L;                                    // the sample's first row of the [Nb L][3 C] matrix
     const int nblocks = (L + KB - 1) / KB;
 
     if (tid == 0) {
-        mbar_init(&bar_mma, 1); mbar_init(&bar_q, 1); mbar_init(&bar_k, 1); mbar_init(&bar_v, 1);
+        mbar_init(&bar_q, 1); mbar_init(&bar_k, 1); mbar_init(&bar_v, 1);
+        mbar_init(&bar_s, 1); mbar_init(&bar_o, 1); mbar_init(&bar_read, 4); mbar_init(&bar_p, 4);
         fence_barrier_init();
         tma_prefetch_desc(&tmQ);
         tma_prefetch_desc(&tmKV);
@@ -359,196 +369,177 @@ attention_tma_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    bool q_flying = false, k_flying = false, v_flying = false;  // thread 0: a load into the buffer is outstanding
-    uint32_t k_par = 0, v_par = 0;                              // ... and the barrier phase it completes
-    if (tid == 0) {
-        mbar_expect_tx(&bar_q, NH * kQHalf);
-#pragma unroll
-        for (int h = 0; h < NH; ++h) tma_load_2d(sQ + h * kQHalf, &tmQ, &bar_q, head * DH + 64 * h, row0 + q0);
-        mbar_expect_tx(&bar_k, NH * kKVHalf);
-#pragma unroll
-        for (int h = 0; h < NH; ++h) tma_load_2d(sK + h * kKVHalf, &tmKV, &bar_k, C + head * DH + 64 * h, row0);
-        mbar_expect_tx(&bar_v, NH * kKVHalf);
-#pragma unroll
-        for (int h = 0; h < NH; ++h) tma_load_2d(sV + h * kKVHalf, &tmKV, &bar_v, 2 * C + head * DH + 64 * h, row0);
-        q_flying = k_flying = v_flying = true;
-    }
     const uint32_t tmem_base = tmem_slot;
-    const uint32_t t_s = tmem_base + (uint32_t(warp * 32) << 16);
-    const uint32_t t_o = t_s + uint32_t(KB);
     constexpr uint32_t kPGroup = (KB / 8) * 128;
-    const uint32_t idesc_s = make_idesc_bf16(kQTile, KB, false);
-    const uint32_t idesc_o = make_idesc_bf16(kQTile, DH, true);
-
-    float m_run = -INFINITY, l_run = 0.f;
-    uint32_t ph_mma = 0;
     bool ok = true;
-    // S of block 0
-    if (warp == 0) {
-        if (tid == 0) {
-            bool ready = mbar_wait(&bar_q, 0, p.dev_status, kStatusAttnTma);
-            if (ready) q_flying = false;
-            ready = ready && mbar_wait(&bar_k, 0, p.dev_status, kStatusAttnTma);
-            if (ready) {
-                k_flying = false;
+
+    if (warp == 4) {
+        if (elect_one()) {
+            const uint32_t idesc_s = make_idesc_bf16(kQTile, KB, false);
+            const uint32_t idesc_o = make_idesc_bf16(kQTile, DH, true);
+            const uint64_t dq = make_sw128_kmajor_desc(smem_u32(sQ)), dk = make_sw128_kmajor_desc(smem_u32(sK));
+            const uint64_t dp = make_desc_noswizzle(smem_u32(sP), 128, kPGroup), dv = make_sw128_mnmajor_desc(smem_u32(sV), kKVHalf);
+            auto load_kv = [&](unsigned char* dst, uint64_t* bar, int part, int key0) {
+                mbar_expect_tx(bar, NH * kKVHalf);
+#pragma unroll
+                for (int h = 0; h < NH; ++h) tma_load_2d(dst + h * kKVHalf, &tmKV, bar, part * C + head * DH + 64 * h, row0 + key0);
+            };
+            auto s_product = [&]() {
+#pragma unroll
+                for (int k = 0; k < DH / 16; ++k)
+                    mma_bf16(tmem_base, dq + uint64_t((k / 4) * (kQHalf >> 4) + 2 * (k & 3)), dk + uint64_t((k / 4) * (kKVHalf >> 4) + 2 * (k & 3)),
+                             idesc_s, k != 0 ? 1u : 0u);
+                mma_commit(&bar_s);
+            };
+            mbar_expect_tx(&bar_q, NH * kQHalf);
+#pragma unroll
+            for (int h = 0; h < NH; ++h) tma_load_2d(sQ + h * kQHalf, &tmQ, &bar_q, head * DH + 64 * h, row0 + q0);
+            load_kv(sK, &bar_k, 1, 0);
+            load_kv(sV, &bar_v, 2, 0);
+            int k_loads = 1, v_loads = 1;                      // begun so far
+            ok = mbar_wait(&bar_q, 0, p.dev_status, kStatusAttnTma) && mbar_wait(&bar_k, 0, p.dev_status, kStatusAttnTma);
+            if (ok) { tc_fence_after(); s_product(); }
+            for (int j = 0; j < nblocks && ok; ++j) {
+                const uint32_t par = uint32_t(j) & 1u;
+                if (j + 1 < nblocks) {
+                    ok = mbar_wait(&bar_s, par, p.dev_status, kStatusAttnWait);                    // the K buffer has been read
+                    if (!ok) break;
+                    load_kv(sK, &bar_k, 1, (j + 1) * KB);
+                    ++k_loads;
+                }
+                if (j > 0) {
+                    ok = mbar_wait(&bar_o, par ^ 1u, p.dev_status, kStatusAttnWait);               // ... and the V buffer
+                    if (!ok) break;
+                    load_kv(sV, &bar_v, 2, j * KB);
+                    ++v_loads;
+                }
+                if (j + 1 < nblocks) {
+                    ok = mbar_wait(&bar_read, par, p.dev_status, kStatusAttnWait) && mbar_wait(&bar_k, par ^ 1u, p.dev_status, kStatusAttnTma);
+                    if (!ok) break;
+                    tc_fence_after();
+                    s_product();
+                }
+                ok = mbar_wait(&bar_v, par, p.dev_status, kStatusAttnTma) && mbar_wait(&bar_p, par, p.dev_status, kStatusAttnWait);
+                if (!ok) break;
                 tc_fence_after();
 #pragma unroll
-                for (int k = 0; k < DH / 16; ++k) {
-                    const uint64_t a = make_sw128_kmajor_desc(smem_u32(sQ + (k / 4) * kQHalf)) + uint64_t(2 * (k & 3));
-                    const uint64_t b = make_sw128_kmajor_desc(smem_u32(sK + (k / 4) * kKVHalf)) + uint64_t(2 * (k & 3));
-                    mma_bf16(tmem_base, a, b, idesc_s, k != 0 ? 1u : 0u);
-                }
-                mma_commit(&bar_mma);
+                for (int k = 0; k < KB / 16; ++k)              // 16 keys on: two core-matrix columns of P, 16 rows of V
+                    mma_bf16(tmem_base + uint32_t(KB), dp + uint64_t(k * 16), dv + uint64_t(k * 128), idesc_o, (j | k) != 0 ? 1u : 0u);
+                mma_commit(&bar_o);
+            }
+            if (!ok) {
+                // a wait ran out: the loads still on their way must land before the CTA's shared memory is given up
+                mbar_wait(&bar_q, 0, nullptr, 0);
+                mbar_wait(&bar_k, uint32_t(k_loads - 1) & 1u, nullptr, 0);
+                mbar_wait(&bar_v, uint32_t(v_loads - 1) & 1u, nullptr, 0);
             }
         }
         __syncwarp();
-    }
-    // Block j: wait for S(j) (and O += P V of block j - 1, issued in the same batch), refill the buffers those MMAs have
-    // read, softmax from registers, then one batch of MMAs again: O += P(j) V(j) and S(j + 1) -- the S columns are free as
-    // soon as every thread holds its row in registers, so the two products share one trip to the tensor core.
-    for (int j = 0; j < nblocks && ok; ++j) {
-        const int k0 = j * KB;
-        const int kvalid = L - k0 < KB ? L - k0 : KB;
-        ok = mbar_wait(&bar_mma, ph_mma, p.dev_status, kStatusAttnWait);
-        ph_mma ^= 1;
-        ok = __syncthreads_and(ok);
-        if (!ok) break;
-        tc_fence_after();
-        if (tid == 0) {
-            if (j + 1 < nblocks) {                             // the K buffer is free: the next block's keys
-                mbar_expect_tx(&bar_k, NH * kKVHalf);
+    } else {
+        const uint32_t t_s = tmem_base + (uint32_t(warp * 32) << 16);
+        const uint32_t t_o = t_s + uint32_t(KB);
+        float m_run = -INFINITY, l_run = 0.f;
+        for (int j = 0; j < nblocks; ++j) {
+            const uint32_t par = uint32_t(j) & 1u;
+            const int k0 = j * KB;
+            const int kvalid = L - k0 < KB ? L - k0 : KB;
+            ok = __all_sync(0xffffffffu, mbar_wait(&bar_s, par, p.dev_status, kStatusAttnWait));
+            if (!ok) break;
+            tc_fence_after();
+            // ---- the row's KB scores come into registers once: maximum, P = exp2(c (S - m)), row sum, P as bf16 to smem
+            const bool full = kvalid == KB;
+            uint32_t sreg[KB];
 #pragma unroll
-                for (int h = 0; h < NH; ++h)
-                    tma_load_2d(sK + h * kKVHalf, &tmKV, &bar_k, C + head * DH + 64 * h, row0 + k0 + KB);
-                k_flying = true;
-                k_par = uint32_t(j + 1) & 1u;
+            for (int c = 0; c < KB / 32; ++c) tmem_ld_32x32(t_s + uint32_t(c * 32), *reinterpret_cast<uint32_t (*)[32]>(&sreg[32 * c]));
+#pragma unroll
+            for (int c = 0; c < KB / 32; ++c) tmem_ld_wait_32(*reinterpret_cast<uint32_t (*)[32]>(&sreg[32 * c]));
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_read);
+            if (!full) {
+#pragma unroll
+                for (int e = 0; e < KB; ++e)
+                    if (e >= kvalid) sreg[e] = 0xFF800000u;                   // -inf: no part in the maximum, weight 0
             }
-            if (j > 0) {                                       // the V buffer is free: this block's values
-                mbar_expect_tx(&bar_v, NH * kKVHalf);
+            float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};        // four chains instead of one of 32 steps
 #pragma unroll
-                for (int h = 0; h < NH; ++h)
-                    tma_load_2d(sV + h * kKVHalf, &tmKV, &bar_v, 2 * C + head * DH + 64 * h, row0 + k0);
-                v_flying = true;
-                v_par = uint32_t(j) & 1u;
+            for (int e = 0; e < KB; e += 8) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) m4[c] = max3(m4[c], __uint_as_float(sreg[e + 2 * c]), __uint_as_float(sreg[e + 2 * c + 1]));
             }
-        }
-        // ---- the row's KB scores come into registers once: maximum, P = exp2(c (S - m)), row sum, P as bf16 to smem
-        const bool full = kvalid == KB;
-        uint32_t sreg[KB];
-#pragma unroll
-        for (int c = 0; c < KB / 32; ++c) tmem_ld_32x32(t_s + uint32_t(c * 32), *reinterpret_cast<uint32_t (*)[32]>(&sreg[32 * c]));
-#pragma unroll
-        for (int c = 0; c < KB / 32; ++c) tmem_ld_wait_32(*reinterpret_cast<uint32_t (*)[32]>(&sreg[32 * c]));
-        if (!full) {
-#pragma unroll
-            for (int e = 0; e < KB; ++e)
-                if (e >= kvalid) sreg[e] = 0xFF800000u;                   // -inf: no part in the maximum, weight 0
-        }
-        float mx = -INFINITY;
-#pragma unroll
-        for (int e = 0; e < KB; e += 2) mx = max3(mx, __uint_as_float(sreg[e]), __uint_as_float(sreg[e + 1]));
-        const float m_new = LAZY ? ((mx - m_run) * p.scale_log2 > 8.0f ? mx : m_run)     // first block: inf > 8
-                                 : fmaxf(m_run, mx);
-        const float mc = m_new * p.scale_log2;
-        const float alpha = ex2(m_run * p.scale_log2 - mc);              // 1 when the maximum stays, 0 on the first block
-        f32x2 sum2 = pk2(0.f, 0.f);
-        const f32x2 sc2 = pk2(p.scale_log2, p.scale_log2), nmc2 = pk2(-mc, -mc);
-        unsigned char* prow = sP + (tid >> 3) * kPGroup + (tid & 7) * 16;
-#pragma unroll
-        for (int g = 0; g < KB / 8; ++g) {
-            uint32_t w[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                float z0, z1;
-                upk2(fma2(pk2(__uint_as_float(sreg[8 * g + 2 * h]), __uint_as_float(sreg[8 * g + 2 * h + 1])), sc2, nmc2), z0, z1);
-                const float p0 = ex2(z0), p1 = ex2(z1);
-                sum2 = add2(sum2, pk2(p0, p1));
-                w[h] = pack_bf16(p0, p1);
+            const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+            const float m_new = LAZY ? ((mx - m_run) * p.scale_log2 > 8.0f ? mx : m_run)     // first block: inf > 8
+                                     : fmaxf(m_run, mx);
+            const float mc = m_new * p.scale_log2;
+            const float alpha = ex2(m_run * p.scale_log2 - mc);              // 1 when the maximum stays, 0 on the first block
+            f32x2 sum2 = pk2(0.f, 0.f);
+            const f32x2 sc2 = pk2(p.scale_log2, p.scale_log2), nmc2 = pk2(-mc, -mc);
+            unsigned char* prow = sP + (tid >> 3) * kPGroup + (tid & 7) * 16;
+            if (j > 0) {                                       // the product before has read P, and O may be rescaled
+                ok = __all_sync(0xffffffffu, mbar_wait(&bar_o, par ^ 1u, p.dev_status, kStatusAttnWait));
+                if (!ok) break;
+                tc_fence_after();
             }
-            *reinterpret_cast<uint4*>(prow + g * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+#pragma unroll
+            for (int g = 0; g < KB / 8; ++g) {
+                uint32_t w[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    float z0, z1;
+                    upk2(fma2(pk2(__uint_as_float(sreg[8 * g + 2 * h]), __uint_as_float(sreg[8 * g + 2 * h + 1])), sc2, nmc2), z0, z1);
+                    const float p0 = ex2(z0), p1 = ex2(z1);
+                    sum2 = add2(sum2, pk2(p0, p1));
+                    w[h] = pack_bf16(p0, p1);
+                }
+                *reinterpret_cast<uint4*>(prow + g * 128) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            float sum_lo, sum_hi;
+            upk2(sum2, sum_lo, sum_hi);
+            l_run = fmaf(l_run, alpha, sum_lo + sum_hi);
+            m_run = m_new;
+            if (j > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
+#pragma unroll
+                for (int c = 0; c < DH / 16; ++c) {
+                    uint32_t r[16];
+                    tmem_ld_32x16(t_o + uint32_t(c * 16), r);
+                    tmem_ld_wait_16(r);
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
+                    tmem_st_32x16(t_o + uint32_t(c * 16), r);
+                }
+                tmem_st_wait();
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_p);
         }
-        float sum_lo, sum_hi;
-        upk2(sum2, sum_lo, sum_hi);
-        l_run = fmaf(l_run, alpha, sum_lo + sum_hi);
-        m_run = m_new;
-        if (j > 0 && __any_sync(0xffffffffu, alpha != 1.0f)) {
+        if (ok) {                                              // the last O += P V
+            ok = __all_sync(0xffffffffu, mbar_wait(&bar_o, uint32_t(nblocks - 1) & 1u, p.dev_status, kStatusAttnWait));
+            tc_fence_after();
+        }
+        if (ok) {
+            const bool row_ok = q0 + tid < L;
+            const float inv = 1.0f / l_run;
+            __nv_bfloat16* dst = p.out + (int64_t(n) * L + (row_ok ? q0 + tid : 0)) * C + head * DH;
 #pragma unroll
             for (int c = 0; c < DH / 16; ++c) {
                 uint32_t r[16];
                 tmem_ld_32x16(t_o + uint32_t(c * 16), r);
                 tmem_ld_wait_16(r);
-#pragma unroll
-                for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * alpha);
-                tmem_st_32x16(t_o + uint32_t(c * 16), r);
-            }
-            tmem_st_wait();
-        }
-        fence_proxy_async_smem();
-        tc_fence_before();
-        __syncthreads();
-        if (warp == 0) {
-            if (tid == 0) {
-                bool ready = mbar_wait(&bar_v, uint32_t(j) & 1u, p.dev_status, kStatusAttnTma);
-                if (ready) v_flying = false;
-                if (ready && j + 1 < nblocks) {
-                    ready = mbar_wait(&bar_k, uint32_t(j + 1) & 1u, p.dev_status, kStatusAttnTma);
-                    if (ready) k_flying = false;
+                uint4 w0, w1;
+                w0.x = pack_bf16(__uint_as_float(r[0]) * inv, __uint_as_float(r[1]) * inv);
+                w0.y = pack_bf16(__uint_as_float(r[2]) * inv, __uint_as_float(r[3]) * inv);
+                w0.z = pack_bf16(__uint_as_float(r[4]) * inv, __uint_as_float(r[5]) * inv);
+                w0.w = pack_bf16(__uint_as_float(r[6]) * inv, __uint_as_float(r[7]) * inv);
+                w1.x = pack_bf16(__uint_as_float(r[8]) * inv, __uint_as_float(r[9]) * inv);
+                w1.y = pack_bf16(__uint_as_float(r[10]) * inv, __uint_as_float(r[11]) * inv);
+                w1.z = pack_bf16(__uint_as_float(r[12]) * inv, __uint_as_float(r[13]) * inv);
+                w1.w = pack_bf16(__uint_as_float(r[14]) * inv, __uint_as_float(r[15]) * inv);
+                if (row_ok) {
+                    reinterpret_cast<uint4*>(dst + c * 16)[0] = w0;
+                    reinterpret_cast<uint4*>(dst + c * 16)[1] = w1;
                 }
-                if (ready) {
-                    tc_fence_after();
-                    const uint64_t a = make_desc_noswizzle(smem_u32(sP), 128, kPGroup);
-                    const uint64_t b = make_sw128_mnmajor_desc(smem_u32(sV), kKVHalf);
-#pragma unroll
-                    for (int k = 0; k < KB / 16; ++k)        // 16 keys on: two core-matrix columns of P, 16 rows of V
-                        mma_bf16(tmem_base + uint32_t(KB), a + uint64_t(k * 16), b + uint64_t(k * 128), idesc_o,
-                                 (j | k) != 0 ? 1u : 0u);
-                    if (j + 1 < nblocks) {
-#pragma unroll
-                        for (int k = 0; k < DH / 16; ++k) {
-                            const uint64_t qa = make_sw128_kmajor_desc(smem_u32(sQ + (k / 4) * kQHalf)) + uint64_t(2 * (k & 3));
-                            const uint64_t kb = make_sw128_kmajor_desc(smem_u32(sK + (k / 4) * kKVHalf)) + uint64_t(2 * (k & 3));
-                            mma_bf16(tmem_base, qa, kb, idesc_s, k != 0 ? 1u : 0u);
-                        }
-                    }
-                    mma_commit(&bar_mma);
-                }
-            }
-            __syncwarp();
-        }
-    }
-    if (ok) {                                                  // the last O += P V
-        ok = mbar_wait(&bar_mma, ph_mma, p.dev_status, kStatusAttnWait);
-        ok = __syncthreads_and(ok);
-        tc_fence_after();
-    }
-    if (!ok && tid == 0) {
-        // a wait ran out: the loads still on their way must land before the CTA's shared memory is given up
-        if (q_flying) mbar_wait(&bar_q, 0, nullptr, 0);
-        if (k_flying) mbar_wait(&bar_k, k_par, nullptr, 0);
-        if (v_flying) mbar_wait(&bar_v, v_par, nullptr, 0);
-    }
-
-    if (ok) {
-        const bool row_ok = q0 + tid < L;
-        const float inv = 1.0f / l_run;
-        __nv_bfloat16* dst = p.out + (int64_t(n) * L + (row_ok ? q0 + tid : 0)) * C + head * DH;
-#pragma unroll
-        for (int c = 0; c < DH / 16; ++c) {
-            uint32_t r[16];
-            tmem_ld_32x16(t_o + uint32_t(c * 16), r);
-            tmem_ld_wait_16(r);
-            uint4 w0, w1;
-            w0.x = pack_bf16(__uint_as_float(r[0]) * inv, __uint_as_float(r[1]) * inv);
-            w0.y = pack_bf16(__uint_as_float(r[2]) * inv, __uint_as_float(r[3]) * inv);
-            w0.z = pack_bf16(__uint_as_float(r[4]) * inv, __uint_as_float(r[5]) * inv);
-            w0.w = pack_bf16(__uint_as_float(r[6]) * inv, __uint_as_float(r[7]) * inv);
-            w1.x = pack_bf16(__uint_as_float(r[8]) * inv, __uint_as_float(r[9]) * inv);
-            w1.y = pack_bf16(__uint_as_float(r[10]) * inv, __uint_as_float(r[11]) * inv);
-            w1.z = pack_bf16(__uint_as_float(r[12]) * inv, __uint_as_float(r[13]) * inv);
-            w1.w = pack_bf16(__uint_as_float(r[14]) * inv, __uint_as_float(r[15]) * inv);
-            if (row_ok) {
-                reinterpret_cast<uint4*>(dst + c * 16)[0] = w0;
-                reinterpret_cast<uint4*>(dst + c * 16)[1] = w1;
             }
         }
     }
@@ -567,7 +558,7 @@ hq_status launch_attention_tma(const AttnParams& p, int Nb, cudaStream_t st) {
     if (cudaFuncSetAttribute(attention_tma_kernel<DH, LAZY>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
         return HQ_ERR_CUDA;
     const dim3 grid(unsigned((p.L + kQTile - 1) / kQTile), unsigned(p.heads), unsigned(Nb));
-    attention_tma_kernel<DH, LAZY><<<grid, 128, smem, st>>>(tmQ, tmKV, p);
+    attention_tma_kernel<DH, LAZY><<<grid, kAttnTmaThreads, smem, st>>>(tmQ, tmKV, p);
     return cudaGetLastError() == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
 }
 

@@ -301,7 +301,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA, its own halves)
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0; uint32_t phase = 0;
             int cur_n = -1, reloads = 0;
             bool ok = true;
@@ -345,7 +345,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = make_idesc_i8(256, kBN);
             int stage = 0; uint32_t phase = 0;
             int cur_n = -1, reloads = 0;
@@ -582,7 +582,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA, its own halves)
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
             if (p.pdl) griddep_wait();                     // the codes come from the kernel before this one
@@ -620,7 +620,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             // A lone lane spends several cycles per instruction, and this lane's path per K block is what paces the
             // kernel: the operand descriptors advance by constants (a stage is 32 KB = 2048 descriptor units on, the
             // weights 1024 units behind the activations), and only the very first MMA of a tile overwrites.

@@ -144,7 +144,7 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     if (warp != 0) cluster_wait();
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             int w0 = 0, h0 = 0, n0 = 0;
             if (CONV) {
                 w0 = (m_tile % p.tiles_w) * p.bw;
@@ -186,7 +186,7 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         cluster_wait();
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t idesc = make_idesc_i8(kBM, kSkCols * LIMBS);
             for (int i = 0; i < count; ++i) {
                 const int st = i % STAGES;
@@ -295,7 +295,7 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     __syncwarp();
     cluster_arrive_relaxed();
     __syncthreads();
-    if (threadIdx.x == 0 && ctl->abort_flag)                    // the copies in flight must land before the ring is given up
+    if (warp == 0 && elect_one() && ctl->abort_flag)            // the copies in flight must land before the ring is given up
         for (int i = armed > STAGES ? armed - STAGES : 0; i < armed; ++i)
             mbar_wait(&ctl->full[i % STAGES], uint32_t(i / STAGES) & 1u, nullptr, 0);
     if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, kSkCols * LIMBS); }
