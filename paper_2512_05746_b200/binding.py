@@ -128,6 +128,10 @@ def _load():
 
 
 lib = _load()
+try:
+    from . import _hqcall
+except ImportError as e:
+    raise ImportError("the extension module _hqcall is missing: build it with `python -m paper_2512_05746_b200.build`") from e
 
 
 def status_string(status: int) -> str:
@@ -172,6 +176,12 @@ def _dtype_code(t):
     return code
 
 
+# The calls of single layers go through a module of native functions: ctypes takes 2.4 us for the arguments of a linear, and the
+# attribute look-ups before it as long again.
+_hqcall.bind(_dtype_code, *(C.cast(getattr(lib, n), C.c_void_p).value for n in ("hq_qlinear", "hq_qconv", "hq_ln_qlinear",
+                                                                                 "hq_hadamard_quant")))
+
+
 def hq_version() -> int:
     return lib.hq_version()
 
@@ -186,16 +196,14 @@ def hq_hadamard_quant(x, had_block: int, bits: int, codes, container: int, scale
                       stream=None, x2=None) -> None:
     """x [rows, cols] (fp32/bf16, last dim contiguous) -> codes (uint8 [rows, pitch]) and scales (fp32).  With x2
     [rows, cols2] the input is the column concatenation [x | x2], read in place."""
-    rows, cols = x.shape
-    mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
     if x2 is not None:
+        rows, cols = x.shape
+        mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
         _check(lib.hq_hadamard_quant_cat(_dptr(x), x.stride(0), _dptr(x2), x2.stride(0), cols, _dtype_code(x), rows,
                                          cols + x2.shape[1], had_block, bits, mode, _dptr(static_scale), _dptr(codes),
                                          container, codes.stride(0), _dptr(scales), _stream(stream)), "hq_hadamard_quant_cat")
         return
-    _check(lib.hq_hadamard_quant(_dptr(x), _dtype_code(x), rows, cols, x.stride(0), had_block, bits, mode,
-                                 _dptr(static_scale), _dptr(codes), container, codes.stride(0), _dptr(scales),
-                                 _stream(stream)), "hq_hadamard_quant")
+    _check(_hqcall.hadamard_quant(x, had_block, bits, codes, container, scales, static_scale, _stream(stream)), "hq_hadamard_quant")
 
 
 class PreparedWeight:
@@ -275,8 +283,8 @@ def hq_layer_workspace_size(pw: PreparedWeight, a_bits: int, rows: int, static: 
 def hq_qlinear(x, pw: PreparedWeight, bias, a_bits: int, y, workspace, static_scale=None, dev_status=None,
                stream=None, residual=None) -> None:
     """residual: bf16 tensor of y's shape added to the rounded output (y bf16 and dense, one scale per row), or None."""
-    M, K = x.shape
     if residual is not None:
+        M, K = x.shape
         if static_scale is not None or y.element_size() != 2 or not (y.is_contiguous() and residual.is_contiguous()) or \
                 residual.shape != y.shape or residual.dtype != y.dtype:
             raise ValueError("hq_qlinear: a residual goes with a dense bf16 output of its shape and one scale per row")
@@ -284,11 +292,7 @@ def hq_qlinear(x, pw: PreparedWeight, bias, a_bits: int, y, workspace, static_sc
                                   _dptr(pw.s_w_dev), _dptr(bias), a_bits, _dptr(residual), _dptr(y), _dptr(workspace),
                                   workspace.nbytes, _dptr(dev_status), _stream(stream)), "hq_qlinear_add")
         return
-    mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
-    _check(lib.hq_qlinear(_dptr(x), _dtype_code(x), M, K, x.stride(0), C.byref(pw.desc), _dptr(pw.blob_dev),
-                          _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode, _dptr(static_scale), _dptr(y), _dtype_code(y),
-                          y.stride(0), _dptr(workspace), workspace.nbytes,
-                          _dptr(dev_status), _stream(stream)), "hq_qlinear")
+    _check(_hqcall.qlinear(x, pw, bias, a_bits, y, workspace, static_scale, dev_status, _stream(stream)), "hq_qlinear")
 
 
 def hq_qlinear_noalloc(x, pw: PreparedWeight, bias, a_bits: int, y, static_scale=None, dev_status=None,
@@ -306,19 +310,16 @@ def hq_qlinear_noalloc(x, pw: PreparedWeight, bias, a_bits: int, y, static_scale
 def hq_qconv(x, pw: PreparedWeight, R: int, S: int, stride: int, pad: int, bias, a_bits: int, y, workspace,
              static_scale=None, dev_status=None, stream=None, x2=None) -> None:
     """The fused convolution layer on x NHWC, or (x2 given) on the channel concatenation [x | x2] read in place."""
-    Nb, H, W, Cin = x.shape
-    mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
     if x2 is not None:
+        Nb, H, W, Cin = x.shape
+        mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
         _check(lib.hq_qconv_cat(_dptr(x), _dptr(x2), Cin, _dtype_code(x), Nb, H, W, Cin + x2.shape[3], C.byref(pw.desc),
                                 _dptr(pw.blob_dev), R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode,
                                 _dptr(static_scale), _dptr(y), _dtype_code(y), _dptr(workspace),
                                 workspace.nbytes, _dptr(dev_status), _stream(stream)),
                "hq_qconv_cat")
         return
-    _check(lib.hq_qconv(_dptr(x), _dtype_code(x), Nb, H, W, Cin, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride,
-                        pad, _dptr(pw.s_w_dev), _dptr(bias), a_bits, mode, _dptr(static_scale), _dptr(y),
-                        _dtype_code(y), _dptr(workspace), workspace.nbytes,
-                        _dptr(dev_status), _stream(stream)), "hq_qconv")
+    _check(_hqcall.qconv(x, pw, R, S, stride, pad, bias, a_bits, y, workspace, static_scale, dev_status, _stream(stream)), "hq_qconv")
 
 
 def hq_gn_silu_quant(x, groups: int, gamma, beta, eps: float, had_block: int, bits: int, codes, container: int,
@@ -389,11 +390,8 @@ def hq_ln_quant(x, weight, bias, rows_per_group: int, eps: float, had_block: int
 def hq_ln_qlinear(x, ln_weight, ln_bias, rows_per_group: int, eps: float, pw: PreparedWeight, bias, a_bits: int, y,
                   workspace, dev_status=None, stream=None) -> None:
     """The fused linear layer with LayerNorm + per-sample affine in front (per-row activation scales)."""
-    M, K = x.shape
-    _check(lib.hq_ln_qlinear(_dptr(x), _dtype_code(x), M, K, x.stride(0), _dptr(ln_weight), _dptr(ln_bias), rows_per_group,
-                             eps, C.byref(pw.desc), _dptr(pw.blob_dev), _dptr(pw.s_w_dev), _dptr(bias), a_bits, _dptr(y),
-                             _dtype_code(y), y.stride(0), _dptr(workspace), workspace.nbytes,
-                             _dptr(dev_status), _stream(stream)), "hq_ln_qlinear")
+    _check(_hqcall.ln_qlinear(x, ln_weight, ln_bias, rows_per_group, eps, pw, bias, a_bits, y, workspace, dev_status, _stream(stream)),
+           "hq_ln_qlinear")
 
 
 def hq_hadamard_quant_width(x, had_block_w: int, bits: int, static_scale, z, scale_out=None, stream=None) -> None:

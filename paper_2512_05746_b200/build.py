@@ -1,4 +1,5 @@
-"""Compile csrc/*.cu for sm_100a into libhq.so next to this file (nvcc cross-compiles without a GPU)."""
+"""Compile csrc/*.cu for sm_100a into libhq.so next to this file (nvcc cross-compiles without a GPU), and csrc/hq_pycall.c
+into the extension module binding.py calls it through."""
 from __future__ import annotations
 
 import glob
@@ -8,21 +9,34 @@ import sys
 
 _DIR = os.path.dirname(os.path.abspath(__file__))
 LIB = os.path.join(_DIR, "libhq.so")
+PYCALL = os.path.join(_DIR, "_hqcall.so")
+PYCALL_SOURCE = os.path.join(_DIR, "csrc", "hq_pycall.c")
 SOURCES = sorted(glob.glob(os.path.join(_DIR, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(_DIR, "csrc", "*.cuh"))) + [os.path.join(os.path.dirname(_DIR), "include", "hq.h")]
 
 
 def stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYCALL):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYCALL))
+    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS + [PYCALL_SOURCE])
+
+
+def build_pycall() -> str:
+    """The native marshalling of binding.py's frequent calls, an extension module of its own (the library links no Python)."""
+    import sysconfig
+    tmp = PYCALL + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-fvisibility=hidden", "-I" + sysconfig.get_paths()["include"],
+                           "-o", tmp, PYCALL_SOURCE])
+    os.replace(tmp, PYCALL)
+    return PYCALL
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compiles every csrc/*.cu to an object file (in parallel) and links them into libhq.so."""
     if not force and not stale():
         return LIB
+    build_pycall()
     from concurrent.futures import ThreadPoolExecutor
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     cflags = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
