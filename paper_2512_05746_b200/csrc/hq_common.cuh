@@ -37,6 +37,14 @@ struct HalvedParity { const uint8_t* row; int64_t pitch; const uint8_t* col; };
 // `done`: the product kernel has added it.
 struct ResidualAdd { const __nv_bfloat16* r; bool done; };
 
+// Whether a transform of `grid` CTAs is launched as a programmatic dependent of whatever precedes it in the stream: its CTAs are placed
+// while that kernel drains and wait (griddep_wait) before they touch anything.  Small layers one after the other: 256 x 256 -> 256
+// 6.4 / 5.4 us, 2 x 1024 -> 1024 6.7 / 5.5, 2 x 8 x 8 x 2048 -> 1024 3x3 12.0 / 11.3; with 256 CTAs (2 x 32 x 32 x 512 3x3) 14.6 / 14.9,
+// and the thousands of large layers cost the kernel in front its place (four transformer linears and a convolution at 32768 rows
+// 10 % slower).  The kernels such layers' products run on let it in (griddep_launch) as they begin.
+int sm_count();             // hq_gemm.cu: SM count of the current device
+inline bool dependent_launch(int64_t grid) { return grid <= int64_t(sm_count()) / 2; }
+
 // hq_gemm_splitk.cu: CTAs a tile's reduction is divided over (0: persistent kernels) and the estimated time of a product.
 struct ProductPlan { int ways; double us; };
 ProductPlan plan_product(int limbs, int64_t out_rows, int tile_rows, int64_t n_pad, int num_kb);
@@ -44,6 +52,18 @@ ProductPlan plan_product(int limbs, int64_t out_rows, int tile_rows, int64_t n_p
 #define HQ_CUDA_OK(expr) do { cudaError_t e__ = (expr); if (e__ != cudaSuccess) return HQ_ERR_CUDA; } while (0)
 
 #ifdef __CUDACC__
+
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, bool dependent, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));

@@ -105,6 +105,7 @@ __device__ __forceinline__ bool wait_splitk(uint64_t* bar, uint32_t parity, Spli
 template <int LIMBS, bool CONV>
 __global__ void __launch_bounds__(kSkThreads, 1)
 qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const SplitKParams p) {
+    griddep_launch();                                  // a small transform behind this kernel may place its CTAs (dependent_launch)
     using Sh = SplitKShape<LIMBS>;
     constexpr int STAGES = Sh::kStages;
     extern __shared__ unsigned char smem_raw[];

@@ -19,7 +19,6 @@
 #include "hq_fwht.cuh"
 
 namespace hq {
-int sm_count();             // hq_gemm.cu: SM count of the current device
 
 namespace {
 
@@ -42,6 +41,7 @@ struct QuantParams {
     uint8_t* z;          // optional second output: the codes with the factors of H_raw that the weights leave to them
     int64_t ld_z;        // (split_codes), one signed byte each, for the one-limb product; z_halved: and behind each row the
     int z_halved;        // further columns of halved weights (halved_columns)
+    int dependent;       // launched as a programmatic dependent: wait before anything is read or written (dependent_launch)
     // optional GroupNorm + SiLU applied to the values as they are loaded (gn_stats == nullptr: off)
     const float* gn_stats;   // [samples][groups][2]: mean, 1/sqrt(var + eps)
     const float* gn_gamma;   // [cols]
@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     constexpr bool LN = PRO == 2 || PRO == 4;
     constexpr bool LN_TABLE = PRO == 2;
     griddep_launch();      // a GEMM launched as a programmatic dependent may start its prologue as this grid drains
+    if (!GN && p.dependent) griddep_wait();
     constexpr int N = 1 << KLOG;
     constexpr int LE = ilog2_c(E);
     constexpr int P = E / 2;                           // two-wide registers per thread
@@ -906,19 +907,8 @@ cudaError_t launch_fast(const QuantParams& p, bool int8_out, int grid, int threa
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
             if (e != cudaSuccess) return e;
         }
-        if (p.gn_stats != nullptr) {
-            // a dependent of the statistics kernel: its rows are on their way before it waits for the statistics (1-2 us)
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(unsigned(grid)); cfg.blockDim = dim3(unsigned(threads));
-            cfg.dynamicSmemBytes = smem; cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr; cfg.numAttrs = 1;
-            return cudaLaunchKernelEx(&cfg, kern, p);
-        }
-        kern<<<grid, threads, smem, st>>>(p);
-        return cudaGetLastError();
+        // with statistics a dependent of the statistics kernel: its rows are on their way before it waits for them (1-2 us)
+        return launch_dependent(kern, dim3(unsigned(grid)), unsigned(threads), smem, st, p.gn_stats != nullptr || p.dependent, p);
     };
     if (p.gn_stats != nullptr && p.gn_silu) {
         if (int8_out) return stat ? go(fwht_quant_fast<KLOG, E, InT, true, true, 1>) : go(fwht_quant_fast<KLOG, E, InT, true, false, 1>);
@@ -1069,6 +1059,7 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
             p.z = zo->z; p.ld_z = zo->ld; p.z_halved = zo->halved;
             zo->written = true;
         }
+        p.dependent = gn == nullptr && dependent_launch(grid);
         cudaError_t e = xdt == HQ_F32
                             ? dispatch_fast<float>(klog, p, cont == HQ_CODES_INT8, grid, threads, smem, st)
                             : dispatch_fast<__nv_bfloat16>(klog, p, cont == HQ_CODES_INT8, grid, threads, smem, st);
