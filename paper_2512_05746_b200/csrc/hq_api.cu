@@ -138,7 +138,8 @@ struct LayerCodes {
     static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows, int more_kb) {
         const int num_kb = int(desc->RS * desc->C_pad / 128), tile_rows = out_rows < 128 ? int(out_rows > 0 ? out_rows : 1) : 128;
         // with two codes per byte the two-limb product unpacks them on one SM a tile (32768 x 2048 -> 512 52 us against 45)
-        const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us * (desc->container == HQ_CODES_NIBBLE ? 1.15 : 1.0);
+        const bool unpacks = desc->container == HQ_CODES_NIBBLE && desc->had_block > 512;
+        const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us * (unpacks ? 1.15 : 1.0);
         const double one = plan_product(1, out_rows, tile_rows, desc->N_pad, num_kb + more_kb).us;
         return two - one > 0.7 + double(rows) * double(cols) / 5.2e6;
     }

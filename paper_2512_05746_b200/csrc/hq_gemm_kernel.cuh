@@ -520,7 +520,6 @@ template <bool NIBBLE, int MODE, bool CONV, int LIMBS_T, int RES_T, bool FRAG>
 __global__ void __launch_bounds__(cta_threads(NIBBLE, FRAG), 1)
 qgemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
              const __grid_constant__ CUtensorMap tmY, const GemmParams p) {
-    griddep_launch();                                  // a small transform behind this kernel may place its CTAs (dependent_launch)
     constexpr bool PERTAP = MODE == kModePerTap;
     static_assert(!PERTAP || LIMBS_T != 0, "the per-tap drain is compiled per number of limbs");
     constexpr int BN = PERTAP ? per_tap_rows(LIMBS_T) : kBN, kBBlock = BN * kBK;      // operand-B rows of a tile, bytes of a K block
