@@ -406,7 +406,9 @@ hq_status hq_qlinear_noalloc(const void* x, hq_dtype xdt, int64_t M, int64_t K, 
  *      or slower);
  *   2  (default) where it measured faster: reductions with streamed weights (K_pad > 512), convolutions, and two-limb
  *      weights at K_pad 512 on problems of at least one 256-row tile per SM; problems of few tiles with a long reduction
- *      run on clusters of 2, 4 or 8 SMs that divide a tile's reduction (one code per byte, bf16 output).
+ *      run on clusters of 2, 4 or 8 SMs that divide a tile's reduction (one code per byte, bf16 output), and hq_qlinear
+ *      as one kernel, transform included, where its CTAs of 16 rows x 64 channels are all resident at once (blocks of
+ *      32 .. 512 channels, reductions of 128 .. 1024 in whole K blocks, an even number of output channels).
  * Results are bit-identical in every mode.  Returns the previous mode.  Process-wide, not thread-safe. */
 int hq_set_pair_gemm(int mode);
 

@@ -46,6 +46,13 @@ hq_status launch_hadamard_quant_width2(const void* x, hq_dtype xdt, int64_t Nb, 
                                        float* scale_out, cudaStream_t st);
 
 int sm_count();             // hq_gemm.cu: SM count of the current device
+// hq_small.cu: a linear layer of few rows as one kernel
+bool small_linear_takes(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc, const void* w_dev,
+                        const float* scale_w, int a_bits, hq_scale_mode mode, const float* static_scale, const void* y, hq_dtype ydt,
+                        int64_t ldy, const void* workspace, int64_t ws_used);
+hq_status launch_small_linear(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc, const void* w_dev,
+                              const float* scale_w, const float* bias, int a_bits, hq_scale_mode mode, const float* static_scale,
+                              float alpha, void* y, int64_t ldy, void* codes, int64_t ld_codes, float* scales, cudaStream_t st);
 
 namespace {
 int64_t code_pitch(int64_t cols, hq_container cont) {
@@ -236,6 +243,11 @@ static hq_status qlinear_impl(const void* x, hq_dtype xdt, int64_t M, int64_t K,
     s = check_residual(residual, y, ydt, desc->N, ldy);
     if (s != HQ_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (residual == nullptr && small_linear_takes(x, xdt, M, K, ldx, desc, w_dev, scale_w, a_bits, mode, static_scale, y, ydt, ldy,
+                                               workspace, int64_t(need)))
+        return launch_small_linear(x, xdt, M, K, ldx, desc, w_dev, scale_w, bias, a_bits, mode, static_scale, hq_alpha_for(desc), y, ldy,
+                                   workspace, code_pitch(K, cont),
+                                   reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + scales_offset(M, K, cont)), st);
     ResidualAdd res{static_cast<const __nv_bfloat16*>(residual), false};
     LayerCodes lc(desc, w_dev, a_bits, mode, M, K, 1, cont, workspace, ws_bytes, halved_product_covers(M, y, ydt, ldy));
     s = launch_hadamard_quant(x, xdt, M, K, ldx, desc->had_block, a_bits, mode, static_scale, lc.codes, cont, lc.ld, lc.scales, st,
