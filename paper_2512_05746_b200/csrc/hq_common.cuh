@@ -279,8 +279,9 @@ __host__ __device__ constexpr uint32_t make_idesc_i8(int M, int N) {
 
 // One lane of a converged warp, the same at every call.  Unlike a comparison of the lane number it tells the compiler that what
 // follows runs on one lane: the operands of tensor-core and copy instructions stay in uniform registers.  Issuing warps of the
-// split and paired products and of the attention core (2 x 8 x 8 x 2048 -> 1024 3x3 13.1 -> 12.0 us, 64 x 64 x 64 x 256 3x3 151 ->
-// 148); in the one-CTA product kernel level or slower (256 x 256 -> 256 6.2 / 6.4 us, 32768 x 256 -> 1024 25-28 / 31-33).
+// split and streamed paired products and of the attention core (2 x 8 x 8 x 2048 -> 1024 3x3 13.1 -> 12.0 us, 64 x 64 x 64 x 256 3x3
+// 151 -> 148, 16001 x 1024 -> 1288 with 8-bit codes 39.65 -> 39.1); level or slower in the one-CTA kernel (256 x 256 -> 256 6.2 / 6.4 us,
+// 32768 x 256 -> 1024 25-28 / 31-33) and in the resident paired one (32768 x 512 -> 1536 59.9 / 60.3).
 __device__ __forceinline__ bool elect_one() {
     uint32_t pred;
     asm volatile(

@@ -301,7 +301,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer (one per CTA, its own halves)
-        if (elect_one()) {
+        if (lane == 0) {
             int stage = 0; uint32_t phase = 0;
             int cur_n = -1, reloads = 0;
             bool ok = true;
@@ -345,7 +345,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (rank == 0 && elect_one()) {
+        if (lane == 0 && rank == 0) {
             const uint32_t idesc = make_idesc_i8(256, kBN);
             int stage = 0; uint32_t phase = 0;
             int cur_n = -1, reloads = 0;
