@@ -141,14 +141,15 @@ struct LayerCodes {
     // no round of tiles is saved it only costs: 256 x 256 -> 256 6.1 / 6.8 us, 8 x 64 x 64 x 256 3x3 stride 2 16.5 / 17.6.
     // Blocks above 512, the same rule: 65536 x 4096 -> 4096 1657 / 1127 us (the second byte costs the transform 84 of its 341 us),
     // 65536 x 4096 -> 1024 536 / 487, 32768 x 2048 -> 2048 195 / 161, 65536 x 1024 -> 1024 125 / 113, 32768 x 2048 -> 512 with two
-    // codes per byte 113 / 111; not taken: the same with one code per byte, 101 / 104.
+    // codes per byte 113 / 111; not taken: the same with one code per byte, 101 / 104 (halved weights; where they fit a byte the product
+    // gains 13.6 us and the transform, whose threads hold 64 values, loses 14.8: 4.6 TB/s).
     static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows, int more_kb) {
         const int num_kb = int(desc->RS * desc->C_pad / 128), tile_rows = out_rows < 128 ? int(out_rows > 0 ? out_rows : 1) : 128;
         // with two codes per byte the two-limb product unpacks them on one SM a tile (32768 x 2048 -> 512 52 us against 45)
         const bool unpacks = desc->container == HQ_CODES_NIBBLE && desc->had_block > 512;
         const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us * (unpacks ? 1.15 : 1.0);
         const double one = plan_product(1, out_rows, tile_rows, desc->N_pad, num_kb + more_kb).us;
-        return two - one > 0.7 + double(rows) * double(cols) / 5.2e6;
+        return two - one > 0.7 + double(rows) * double(cols) / (desc->had_block > 512 ? 4.6e6 : 5.2e6);
     }
     const void* a() const { return z.written ? z.z : codes; }
     int64_t lda() const { return z.written ? z.ld : ld; }
