@@ -151,8 +151,10 @@ __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bul
 // one be scheduled once every CTA has called it or exited.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// A load of what the kernel before this one wrote, for use behind griddep_wait(): through the non-coherent path (__ldg) the
-// compiler may move the load in front of the wait, which gave a layer the scale that the workspace held before.
+// Loads of what a kernel before this one wrote, for use behind griddep_wait(): through the non-coherent path (__ldg) the
+// compiler may move the load in front of the wait, which gave a layer the scale that the workspace held before, and the path
+// itself is for data that nothing writes while the kernel runs; the intrinsics with a caching hint (__ldcs, __ldcg) promise no
+// order against the wait either.  The _cs forms carry the hint of a load that nothing reads again, the _cg forms stay out of L1.
 __device__ __forceinline__ float ld_dependent(const float* p) {
     float v;
     asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
@@ -168,6 +170,20 @@ __device__ __forceinline__ float2 ld_dependent2(const float2* p) {
     asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
     return v;
 }
+#define HQ_LD_DEPENDENT(HINT)                                                                                                          \
+    __device__ __forceinline__ float4 ld_dependent_##HINT(const float4* p) {                                                           \
+        float4 v;                                                                                                                      \
+        asm volatile("ld.global." #HINT ".v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory"); \
+        return v;                                                                                                                      \
+    }                                                                                                                                  \
+    __device__ __forceinline__ uint2 ld_dependent_##HINT(const uint2* p) {                                                             \
+        uint2 v;                                                                                                                       \
+        asm volatile("ld.global." #HINT ".v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");                         \
+        return v;                                                                                                                      \
+    }
+HQ_LD_DEPENDENT(cs)
+HQ_LD_DEPENDENT(cg)
+#undef HQ_LD_DEPENDENT
 // at most one bulk store group of this thread may still be reading shared memory
 __device__ __forceinline__ void bulk_wait_read_1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }

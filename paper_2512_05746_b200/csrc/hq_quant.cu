@@ -193,8 +193,14 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
                              ? reinterpret_cast<const InT*>(p.x2) + r * p.ldx2 + (c0 - p.split)
                              : reinterpret_cast<const InT*>(p.x) + r * p.ldx + c0;
 #pragma unroll
-        for (int i = 0; i < E / 4; ++i) cur[i] = __ldcs(reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i)));
+        for (int i = 0; i < E / 4; ++i) {
+            const Raw* from = reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i));
+            cur[i] = PRO == 0 ? ld_dependent_cs(from) : __ldcs(from);
+        }
     }
+    // A plain transform's scale may come from the kernel in front like its rows; with a prologue both were complete before the launch
+    // (the statistics kernel, which is never a dependent, or none is in front).
+    const float given = STATIC && PRO == 0 ? ld_dependent(p.static_scale) : 0.f;
     const int64_t ln_group = LN && p.ln_rows_per_group > 0 ? (int64_t(blockIdx.x) * p.rows_per_cta) / p.ln_rows_per_group : 0;
     if (LN_TABLE) {
         // The affine vectors are copied asynchronously while the row statistics are taken.
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
             inv = 0.f;
         }
     } else {
-        scale = __ldg(p.static_scale);
+        scale = PRO == 0 ? given : __ldg(p.static_scale);
         inv = p.norm / scale;
     }
 

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
         using Raw = typename std::conditional<sizeof(InT) == 4, float4, uint2>::type;
         Raw raw[E / 4];
 #pragma unroll
-        for (int i = 0; i < E / 4; ++i) raw[i] = valid ? __ldcg(reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i))) : Raw{};
+        for (int i = 0; i < E / 4; ++i) raw[i] = valid ? ld_dependent_cg(reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i))) : Raw{};
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) {
             float4 f;
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
             inv = 0.f;
         }
     } else {
-        scale = __ldcg(p.static_scale);
+        scale = ld_dependent(p.static_scale);
         inv = p.norm / scale;
     }
     {

@@ -1,0 +1,67 @@
+"""A fused call may be launched while the kernel in front of it on the stream is still running.  What that kernel wrote, it reads as
+if the two were synchronised in between: calls chained through an operand, many times over changing values and in a graph, give
+what the same calls give one at a time."""
+import pytest
+
+from paper_2512_05746_b200 import inputs
+
+
+def chained(torch, step, values, outputs):
+    """`step(value)` for every value: one at a time, back to back, and as one graph; the `outputs` of each must agree."""
+    def collect(sync=False):
+        out = []
+        for v in values:
+            step(v)
+            if sync:
+                torch.cuda.synchronize()
+            out.append([t.clone() for t in outputs])
+        return out
+
+    apart, together = collect(sync=True), collect()
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        graph.capture_begin()
+        try:
+            captured = collect()
+        finally:
+            graph.capture_end()
+    torch.cuda.current_stream().wait_stream(stream)
+    graph.replay()
+    torch.cuda.synchronize()
+    for i, want in enumerate(apart):
+        for a, b, c in zip(want, together[i], captured[i]):
+            assert torch.equal(a, b) and torch.equal(a, c), i
+    assert any(not torch.equal(a, b) for a, b in zip(apart[0], apart[1])), "the values were meant to matter"
+
+
+def inputs_of(torch, shape, n, dtype=None):
+    gen = torch.Generator(device="cuda").manual_seed(shape[-1])
+    x = torch.randn((n, *shape), generator=gen, device="cuda") * torch.rand((n, *[1] * len(shape)), generator=gen, device="cuda").mul(4).exp()
+    return list(x if dtype is None else x.to(dtype))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["quantize", "linear", "linear of 2048", "convolution"])
+def test_static_scale_from_the_transform_in_front(kind):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    K = 2048 if kind == "linear of 2048" else 256
+    rows, N = 128, 256
+    pw = hq.hq_weight_prepare(inputs.weights((N, 3, 3, K) if kind == "convolution" else (N, K), seed=1), 4, 256, hq.HQ_W_FOLDED,
+                              hq.HQ_CODES_INT8).to_device()
+    codes, own = (torch.zeros((rows, K), dtype=torch.uint8, device="cuda") for _ in range(2))
+    s = torch.ones((rows,), device="cuda")
+    ws = torch.zeros((hq.hq_workspace_size(rows, K, hq.HQ_CODES_INT8),), dtype=torch.uint8, device="cuda")
+    y = torch.zeros((rows, N), dtype=torch.bfloat16, device="cuda")
+
+    def step(x):
+        hq.hq_hadamard_quant(x, 256, 4, codes, hq.HQ_CODES_INT8, scales=s)
+        if kind == "quantize":
+            hq.hq_hadamard_quant(x, 256, 4, own, hq.HQ_CODES_INT8, static_scale=s[:1])
+        elif kind == "convolution":
+            hq.hq_qconv(x.view(2, 8, 8, K), pw, 3, 3, 1, 1, None, 4, y.view(2, 8, 8, N), ws, static_scale=s[:1])
+        else:
+            hq.hq_qlinear(x, pw, None, 4, y, ws, static_scale=s[:1])
+
+    chained(torch, step, inputs_of(torch, (rows, K), 200), [own if kind == "quantize" else y])
