@@ -180,6 +180,11 @@ __device__ __forceinline__ float2 ld_dependent2(const float2* p) {
         uint2 v;                                                                                                                       \
         asm volatile("ld.global." #HINT ".v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");                         \
         return v;                                                                                                                      \
+    }                                                                                                                                  \
+    __device__ __forceinline__ uint4 ld_dependent_##HINT(const uint4* p) {                                                             \
+        uint4 v;                                                                                                                       \
+        asm volatile("ld.global." #HINT ".v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory"); \
+        return v;                                                                                                                      \
     }
 HQ_LD_DEPENDENT(cs)
 HQ_LD_DEPENDENT(cg)

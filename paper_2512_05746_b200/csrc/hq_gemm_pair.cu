@@ -173,7 +173,7 @@ __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg
     auto request = [&](int st) {
 #pragma unroll
         for (int j = 0; j < 2; ++j)
-            rn[RES ? j : 0] = res != nullptr && st * 16 + 8 * j < ncols ? __ldcs(reinterpret_cast<const uint4*>(res + st * 16 + 8 * j))
+            rn[RES ? j : 0] = res != nullptr && st * 16 + 8 * j < ncols ? ld_dependent_cs(reinterpret_cast<const uint4*>(res + st * 16 + 8 * j))
                                                                         : make_uint4(0u, 0u, 0u, 0u);
     };
     if constexpr (RES) request(0);

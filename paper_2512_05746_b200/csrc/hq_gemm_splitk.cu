@@ -213,13 +213,14 @@ qgemm_splitk_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         if (p.pdl) griddep_wait();                     // scale_a comes from the kernel before this one
         if ((e & 127) < rows) sa_eff = p.alpha * ld_dependent(p.scale_a + (p.sa_scalar ? 0 : row0 + (e & 127)));
         // from here on every CTA's ring is its receive buffer: [from CTA][4-column group][row] of 16-byte pieces
-        uint4 resid[4];                                // the residual's share, 8 columns each (cw <= 64), requested ahead
+        uint4 resid[4];                                // the residual's share, 8 columns each (cw <= 64), requested ahead; the kernel
+                                                       // in front of the transform may have written it
         if (p.res != nullptr) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const int g = (e >> 7) + 2 * i, col0 = n_tile * kSkCols + rank * cw + g * 8;
                 resid[i] = g < cw / 8 && col0 < p.N && (e & 127) < rows
-                               ? __ldg(reinterpret_cast<const uint4*>(p.res + (row0 + (e & 127)) * p.ldy + col0)) : make_uint4(0u, 0u, 0u, 0u);
+                               ? ld_dependent_cs(reinterpret_cast<const uint4*>(p.res + (row0 + (e & 127)) * p.ldy + col0)) : make_uint4(0u, 0u, 0u, 0u);
             }
         }
         ok = wait_splitk<true>(&ctl->ready, 0, ctl, p.dev_status, kStatusAccumWait);

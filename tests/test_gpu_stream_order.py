@@ -65,3 +65,29 @@ def test_static_scale_from_the_transform_in_front(kind):
             hq.hq_qlinear(x, pw, None, 4, y, ws, static_scale=s[:1])
 
     chained(torch, step, inputs_of(torch, (rows, K), 200), [own if kind == "quantize" else y])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,K,N,room", [
+    (2, 1024, 1024, False),        # both products divided over clusters, the transform between them a dependent
+    (64, 256, 256, False),         # the layer in front is one kernel
+    (300, 768, 264, False),
+    (4096, 1024, 1024, True),      # pairs of SMs
+])
+def test_residual_from_the_layer_in_front(M, K, N, room):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    first, second = (hq.hq_weight_prepare(inputs.weights((N, K), seed=i), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device()
+                     for i in (1, 2))
+    ws1, ws2 = (torch.zeros((max(hq.hq_layer_workspace_size(first, 4, M), hq.hq_workspace_size(M, K, 1)) if room else
+                             (M * K + 255) // 256 * 256 + 4 * M,), dtype=torch.uint8, device="cuda") for _ in range(2))
+    x2 = inputs_of(torch, (M, K), 1, torch.bfloat16)[0]
+    r, y = (torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+
+    def step(x):
+        hq.hq_qlinear(x, first, None, 4, r, ws1, dev_status=status)
+        hq.hq_qlinear(x2, second, None, 4, y, ws2, dev_status=status, residual=r)
+
+    chained(torch, step, inputs_of(torch, (M, K), 200 if M < 1000 else 20, torch.bfloat16), [y])
+    hq.hq_check_status(status)
