@@ -280,13 +280,18 @@ def hq_layer_workspace_size(pw: PreparedWeight, a_bits: int, rows: int, static: 
     return int(out.value)
 
 
+def _takes_residual(y, residual) -> bool:
+    """Whether `residual` can be added to the output y: both dense, of one shape, and bf16 (the only type the entry points that add
+    one read and write; two bytes of another type would be taken for it)."""
+    return _dtype_code(y) == _dtype_code(residual) == HQ_BF16 and residual.shape == y.shape and y.is_contiguous() and residual.is_contiguous()
+
+
 def hq_qlinear(x, pw: PreparedWeight, bias, a_bits: int, y, workspace, static_scale=None, dev_status=None,
                stream=None, residual=None) -> None:
     """residual: bf16 tensor of y's shape added to the rounded output (y bf16 and dense, one scale per row), or None."""
     if residual is not None:
         M, K = x.shape
-        if static_scale is not None or y.element_size() != 2 or not (y.is_contiguous() and residual.is_contiguous()) or \
-                residual.shape != y.shape or residual.dtype != y.dtype:
+        if static_scale is not None or not _takes_residual(y, residual) or tuple(y.shape) != (M, pw.desc.N):
             raise ValueError("hq_qlinear: a residual goes with a dense bf16 output of its shape and one scale per row")
         _check(lib.hq_qlinear_add(_dptr(x), _dtype_code(x), M, K, x.stride(0), C.byref(pw.desc), _dptr(pw.blob_dev),
                                   _dptr(pw.s_w_dev), _dptr(bias), a_bits, _dptr(residual), _dptr(y), _dptr(workspace),
@@ -350,8 +355,7 @@ def hq_gn_silu_qconv(x, groups: int, gamma, beta, eps: float, pw: PreparedWeight
     Nb, H, W, Cin = x.shape
     mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
     if residual is not None:
-        if x2 is not None or y.element_size() != 2 or not (y.is_contiguous() and residual.is_contiguous()) or \
-                residual.shape != y.shape or residual.dtype != y.dtype:
+        if x2 is not None or not _takes_residual(y, residual) or y.shape[-1] != pw.desc.N:
             raise ValueError("hq_gn_silu_qconv: a residual goes with a dense bf16 output of its shape and a single input")
         _check(lib.hq_gn_silu_qconv_add(_dptr(x), _dtype_code(x), Nb, H, W, Cin, groups, _dptr(gamma), _dptr(beta), _dptr(pre_bias),
                                         Cin if pre_bias is None else pre_bias.stride(0), eps, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias),

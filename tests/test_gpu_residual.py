@@ -95,3 +95,28 @@ def test_residuals_that_cannot_be_added_are_refused_before_a_launch():
     assert call(odd, p(0x3000), p(0x2000)) == 2                       # 36 columns
     assert call(lin, p(0x3008), p(0x2000)) == 4
     assert call(lin, p(0x3000), p(0x2008)) == 4
+
+
+def test_a_residual_of_another_type_or_shape_is_refused():
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    lin = hq.hq_weight_prepare(inputs.weights((64, 256), seed=1), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device("cpu")
+    conv = hq.hq_weight_prepare(inputs.weights((64, 3, 3, 256), seed=1), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device("cpu")
+    x, px = torch.zeros((8, 256)), torch.zeros((1, 4, 4, 256))
+    g, ws, scr = torch.zeros(256), torch.zeros(1 << 16, dtype=torch.uint8), torch.zeros(1 << 10, dtype=torch.uint8)
+
+    class Stream:
+        cuda_stream = 0
+
+    def both(error, y, residual):
+        with pytest.raises(error):
+            hq.hq_qlinear(x, lin, None, 4, y, ws, residual=residual, stream=Stream)
+        with pytest.raises(error):
+            hq.hq_gn_silu_qconv(px, 32, g, g, 1e-5, conv, 3, 3, 1, 1, None, 4, y.view(1, -1, 4, y.shape[-1]), ws, scr, stream=Stream,
+                                residual=residual.view(1, -1, 4, residual.shape[-1]))
+    both(TypeError, *(torch.zeros((8, 64), dtype=torch.float16) for _ in range(2)))
+    both(TypeError, *(torch.zeros((8, 64), dtype=torch.int16) for _ in range(2)))
+    both(ValueError, *(torch.zeros((8, 64)) for _ in range(2)))
+    both(ValueError, torch.zeros((8, 64), dtype=torch.bfloat16), torch.zeros((8, 64)))
+    both(ValueError, *(torch.zeros((8, 72), dtype=torch.bfloat16) for _ in range(2)))        # rows longer than the layer's
+    both(ValueError, torch.zeros((8, 64), dtype=torch.bfloat16), torch.zeros((4, 64), dtype=torch.bfloat16))
