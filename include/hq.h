@@ -169,8 +169,10 @@ hq_status hq_qconv2d(const void* a_codes, hq_container cont, int a_bits, int64_t
  *    more at 2048 and 4096 columns for the further columns of halved weights).
  * alpha is derived from the descriptor.  y pitch ldy elements.
  * The product kernel is launched so that it may begin (set-up, first weight tile) while the transform kernel is still
- * running; it waits for the transform before it touches codes or activation scales.  Work enqueued on the stream before
- * the call has completed before either kernel starts, as usual. */
+ * running; it waits for the transform before it touches codes or activation scales.  The first kernel of a call may itself be
+ * placed on the device while the kernel in front of it in the stream still runs, but reads and writes nothing, and lets nothing
+ * behind it begin, until that has completed: work enqueued on the stream before the call is complete before any operand
+ * of the call (inputs, weights, scales, bias, residual) is read, as usual. */
 hq_status hq_workspace_size(int64_t rows, int64_t cols, hq_container cont, size_t* bytes);
 hq_status hq_layer_workspace_size(const hq_weight_desc* desc, int a_bits, hq_scale_mode mode, int64_t rows, int stride,
                                   size_t* bytes);

@@ -39,7 +39,7 @@ struct ResidualAdd { const __nv_bfloat16* r; bool done; };
 
 // Whether a plain transform of `grid` CTAs is launched as a programmatic dependent of whatever precedes it in the stream: its CTAs are
 // placed while that kernel drains and wait (griddep_wait) before they touch anything.  Small layers one after the other: 2 x 2048 -> 1024
-// 8.2 / 6.7 us a call, 2 x 8 x 8 x 2048 -> 1024 3x3 15.1 / 13.7; with 256 CTAs (2 x 32 x 32 x 512 3x3) 14.6 / 14.9, and the thousands of
+// 8.2 / 6.3 us a call, 2 x 8 x 8 x 2048 -> 1024 3x3 15.1 / 13.2; with 256 CTAs (2 x 32 x 32 x 512 3x3) 14.6 / 14.9, and the thousands of
 // large layers cost the kernel in front its place (four transformer linears and a convolution at 32768 rows 10 % slower).  The split
 // product such layers run on lets it in (griddep_launch) as it begins; in the one-CTA product that cost 2 x 48 x 48 x 768 -> 944 1x1
 // stride 2 12.5 / 12.8.

@@ -144,7 +144,10 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     constexpr bool GN_SILU = PRO == 1;
     constexpr bool LN = PRO == 2 || PRO == 4;
     constexpr bool LN_TABLE = PRO == 2;
-    griddep_launch();      // a GEMM launched as a programmatic dependent may start its prologue as this grid drains
+    // A GEMM launched as a programmatic dependent may start its prologue, weights included, as this grid drains.  A plain transform,
+    // which may itself have been let in by the kernel in front, lets it in behind its own wait only: weights, their scales and the
+    // bias are then read when everything older than the transform is complete.
+    if (PRO != 0) griddep_launch();
     constexpr int N = 1 << KLOG;
     constexpr int LE = ilog2_c(E);
     constexpr int P = E / 2;                           // two-wide registers per thread
@@ -186,7 +189,7 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     Raw cur[E / 4];
     // Waits where the launch was a dependent one, and is nothing otherwise.  Without a look at p.dependent, which cost the first loads
     // 0.3 us in every launch (109 x 8 x 8 x 1024 -> 216 1x1 14.69 / 14.40 us a call).
-    if (PRO == 0) griddep_wait();
+    if (PRO == 0) { griddep_wait(); griddep_launch(); }
     {
         const int64_t c0 = int64_t(blk) * N, r = valid ? row : 0;
         const InT* src = (p.x2 != nullptr && c0 >= p.split)

@@ -1,15 +1,18 @@
 // A linear layer of few rows as ONE kernel: transform, quantization, integer product and rescale (Eq. 10, Eq. 3, Eq. 12).
 //
 // Latency bound: the two kernels of such a layer (256 x 256 -> 256: 5.4 us on the device one after the other, two launches of
-// 2.5 us each on the host) are longer than their work.  A CTA takes 16 rows and 64 output channels.  Its weights are on their way into
-// shared memory (`cp.async`) before anything else; K / 32 threads a row transform and quantize as the transform kernel does (the same
+// 2.5 us each on the host) are longer than their work.  A CTA takes 16 rows and 64 output channels; its weights land in shared
+// memory (`cp.async`) while K / 32 threads a row transform and quantize as the transform kernel does (the same
 // building blocks in the same order, so the same codes), every column's CTA over again -- a few hundred cycles against a trip of the
 // codes through memory and a launch -- and the first column's CTA leaves codes and scales in the workspace.  The product of 16 x 64 x K
 // is too small for a tensor-memory accumulator to pay its set-up: `mma.sync` m16n8k32 on fragments read from shared memory
 // (rows 16 bytes apart from a multiple of 128: conflict-free), both limbs in accumulators of their own.
-// Launched as a programmatic dependent, and letting the next kernel in at its start: only weights are touched before the wait.
-// Two kernels / one, in a graph: 256 x 256 -> 256 5.3 / 3.0 us (a call 7.1 / 6.5), 70 x 512 -> 1024 6.0 / 3.7, 200 x 768 -> 640 6.5 / 5.2,
-// 2 x 1024 -> 1024 5.3 / 4.2, 128 x 1024 -> 1024 7.3 / 6.2, 2000 x 128 -> 64 5.1 / 3.7.
+// Launched as a programmatic dependent, and letting the next kernel in at its start: nothing is read before the wait, weights
+// included, since the kernel in front may be the one that writes them.
+// Two kernels / one, in a graph: 256 x 256 -> 256 5.4 / 3.2 us (a call 6.3 / 4.2), 70 x 512 -> 1024 6.5 / 5.3, 200 x 768 -> 640 6.4 / 4.6,
+// 2 x 1024 -> 1024 5.9 / 5.1, 128 x 1024 -> 1024 7.3 / 5.9, 2000 x 128 -> 64 5.1 / 3.6.  With a division per 16 bytes copied instead of
+// one per thread 4.2, 6.4, 5.7, 6.2, 6.9 and 4.6; with one bulk copy a channel and limb, 55 cycles each from the warp that
+// issues them, 6.3, 7.4, 7.1, 7.2, 7.8 and 6.8.
 #include <type_traits>
 
 #include "hq_common.cuh"
@@ -46,10 +49,11 @@ __host__ __device__ inline SmallLayout small_layout(int K, int limbs, int gs_byt
 __host__ __device__ constexpr int small_xch_bytes(int m, int gs) { return m * gs * 16; }
 template <int KLOG>
 __host__ __device__ constexpr int small_xch_bytes(int m) { return small_xch_bytes(m, FwhtShape<KLOG, 32>::GS); }
+constexpr int kSmStatic = 8 * kSmRows + 8 * kSmCols;    // the kernel's other shared arrays
 // CTAs of the kernel that an SM holds at once, by its shared memory (227 KB, 1 KB of it a CTA's own) and the registers of 128 a thread
 int small_resident(int K, int limbs, int block) {
     constexpr int gs[] = {FwhtShape<5, 32>::GS, FwhtShape<6, 32>::GS, FwhtShape<7, 32>::GS, FwhtShape<8, 32>::GS, FwhtShape<9, 32>::GS};
-    const int smem = small_layout(K, limbs, small_xch_bytes(K / block, gs[ilog2(block) - 5])).total + 1024;
+    const int smem = small_layout(K, limbs, small_xch_bytes(K / block, gs[ilog2(block) - 5])).total + kSmStatic + 1024;
     const int by_smem = 227 * 1024 / smem, by_regs = 1024 / K, most = by_smem < by_regs ? by_smem : by_regs;
     return most < 4 ? most : 4;
 }
@@ -69,7 +73,7 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
     using Sh = FwhtShape<KLOG, E>;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned int rowmax[kSmRows];
-    __shared__ float sScale[kSmRows];
+    __shared__ float sScale[kSmRows], sSw[kSmCols], sBias[kSmCols];
     const int K = p.K, pitch = K + 16;
     const SmallLayout L = small_layout(K, LIMBS, small_xch_bytes<KLOG>(p.m));
     unsigned char* sA = smem + L.a_off;
@@ -79,20 +83,9 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
     const int n0 = blockIdx.x * kSmCols;
     const int64_t m0 = int64_t(blockIdx.y) * kSmRows;
 
-    griddep_launch();
-    // channel n's rows in the blob: group n / 128 of 128 * LIMBS rows, "hi" in front of "lo"; rows past the last group are never read
-    {
-        const int chunks = K / 16;
-        for (int e = tid; e < kSmCols * LIMBS * chunks; e += blockDim.x) {
-            const int r = e / chunks, c = e - r * chunks;             // r: limb * 64 + channel
-            const int n = n0 + (r & (kSmCols - 1)), limb = r / kSmCols;
-            const int64_t row = int64_t(n >> 7) * (128 * LIMBS) + limb * 128 + (n & 127);
-            cp_async_cg_16(sB + r * pitch + c * 16, p.w + row * K + c * 16);
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
+    griddep_launch();                                  // whoever it lets in waits for this kernel before it reads anything
     if (tid < kSmRows) rowmax[tid] = 0u;
-    griddep_wait();                                    // the input, and whoever used the workspace and the output before
+    griddep_wait();                                    // the operands, and whoever used the workspace and the output before
 
     const int tpr = K / E;                             // threads per row; a Hadamard block's are neighbours in one warp
     const int r = tid / tpr, tr = tid - r * tpr;
@@ -101,12 +94,26 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
     const bool valid = row < p.M;                      // rows past the end are zeros (nothing is read for them: 64 CTAs all reading one
                                                        // last row again cost 2 x 1024 -> 4096 2.4 us) and store nothing
     f32x2 v[P];
+    float sw = 0.f, bias = 0.f, given = 0.f;           // of column tid; the static scale
     {
         const InT* src = reinterpret_cast<const InT*>(p.x) + (valid ? row : 0) * p.ldx + blk * N;
         using Raw = typename std::conditional<sizeof(InT) == 4, float4, uint2>::type;
         Raw raw[E / 4];
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) raw[i] = valid ? ld_dependent_cg(reinterpret_cast<const Raw*>(src + 4 * (tb + TB * i))) : Raw{};
+        // The weights, behind the rows: every thread the same 16 bytes of each eighth channel.  Channel n's rows in the blob: group n / 128
+        // of 128 * LIMBS rows, "hi" in front of "lo"; rows past the last group are never read.
+        const int w8 = r >> 1, c = (tid - w8 * (K / 16)) * 16;       // K / 2 threads: eight channels at a time
+        const unsigned char* from = p.w + (int64_t(n0 >> 7) * (128 * LIMBS) + (n0 & 127) + w8) * K + c;
+#pragma unroll
+        for (int i = 0; i < 8 * LIMBS; ++i) cp_async_cg_16(sB + (w8 + 8 * i) * pitch + c, from + ((i >> 3) * 128 + 8 * (i & 7)) * K);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (tid < kSmCols) {
+            const int col = n0 + tid;
+            sw = col < p.N ? ld_dependent(p.scale_w + col) : 0.f;
+            bias = col < p.N && p.bias != nullptr ? ld_dependent(p.bias + col) : 0.f;
+        }
+        if (STATIC) given = ld_dependent(p.static_scale);
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) {
             float4 f;
@@ -143,7 +150,7 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
             inv = 0.f;
         }
     } else {
-        scale = ld_dependent(p.static_scale);
+        scale = given;
         inv = p.norm / scale;
     }
     {
@@ -161,6 +168,7 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
             else if (row == 0 && tr == 0) p.scales[0] = scale;
         }
         if (tr == 0) sScale[r] = scale;
+        if (tid < kSmCols) { sSw[tid] = sw; sBias[tid] = bias; }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -187,8 +195,7 @@ __global__ void __launch_bounds__(512) qlinear_small_kernel(const SmallParams p)
         }
         const int col = n0 + nt * 8 + 2 * (lane & 3);                 // and the next one: N is even
         if (col < p.N) {
-            const float sw0 = __ldg(p.scale_w + col), sw1 = __ldg(p.scale_w + col + 1);
-            const float b0 = p.bias != nullptr ? __ldg(p.bias + col) : 0.f, b1 = p.bias != nullptr ? __ldg(p.bias + col + 1) : 0.f;
+            const float sw0 = sSw[col - n0], sw1 = sSw[col - n0 + 1], b0 = sBias[col - n0], b1 = sBias[col - n0 + 1];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int rr = g + 8 * h;
@@ -240,8 +247,8 @@ cudaError_t dispatch_small(int klog, const SmallParams& p, int limbs, cudaStream
 // weights of 64 channels and the rows' exchange buffers fill the shared memory there), an even number of bf16 output channels in
 // rows of whole pairs, and no more CTAs than the SMs hold at once
 // (small_resident): within one round of CTAs it was the faster of the two at every size looked at (K = 128 to 1024, both numbers of limbs,
-// M = 2 to 2048, N = 64 to 8192), beyond it the slower one almost everywhere: 512 x 512 -> 512 6.2 / 5.6 us on 256 of 296 CTAs, 48 x 512 ->
-// 8192 6.1 / 8.9 on 384, 512 x 768 -> 512 7.7 / 10.1 on 256 of 148.
+// M = 2 to 2000, N = 64 to 4096), beyond it the slower one almost everywhere: 512 x 512 -> 512 6.5 / 5.7 us on 256 of 296 CTAs, 48 x 512 ->
+// 8192 6.4 / 8.5 on 384, 512 x 768 -> 512 7.5 / 8.6 on 256 of 148.
 bool small_linear_takes(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64_t ldx, const hq_weight_desc* desc, const void* w_dev,
                         const float* scale_w, int a_bits, hq_scale_mode mode, const float* static_scale, const void* y, hq_dtype ydt,
                         int64_t ldy, const void* workspace, int64_t ws_used) {

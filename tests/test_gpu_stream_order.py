@@ -91,3 +91,33 @@ def test_residual_from_the_layer_in_front(M, K, N, room):
 
     chained(torch, step, inputs_of(torch, (M, K), 200 if M < 1000 else 20, torch.bfloat16), [y])
     hq.hq_check_status(status)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["one kernel", "divided over clusters", "convolution", "resident", "streamed"])
+def test_weights_from_the_transform_in_front(kind):
+    """Codes are weights as a layer of one limb reads them: the transform's rows of codes are the prepared rows, its scales theirs."""
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    M, K, taps = {"one kernel": (64, 256, 1), "divided over clusters": (64, 2048, 1), "convolution": (128, 256, 9),
+                  "resident": (4096, 256, 1), "streamed": (4096, 768, 1)}[kind]
+    N = 256
+    pw = hq.hq_weight_prepare(inputs.weights((N, 3, 3, K) if taps == 9 else (N, K), seed=1), 4, 256, hq.HQ_W_PLAIN, hq.HQ_CODES_INT8)
+    assert pw.desc.limbs == 1 and pw.desc.N_pad == N and pw.desc.max_abs_b == 7
+    pw.blob_dev = torch.zeros((N, taps * K), dtype=torch.uint8, device="cuda")
+    pw.s_w_dev = torch.ones((N,), device="cuda")
+    x = inputs_of(torch, (M, K), 1, torch.bfloat16)[0]
+    ws = torch.zeros((hq.hq_workspace_size(M, K, hq.HQ_CODES_INT8),), dtype=torch.uint8, device="cuda")
+    y = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    ss = torch.tensor([0.1], device="cuda")
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+
+    def step(w):
+        hq.hq_hadamard_quant(w, 256, 4, pw.blob_dev, hq.HQ_CODES_INT8, scales=pw.s_w_dev)
+        if taps == 9:
+            hq.hq_qconv(x.view(2, 8, 8, K), pw, 3, 3, 1, 1, pw.s_w_dev, 4, y.view(2, 8, 8, N), ws, static_scale=ss, dev_status=status)
+        else:
+            hq.hq_qlinear(x, pw, pw.s_w_dev, 4, y, ws, dev_status=status)
+
+    chained(torch, step, inputs_of(torch, (N, taps * K), 100, torch.bfloat16), [y])
+    hq.hq_check_status(status)
