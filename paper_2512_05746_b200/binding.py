@@ -327,12 +327,23 @@ def hq_qconv(x, pw: PreparedWeight, R: int, S: int, stride: int, pad: int, bias,
     _check(_hqcall.qconv(x, pw, R, S, stride, pad, bias, a_bits, y, workspace, static_scale, dev_status, _stream(stream)), "hq_qconv")
 
 
+def _pre_bias_pitch(pre_bias, Nb: int, channels: int, pitched: bool = False) -> int:
+    """Elements between two samples' rows of a GroupNorm call's addend [Nb, channels].  Rows further apart than `channels` go to
+    the entry point that takes a pitch alone."""
+    if pre_bias is None or pre_bias.is_contiguous():
+        return channels
+    if tuple(pre_bias.shape) == (Nb, channels) and pre_bias.stride(1) == 1 and (pitched or Nb == 1):
+        return channels if Nb == 1 else pre_bias.stride(0)
+    raise ValueError("pre_bias: dense rows [Nb, C] (with a pitch of their own where a residual is given)")
+
+
 def hq_gn_silu_quant(x, groups: int, gamma, beta, eps: float, had_block: int, bits: int, codes, container: int,
                      scratch, scales=None, static_scale=None, stream=None, pre_bias=None, x2=None) -> None:
     """GroupNorm(groups) + SiLU of x NHWC (of x + pre_bias[n, c] when a bf16 [Nb, C] addend is given; of the channel
     concatenation [x | x2] when x2 is given), then transform over channels + quantization into codes [Nb*H*W, pitch]."""
     Nb, H, W, Cin = x.shape
     mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
+    _pre_bias_pitch(pre_bias, Nb, Cin + (x2.shape[3] if x2 is not None else 0))
     if x2 is not None:
         _check(lib.hq_gn_silu_quant_cat(_dptr(x), _dptr(x2), Cin, _dtype_code(x), Nb, H, W, Cin + x2.shape[3], groups,
                                         _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps, had_block, bits, mode,
@@ -350,7 +361,7 @@ def hq_gn_silu_qconv(x, groups: int, gamma, beta, eps: float, pw: PreparedWeight
                      bias, a_bits: int, y, workspace, scratch, static_scale=None, dev_status=None, stream=None,
                      pre_bias=None, x2=None, residual=None) -> None:
     """The fused convolution layer with GroupNorm + SiLU in front (x NHWC; pre_bias: bf16 [Nb, C] added to x before the
-    normalisation, or None; x2: the input is the channel concatenation [x | x2], read in place; residual: bf16 tensor of y's
+    normalisation, or None, with rows further apart than C only beside a residual; x2: the input is the channel concatenation [x | x2], read in place; residual: bf16 tensor of y's
     shape added to the rounded output, or None -- with it y is bf16 and x2 None)."""
     Nb, H, W, Cin = x.shape
     mode = HQ_SCALE_PER_ROW if static_scale is None else HQ_SCALE_STATIC
@@ -358,11 +369,13 @@ def hq_gn_silu_qconv(x, groups: int, gamma, beta, eps: float, pw: PreparedWeight
         if x2 is not None or not _takes_residual(y, residual) or y.shape[-1] != pw.desc.N:
             raise ValueError("hq_gn_silu_qconv: a residual goes with a dense bf16 output of its shape and a single input")
         _check(lib.hq_gn_silu_qconv_add(_dptr(x), _dtype_code(x), Nb, H, W, Cin, groups, _dptr(gamma), _dptr(beta), _dptr(pre_bias),
-                                        Cin if pre_bias is None else pre_bias.stride(0), eps, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride, pad, _dptr(pw.s_w_dev), _dptr(bias),
+                                        _pre_bias_pitch(pre_bias, Nb, Cin, pitched=True), eps, C.byref(pw.desc), _dptr(pw.blob_dev), R, S, stride,
+                                        pad, _dptr(pw.s_w_dev), _dptr(bias),
                                         a_bits, mode, _dptr(static_scale), _dptr(residual), _dptr(y), _dptr(workspace),
                                         workspace.nbytes, _dptr(scratch), scratch.nbytes, _dptr(dev_status), _stream(stream)),
                "hq_gn_silu_qconv_add")
         return
+    _pre_bias_pitch(pre_bias, Nb, Cin + (x2.shape[3] if x2 is not None else 0))
     if x2 is not None:
         _check(lib.hq_gn_silu_qconv_cat(_dptr(x), _dptr(x2), Cin, _dtype_code(x), Nb, H, W, Cin + x2.shape[3], groups,
                                         _dptr(gamma), _dptr(beta), _dptr(pre_bias), eps, C.byref(pw.desc), _dptr(pw.blob_dev),

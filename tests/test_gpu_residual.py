@@ -120,3 +120,58 @@ def test_a_residual_of_another_type_or_shape_is_refused():
     both(ValueError, torch.zeros((8, 64), dtype=torch.bfloat16), torch.zeros((8, 64)))
     both(ValueError, *(torch.zeros((8, 72), dtype=torch.bfloat16) for _ in range(2)))        # rows longer than the layer's
     both(ValueError, torch.zeros((8, 64), dtype=torch.bfloat16), torch.zeros((4, 64), dtype=torch.bfloat16))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("Nb,H,W,Cin,Cout", [
+    (3, 16, 16, 768, 776),              # statistics by runs of groups
+    (7, 32, 32, 512, 512),
+    (1, 256, 256, 256, 256),            # one wave over the pixels
+])
+def test_an_addend_with_a_pitch_of_its_own_is_its_dense_copy(Nb, H, W, Cin, Cout):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    gen = torch.Generator(device="cuda").manual_seed(Cin + Nb)
+    x = torch.randn((Nb, H, W, Cin), generator=gen, device="cuda").to(torch.bfloat16)
+    wide = (2 * torch.randn((Nb, 3 * Cin + 128), generator=gen, device="cuda")).to(torch.bfloat16)
+    pw = hq.hq_weight_prepare(inputs.weights((Cout, 3, 3, Cin), seed=Cin), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device()
+    g, bt = torch.ones(Cin, device="cuda"), torch.zeros(Cin, device="cuda")
+    r = (3 * torch.randn((Nb, H, W, Cout), generator=gen, device="cuda")).to(torch.bfloat16)
+    ws = torch.zeros((hq.hq_workspace_size(Nb * H * W, Cin, 1),), dtype=torch.uint8, device="cuda")
+    scr, ss = torch.zeros((Nb * 32 * 24,), dtype=torch.uint8, device="cuda"), torch.tensor([0.3], device="cuda")
+
+    def call(e, residual):
+        y = torch.zeros((Nb, H, W, Cout), dtype=torch.bfloat16, device="cuda")
+        hq.hq_gn_silu_qconv(x, 32, g, bt, 1e-5, pw, 3, 3, 1, 1, None, 4, y, ws, scr, static_scale=ss, pre_bias=e, residual=residual)
+        return y
+    sliced = wide[:, Cin + 64: 2 * Cin + 64]
+    want = torch.empty_like(r)
+    hq.hq_add(call(sliced.contiguous(), None).view(-1), r.view(-1), want.view(-1))
+    assert torch.equal(call(sliced, r), want) and torch.equal(call(sliced.contiguous(), r), want)
+
+
+def test_an_addend_that_cannot_be_read_is_refused():
+    """The calls without a pitch for it (no residual; codes alone; two inputs) would take its rows from the wrong places."""
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    conv = hq.hq_weight_prepare(inputs.weights((64, 3, 3, 256), seed=1), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device("cpu")
+    x, half = torch.zeros((2, 4, 4, 256)), torch.zeros((2, 4, 4, 128))
+    g, ws, scr = torch.zeros(256), torch.zeros(1 << 16, dtype=torch.uint8), torch.zeros(1 << 10, dtype=torch.uint8)
+    y, r = (torch.zeros((2, 4, 4, 64), dtype=torch.bfloat16) for _ in range(2))
+    codes, sc = torch.zeros((32, 256), dtype=torch.uint8), torch.zeros(32)
+    wide = torch.zeros((2, 512), dtype=torch.bfloat16)
+
+    class Stream:
+        cuda_stream = 0
+
+    def conv_call(e, xs=(x, None), residual=None):
+        hq.hq_gn_silu_qconv(xs[0], 32, g, g, 1e-5, conv, 3, 3, 1, 1, None, 4, y, ws, scr, stream=Stream, pre_bias=e, x2=xs[1], residual=residual)
+    for e in (wide[:, :256], wide[:, ::2], wide.view(4, 256)[::2], wide[:1, :256].expand(2, 256)):
+        with pytest.raises(ValueError):
+            conv_call(e)
+        with pytest.raises(ValueError):
+            conv_call(e, (half, half))
+        with pytest.raises(ValueError):
+            hq.hq_gn_silu_quant(x, 32, g, g, 1e-5, 256, 4, codes, 1, scr, scales=sc, pre_bias=e, stream=Stream)
+    with pytest.raises(ValueError):
+        conv_call(wide[:, ::2], residual=r)
