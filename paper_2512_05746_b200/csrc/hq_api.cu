@@ -329,6 +329,7 @@ static hq_status gn_silu_qconv_impl(const void* x, const void* x2, int64_t split
     s = launch_qconv2d(lc.a(), lc.container(cont), a_bits, Nb, H, W, C, lc.desc(desc), lc.w(w_dev), R, S, stride, pad, lc.scales,
                        mode == HQ_SCALE_STATIC, scale_w, bias, hq_alpha_for(desc), nullptr, y, ydt, dev_status, st, true,
                        residual != nullptr ? &res : nullptr);
+    if (s != HQ_OK) return s;                              // a stride of 0 is refused there
     const int64_t Ho = (H + 2 * pad - R) / stride + 1, Wo = (W + 2 * pad - S) / stride + 1;
     return finish_residual(s, res, y, Nb * Ho * Wo * desc->N, stream);
 }

@@ -175,3 +175,21 @@ def test_an_addend_that_cannot_be_read_is_refused():
             hq.hq_gn_silu_quant(x, 32, g, g, 1e-5, 256, 4, codes, 1, scr, scales=sc, pre_bias=e, stream=Stream)
     with pytest.raises(ValueError):
         conv_call(wide[:, ::2], residual=r)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("stride", [0, 3, -1])
+@pytest.mark.parametrize("with_residual", [False, True])
+def test_a_stride_that_is_refused_is_refused(stride, with_residual):
+    """The size of the output is worked out for the residual: not from a stride that the product has refused."""
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    pw = hq.hq_weight_prepare(inputs.weights((64, 3, 3, 256), seed=1), 4, 256, hq.HQ_W_FOLDED, hq.HQ_CODES_INT8).to_device()
+    x = torch.zeros((1, 8, 8, 256), dtype=torch.bfloat16, device="cuda")
+    y, r = (torch.full((1, 8, 8, 64), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    g, ws = torch.ones(256, device="cuda"), torch.zeros((hq.hq_workspace_size(64, 256, 1),), dtype=torch.uint8, device="cuda")
+    scr = torch.zeros((32 * 24,), dtype=torch.uint8, device="cuda")
+    with pytest.raises(hq.HqError) as e:
+        hq.hq_gn_silu_qconv(x, 32, g, g, 1e-5, pw, 3, 3, stride, 1, None, 4, y, ws, scr, static_scale=torch.tensor([0.3], device="cuda"),
+                            residual=r if with_residual else None)
+    assert e.value.status == 3 and bool((y == 7).all())
