@@ -84,10 +84,10 @@ typedef struct {
     int32_t container;  /* hq_container of the activation codes this blob pairs with (fixes the byte order along K) */
     int64_t C_pad;      /* C rounded up to the kernel's K tile (128); padding is zero */
     int64_t N_pad;      /* N rounded up to 128; padding rows are zero */
-    int64_t bytes;      /* size of the blob */
+    int64_t bytes;      /* bytes of the blob in use; blocks above 512: the one-limb section is there, in the form whose size this is */
     int32_t max_abs_b;  /* largest |B| entry, for the accumulator-range check */
-    int32_t reserved;   /* 1: the one-limb section of the split fold follows (see hq_weight_prepare); 0: it does not (blocks above
-                           512: see bytes) */
+    int32_t reserved;   /* 1: the one-limb section of the split fold follows (see hq_weight_prepare); 0: it does not.  Blocks
+                           above 512: 0, see bytes */
 } hq_weight_desc;
 
 int hq_version(void);
@@ -119,8 +119,9 @@ hq_status hq_hadamard_quant(const void* x, hq_dtype xdt, int64_t rows, int64_t c
  *   weights with four of the log2(had_block) factors of H_raw applied, for the fused layer calls, which give the other
  *   factors to the codes (same integers, half the tensor work).  Blocks of 1024 .. 4096 channels get one too (four factors to
  *   the codes, the rest applied here) where the integers of these weights fit a byte, or, for linear layers of one block of
- *   2048 or 4096, where they do when halved; desc->bytes says which (hq_weight_blob_bytes is the most it may be).  A blob_bytes
- *   that holds only the first section is taken as well; the layer then always runs on two limbs.
+ *   2048 or 4096, where they do when halved; desc->bytes, the end of the last section, says which.  hq_weight_blob_bytes is more
+ *   than either form takes: with any other size in desc->bytes the layer runs on two limbs.  A blob_bytes that holds only the first
+ *   section is taken as well; the layer then always runs on two limbs.
  * Errors: FOLDED/DOUBLE with C % had_block != 0; FOLDED whose integers need more than 2 limbs -> HQ_ERR_OVERFLOW_RISK. */
 int64_t hq_weight_blob_bytes(int64_t N, int32_t RS, int64_t C, int32_t w_bits, int32_t had_block,
                              hq_weight_mode mode);

@@ -89,6 +89,10 @@ int halve_channel(const int16_t* b, int n, int8_t* dst, int8_t* ext) {
     return odd;
 }
 
+// Above 512 channels desc->bytes tells the fused calls whether and in which form the section is there.  The buffer asked for is
+// a little longer than either form, so that a descriptor that was given the buffer's size instead says that there is none.
+constexpr int64_t kWideSpare = 16;
+
 void quantize_channel(const double* w, int64_t count, int w_bits, int32_t* out, float* scale) {
     const int qmax = kQmax(w_bits), qmin = kQmin(w_bits);
     double amax = 0.0;
@@ -114,7 +118,8 @@ extern "C" int64_t hq_weight_blob_bytes(int64_t N, int32_t RS, int64_t C, int32_
     const int64_t limb = hq::round_up(N, hq::kTileN) * RS * hq::round_up(Ck, hq::kTileK);
     const bool wide = limbs == 2 && hq::wide_section(w_bits, had_block, mode);
     return limb * (limbs + (wide || (limbs == 2 && hq::split_section(w_bits, had_block, mode)) ? 1 : 0)) +
-           (wide && hq::halved_layer(RS, C, had_block) ? hq::round_up(N, hq::kTileN) * (hq::kHalvedCols + 1) : 0);
+           (wide && hq::halved_layer(RS, C, had_block) ? hq::round_up(N, hq::kTileN) * (hq::kHalvedCols + 1) : 0) +
+           (wide ? hq::kWideSpare : 0);
 }
 
 extern "C" hq_status hq_weight_prepare(const float* w, int64_t N, int32_t RS, int64_t C, int32_t w_bits,

@@ -223,3 +223,15 @@ def test_split_section_holds_the_extreme_integers(hq, n, kind):
         v = B1.reshape(N, -1, 2, 1 << bit)
         B1 = np.stack([v[:, :, 0] + v[:, :, 1], v[:, :, 0] - v[:, :, 1]], axis=2).reshape(N, n)
     assert np.array_equal(B1, B)
+
+
+@pytest.mark.parametrize("n", [1024, 2048, 4096])
+@pytest.mark.parametrize("blocks,taps,N", [(1, 1, 130), (2, 1, 64), (1, 9, 8)])
+def test_the_size_of_a_buffer_never_says_that_a_section_is_there(hq, n, blocks, taps, N):
+    """Above 512 channels the one-limb section is known by desc->bytes alone: a descriptor that was given the size of the buffer
+    must not equal one of a blob with a section (its bytes, or halved with 128 further columns and a parity)."""
+    C, N_pad = n * blocks, (N + 127) // 128 * 128
+    rows = N_pad * taps * C
+    section = hq.hq_weight_blob_bytes(N, taps, C, 4, n, hq.HQ_W_FOLDED) - 2 * rows
+    halved = N_pad * (C + 129) if blocks == taps == 1 and n > 1024 else 0
+    assert section > max(rows, halved) and section % 16 == 0
