@@ -263,13 +263,15 @@ bool small_linear_takes(const void* x, hq_dtype xdt, int64_t M, int64_t K, int64
     if (ldx < K || ldx % 4 != 0 || reinterpret_cast<uintptr_t>(x) % (4 * elt) != 0 || !aligned16(w_dev)) return false;
     if (ldy < desc->N || ldy % 2 != 0 || reinterpret_cast<uintptr_t>(y) % 4 != 0) return false;
     if (double(K) * double(1 << (a_bits - 1)) * double(desc->max_abs_b > 0 ? desc->max_abs_b : 1) >= 2147483648.0) return false;
-    // a CTA reads its rows while others already write: the two kernels take an output or a workspace on top of the input, this one not
+    // a CTA reads its rows and the static scale while others already write: the two kernels take an output on top of either and a
+    // workspace on top of the input, this one not
     const auto apart = [](const void* a, int64_t an, const void* b, int64_t bn) {
         const uintptr_t i = reinterpret_cast<uintptr_t>(a), j = reinterpret_cast<uintptr_t>(b);
         return i + uintptr_t(an) <= j || j + uintptr_t(bn) <= i;
     };
-    const int64_t x_bytes = ((M - 1) * ldx + K) * elt;
-    if (!apart(x, x_bytes, y, ((M - 1) * ldy + desc->N) * 2) || !apart(x, x_bytes, workspace, ws_used)) return false;
+    const int64_t x_bytes = ((M - 1) * ldx + K) * elt, y_bytes = ((M - 1) * ldy + desc->N) * 2;
+    if (!apart(x, x_bytes, y, y_bytes) || !apart(x, x_bytes, workspace, ws_used)) return false;
+    if (mode == HQ_SCALE_STATIC && !apart(static_scale, sizeof(float), y, y_bytes)) return false;
     return ((M + kSmRows - 1) / kSmRows) * ((desc->N + kSmCols - 1) / kSmCols) <= int64_t(sm_count()) * small_resident(int(K), desc->limbs, desc->had_block);
 }
 

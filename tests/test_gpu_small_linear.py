@@ -68,3 +68,22 @@ def test_output_over_the_input():
         y = x.clone()
         hq.hq_qlinear(y, pw, None, 4, y, ws)
         assert torch.equal(y, want)
+
+
+@pytest.mark.gpu
+def test_output_over_the_static_scale():
+    """Likewise an output on top of the static scale, which the first of the two kernels has copied by then."""
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    M = K = N = 256
+    x = torch.randn((M, K), generator=torch.Generator(device="cuda").manual_seed(6), device="cuda").to(torch.bfloat16)
+    pw = hq.hq_weight_prepare(inputs.weights((N, K), seed=N), 4, 256, hq.WEIGHT_MODES["folded"], hq.HQ_CODES_INT8).to_device()
+    ws = torch.empty((hq.hq_workspace_size(M, K, hq.HQ_CODES_INT8),), dtype=torch.uint8, device="cuda")
+    want, y = (torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    hq.hq_qlinear(x, pw, None, 4, want, ws, static_scale=torch.tensor([0.3], device="cuda"))
+    for i in (0, M * N // 2 - 1):
+        inside = y.view(-1).view(torch.float32)[i: i + 1]
+        for _ in range(20):
+            inside.fill_(0.3)
+            hq.hq_qlinear(x, pw, None, 4, y, ws, static_scale=inside)
+            assert torch.equal(y, want)
