@@ -131,7 +131,8 @@ lib = _load()
 try:
     from . import _hqcall
 except ImportError as e:
-    raise ImportError("the extension module _hqcall is missing: build it with `python -m paper_2512_05746_b200.build`") from e
+    raise ImportError(f"the extension module _hqcall cannot be loaded ({e}): build it with this Python, `python -m "
+                      "paper_2512_05746_b200.build --force`") from e
 
 
 def status_string(status: int) -> str:

@@ -6,10 +6,12 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 _DIR = os.path.dirname(os.path.abspath(__file__))
 LIB = os.path.join(_DIR, "libhq.so")
-PYCALL = os.path.join(_DIR, "_hqcall.so")
+# named for the Python it is compiled against: another one does not find it, where it would load a plain ".so" and crash
+PYCALL = os.path.join(_DIR, "_hqcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 PYCALL_SOURCE = os.path.join(_DIR, "csrc", "hq_pycall.c")
 SOURCES = sorted(glob.glob(os.path.join(_DIR, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(_DIR, "csrc", "*.cuh"))) + [os.path.join(os.path.dirname(_DIR), "include", "hq.h")]
@@ -24,11 +26,13 @@ def stale() -> bool:
 
 def build_pycall() -> str:
     """The native marshalling of binding.py's frequent calls, an extension module of its own (the library links no Python)."""
-    import sysconfig
     tmp = PYCALL + f".tmp{os.getpid()}"
     subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-fvisibility=hidden", "-I" + sysconfig.get_paths()["include"],
                            "-o", tmp, PYCALL_SOURCE])
     os.replace(tmp, PYCALL)
+    plain = os.path.join(_DIR, "_hqcall.so")               # of an earlier build
+    if os.path.exists(plain):
+        os.remove(plain)
     return PYCALL
 
 

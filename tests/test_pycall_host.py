@@ -101,3 +101,16 @@ def test_what_was_refused_is_refused(taken):
     with pytest.raises(hq.HqError) as e:
         hq.hq_qlinear(x, pw, None, 4, y, ws, stream=Stream)
     assert e.value.status == 5
+
+
+def test_the_module_belongs_to_this_python_and_says_why_it_cannot_be_loaded():
+    import os
+    import subprocess
+    import sys
+    import sysconfig
+
+    from paper_2512_05746_b200 import binding, build
+    assert os.path.samefile(binding._hqcall.__file__, build.PYCALL) and build.PYCALL.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    r = subprocess.run([sys.executable, "-c", "import sys; sys.modules['paper_2512_05746_b200._hqcall'] = None\n"
+                        "import paper_2512_05746_b200.binding"], capture_output=True, text=True, cwd=os.path.dirname(os.path.dirname(build.LIB)))
+    assert r.returncode != 0 and "_hqcall cannot be loaded" in r.stderr and "halted" in r.stderr
