@@ -68,16 +68,22 @@ def ws_views(torch, ws, rows, cols):
     return ws[: rows * pitch].view(rows, pitch), ws[off: off + rows * 4].view(torch.float32)
 
 
-def limbs_run(hq, pw, a_bits, rows, ws, static=False, stride=1):
+def limbs_run(hq, pw, a_bits, rows, ws, static=False, stride=1, call=None):
     """Weight limbs a fused call of this layer runs on in this workspace: one where it takes the split fold (the query asks
-    for the room its codes need; 8-bit codes never fold, so theirs is codes and scales alone), else the descriptor's."""
+    for the room its codes need; 8-bit codes never fold, so theirs is codes and scales alone), else the descriptor's.  The query
+    never asks for blocks above 512: there `call` makes the layer's call, which writes split-fold codes behind the scales or not."""
     alone = hq.hq_layer_workspace_size(pw, 8, rows, static, stride)
+    if call is not None and pw.desc.had_block > 512 and pw.desc.limbs == 2:
+        row = ws[(alone + 255) // 256 * 256:][: pw.desc.C]
+        row.fill_(0x11)
+        call()
+        return 1 if bool((row != 0x11).any()) else 2
     need = hq.hq_layer_workspace_size(pw, a_bits, rows, static, stride)
     return 1 if alone < need <= ws.nbytes else pw.desc.limbs
 
 
 STEP_KERNEL_SOURCES = ("hq_common.cuh", "hq_cluster.cuh", "hq_fwht.cuh", "hq_quant.cu", "hq_gemm_kernel.cuh", "hq_gemm.cu",
-                       "hq_gemm_pair.cu", "hq_gemm_splitk.cu", "hq_api.cu",
+                       "hq_gemm_pair.cu", "hq_gemm_splitk.cu", "hq_small.cu", "hq_api.cu",
                        "hq_gemm_inst_i8_gemm.cu", "hq_gemm_inst_i8_conv.cu", "hq_gemm_inst_nibble_gemm.cu",
                        "hq_gemm_inst_nibble_conv.cu")
 
@@ -213,7 +219,8 @@ def build_layers(torch, hq, device, seed, cont=None, share=None, weight_mode=Non
         L["cont"] = cont
         L["ws"] = torch.empty((hq.hq_workspace_size(rows, cols, cont),), dtype=torch.uint8, device=device)
         # what the fused call issues: its weight limbs, and one byte per code where it reads the split-fold codes
-        L["limbs"] = limbs_run(hq, pw, A_BITS, rows, L["ws"], static=L["kind"] == "conv")
+        L["limbs"] = limbs_run(hq, pw, A_BITS, rows, L["ws"], static=L["kind"] == "conv",
+                               call=(lambda L=L: fused_layer(hq, L, None)) if L["kind"] == "linear" else None)
         L["split"] = L["limbs"] < pw.desc.limbs
         L["ops"] = 2.0 * L["M"] * L["N"] * L["K"] * L["limbs"]
         L["ops_1limb"] = 2.0 * L["M"] * L["N"] * L["K"]
