@@ -140,16 +140,22 @@ struct LayerCodes {
     // 8192 x 1152 -> 4608 57.9 / 44.2 us, 64 x 32 x 32 x 512 3x3 176 / 117 us, 2 x 16 x 16 x 768 3x3 13.1 / 11.8 us; where
     // no round of tiles is saved it only costs: 256 x 256 -> 256 6.1 / 6.8 us, 8 x 64 x 64 x 256 3x3 stride 2 16.5 / 17.6.
     // Blocks above 512, the same rule: 65536 x 4096 -> 4096 1657 / 1127 us (the second byte costs the transform 84 of its 341 us),
-    // 65536 x 4096 -> 1024 536 / 487, 32768 x 2048 -> 2048 195 / 161, 65536 x 1024 -> 1024 125 / 113, 32768 x 2048 -> 512 with two
-    // codes per byte 113 / 111; not taken: the same with one code per byte, 101 / 104 (halved weights; where they fit a byte the product
-    // gains 13.6 us and the transform, whose threads hold 64 values, loses 14.8: 4.6 TB/s).
+    // 65536 x 4096 -> 1024 536 / 487, 32768 x 2048 -> 2048 195 / 161, 65536 x 1024 -> 1024 125 / 113.  The transform's threads hold 64
+    // values, and the second byte travels at about 4.6 TB/s; at 4096 with one code per byte, where both bytes change lanes before
+    // they are stored, at 3.4.  With one code per byte, taken: 65536 x 2048 -> 512 187.6 / 185 (bf16 input 172 / 166), 32768 x 1024 ->
+    // 1024 70.0 / 66.5, 32768 x 2048 -> 768 114.6 / 109; not taken: 32768 x 2048 -> 512 95.5 / 99.0, 32768 x 1024 -> 512 50.8 / 57.8,
+    // 16384 x 4096 -> 512 103.5 / 108.5, 32768 x 4096 -> 512 194 / 204.5.  At 28 shapes of 4096 to 65536 rows and 256 to 2048 channels, both
+    // containers and input types, what it takes is within 3 % of the faster form.
     static bool split_pays(const hq_weight_desc* desc, int64_t rows, int64_t cols, int64_t out_rows, int more_kb) {
         const int num_kb = int(desc->RS * desc->C_pad / 128), tile_rows = out_rows < 128 ? int(out_rows > 0 ? out_rows : 1) : 128;
-        // with two codes per byte the two-limb product unpacks them on one SM a tile (32768 x 2048 -> 512 52 us against 45)
+        // with two codes per byte the two-limb product unpacks them on one SM a tile (32768 x 2048 -> 512 52 us against 45): the whole
+        // layer taken at 32768 x 1024 -> 512 53.6 / 50.0, 32768 x 2048 -> 512 96.0 / 91.3, 32768 x 4096 -> 512 199.4 / 197.4, 16384 x
+        // 4096 -> 512 105.4 / 102.1; not taken at 65536 x 1024 -> 256 76.0 / 82.4, 65536 x 4096 -> 384 354 / 372
         const bool unpacks = desc->container == HQ_CODES_NIBBLE && desc->had_block > 512;
         const double two = plan_product(2, out_rows, tile_rows, desc->N_pad, num_kb).us * (unpacks ? 1.15 : 1.0);
         const double one = plan_product(1, out_rows, tile_rows, desc->N_pad, num_kb + more_kb).us;
-        return two - one > 0.7 + double(rows) * double(cols) / (desc->had_block > 512 ? 4.6e6 : 5.2e6);
+        const bool lanes = desc->had_block == 4096 && !unpacks;              // staged_stores in hq_quant.cu
+        return two - one > 0.7 + double(rows) * double(cols) / (desc->had_block <= 512 ? 5.2e6 : lanes ? 3.4e6 : 4.6e6);
     }
     const void* a() const { return z.written ? z.z : codes; }
     int64_t lda() const { return z.written ? z.ld : ld; }

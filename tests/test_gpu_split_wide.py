@@ -152,3 +152,26 @@ def test_linear_on_wide_split_weights_is_the_linear_on_two_limbs(M, n, N, a_bits
     yf = torch.zeros((M, N), dtype=torch.float32, device="cuda")
     hq.hq_qlinear(x, pw, b, a_bits, yf, ws2[:full], static_scale=ss, dev_status=status)
     assert torch.equal(yf.to(torch.bfloat16), y1)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,n,N,container,taken", [
+    (16384, 4096, 512, 1, False),       # two limbs / one: 103.5 / 108.5 us
+    (32768, 4096, 512, 1, False),       # 194 / 204.5
+    (16384, 4096, 1024, 1, True),
+    (16384, 4096, 512, 0, True),        # 105.4 / 102.1
+    (32768, 2048, 512, 1, False),       # 95.5 / 99.0
+    (32768, 2048, 768, 1, True),        # 114.6 / 109
+])
+def test_one_limb_only_where_it_is_the_faster(M, n, N, container, taken):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    pw = hq.hq_weight_prepare(layer_weights(N, n, "gaussian"), 4, n, hq.HQ_W_FOLDED, container)
+    assert section(pw) is not None
+    pw = pw.to_device()
+    x = torch.randn((M, n), generator=torch.Generator(device="cuda").manual_seed(n), device="cuda").to(torch.bfloat16)
+    ws = torch.full((hq.hq_workspace_size(M, n, container),), 0x11, dtype=torch.uint8, device="cuda")
+    y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    hq.hq_qlinear(x, pw, None, 4, y, ws)
+    behind = ws[(_codes_bytes(M, n, container) + 255) // 256 * 256:]
+    assert bool((behind[:n] != 0x11).any()) == taken
