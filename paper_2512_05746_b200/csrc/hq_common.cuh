@@ -63,7 +63,9 @@ cudaError_t launch_dependent(void (*kern)(Params...), dim3 grid, unsigned thread
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = dependent ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();    // reported here: not again by the next call's look at the last error
+    return e;
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

@@ -219,3 +219,17 @@ def test_quant_of_a_concatenation_refuses_a_block_across_the_seam(env):
     scales = torch.zeros((32,), dtype=torch.float32, device="cuda")
     with pytest.raises(hq.HqError):
         hq.hq_hadamard_quant(ta, 256, 4, codes, hq.HQ_CODES_NIBBLE, scales=scales, x2=tb)     # 128 is not a multiple of 256
+
+
+@pytest.mark.gpu
+def test_a_launch_that_fails_fails_one_call():
+    """Rows beyond any grid are refused by the launch; the call after it has nothing to do with that."""
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    x, y = torch.ones((8, 32), device="cuda"), torch.ones(64, dtype=torch.bfloat16, device="cuda")
+    codes, s = torch.zeros((8, 32), dtype=torch.uint8, device="cuda"), torch.zeros(8, device="cuda")
+    rows = 1 << 39                                  # 2^32 CTAs of 128 rows: none by the launch's 32 bits
+    assert hq.lib.hq_hadamard_quant(x.data_ptr(), 0, rows, 32, 32, 32, 4, 0, None, codes.data_ptr(), 1, 32, s.data_ptr(), None) == 7
+    hq.hq_add(y, y, y)
+    torch.cuda.synchronize()
+    assert bool((y == 2).all()) and not bool(codes.any())
