@@ -178,11 +178,11 @@ def test_fused_layers_refuse_null_weights_before_a_launch(hq, had_block):
     (4096, 1152, 128, "folded", 4, 1, 4, False, 1, 1, True),        # 4.5 MiB of codes, runs on one limb
     (4096, 1152, 128, "folded", 4, 0, 3, True, 1, 1, True),         # two codes per byte
     (65536, 1152, 128, "folded", 4, 1, 8, False, 1, 1, False),      # 8-bit codes need two limbs
-    (65536, 1024, 1024, "folded", 4, 1, 4, False, 1, 1, False),     # so do blocks above 512
+    (65536, 1024, 1024, "folded", 4, 1, 4, False, 1, 1, False),     # one limb where it is given the room: the query does not ask above 512
     (65536, 1152, 128, "double", 4, 1, 4, False, 1, 1, False),      # one limb anyhow
     (256, 256, 256, "folded", 4, 1, 4, False, 1, 1, False),         # nothing to gain
     (15 * 32 * 32, 512, 256, "folded", 4, 1, 4, True, 1, 9, True),  # 7.6 MiB
-    (64 * 32 * 32, 512, 256, "folded", 4, 1, 4, False, 1, 9, False),    # one scale per pixel under a 3x3 window
+    (64 * 32 * 32, 512, 256, "folded", 4, 1, 4, False, 1, 9, False),    # likewise one scale per pixel under a 3x3 window
 ])
 def test_layer_workspace_asks_for_what_the_layer_uses(hq, rows, cols, n, mode, w_bits, container, a_bits, static, stride, taps, room):
     N = {1152: 4608, 256: 256}.get(cols, 1024)
