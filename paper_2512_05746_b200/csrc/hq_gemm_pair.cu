@@ -149,7 +149,7 @@ __device__ __forceinline__ bool wait_pair(uint64_t* bar, uint32_t parity, PairCt
 // loads them once per column tile).  Every lane needs all of them, so from shared memory they arrive as broadcast reads,
 // 128 wavefronts per warp and tile, 1024 per tile on the data pipe that also feeds the tensor core its operands (1024 per
 // tile) and takes the staging stores and the bulk stores' reads (520): together more than the 2144 cycles of a tile's MMAs.
-// NBUF: the warp's staging buffers (two used in turn, or one).
+// NBUF: the warp's staging buffers (two used in turn, or one); `tile` counts the tiles that the warp has finished.
 // BN: operand-B rows (accumulator columns) of the tile.
 // HALVED (halved weights, hq_fwht.cuh): the integer is twice the accumulator plus the column's bit in `odd` (the column parities
 // of the warp, 32 to a word, zero for a row of parity 0).
@@ -158,13 +158,14 @@ __device__ __forceinline__ bool wait_pair(uint64_t* bar, uint32_t parity, PairCt
 template <int LIMBS, int PREG = 0, int NBUF = 2, int BN = kBN, bool HALVED = false, bool RES = false>
 __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg, int lane, const float* prm_sw,
                                               const float* prm_b, float sa_eff, const CUtensorMap* tmY, int col0, int row0,
-                                              uint32_t tempty_leader, const float (&rsw)[PREG > 0 ? PREG * 16 : 1] = {0.f},
+                                              uint32_t tempty_leader, int tile, const float (&rsw)[PREG > 0 ? PREG * 16 : 1] = {0.f},
                                               const float (&rb)[PREG > 0 ? PREG * 16 : 1] = {0.f},
                                               const uint32_t (&odd)[HALVED ? BN / 64 : 1] = {0u},
                                               const __nv_bfloat16* res = nullptr, int ncols = 0) {
     static_assert(!HALVED || LIMBS == 1, "halved weights are one limb");
     static_assert(LIMBS == 1 || BN == kBN, "narrower tiles exist with one limb");
     constexpr int NSTEPS = LIMBS == 2 ? kBN / 2 / 2 / 16 : BN / 2 / 16;
+    constexpr bool ODD_STORES = (NSTEPS / 2) % 2 != 0;
     const uint32_t wsw = (lane >> 1) & 3;
     uint32_t hi[16], lo[16];
     tmem_ld_32x16(t_row, hi);
@@ -203,8 +204,9 @@ __device__ __forceinline__ void epilogue_pair(uint32_t t_row, unsigned char* stg
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(tempty_leader);
         }
-        // two staging buffers, used in turn: the copy engine must be done reading the one written two stores ago
-        unsigned char* buf = NBUF == 2 ? stg + ((st >> 1) & 1) * kStagingBytes : stg;
+        // two staging buffers, used in turn, from tile to tile too (an odd number of stores leaves the turn with the other one): the
+        // copy engine must be done reading the one written two stores ago
+        unsigned char* buf = NBUF == 2 ? stg + (((st >> 1) + (ODD_STORES ? tile : 0)) & 1) * kStagingBytes : stg;
         unsigned char* wr = buf + lane * 64;
         if ((st & 1) == 0) {
             if (lane == 0) { if (NBUF == 2) bulk_wait_read_1(); else bulk_wait_read_all(); }
@@ -484,7 +486,7 @@ qgemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             const float sa_eff = p.alpha * sa;
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
             const uint32_t t_fast = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as * kBN + wc0);
-            epilogue_pair<LIMBS, PREG>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as], rsw, rb);
+            epilogue_pair<LIMBS, PREG>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as], i, rsw, rb);
         }
         if (lane == 0) bulk_wait_read_all();           // shared memory must outlive the copy engine's reads
     }
@@ -712,11 +714,11 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
             const uint32_t t_fast = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as * kBN + wc0);
             if (!HALVED && p.res != nullptr)
-                epilogue_pair<LIMBS, 0, NBUF, BN, HALVED, true>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as],
+                epilogue_pair<LIMBS, 0, NBUF, BN, HALVED, true>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as], i,
                                                                 {0.f}, {0.f}, odd,
                                                                 my_row < p.M ? p.res + my_row * p.ldr + col_base + wc0 : nullptr, p.N - col_base - wc0);
             else
-                epilogue_pair<LIMBS, 0, NBUF, BN, HALVED>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as],
+                epilogue_pair<LIMBS, 0, NBUF, BN, HALVED>(t_fast, stg, lane, prm_sw, prm_b, sa_eff, &tmY, col_base + wc0, row0, tempty_leader[as], i,
                                                           {0.f}, {0.f}, odd);
         }
         if (lane == 0) bulk_wait_read_all();           // shared memory must outlive the copy engine's reads

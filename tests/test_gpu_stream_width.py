@@ -37,3 +37,26 @@ def test_convolution_on_narrow_tiles(Nb, H, C, Cout):
     sa, b = torch.rand((1,), generator=gen, device="cuda") + 0.5, torch.from_numpy(inputs.bias(Cout, seed=1)).cuda()
     both(torch, hq, lambda y, st: hq.hq_qconv2d(q, hq.HQ_CODES_INT8, 8, Nb, H, H, C, pw, 3, 3, 1, 1, scale_a=sa, bias=b, y=y,
                                                 dev_status=st), (Nb, H, H, Cout))
+
+
+@pytest.mark.parametrize("M,K,N", [(16001, 640, 1288), (32768, 640, 960), (9000, 1152, 3456)])
+def test_narrow_tiles_one_after_the_other_keep_their_staging_apart(M, K, N):
+    # three stores a tile and two staging buffers: the turn passes from tile to tile, and every pass gives the same bytes
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    pw = hq.hq_weight_prepare(inputs.weights((N, K), seed=N), 8, 128, hq.HQ_W_DOUBLE, hq.HQ_CODES_INT8).to_device()
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    q = torch.randint(-128, 128, (M, K), generator=gen, device="cuda", dtype=torch.int8).view(torch.uint8)
+    sa = torch.rand((M,), generator=gen, device="cuda") + 0.5
+    status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+    ys = [torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(13)]
+    hq.hq_set_pair_gemm(0)
+    try:
+        hq.hq_qgemm(q, hq.HQ_CODES_INT8, 8, K, pw, scale_a=sa, y=ys[0], dev_status=status)
+    finally:
+        hq.hq_set_pair_gemm(2)
+    for y in ys[1:]:
+        hq.hq_qgemm(q, hq.HQ_CODES_INT8, 8, K, pw, scale_a=sa, y=y, dev_status=status)
+    assert int(status) == 0
+    for y in ys[1:]:
+        assert torch.equal(y, ys[0])
