@@ -19,6 +19,15 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { f32x2 r; asm("sub.rn.f
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 
+// Two pairs to 16 bytes of shared memory, as four 32-bit operands: stored as a vector of two 64-bit values, every value was moved to
+// another register first (0.8 instructions per value; 32768 x 2048 bf16, two codes per byte, 43.3 -> 41.2 us).
+__device__ __forceinline__ void st_shared_pairs(ulonglong2* to, f32x2 a, f32x2 b) {
+    float x0, x1, x2, x3;
+    upk2(a, x0, x1);
+    upk2(b, x2, x3);
+    *reinterpret_cast<float4*>(to) = make_float4(x0, x1, x2, x3);
+}
+
 // The largest of three values in one instruction.
 __device__ __forceinline__ float max3(float a, float b, float c) { float r; asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c)); return r; }
 
@@ -37,6 +46,18 @@ __device__ __forceinline__ void butterflies_pairs(f32x2 (&v)[P]) {
         }
     }
 }
+// Sums with one operand in bf16 (converted exactly by the adder itself, at the rate of a plain addition): the low or the high half
+// of a word.  A conversion by a shift or a mask takes a slot of the pipe that the packing needs, at half the rate.
+__device__ __forceinline__ float add_bf16_lo(uint32_t w, float c) { float r; asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; add.rn.f32.bf16 %0, l, %2;}" : "=f"(r) : "r"(w), "f"(c)); return r; }
+__device__ __forceinline__ float add_bf16_hi(uint32_t w, float c) { float r; asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; add.rn.f32.bf16 %0, h, %2;}" : "=f"(r) : "r"(w), "f"(c)); return r; }
+__device__ __forceinline__ float sub_bf16_lo(uint32_t w, float c) { float r; asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; sub.rn.f32.bf16 %0, l, %2;}" : "=f"(r) : "r"(w), "f"(c)); return r; }
+__device__ __forceinline__ float sub_bf16_hi(uint32_t w, float c) { float r; asm("{.reg .b16 l, h; mov.b32 {l, h}, %1; sub.rn.f32.bf16 %0, h, %2;}" : "=f"(r) : "r"(w), "f"(c)); return r; }
+// The stage between two neighbouring bf16 values.
+__device__ __forceinline__ f32x2 butterfly_bf16(uint32_t w) {
+    const float b = __uint_as_float(w & 0xFFFF0000u);
+    return pk2(add_bf16_lo(w, b), sub_bf16_lo(w, b));
+}
+
 // The stage between the two values of each pair.
 template <int P>
 __device__ __forceinline__ void butterfly_within_pairs(f32x2 (&v)[P]) {
@@ -51,31 +72,46 @@ __device__ __forceinline__ void butterfly_within_pairs(f32x2 (&v)[P]) {
 __host__ __device__ constexpr int ilog2_c(int v) { return v <= 1 ? 0 : 1 + ilog2_c(v >> 1); }
 
 // Rounds E values held as pairs (ties to even, optional clamp) and packs them in register order into words: 8
-// four-bit codes or 4 bytes per word.  Adding kMagic + bias leaves code + bias in the low mantissa bits.  The second
-// value of every pair is rounded F times larger (F = 256 for bytes, 16 for four-bit codes): scaling the multiplier and
+// four-bit codes or 4 bytes per word.  Adding kMagic + bias leaves code + bias in the low mantissa bits.  One of two
+// values is rounded F times larger (F = 256 for bytes, 16 for four-bit codes): scaling the multiplier and
 // the magic number by a power of two scales the sum exactly, so the code is the same, and it lands F units up.  Taking
-// the scaled magic number off again (exact) and adding the first value (exact: the sum stays below 2^22 units) leaves
+// the scaled magic number off again (exact) and adding the other value (exact: the sum stays below 2^22 units) leaves
 // both biased codes side by side in the low bits of one float, on the floating-point pipe; byte permutes then gather
-// the fields of a word, and one XOR turns the biased fields into two's complement.
+// the fields of a word, and one XOR turns the biased fields into two's complement.  Bytes: the two values come from
+// neighbouring pairs, so that the additions are two-wide as well.
 template <int E, bool INT8_OUT, bool CLAMP>
 __device__ __forceinline__ void round_pack(const f32x2 (&v)[E / 2], float inv, int bits, uint32_t (&out)[INT8_OUT ? E / 4 : E / 8]) {
     constexpr float F = INT8_OUT ? 256.0f : 16.0f;
     const float bias = INT8_OUT ? 128.0f : 8.0f;
     const float mb = kMagic + bias;
     const float lo = mb + float(-(1 << (bits - 1))), hi = mb + float((1 << (bits - 1)) - 1);
-    const f32x2 inv2 = pk2(inv, F * inv), mb2 = pk2(mb, F * mb);
-    uint32_t u[E / 2];                                 // per pair: kMagicBits + (c0 + bias) + F (c1 + bias)
-#pragma unroll
-    for (int e = 0; e < E / 2; ++e) {
-        float f0, f1;
-        upk2(fma2(v[e], inv2, mb2), f0, f1);
-        if (CLAMP) { f0 = fminf(fmaxf(f0, lo), hi); f1 = fminf(fmaxf(f1, F * lo), F * hi); }
-        u[e] = __float_as_uint(f0 + (f1 - F * kMagic));
-    }
     if (INT8_OUT) {
+        const f32x2 inv0 = pk2(inv, inv), inv1 = pk2(F * inv, F * inv), mb0 = pk2(mb, mb), mb1 = pk2(F * mb, F * mb);
+        const f32x2 off = pk2(-F * kMagic, -F * kMagic);
 #pragma unroll
-        for (int w = 0; w < E / 4; ++w) out[w] = __byte_perm(u[2 * w], u[2 * w + 1], 0x5410) ^ 0x80808080u;
+        for (int w = 0; w < E / 4; ++w) {
+            f32x2 a = fma2(v[2 * w], inv0, mb0), b = fma2(v[2 * w + 1], inv1, mb1);
+            if (CLAMP) {
+                float a0, a1, b0, b1;
+                upk2(a, a0, a1);
+                upk2(b, b0, b1);
+                a = pk2(fminf(fmaxf(a0, lo), hi), fminf(fmaxf(a1, lo), hi));
+                b = pk2(fminf(fmaxf(b0, F * lo), F * hi), fminf(fmaxf(b1, F * lo), F * hi));
+            }
+            float u0, u1;                              // kMagicBits + (c0 + bias) + F (c2 + bias), and c1, c3
+            upk2(add2(a, add2(b, off)), u0, u1);
+            out[w] = __byte_perm(__float_as_uint(u0), __float_as_uint(u1), 0x5140) ^ 0x80808080u;
+        }
     } else {
+        const f32x2 inv2 = pk2(inv, F * inv), mb2 = pk2(mb, F * mb);
+        uint32_t u[E / 2];                             // per pair: kMagicBits + (c0 + bias) + F (c1 + bias)
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) {
+            float f0, f1;
+            upk2(fma2(v[e], inv2, mb2), f0, f1);
+            if (CLAMP) { f0 = fminf(fmaxf(f0, lo), hi); f1 = fminf(fmaxf(f1, F * lo), F * hi); }
+            u[e] = __float_as_uint(f0 + (f1 - F * kMagic));
+        }
 #pragma unroll
         for (int w = 0; w < E / 8; ++w)
             out[w] = __byte_perm(__byte_perm(u[4 * w], u[4 * w + 1], 0x0040), __byte_perm(u[4 * w + 2], u[4 * w + 3], 0x0040),
@@ -105,19 +141,26 @@ struct FwhtShape {
 // values make one trip through the block's exchange buffer `grp` (float4 slot f at f + f / J, conflict-free both ways),
 // and phase B covers the remaining bits in registers (KLOG = 12: one lane exchange more).  On exit thread u holds the E
 // contiguous channels E u .. (or, PAIR, the channel pairs {4 j, 4 j + 1} + 2 (u & 1) of a 2E-channel group).
+// (PAIR: the odd thread of a group holds its rows with the upper and the lower half of the pair-index range exchanged, so that
+// pack_codes finds what a thread keeps and what it hands over in the same registers of both.)
 // CTA_SYNC: the block's threads span more than one warp (or the caller needs a CTA-wide barrier here anyway).
-template <int KLOG, int E, bool CTA_SYNC>
+// FIRST_DONE: the stage of index bit 0 has been taken as the values were read.  PAIR_STORE: without st_shared_pairs.
+template <int KLOG, int E, bool CTA_SYNC, bool FIRST_DONE = false, bool PAIR_STORE = false>
 __device__ __forceinline__ void fwht_stages(f32x2 (&v)[E / 2], float4* grp, int tb) {
     using Sh = FwhtShape<KLOG, E>;
     constexpr int P = Sh::P, TB = Sh::TB, J = Sh::J, S = Sh::S, R = Sh::R;
-    butterfly_within_pairs<P>(v);                      // index bit 0
+    if (!FIRST_DONE) butterfly_within_pairs<P>(v);     // index bit 0
     butterflies_pairs<P, 1, P / 2>(v);                 // index bit 1 and the top LE-2 bits
     {
         // slot f = tb + TB i sits at f + f / J; with TB and J dividing one another that is a per-thread base plus a
         // compile-time offset
         ulonglong2* wr = reinterpret_cast<ulonglong2*>(grp + tb + (tb >> S));
 #pragma unroll
-        for (int i = 0; i < E / 4; ++i) wr[TB * i + ((TB * i) >> S)] = make_ulonglong2(v[2 * i], v[2 * i + 1]);
+        for (int i = 0; i < E / 4; ++i) {
+            ulonglong2* to = wr + TB * i + ((TB * i) >> S);
+            if (PAIR_STORE) *to = make_ulonglong2(v[2 * i], v[2 * i + 1]);
+            else st_shared_pairs(to, v[2 * i], v[2 * i + 1]);
+        }
     }
     if (CTA_SYNC) __syncthreads(); else __syncwarp();
     if (!Sh::PAIR) {
@@ -130,9 +173,21 @@ __device__ __forceinline__ void fwht_stages(f32x2 (&v)[E / 2], float4* grp, int 
         butterflies_pairs<P, 2, (2 << R) / 2>(v);      // index bits 2 .. R+1 are pair-index bits 1 .. R
     } else {
         const f32x2* rd = reinterpret_cast<const f32x2*>(grp + (J + 1) * (tb >> 1)) + (tb & 1);
+        const f32x2* rd_lo = rd + (tb & 1) * P;
+        const f32x2* rd_hi = rd - (tb & 1) * P;
 #pragma unroll
-        for (int j = 0; j < P; ++j) v[j] = rd[2 * j];
-        butterflies_pairs<P, 1, P / 2>(v);             // index bits 2 .. LE are pair-index bits 0 .. LE-2
+        for (int j = 0; j < P; ++j) v[j] = (j < P / 2 ? rd_lo : rd_hi)[2 * j];
+        butterflies_pairs<P, 1, P / 4>(v);             // index bits 2 .. LE are pair-index bits 0 .. LE-2
+        {                                              // the last of them, whose operands the odd thread holds exchanged
+            const float sg = (tb & 1) ? -1.0f : 1.0f;
+            const f32x2 sg2 = pk2(sg, sg), msg2 = pk2(-sg, -sg);
+#pragma unroll
+            for (int i = 0; i < P / 2; ++i) {
+                const f32x2 a = v[i], b = v[i + P / 2];
+                v[i] = fma2(sg2, a, b);
+                v[i + P / 2] = fma2(msg2, b, a);
+            }
+        }
         if (Sh::SHUF) {                                // index bit LE+1 lives in lane bit 1
             const float sgn = (tb & 2) ? -1.0f : 1.0f;
             const f32x2 sgn2 = pk2(sgn, sgn);
@@ -148,7 +203,8 @@ __device__ __forceinline__ void fwht_stages(f32x2 (&v)[E / 2], float4* grp, int 
 // Rounds and packs the E values a thread holds after fwht_stages into words of codes for the E contiguous channels
 // E tb .. of the block (8 four-bit codes or 4 bytes per word).  In the PAIR layout the two threads of a group first
 // exchange halves: w holds the codes of channel pairs {4j, 4j+1} (+2 for the odd thread); the even thread emits the first
-// half of the group's bytes, the odd thread the second half, interleaved at pair granularity (1 byte or 2 bytes).
+// half of the group's bytes, the odd thread the second half (the first half of its registers), interleaved at pair granularity
+// (1 byte or 2 bytes).
 template <int KLOG, int E, bool INT8_OUT, bool CLAMP>
 __device__ __forceinline__ void pack_codes(const f32x2 (&v)[E / 2], float inv, int bits, int tb,
                                            uint32_t (&w)[INT8_OUT ? E / 4 : E / 8]) {
@@ -156,16 +212,14 @@ __device__ __forceinline__ void pack_codes(const f32x2 (&v)[E / 2], float inv, i
     round_pack<E, INT8_OUT, CLAMP>(v, inv, bits, w);
     if (FwhtShape<KLOG, E>::PAIR) {
         constexpr int H = NW / 2;
-        const bool odd = tb & 1;
+        // first and second word of two: bytes (or nibbles) of the even and the odd thread in turn
+        const uint32_t first = INT8_OUT ? 0x5410 : 0x5140, second = INT8_OUT ? 0x7632 : 0x7362, swap = (tb & 1) ? 0x4444 : 0;
         uint32_t o[NW];
 #pragma unroll
         for (int i = 0; i < H; ++i) {
-            const uint32_t send = odd ? w[i] : w[i + H];
-            const uint32_t keep = odd ? w[i + H] : w[i];
-            const uint32_t recv = __shfl_xor_sync(0xffffffffu, send, 1);
-            const uint32_t ev = odd ? recv : keep, od = odd ? keep : recv;
-            o[2 * i + 0] = __byte_perm(ev, od, INT8_OUT ? 0x5410 : 0x5140);
-            o[2 * i + 1] = __byte_perm(ev, od, INT8_OUT ? 0x7632 : 0x7362);
+            const uint32_t recv = __shfl_xor_sync(0xffffffffu, w[i + H], 1);
+            o[2 * i + 0] = __byte_perm(w[i], recv, first ^ swap);
+            o[2 * i + 1] = __byte_perm(w[i], recv, second ^ swap);
         }
 #pragma unroll
         for (int i = 0; i < NW; ++i) w[i] = o[i];

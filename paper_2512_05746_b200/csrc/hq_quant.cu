@@ -13,6 +13,12 @@
 //                       followed by the integer factor q * H_raw.
 //   gn_stats_kernel     per-(sample, group) mean and 1/sqrt(var + eps) for the GroupNorm prologue, in one launch.
 // The butterflies run unnormalised (H_raw); 2^(-k/2) is folded into the scale (Eq. 7).
+// What bounds the rows of two-byte input: the two half-rate pipes together (two-wide additions 2 cycles a warp instruction, logic, permutes
+// and conversions 2 cycles on the other; neither above 60 %) at the 20 to 32 warps that the registers allow.  So instructions count: 15.0
+// per element at 2048 channels, 12.2 now (first stage on bf16 operands, two-wide packing, no selects or moves around the exchange, no
+// integer division): 65536 x 2048 bf16 92 -> 85 us, 131072 x 512 45.7 -> 42.5, GroupNorm + SiLU 262144 x 256 98 -> 93, LayerNorm 8192 x
+// 1152 18.7 -> 16.7.  A CTA that takes several sets of rows and requests the next ones early (cp.async) was 2-10 % slower on most shapes:
+// the loads are not what is waited for.
 #include <type_traits>
 
 #include "hq_common.cuh"
@@ -32,8 +38,10 @@ struct QuantParams {
     int m;               // Hadamard blocks per row
     int rows_per_cta;
     int threads_per_row;
+    uint32_t row_magic;  // ceil(2^20 / threads_per_row): a thread's row in its CTA without a division (at most 320 threads)
     int bits;
     float norm;          // 2^(-k/2) (1 for the identity)
+    float norm_q;        // norm / qmax
     const float* static_scale;
     uint8_t* codes;
     int64_t ld_codes;
@@ -164,11 +172,12 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     unsigned int* rowmax = reinterpret_cast<unsigned int*>(smem_raw + size_t(blockDim.x / TB) * GS * 16);
 
     const int tid = threadIdx.x;
-    const int row_in_cta = tid / p.threads_per_row;
+    const int row_in_cta = int((uint32_t(tid) * p.row_magic) >> 20);
     const int tr = tid - row_in_cta * p.threads_per_row;
     const int blk = tr / TB;
     const int tb = tr & (TB - 1);
     const bool shared_max = (p.m > 1) || (TB > 32);
+    const bool cta_wide = TB > 32 || (!STATIC && shared_max);      // barriers of the CTA; else a warp's blocks are its own
 
     if (!STATIC && tid < p.rows_per_cta) rowmax[tid] = 0u;
 
@@ -241,7 +250,14 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
     }
 
     f32x2 v[P];
-    {
+    // bf16: the first stage, or LayerNorm's sums, take the values as they came (add_bf16_lo)
+    constexpr bool BF16 = sizeof(InT) == 2, FIRST_DONE = BF16 && PRO == 0;
+    if constexpr (BF16 && (PRO == 0 || LN)) {
+        if (PRO == 0) {
+#pragma unroll
+            for (int i = 0; i < E / 4; ++i) { v[2 * i] = butterfly_bf16(cur[i].x); v[2 * i + 1] = butterfly_bf16(cur[i].y); }
+        }
+    } else {
 #pragma unroll
         for (int i = 0; i < E / 4; ++i) {
             float4 f;
@@ -279,16 +295,35 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
             for (int i = 0; i < parts; ++i) sum += buf[row_in_cta * parts + i];
             return sum;
         };
-        f32x2 acc = v[0];
-#pragma unroll
-        for (int i = 1; i < P; ++i) acc = add2(acc, v[i]);
         float lo, hi;
-        upk2(acc, lo, hi);
+        if constexpr (BF16) {
+            lo = __uint_as_float(cur[0].x << 16);
+            hi = __uint_as_float(cur[0].x & 0xFFFF0000u);
+#pragma unroll
+            for (int i = 1; i < P; ++i) {
+                const uint32_t w = (i & 1) ? cur[i / 2].y : cur[i / 2].x;
+                lo = add_bf16_lo(w, lo);
+                hi = add_bf16_hi(w, hi);
+            }
+        } else {
+            f32x2 acc = v[0];
+#pragma unroll
+            for (int i = 1; i < P; ++i) acc = add2(acc, v[i]);
+            upk2(acc, lo, hi);
+        }
         const float mean = row_sum(lo + hi, ln_part) / float(p.cols);
         const f32x2 mean2 = pk2(mean, mean);
-        acc = pk2(0.f, 0.f);
+        f32x2 acc = pk2(0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < P; ++i) { v[i] = sub2(v[i], mean2); acc = fma2(v[i], v[i], acc); }
+        for (int i = 0; i < P; ++i) {
+            if constexpr (BF16) {
+                const uint32_t w = (i & 1) ? cur[i / 2].y : cur[i / 2].x;
+                v[i] = pk2(sub_bf16_lo(w, mean), sub_bf16_hi(w, mean));
+            } else {
+                v[i] = sub2(v[i], mean2);
+            }
+            acc = fma2(v[i], v[i], acc);
+        }
         upk2(acc, lo, hi);
         if (LN_TABLE) cp_async_wait_all();             // this thread's pieces of the table; the barrier covers the others'
         const float rstd = rsqrtf(row_sum(lo + hi, ln_part + blockDim.x) / float(p.cols) + p.ln_eps);
@@ -313,8 +348,10 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
         }
     }
     float4* grp = xch + (tid / TB) * GS;
-    if (TB > 32 || shared_max) fwht_stages<KLOG, E, true>(v, grp, tb);
-    else fwht_stages<KLOG, E, false>(v, grp, tb);
+    // fp32 rows of narrow blocks are at the memory's rate either way: 262144 x 256 51.9 us so, 53.5 with st_shared_pairs
+    constexpr bool PAIR_STORE = !BF16 && KLOG <= 8;
+    if (cta_wide) fwht_stages<KLOG, E, true, FIRST_DONE, PAIR_STORE>(v, grp, tb);
+    else fwht_stages<KLOG, E, false, FIRST_DONE, PAIR_STORE>(v, grp, tb);
 
     float inv, scale;
     if (!STATIC) {
@@ -335,7 +372,7 @@ __global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast
         }
         const float qmaxf = float((1 << (p.bits - 1)) - 1);
         if (amax > 0.f) {
-            scale = amax * (p.norm / qmaxf);
+            scale = amax * p.norm_q;
             inv = qmaxf / amax;
             if (!(scale > 0.f)) { scale = 1.0f; inv = p.norm; }   // scale underflowed: same rule as an all-zero row
         } else {
@@ -1015,6 +1052,7 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
     p.m = int(cols / n);
     p.bits = bits;
     p.norm = float(exp2(-0.5 * double(klog)));
+    p.norm_q = p.norm / float((1 << (bits - 1)) - 1);
     p.static_scale = mode == HQ_SCALE_STATIC ? static_scale : nullptr;
     p.codes = static_cast<uint8_t*>(codes);
     p.ld_codes = ld_codes;
@@ -1045,6 +1083,7 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         const int base = rpc;
         while ((rpc + base) * tr <= 128) rpc += base;
         p.threads_per_row = tr;
+        p.row_magic = uint32_t(((1 << 20) + tr - 1) / tr);
         p.rows_per_cta = rpc;
         const int threads = rpc * tr;
         if (gn != nullptr) {
