@@ -905,8 +905,14 @@ bool pair_stream_stages(PairStreamParams& p, size_t& smem, int kps) {
 
 // Whether the streamed pair kernel covers a plain GEMM / a convolution planned by the one-CTA path (`g`: that plan).
 bool pair_stream_covers_gemm(hq_container cont, const hq_weight_desc* desc, int64_t M, const void* y, hq_dtype ydt, int64_t ldy,
-                             const int32_t* acc_out, bool combine_fast) {
-    return cont == HQ_CODES_INT8 && desc->RS == 1 && desc->C_pad > int64_t(kResidentKb) * kBK && y != nullptr &&
+                             const int32_t* acc_out, bool combine_fast, bool residual) {
+    if (desc->C_pad < int64_t(kResidentKb) * kBK) return false;
+    // One limb at K_pad = 512, where the one-CTA kernel keeps the weights: the streamed pair is as fast on 1000 tiles of 256 x 256 and faster
+    // beyond (32768 x 512 -> 1536 33.7 / 34.5 us, -> 2048 42.8 / 42.7, 65536 x 512 -> 512 24.8 / 24.5, -> 1536 65.8 / 60.0), and it adds a
+    // residual as it stores, which the other leaves to a launch of its own (65536 x 512 -> 512 another 24 us).
+    if (desc->C_pad == int64_t(kResidentKb) * kBK &&
+        (desc->limbs != 1 || !(residual || (M + 255) / 256 * ((desc->N + kBN - 1) / kBN) > 1024))) return false;
+    return cont == HQ_CODES_INT8 && desc->RS == 1 && y != nullptr &&
            acc_out == nullptr && ydt == HQ_BF16 && aligned16(y) && (ldy * 2) % 16 == 0 && combine_fast && M >= 256;
 }
 bool pair_stream_covers_conv(hq_container cont, const gemm::GemmParams& g) {

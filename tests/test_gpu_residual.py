@@ -17,7 +17,8 @@ from paper_2512_05746_b200 import inputs
     (1001, 2304, 1160, 256, True),      # ... rows of the last tile missing, a column tile cut off inside a 32-column store
     (16385, 768, 200, 256, True),       # ... narrower column tiles
     (5000, 1024, 776, 256, False),      # ... two limbs
-    (4096, 512, 512, 256, True),        # resident weights: a launch of its own
+    (4096, 512, 512, 256, True),        # ... four K blocks, which a layer without a residual runs on one CTA
+    (1001, 512, 200, 256, True),
     (8200, 2048, 520, 2048, True),      # halved weights: likewise
 ])
 def test_linear_with_a_residual_is_the_linear_and_an_addition(M, K, N, n, room):

@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
     (5000, 4096, 520),        # 192 wide, two K blocks per stage
     (20000, 1280, 136),       # 192 wide, as many tiles as 256 wide ones
     (8192, 4608, 1152),       # 192 wide, whole tiles
+    (53000, 512, 1288),       # four K blocks: the one-CTA kernel's weights stay in its shared memory up to 1024 tiles
 ])
 def test_linear_on_narrow_tiles(M, K, N):
     import torch
