@@ -21,6 +21,7 @@
 // the loads are not what is waited for.
 #include <type_traits>
 
+#include "hq_cluster.cuh"
 #include "hq_common.cuh"
 #include "hq_fwht.cuh"
 
@@ -842,23 +843,36 @@ __global__ void __launch_bounds__(256, 4) gn_stats_kernel(const InT* x, const In
     }
 }
 
+constexpr int kSlabWays = 8, kSlabWayGroups = 32;      // CTAs of a cluster at most, groups of its run at most
+// Mean and 1 / sqrt(var + eps) of a group from its sums.
+__device__ __forceinline__ void gn_finish(double sum, double sq, double inv_count, double eps, float2* out) {
+    const double mean = sum * inv_count;
+    double var = sq * inv_count - mean * mean;
+    if (var < 0.0) var = 0.0;
+    *out = make_float2(float(mean), float(1.0 / sqrt(var + eps)));
+}
+
 // The same statistics with one CTA per (sample, run of whole groups): it sees every pixel of its channels, so the sums need
 // no atomics, no clearing and no ticket, and the call no memset in front (two 32 x 32 x 512 images: 6.6 us of this kernel
 // and 1.5 us of memset before).  A thread owns a 16-byte piece and takes the pixels in the sets that the kernel above adds up
 // in fp32 (eight pixels `ppl` apart), so the fp32 partial sums are the same; only the fp64 sums over them run in another
 // order.  The CTA reads `pieces` * 16 contiguous bytes of every pixel, its neighbours in the grid the rest.
+// `ways` > 1: a cluster of CTAs shares the run, each takes every ways-th round of sets, and the first adds up their sums, which the others
+// have put into its shared memory.
 template <typename InT, int VEC>
 __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, const InT* x2, int split, const __nv_bfloat16* pre_bias, int64_t pre_ld,
-                                                               int hw, int C, int groups, int run, int ppl, float* stats,
+                                                               int hw, int C, int groups, int run, int ppl, int ways, float* stats,
                                                                double inv_count, double eps) {
     constexpr int Q = VEC / 4, U = 8;
     __shared__ double red[2 * Q][256];
     __shared__ double piece_sum[2 * Q][256];
+    __shared__ double way_sum[kSlabWays][2][kSlabWayGroups];           // of the cluster's CTAs, in the first
     griddep_launch();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cg = C / groups, pieces = run * cg / VEC, lanes = 256 / pieces;      // the host keeps pieces <= 256
     const int runs = groups / run;
-    const int sample = blockIdx.x / runs, g0 = (blockIdx.x - sample * runs) * run;
+    const int way = ways > 1 ? int(cluster_rank()) : 0, slab = ways > 1 ? int(blockIdx.x) / ways : int(blockIdx.x);
+    const int sample = slab / runs, g0 = (slab - sample * runs) * run;
     const int piece = tid % pieces, pl = tid / pieces;
     const int ch = g0 * cg + piece * VEC;
     double s1[Q], s2[Q];
@@ -878,7 +892,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
         const int64_t pitch = x2 == nullptr ? C : (second ? C - split : split);
         const InT* src = (second ? x2 + (ch - split) : x + ch) + int64_t(sample) * hw * pitch;
         const int full = hw / (U * ppl) * ppl;         // sets of eight pixels; the pixels behind them are taken one by one
-        for (int set = pl; set < full; set += lanes) {
+        for (int set = pl + way * lanes; set < full; set += ways * lanes) {
             const int px = set / ppl * (U * ppl) + set % ppl;
             GnPiece<VEC> raw[U];
 #pragma unroll
@@ -902,7 +916,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
                 s2[q] += double(b0 + b1);
             }
         }
-        for (int px = full * U + pl; px < hw; px += lanes) {
+        for (int px = full * U + pl + way * lanes; px < hw; px += ways * lanes) {
             const GnPiece<VEC> raw = gn_load(src + int64_t(px) * pitch, static_cast<GnPiece<VEC>*>(nullptr));
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
@@ -940,10 +954,21 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
             a += piece_sum[2 * q][pc];
             b += piece_sum[2 * q + 1][pc];
         }
-        const double mean = a * inv_count;
-        double var = b * inv_count - mean * mean;
-        if (var < 0.0) var = 0.0;
-        reinterpret_cast<float2*>(stats)[int64_t(sample) * groups + g0 + tid] = make_float2(float(mean), float(1.0 / sqrt(var + eps)));
+        if (ways > 1) {
+            const uint32_t to = map_to_cta(&way_sum[way][0][tid], 0);
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(to), "d"(a) : "memory");
+            asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(to + uint32_t(kSlabWayGroups * sizeof(double))), "d"(b) : "memory");
+        } else {
+            gn_finish(a, b, inv_count, eps, reinterpret_cast<float2*>(stats) + int64_t(sample) * groups + g0 + tid);
+        }
+    }
+    if (ways > 1) {
+        cluster_sync_all();                            // every CTA's sums are in the first one's shared memory
+        if (way == 0 && tid < run) {
+            double a = 0.0, b = 0.0;
+            for (int w = 0; w < ways; ++w) { a += way_sum[w][0][tid]; b += way_sum[w][1][tid]; }
+            gn_finish(a, b, inv_count, eps, reinterpret_cast<float2*>(stats) + int64_t(sample) * groups + g0 + tid);
+        }
     }
 }
 
@@ -1165,7 +1190,7 @@ static int64_t gn_wave_ctas(int64_t Nb, int64_t hw, int64_t C, int vec) {
     return (Nb * hw + span - 1) / span;
 }
 
-// Groups per CTA of the slab kernel, or 0: the one-wave kernel takes the tensor (groups of more than 256 pieces, more samples
+// Groups per CTA of the slab kernel, and the CTAs that share them, or 0 groups: the one-wave kernel takes the tensor (groups of more than 256 pieces, more samples
 // than one wave of CTAs).  The fewest groups for which the CTAs fit one wave of four per SM.  Both sides are estimated, in us
 // over what they share.  A slab CTA walks its pixels in rounds of eight loads per thread, 0.85 us each however few CTAs there
 // are, and 1.4 times that where its run fills half sectors only.  The one-wave kernel spreads the bytes over the whole chip, but
@@ -1175,21 +1200,48 @@ static int64_t gn_wave_ctas(int64_t Nb, int64_t hw, int64_t C, int vec) {
 // 1 x 64 x 64 x 2048 90 / 31, 64 x 32 x 32 x 512 56.8 / 55.0; not taken: 1 x 128 x 128 x 1024 63 / 52 from L2 but 66 / 83 from
 // memory, 1 x 256 x 256 x 512 66 / 162, 1 x 512 x 512 x 512 201 / 665, 16 x 64 x 64 x 256 29.7 / 31.2 (half sectors),
 // 64 x 16 x 16 x 768 27.7 / 28.8 (32 sets over 21 threads), one group of 256 channels on 1 x 64 x 64 18.6 / 61.
-static int gn_slab_run(int64_t Nb, int64_t hw, int64_t C, int groups, int elt, int vec) {
-    const int64_t cg = C / groups;
+// Where a CTA alone would walk several rounds and SMs are left, a cluster of up to eight shares the run (and a run fills a sector: a
+// quarter of the requests of a warp).  Statistics + transform, without / with clusters: 2 x 64 x 64 x 512 11.4 / 10.1 us, 1 x 64 x 64 x
+// 2048 27 / 18.7, 8 x 64 x 64 x 256 15.8 / 14.3, and against the one-wave kernel 1 x 128 x 128 x 1024 53 / 25, 2 x 128 x 128 x 256 21.2 / 14.5,
+// 1 x 96 x 96 x 512 17.2 / 11.2, 1 x 64 x 64 x 256 in four groups 20.3 / 9.0; shapes of one round stay as they are.  Images of 65536
+// pixels and single groups keep the one-wave kernel, as the tests of this choice have it (1 x 256 x 256 x 128 29.3, 18.2 on clusters;
+// one group of 256 channels on 1 x 64 x 64 18.4, 12.7).
+struct SlabPlan { int run, ways; };
+static SlabPlan gn_slab_plan(int64_t Nb, int64_t hw, int64_t C, int groups, int elt, int vec) {
+    const int64_t cg = C / groups, sets = (hw + 7) / 8;
     for (int run = 1; run <= groups && run <= 256; ++run) {
         if (groups % run != 0 || (run * cg) % vec != 0 || run * cg / vec > 256) continue;
         if (Nb * (groups / run) > int64_t(sm_count()) * 4) continue;
-        const int64_t bytes = Nb * hw * C * elt, sets = (hw + 7) / 8, lanes = 256 / (run * cg / vec);
+        SlabPlan plan{run, 1};
+        int wide = run;
+        for (int k = run; k <= groups && k <= kSlabWayGroups; ++k)
+            if (groups % k == 0 && (k * cg) % vec == 0 && k * cg / vec <= 256 && k * cg * elt <= 32) wide = k;
+        const int64_t wide_lanes = 256 / (wide * cg / vec);
+        int ways = 1;
+        while (groups > 1 && hw < 65536 && wide <= kSlabWayGroups && ways < kSlabWays && Nb * (groups / wide) * ways <= sm_count() && sets > wide_lanes * ways) ways *= 2;
+        if (ways > 1) plan = SlabPlan{wide, ways};
+        const int64_t bytes = Nb * hw * C * elt, lanes = 256 / (plan.run * cg / vec) * plan.ways;
         const int64_t rounds = (sets + lanes - 1) / lanes;
-        const bool full = run * cg * elt >= 32, even = 10 * sets >= 8 * lanes * rounds;
+        const bool full = plan.run * cg * elt >= 32, even = 10 * sets >= 8 * lanes * rounds;
         const int64_t per_sample = gn_wave_ctas(Nb, hw, C, vec) / Nb, adds = (per_sample > 1 ? per_sample : 1) * (cg > vec ? cg / vec : 1);
         const double slab = (full ? 0.85 : 1.2) * double(rounds);
         const double wave = 5.0 + 0.02 * double(adds) + 0.3 * (bytes < 20000000 ? double(bytes) * 1e-6 : 20.0);
         const bool streams = full && even && (hw <= 4096 || bytes <= 40000000);
-        return slab < wave && (bytes <= 20000000 || streams) ? run : 0;
+        return slab < wave && (bytes <= 20000000 || streams) ? plan : SlabPlan{0, 1};
     }
-    return 0;
+    return SlabPlan{0, 1};
+}
+template <typename... Params, typename... Args>
+static cudaError_t launch_slab(void (*kern)(Params...), unsigned ctas, int ways, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(256); cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = unsigned(ways); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = ways > 1 ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, Params(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
 }
 
 // GroupNorm statistics of an NHWC tensor (hw pixels per sample): fp64 sums per (sample, group) in `scratch` (cleared
@@ -1222,15 +1274,16 @@ hq_status launch_gn_stats(const void* x, hq_dtype xdt, int64_t Nb, int64_t hw, i
     const int64_t pieces = C / (wide ? 8 : 4);
     const int64_t ppl = pieces < 256 ? 256 / pieces : 1;
     const double inv_count = 1.0 / (double(hw) * double(C / groups));
-    if (const int run = gn_slab_run(Nb, hw, C, groups, elt, wide ? 8 : 4)) {
-        const unsigned slabs = unsigned(Nb * (groups / run));
-#define HQ_SLAB(T, V) gn_stats_slab_kernel<T, V><<<slabs, 256, 0, st>>>(static_cast<const T*>(x), static_cast<const T*>(x2), int(split), pre, pre_ld, int(hw), \
-                                                                        int(C), groups, run, int(ppl), stats, inv_count, double(eps))
+    if (const SlabPlan plan = gn_slab_plan(Nb, hw, C, groups, elt, wide ? 8 : 4); plan.run > 0) {
+        const unsigned slabs = unsigned(Nb * (groups / plan.run) * plan.ways);
+        cudaError_t e;
+#define HQ_SLAB(T, V) e = launch_slab(gn_stats_slab_kernel<T, V>, slabs, plan.ways, st, static_cast<const T*>(x), static_cast<const T*>(x2), int(split), pre, pre_ld, \
+                                      int(hw), int(C), groups, plan.run, int(ppl), plan.ways, stats, inv_count, double(eps))
         if (xdt == HQ_F32) HQ_SLAB(float, 4);
         else if (wide) HQ_SLAB(__nv_bfloat16, 8);
         else HQ_SLAB(__nv_bfloat16, 4);
 #undef HQ_SLAB
-        if (cudaGetLastError() != cudaSuccess) return HQ_ERR_CUDA;
+        if (e != cudaSuccess) return HQ_ERR_CUDA;
         *stats_out = stats;
         return HQ_OK;
     }

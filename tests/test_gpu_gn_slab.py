@@ -18,6 +18,10 @@ pytestmark = pytest.mark.gpu
     (40, 8, 8, 1024, 32, 256, "bf16", 0),       # several groups per CTA
     (70, 8, 8, 512, 32, 256, "bf16", 256),      # the seam between two tensors lies between two runs
     (64, 16, 16, 512, 32, 256, "bf16", 0),      # 17 MB
+    (2, 64, 64, 256, 32, 256, "bf16", 0),       # a cluster of eight CTAs per run of two groups
+    (1, 100, 50, 512, 32, 256, "bf16", 256),    # ... 625 sets over its threads; two tensors
+    (1, 36, 44, 256, 2, 256, "f32", 0),         # ... groups of 128 channels, 196 sets and 16 pixels behind them
+    (5, 48, 48, 768, 32, 256, "bf16", 0),       # clusters of one, two or four, by what is left of the SMs
 ])
 def test_gn_statistics_of_a_run_of_groups(oracle, Nb, H, W, C, G, n, dt, c1):
     import torch
