@@ -417,7 +417,7 @@ hq_status launch_qconv2d(const void* a_codes, hq_container cont, int a_bits, int
     if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, uint32_t(per_tap ? per_tap_rows(desc->limbs) : kBN), true))
         return HQ_ERR_CUDA;
     if (g_pair_gemm && pair_stream_covers_conv(cont, p)) {
-        if (res != nullptr) { p.res = res->r; res->done = true; }
+        if (res != nullptr && !per_tap) { p.res = res->r; res->done = true; }
         return launch_qconv_pair(p, tmA, tmY, desc, w_dev, st);
     }
     return launch(nib, tmA, tmB, tmY, p, st);

@@ -518,6 +518,9 @@ struct PairStreamParams {
     int64_t ldr;
     // convolution geometry (CONV instantiations)
     int kb_per_tap, S, stride, pad, bw, bh, bn, tiles_w, tiles_h;
+    // one scale per input pixel (PERTAP instantiations)
+    int Nb, H, W, Ho, Wo;
+    void* y; int y_bf16, y_vec_ok; int64_t ldy;
 };
 
 constexpr int kPairStageBytes = kABytes + kPairBBytes;      // 32 KB: this CTA's activation rows and its half of the weights
@@ -549,7 +552,11 @@ __device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const void* tma
 // least, see stream_width); a narrower tile's weight half fills only part of its place in the stage.
 // HALVED: halved weights (hq_fwht.cuh); the further columns are the last K block of both operands.  65536 x 4096 -> 4096 1195 us
 // on two limbs, 653 so (the whole layer 1657 / 1127; tensor pipe 88 % active, 92 on two limbs).
-template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED>
+// PERTAP: one activation scale per input pixel under a window: as in the one-CTA kernel, a tap's sums are an accumulator of their own,
+// drained, scaled and added up in registers; 128 output channels a tile.  There a K block of two limbs is 48 KB for 536 cycles of MMAs, more
+// than an SM gets from L2, here 32.  Whole layer, one CTA / pairs: 8 x 32 x 32 x
+// 256 18.8 / 16.7 us, 64 x 16 x 16 x 768 (one limb) 127.6 / 97.1, 64 x 32 x 32 x 512 (one limb) 224.7 / 178.4, 2 x 32 x 32 x 256 16.7 / 14.9.
+template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED, bool PERTAP = false>
 __global__ void __launch_bounds__(kPairThreads, 1)
 qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                          const __grid_constant__ CUtensorMap tmY, const PairStreamParams p) {
@@ -574,7 +581,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         fence_barrier_init();
         tma_prefetch_desc(&tmA);
         tma_prefetch_desc(&tmB);
-        tma_prefetch_desc(&tmY);
+        if (!PERTAP) tma_prefetch_desc(&tmY);          // rows are stored from registers there
     }
     if (warp == 1) { __syncwarp(); tmem_alloc_pair(&ctl->tmem_base, kTmemCols); tmem_relinquish_pair(); }
     tc_fence_before();
@@ -633,13 +640,15 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
             uint64_t a_desc = desc0;
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
-            for (int i = 0; i < count && ok; ++i) {
+            // accumulators in turn: one per tile, or (PERTAP) per tap of a tile
+            const int kb_each = PERTAP ? p.kb_per_tap : num_kb, accs = PERTAP ? count * (num_kb / kb_each) : count;
+            for (int i = 0; i < accs && ok; ++i) {
                 const int as = i & 1;
                 if (!wait_pair(&ctl->tempty[as], (uint32_t(i >> 1) & 1u) ^ 1u, ctl, p.dev_status, kStatusAccumFree)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + uint32_t(as * kBN);
-                uint32_t acc = 0;                          // 0 for the first MMA of the tile only
-                for (int kb = 0; kb < num_kb; kb += KPS) {
+                uint32_t acc = 0;                          // 0 for the first MMA of the accumulator only
+                for (int kb = 0; kb < kb_each; kb += KPS) {
                     if (!wait_pair(&ctl->full[stage], phase, ctl, p.dev_status, kStatusTmaWait)) { ok = false; break; }
                     tc_fence_after();
                     const uint64_t b_desc = a_desc + kBUnits;
@@ -701,7 +710,7 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
         };
         if (count > 0) request_columns(0);
         if (p.pdl) griddep_wait();                    // scale_a comes from the kernel before this one
-        if (count > 0) request_row(0);
+        if (!PERTAP && count > 0) request_row(0);
         for (int i = 0; i < count && ok; ++i) {
             const int u = c + i * G;
             const int m2 = u / p.tiles_n, n_tile = u - m2 * p.tiles_n;
@@ -721,7 +730,71 @@ qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
 #pragma unroll
                 for (int j = 0; j < BN / 64; ++j) odd[j] = next_row_odd ? col_odd[j] : 0u;
             }
-            if (i + 1 < count) { request_columns(i + 1); request_row(i + 1); }
+            if (i + 1 < count) { request_columns(i + 1); if (!PERTAP) request_row(i + 1); }
+            if constexpr (PERTAP) {
+                const int m_tile = m2 * 2 + int(rank), r_tile = q * 32 + lane;
+                const int tw = m_tile % p.tiles_w, th = (m_tile / p.tiles_w) % p.tiles_h, tn = m_tile / (p.tiles_w * p.tiles_h);
+                const int iw = r_tile % p.bw, ih = (r_tile / p.bw) % p.bh, in_ = r_tile / (p.bw * p.bh);
+                const int n = tn * p.bn + in_, ho = th * p.bh + ih, wo = tw * p.bw + iw;
+                const bool row_ok = n < p.Nb && ho < p.Ho && wo < p.Wo;        // a tile is bw x bh x bn = 128 pixels
+                auto tap_scale = [&](int g) -> float {
+                    const int r = g / p.S, sx = g - r * p.S;
+                    const int hi_ = ho * p.stride + r - p.pad, wi_ = wo * p.stride + sx - p.pad;
+                    if (!row_ok || hi_ < 0 || hi_ >= p.H || wi_ < 0 || wi_ >= p.W) return 0.f;
+                    return ld_dependent(p.scale_a + (int64_t(n) * p.H + hi_) * p.W + wi_);
+                };
+                const int taps = num_kb / p.kb_per_tap;
+                float run[64];
+#pragma unroll
+                for (int j = 0; j < 64; ++j) run[j] = 0.f;
+                float s_next = tap_scale(0);
+                for (int g = 0; g < taps; ++g) {
+                    const int seq = i * taps + g, as2 = seq & 1;
+                    const float s_g = s_next;
+                    if (g + 1 < taps) s_next = tap_scale(g + 1);
+                    if (!wait_pair(&ctl->tfull[as2], uint32_t(seq >> 1) & 1u, ctl, p.dev_status, kStatusAccumWait)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t t_tap = tmem_base + (uint32_t(q * 32) << 16) + uint32_t(as2 * kBN + wc0);
+                    uint32_t hi[16], lo[16];
+                    tmem_ld_32x16(t_tap, hi);
+                    if (LIMBS == 2) tmem_ld_32x16(t_tap + uint32_t(kBN / 2), lo);
+#pragma unroll
+                    for (int st = 0; st < 4; ++st) {
+                        int32_t w[16];
+                        tmem_ld_wait_16(hi);
+                        if (LIMBS == 2) tmem_ld_wait_16(lo);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) w[j] = LIMBS == 2 ? int32_t(hi[j]) * 256 + int32_t(lo[j]) : int32_t(hi[j]);
+                        if (st < 3) {
+                            tmem_ld_32x16(t_tap + uint32_t((st + 1) * 16), hi);
+                            if (LIMBS == 2) tmem_ld_32x16(t_tap + uint32_t(kBN / 2 + (st + 1) * 16), lo);
+                        } else {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive_cluster(tempty_leader[as2]);
+                        }
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) run[st * 16 + j] = fmaf(float(w[j]), s_g, run[st * 16 + j]);
+                    }
+                }
+                if (!ok) break;
+                if (row_ok) {
+                    unsigned char* y_row = static_cast<unsigned char*>(p.y) + (int64_t(n * p.Ho + ho) * p.Wo + wo) * p.ldy * (p.y_bf16 ? 2 : 4);
+#pragma unroll
+                    for (int st = 0; st < 4; ++st) {
+                        uint32_t f[16];
+#pragma unroll
+                        for (int j = 0; j < 16; ++j)
+                            f[j] = __float_as_uint(fmaf(run[st * 16 + j] * prm_sw[st * 16 + j], p.alpha, prm_b[st * 16 + j]));
+                        const int col = col_base + wc0 + st * 16;
+                        if (col < p.N) {
+                            if (p.y_bf16) store_row16<2>(y_row, f, col, p.N, p.y_vec_ok != 0);
+                            else store_row16<4>(y_row, f, col, p.N, p.y_vec_ok != 0);
+                        }
+                    }
+                }
+                continue;
+            }
             const int row0 = m2 * 256 + int(rank) * 128 + q * 32;
             const int64_t my_row = row0 + lane;
             const __nv_bfloat16* res = !HALVED && p.res != nullptr && my_row < p.M ? p.res + my_row * p.ldr + col_base + wc0 : nullptr;
@@ -826,10 +899,10 @@ int max_pairs(size_t smem) {
     return slot;
 }
 
-template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED = false>
+template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED = false, bool PERTAP = false>
 cudaError_t launch_pair_stream(int pairs_wanted, size_t smem, cudaStream_t st, const CUtensorMap& tmA, const CUtensorMap& tmB,
                                const CUtensorMap& tmY, const PairStreamParams& p) {
-    auto kern = qgemm_pair_stream_kernel<LIMBS, CONV, KPS, BN, HALVED>;
+    auto kern = qgemm_pair_stream_kernel<LIMBS, CONV, KPS, BN, HALVED, PERTAP>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -916,8 +989,8 @@ bool pair_stream_covers_gemm(hq_container cont, const hq_weight_desc* desc, int6
            acc_out == nullptr && ydt == HQ_BF16 && aligned16(y) && (ldy * 2) % 16 == 0 && combine_fast && M >= 256;
 }
 bool pair_stream_covers_conv(hq_container cont, const gemm::GemmParams& g) {
-    // one static scale, or one scale per output pixel of a 1x1 convolution (per_tap marks per-pixel scales under a window)
-    return cont == HQ_CODES_INT8 && g.conv && g.tma_store && !g.per_tap && g.bw * g.bh * g.bn == kBM &&
+    // one static scale, or one scale per output pixel of a 1x1 convolution; per_tap marks per-pixel scales under a window
+    return cont == HQ_CODES_INT8 && g.conv && (g.per_tap ? g.combine_fast != 0 : g.tma_store != 0) && g.bw * g.bh * g.bn == kBM &&
            g.kb_per_tap * g.taps > kResidentKb && int64_t(g.tiles_m) >= 2;
 }
 
@@ -964,20 +1037,30 @@ hq_status launch_qconv_pair(const gemm::GemmParams& g, const CUtensorMap& tmA, c
     p.res = g.res; p.ldr = g.ldy;
     p.num_kb = g.kb_per_tap * g.taps;
     p.tiles_m2 = (g.tiles_m + 1) / 2;
-    const int bn = g.limbs == 2 ? kBN : stream_width(p.tiles_m2, g.N);
-    p.tiles_n = g.limbs == 2 ? g.tiles_n : (g.N + bn - 1) / bn;
+    const int bn = g.limbs == 2 ? kBN : g.per_tap ? kBN / 2 : stream_width(p.tiles_m2, g.N);
+    p.tiles_n = g.limbs == 2 || g.per_tap ? g.tiles_n : (g.N + bn - 1) / bn;
     p.scale_a = g.scale_a; p.sa_scalar = g.sa_scalar; p.scale_w = g.scale_w; p.bias = g.bias; p.alpha = g.alpha;
     p.pdl = g.pdl; p.dev_status = g.dev_status;
     p.kb_per_tap = g.kb_per_tap; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
     p.bw = g.bw; p.bh = g.bh; p.bn = g.bn; p.tiles_w = g.tiles_w; p.tiles_h = g.tiles_h;
     size_t smem = 0;
-    const int kps = p.num_kb % 2 == 0 ? 2 : 1;      // two K blocks per ring stage: 6 % faster on the 3x3 convolutions
+    p.Nb = g.Nb; p.H = g.H; p.W = g.W; p.Ho = g.Ho; p.Wo = g.Wo;
+    p.y = g.y; p.y_bf16 = g.y_bf16; p.y_vec_ok = g.y_vec_ok; p.ldy = g.ldy;
+    // two K blocks per ring stage: 6 % faster on the 3x3 convolutions
+    const int kps = (g.per_tap ? p.kb_per_tap : p.num_kb) % 2 == 0 ? 2 : 1;
     if (!pair_stream_stages(p, smem, kps)) return HQ_ERR_UNSUPPORTED;
     CUtensorMap tmB;
     const uint64_t Kp = uint64_t(desc->C_pad) * desc->RS;
     if (!encode_2d(&tmB, w_dev, Kp, uint64_t(desc->N_pad) * desc->limbs, Kp, kBK, uint32_t(bn / 2), true)) return HQ_ERR_CUDA;
     const int tiles = p.tiles_m2 * p.tiles_n;
     cudaError_t e;
+    if (g.per_tap) {
+        if (kps == 2) e = g.limbs == 2 ? launch_pair_stream<2, true, 2, kBN, false, true>(tiles, smem, st, tmA, tmB, tmY, p)
+                                       : launch_pair_stream<1, true, 2, kBN / 2, false, true>(tiles, smem, st, tmA, tmB, tmY, p);
+        else e = g.limbs == 2 ? launch_pair_stream<2, true, 1, kBN, false, true>(tiles, smem, st, tmA, tmB, tmY, p)
+                              : launch_pair_stream<1, true, 1, kBN / 2, false, true>(tiles, smem, st, tmA, tmB, tmY, p);
+        return e == cudaSuccess ? HQ_OK : HQ_ERR_CUDA;
+    }
     if (kps == 2) e = desc->limbs == 2 ? launch_pair_stream_bn<2, true, 2>(bn, tiles, smem, st, tmA, tmB, tmY, p)
                                        : launch_pair_stream_bn<1, true, 2>(bn, tiles, smem, st, tmA, tmB, tmY, p);
     else e = desc->limbs == 2 ? launch_pair_stream_bn<2, true, 1>(bn, tiles, smem, st, tmA, tmB, tmY, p)

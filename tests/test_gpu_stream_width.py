@@ -61,3 +61,32 @@ def test_narrow_tiles_one_after_the_other_keep_their_staging_apart(M, K, N):
     assert int(status) == 0
     for y in ys[1:]:
         assert torch.equal(y, ys[0])
+
+
+@pytest.mark.parametrize("Nb,H,W,C,Cout,stride,mode", [
+    (8, 32, 32, 256, 256, 1, "folded"),      # two limbs, two K blocks a stage, one wave
+    (5, 32, 32, 384, 264, 1, "folded"),      # ... three K blocks a tap, an odd number of row tiles, a column tile cut off
+    (7, 16, 16, 256, 136, 2, "plain"),       # one limb, stride 2, two images a tile and one missing
+    (40, 16, 16, 512, 520, 1, "plain"),      # ... several tiles a pair
+])
+@pytest.mark.parametrize("f32", [False, True])
+def test_per_pixel_scales_on_pairs(Nb, H, W, C, Cout, stride, mode, f32):
+    import torch
+    from paper_2512_05746_b200 import binding as hq
+    pw = hq.hq_weight_prepare(inputs.weights((Cout, 3, 3, C), seed=C), 4, 128, hq.WEIGHT_MODES[mode], hq.HQ_CODES_INT8).to_device()
+    gen = torch.Generator(device="cuda").manual_seed(C)
+    q = torch.randint(-8, 8, (Nb, H, W, C), generator=gen, device="cuda", dtype=torch.int8).view(torch.uint8)
+    sa = torch.rand((Nb * H * W,), generator=gen, device="cuda") + 0.5
+    b = torch.from_numpy(inputs.bias(Cout, seed=1)).cuda()
+    out = []
+    for pair in (0, 2):
+        y = torch.full((Nb, H // stride, W // stride, Cout), 7.0, dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+        status = torch.zeros((1,), dtype=torch.int32, device="cuda")
+        before = hq.hq_set_pair_gemm(pair)
+        try:
+            hq.hq_qconv2d(q, hq.HQ_CODES_INT8, 4, Nb, H, W, C, pw, 3, 3, stride, 1, scale_a=sa, bias=b, y=y, dev_status=status)
+        finally:
+            hq.hq_set_pair_gemm(before)
+        assert int(status) == 0
+        out.append(y)
+    assert torch.equal(out[0], out[1])
