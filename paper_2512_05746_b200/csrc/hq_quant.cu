@@ -1107,6 +1107,11 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         while ((rpc * tr) % 32 != 0) ++rpc;                 // whole warps
         const int base = rpc;
         while ((rpc + base) * tr <= 128) rpc += base;
+        // With GroupNorm every CTA builds the table of its sample's channels, an eighth to a quarter of its work on wide pixels: twice the
+        // rows there, where a sample's rows divide.  Statistics + transform, so many / twice: 64 x 16 x 16 x 1536 46.9 / 41.9 us, 64 x 8 x 8 x
+        // 2048 19.1 / 17.3, 64 x 16 x 16 x 768 23.6 / 22.8, 64 x 32 x 32 x 1024 95.5 / 94.8; narrower ones lose resident CTAs (64 x 64 x 64 x
+        // 256 87.2 / 91.0, 64 x 32 x 32 x 512 44.8 / 46.4).
+        if (gn != nullptr && cols >= 768 && 2 * rpc * tr <= 256 && gn->rows_per_sample % (2 * rpc) == 0) rpc *= 2;
         p.threads_per_row = tr;
         p.row_magic = uint32_t(((1 << 20) + tr - 1) / tr);
         p.rows_per_cta = rpc;

@@ -22,6 +22,8 @@ pytestmark = pytest.mark.gpu
     (1, 100, 50, 512, 32, 256, "bf16", 256),    # ... 625 sets over its threads; two tensors
     (1, 36, 44, 256, 2, 256, "f32", 0),         # ... groups of 128 channels, 196 sets and 16 pixels behind them
     (5, 48, 48, 768, 32, 256, "bf16", 0),       # clusters of one, two or four, by what is left of the SMs
+    (3, 4, 5, 768, 32, 256, "bf16", 0),         # 20 rows a sample: four to a CTA of the transform, and not eight
+    (2, 6, 4, 1536, 32, 256, "f32", 0),         # 24: four and not two
 ])
 def test_gn_statistics_of_a_run_of_groups(oracle, Nb, H, W, C, G, n, dt, c1):
     import torch
