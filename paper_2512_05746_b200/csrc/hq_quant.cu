@@ -858,7 +858,8 @@ __device__ __forceinline__ void gn_finish(double sum, double sq, double inv_coun
 // in fp32 (eight pixels `ppl` apart), so the fp32 partial sums are the same; only the fp64 sums over them run in another
 // order.  The CTA reads `pieces` * 16 contiguous bytes of every pixel, its neighbours in the grid the rest.
 // `ways` > 1: a cluster of CTAs shares the run, each takes every ways-th round of sets, and the first adds up their sums, which the others
-// have put into its shared memory.
+// have put into its shared memory: behind a barrier that every CTA arrives at as it starts, since a CTA that has not begun has no
+// shared memory to write to, and one with no set left to walk is there at once.
 template <typename InT, int VEC>
 __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, const InT* x2, int split, const __nv_bfloat16* pre_bias, int64_t pre_ld,
                                                                int hw, int C, int groups, int run, int ppl, int ways, float* stats,
@@ -867,6 +868,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
     __shared__ double red[2 * Q][256];
     __shared__ double piece_sum[2 * Q][256];
     __shared__ double way_sum[kSlabWays][2][kSlabWayGroups];           // of the cluster's CTAs, in the first
+    if (ways > 1) cluster_arrive_relaxed();            // waited for before the first store into another CTA
     griddep_launch();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cg = C / groups, pieces = run * cg / VEC, lanes = 256 / pieces;      // the host keeps pieces <= 256
@@ -946,6 +948,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
         if (sub == 0 && j < 2 * Q * pieces) piece_sum[k][pc] = t;
     }
     __syncthreads();
+    if (ways > 1) cluster_wait();                      // every CTA of the cluster has begun
     if (tid < run) {                                   // the host keeps run <= 256
         const int quads = cg / 4;
         double a = 0.0, b = 0.0;
@@ -963,6 +966,7 @@ __global__ void __launch_bounds__(256, 4) gn_stats_slab_kernel(const InT* x, con
         }
     }
     if (ways > 1) {
+        __syncwarp();                                  // the barrier is taken by whole warps
         cluster_sync_all();                            // every CTA's sums are in the first one's shared memory
         if (way == 0 && tid < run) {
             double a = 0.0, b = 0.0;

@@ -21,6 +21,7 @@ pytestmark = pytest.mark.gpu
     (2, 64, 64, 256, 32, 256, "bf16", 0),       # a cluster of eight CTAs per run of two groups
     (1, 100, 50, 512, 32, 256, "bf16", 256),    # ... 625 sets over its threads; two tensors
     (1, 36, 44, 256, 2, 256, "f32", 0),         # ... groups of 128 channels, 196 sets and 16 pixels behind them
+    (3, 48, 48, 256, 32, 128, "bf16", 128),     # a cluster of four CTAs per run of two groups, no set left for the last; two tensors
     (5, 48, 48, 768, 32, 256, "bf16", 0),       # clusters of one, two or four, by what is left of the SMs
     (3, 4, 5, 768, 32, 256, "bf16", 0),         # 20 rows a sample: four to a CTA of the transform, and not eight
     (2, 6, 4, 1536, 32, 256, "f32", 0),         # 24: four and not two
