@@ -1199,8 +1199,8 @@ static int64_t gn_wave_ctas(int64_t Nb, int64_t hw, int64_t C, int vec) {
     return (Nb * hw + span - 1) / span;
 }
 
-// Groups per CTA of the slab kernel, and the CTAs that share them, or 0 groups: the one-wave kernel takes the tensor (groups of more than 256 pieces, more samples
-// than one wave of CTAs).  The fewest groups for which the CTAs fit one wave of four per SM.  Both sides are estimated, in us
+// Groups per CTA of the slab kernel, and the CTAs that share them, or 0 groups: the one-wave kernel takes the tensor (groups of more than 256
+// pieces, more samples than one wave of CTAs).  The fewest groups for which the CTAs fit one wave of four per SM.  Both sides are estimated, in us
 // over what they share.  A slab CTA walks its pixels in rounds of eight loads per thread, 0.85 us each however few CTAs there
 // are, and 1.4 times that where its run fills half sectors only.  The one-wave kernel spreads the bytes over the whole chip, but
 // its CTAs add their sums to one address per group in turn (20 ns each), behind a memset.  On tensors of more than 20 MB
@@ -1210,35 +1210,50 @@ static int64_t gn_wave_ctas(int64_t Nb, int64_t hw, int64_t C, int vec) {
 // memory, 1 x 256 x 256 x 512 66 / 162, 1 x 512 x 512 x 512 201 / 665, 16 x 64 x 64 x 256 29.7 / 31.2 (half sectors),
 // 64 x 16 x 16 x 768 27.7 / 28.8 (32 sets over 21 threads), one group of 256 channels on 1 x 64 x 64 18.6 / 61.
 // Where a CTA alone would walk several rounds and SMs are left, a cluster of up to eight shares the run (and a run fills a sector: a
-// quarter of the requests of a warp).  Statistics + transform, without / with clusters: 2 x 64 x 64 x 512 11.4 / 10.1 us, 1 x 64 x 64 x
-// 2048 27 / 18.7, 8 x 64 x 64 x 256 15.8 / 14.3, and against the one-wave kernel 1 x 128 x 128 x 1024 53 / 25, 2 x 128 x 128 x 256 21.2 / 14.5,
-// 1 x 96 x 96 x 512 17.2 / 11.2, 1 x 64 x 64 x 256 in four groups 20.3 / 9.0; shapes of one round stay as they are.  Images of 65536
-// pixels and single groups keep the one-wave kernel, as the tests of this choice have it (1 x 256 x 256 x 128 29.3, 18.2 on clusters;
-// one group of 256 channels on 1 x 64 x 64 18.4, 12.7).
+// quarter of the requests of a warp): 2 x 64 x 64 x 512 11.4 / 10.1 us, 1 x 64 x 64 x 2048 27 / 18.7, 8 x 64 x 64 x 256 15.8 / 14.3, and
+// against the one-wave kernel 1 x 128 x 128 x 1024 53 / 25, 2 x 128 x 128 x 256 21.2 / 14.5, 1 x 96 x 96 x 512 17.2 / 11.2, 1 x 64 x 64 x 256
+// in four groups 20.3 / 9.0.  It has to save more than it costs: 1.5 units, 4 on more than 100 CTAs, where the transform's first loads, let in
+// early, no longer find SMs of their own; a round (a last one by its share) 3 units in eight-channel pieces, 0.8 in four, 1.6 times that on
+// half sectors and more the more bytes are shared.  These are fitted to every choice's time on 1126 shapes (up to 50 MB, in L2 and from
+// memory): within 6.8 % of a CTA alone or the one-wave kernel at the worst.  A cluster at every chance, and the one-wave kernel where only the cluster
+// failed the test above, was 1.02 to 10.5 times slower than those on 117 of them: 2 x 40 x 40 x 2048 fp32 19.2 us alone, 203 so, 2 x 64 x 64 x
+// 1536 31.9 / 53, 2 x 24 x 24 x 512 fp32 6.5 / 9.1, 2 x 48 x 48 x 256 8.6 / 9.7.  In place of the one-wave kernel a cluster walks at most 16
+// rounds of eight-channel pieces in groups of up to 16 of them, whose sums that kernel adds up faster than estimated (1 x 200 x 200 x 256 in two groups from memory 42
+// / 63 us on clusters; in groups of 32 pieces 2 x 128 x 128 x 512 111 / 67).
+// Images of 65536 pixels and single groups were left to the one-wave kernel when there were no clusters, and still are: no cost says
+// so (1 x 256 x 256 x 128 29.3, 18.2 on clusters; one group of 256 channels on 1 x 64 x 64 18.4, 12.7).
 struct SlabPlan { int run, ways; };
 static SlabPlan gn_slab_plan(int64_t Nb, int64_t hw, int64_t C, int groups, int elt, int vec) {
-    const int64_t cg = C / groups, sets = (hw + 7) / 8;
-    for (int run = 1; run <= groups && run <= 256; ++run) {
-        if (groups % run != 0 || (run * cg) % vec != 0 || run * cg / vec > 256) continue;
-        if (Nb * (groups / run) > int64_t(sm_count()) * 4) continue;
-        SlabPlan plan{run, 1};
-        int wide = run;
-        for (int k = run; k <= groups && k <= kSlabWayGroups; ++k)
-            if (groups % k == 0 && (k * cg) % vec == 0 && k * cg / vec <= 256 && k * cg * elt <= 32) wide = k;
-        const int64_t wide_lanes = 256 / (wide * cg / vec);
-        int ways = 1;
-        while (groups > 1 && hw < 65536 && wide <= kSlabWayGroups && ways < kSlabWays && Nb * (groups / wide) * ways <= sm_count() && sets > wide_lanes * ways) ways *= 2;
-        if (ways > 1) plan = SlabPlan{wide, ways};
-        const int64_t bytes = Nb * hw * C * elt, lanes = 256 / (plan.run * cg / vec) * plan.ways;
-        const int64_t rounds = (sets + lanes - 1) / lanes;
-        const bool full = plan.run * cg * elt >= 32, even = 10 * sets >= 8 * lanes * rounds;
-        const int64_t per_sample = gn_wave_ctas(Nb, hw, C, vec) / Nb, adds = (per_sample > 1 ? per_sample : 1) * (cg > vec ? cg / vec : 1);
-        const double slab = (full ? 0.85 : 1.2) * double(rounds);
-        const double wave = 5.0 + 0.02 * double(adds) + 0.3 * (bytes < 20000000 ? double(bytes) * 1e-6 : 20.0);
-        const bool streams = full && even && (hw <= 4096 || bytes <= 40000000);
-        return slab < wave && (bytes <= 20000000 || streams) ? plan : SlabPlan{0, 1};
+    const int64_t cg = C / groups, sets = (hw + 7) / 8, bytes = Nb * hw * C * elt;
+    const auto fits = [&](int run) { return groups % run == 0 && (run * cg) % vec == 0 && run * cg / vec <= 256; };
+    int run = 1;
+    while (run <= groups && run <= 256 && !(fits(run) && Nb * (groups / run) <= int64_t(sm_count()) * 4)) ++run;
+    if (run > groups || run > 256) return SlabPlan{0, 1};
+    const auto lanes = [&](SlabPlan p) { return 256 / (p.run * cg / vec) * p.ways; };
+    const auto rounds = [&](SlabPlan p) { return (sets + lanes(p) - 1) / lanes(p); };
+    const auto full = [&](SlabPlan p) { return p.run * cg * elt >= 32; };
+    const int64_t per_sample = gn_wave_ctas(Nb, hw, C, vec) / Nb, adds = (per_sample > 1 ? per_sample : 1) * (cg > vec ? cg / vec : 1);
+    const double wave = 5.0 + 0.02 * double(adds) + 0.3 * (bytes < 20000000 ? double(bytes) * 1e-6 : 20.0);
+    const auto beats_wave = [&](SlabPlan p) {
+        const bool even = 10 * sets >= 8 * lanes(p) * rounds(p), streams = full(p) && even && (hw <= 4096 || bytes <= 40000000);
+        return (full(p) ? 0.85 : 1.2) * double(rounds(p)) < wave && (bytes <= 20000000 || streams);
+    };
+    const auto cost = [&](SlabPlan p) {
+        const double share = double(sets) / double(lanes(p));
+        return (vec == 8 ? 3.0 : 0.8) * (full(p) ? 1.0 : 1.6) * (1.0 + 0.2e-6 * double(bytes)) * (share > 1.0 ? share : 1.0) +
+               (p.ways == 1 ? 0.0 : Nb * (groups / p.run) * p.ways > 100 ? 4.0 : 1.5);
+    };
+    SlabPlan best = beats_wave({run, 1}) ? SlabPlan{run, 1} : SlabPlan{0, 1};
+    if (groups == 1 || hw >= 65536) return best;
+    int wide = run;
+    for (int k = run; k <= groups && k <= kSlabWayGroups; ++k)
+        if (fits(k) && k * cg * elt <= 32) wide = k;
+    if (wide > kSlabWayGroups) return best;
+    for (int w = 1; w < kSlabWays && Nb * (groups / wide) * w <= sm_count() && sets > lanes({wide, w}); w *= 2) {
+        const SlabPlan p{wide, 2 * w};
+        if (beats_wave(p) && (best.run == 0 ? vec == 4 || cg / vec > 16 || rounds(p) <= 16 : cost(p) < cost(best))) best = p;
     }
-    return SlabPlan{0, 1};
+    return best;
 }
 template <typename... Params, typename... Args>
 static cudaError_t launch_slab(void (*kern)(Params...), unsigned ctas, int ways, cudaStream_t st, Args... args) {

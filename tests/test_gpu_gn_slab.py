@@ -18,11 +18,12 @@ pytestmark = pytest.mark.gpu
     (40, 8, 8, 1024, 32, 256, "bf16", 0),       # several groups per CTA
     (70, 8, 8, 512, 32, 256, "bf16", 256),      # the seam between two tensors lies between two runs
     (64, 16, 16, 512, 32, 256, "bf16", 0),      # 17 MB
-    (2, 64, 64, 256, 32, 256, "bf16", 0),       # a cluster of eight CTAs per run of two groups
-    (1, 100, 50, 512, 32, 256, "bf16", 256),    # ... 625 sets over its threads; two tensors
+    (2, 64, 64, 256, 32, 256, "bf16", 0),       # a cluster of four CTAs per run of two groups
+    (1, 100, 50, 512, 32, 256, "bf16", 256),    # ... of eight, 625 sets over its threads: none left for the last three; two tensors
     (1, 36, 44, 256, 2, 256, "f32", 0),         # ... groups of 128 channels, 196 sets and 16 pixels behind them
-    (3, 48, 48, 256, 32, 128, "bf16", 128),     # a cluster of four CTAs per run of two groups, no set left for the last; two tensors
-    (5, 48, 48, 768, 32, 256, "bf16", 0),       # clusters of one, two or four, by what is left of the SMs
+    (3, 48, 48, 256, 32, 128, "bf16", 128),     # ... of two per run of two groups; two tensors
+    (5, 48, 48, 768, 32, 256, "bf16", 0),       # more runs than SMs: one CTA each, four rounds of sets over 85 threads
+    (2, 64, 64, 768, 32, 256, "f32", 0),        # ... of two, where four would share the sets unevenly
     (3, 4, 5, 768, 32, 256, "bf16", 0),         # 20 rows a sample: four to a CTA of the transform, and not eight
     (2, 6, 4, 1536, 32, 256, "f32", 0),         # 24: four and not two
 ])
@@ -58,6 +59,8 @@ def test_gn_statistics_of_a_run_of_groups(oracle, Nb, H, W, C, G, n, dt, c1):
 @pytest.mark.parametrize("Nb,H,W,C,G,slab", [
     (2, 32, 32, 512, 32, True),         # 32 pixel rows on 64 CTAs
     (1, 64, 64, 2048, 32, True),        # long runs, but the one-wave kernel's sums meet at 32 addresses
+    (4, 40, 40, 2048, 32, True),        # 26 MB, shared evenly by single CTAs and unevenly by clusters of two
+    (2, 64, 64, 1536, 32, True),        # 25 MB: clusters of two, unevenly shared by four
     (1, 256, 256, 128, 32, False),      # 16 CTAs of 65536 pixels each
     (1, 64, 64, 256, 1, False),         # one group: one CTA for the whole image
     (1, 160, 256, 512, 32, False),      # 42 MB on 32 CTAs
