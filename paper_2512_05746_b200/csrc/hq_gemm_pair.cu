@@ -976,15 +976,27 @@ bool pair_stream_stages(PairStreamParams& p, size_t& smem, int kps) {
 
 }  // namespace
 
+// K_pad = 512, where the one-CTA kernel keeps the weights of a column tile in shared memory and walks rows under them.  One limb there:
+// with a residual, which that kernel leaves to a launch of its own, the streamed pair adds it as it stores, but waits for memory at every 16
+// columns with four K blocks of work to hide it: taken within one round of tiles over the pairs (whole layer, apart / added here: 4096 x 512 ->
+// 512 11.0 / 8.7 us, 18944 -> 256 18.6 / 18.0; beyond it 4736 -> 1024 13.4 / 15.0, 16384 -> 512 21.6 / 23.6, 65536 -> 512 62.6 / 73.8).
+// Without one beyond 1024 tiles of 256 x 256: 68196 x 512 -> 1536 68.9 / 62.3, 263780 -> 136 41.0 / 35.4, 131940 -> 512
+// 43.6 / 42.1 (up to there level: 32768 -> 2048 42.8 / 42.7).  Not on one or four column tiles that are three
+// quarters full and whole cache lines (537700 -> 256 91.3 / 104.2, 192256 -> 1024 3.7 % slower, -> 896 5.5 %; two such tiles 3 % faster to 6 %
+// slower, ragged ones 6 to 16 % faster), nor on more than eight (16740 -> 4096 39.0 / 43.6, 17920 -> 3584 9 % slower, level at 3000 tiles).
+static bool pair_stream_pays_resident(const hq_weight_desc* desc, int64_t M, bool residual) {
+    const int64_t tiles_n = (desc->N + kBN - 1) / kBN, tiles = (M + 255) / 256 * tiles_n;
+    if (desc->limbs != 1) return false;
+    if (residual) return tiles <= sm_count() / 2;
+    if ((tiles_n == 1 || tiles_n == 4) && desc->N % 64 == 0 && desc->N >= 192 * tiles_n) return false;
+    return tiles > 1024 && tiles_n <= 8;
+}
+
 // Whether the streamed pair kernel covers a plain GEMM / a convolution planned by the one-CTA path (`g`: that plan).
 bool pair_stream_covers_gemm(hq_container cont, const hq_weight_desc* desc, int64_t M, const void* y, hq_dtype ydt, int64_t ldy,
                              const int32_t* acc_out, bool combine_fast, bool residual) {
     if (desc->C_pad < int64_t(kResidentKb) * kBK) return false;
-    // One limb at K_pad = 512, where the one-CTA kernel keeps the weights: the streamed pair is as fast on 1000 tiles of 256 x 256 and faster
-    // beyond (32768 x 512 -> 1536 33.7 / 34.5 us, -> 2048 42.8 / 42.7, 65536 x 512 -> 512 24.8 / 24.5, -> 1536 65.8 / 60.0), and it adds a
-    // residual as it stores, which the other leaves to a launch of its own (65536 x 512 -> 512 another 24 us).
-    if (desc->C_pad == int64_t(kResidentKb) * kBK &&
-        (desc->limbs != 1 || !(residual || (M + 255) / 256 * ((desc->N + kBN - 1) / kBN) > 1024))) return false;
+    if (desc->C_pad == int64_t(kResidentKb) * kBK && !pair_stream_pays_resident(desc, M, residual)) return false;
     return cont == HQ_CODES_INT8 && desc->RS == 1 && y != nullptr &&
            acc_out == nullptr && ydt == HQ_BF16 && aligned16(y) && (ldy * 2) % 16 == 0 && combine_fast && M >= 256;
 }

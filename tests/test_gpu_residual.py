@@ -19,6 +19,9 @@ from paper_2512_05746_b200 import inputs
     (5000, 1024, 776, 256, False),      # ... two limbs
     (4096, 512, 512, 256, True),        # ... four K blocks, which a layer without a residual runs on one CTA
     (1001, 512, 200, 256, True),
+    (9500, 512, 512, 256, True),        # ... beyond one round of tiles: a launch of its own, behind the one-CTA kernel that keeps the weights
+    (20000, 256, 264, 256, True),       # two K blocks: likewise
+    (5000, 512, 776, 512, False),       # two limbs, weights kept by pairs of SMs: likewise
     (8200, 2048, 520, 2048, True),      # halved weights: likewise
 ])
 def test_linear_with_a_residual_is_the_linear_and_an_addition(M, K, N, n, room):
