@@ -143,12 +143,17 @@ __device__ __forceinline__ void store_staged(const uint4 (&w)[4], uint4* stage, 
 // memory, 3 GroupNorm alone (the normalisation in front of an attention block's QKV projection), 4 LayerNorm that reads the affine
 // vectors where it uses them (ln_table says which of the two a launch takes).
 // Blocks per SM the registers are bounded for: three for LayerNorm on 32 values (64 registers; unbounded 26 us on 8192 x 1152,
-// two 18.4, three 15.8, four 18.2); none stated for the GroupNorm prologues (56 registers; stating one lets the compiler take
+// two 18.4, three 15.8, four 18.2); none stated for the GroupNorm prologues (58 to 64 registers; stating one lets the compiler take
 // 84, 2.1 ms instead of 1.8 for the 44 launches of a UNet forward at batch 64); one for the plain transform (level at 256 and
 // 512 channels, 60.9 -> 54.7 us on 65536 x 1152).
-__host__ __device__ constexpr int quant_min_blocks(int pro, int e) { return (pro == 2 || pro == 4) && e == 32 ? 3 : (pro == 0 ? 1 : 0); }
+// LayerNorm on 64 values that reads its affine vectors: two (at most 96 registers), which it kept by itself until a few more put it at 98 to 108
+// and cost resident CTAs: bf16 8192 x 3072 in blocks of 1024 36.5 us then, 38.9 at 98 registers, 36.0 bounded, 8192 x 4096 in blocks of 2048 47.9
+// / 50.5 / 45.8; blocks of 4096 fp32 245 / 247 / 238.  fp32 in narrower blocks is left free, bounded it is slower (8192 x 3072 40.0 / 41.9 / 44.6).
+__host__ __device__ constexpr int quant_min_blocks(int pro, int e, int klog, bool bf16) {
+    return pro == 4 && e == 64 && (bf16 || klog == 12) ? 2 : (pro == 2 || pro == 4) && e == 32 ? 3 : (pro == 0 ? 1 : 0);
+}
 template <int KLOG, int E, typename InT, bool INT8_OUT, bool STATIC, int PRO>
-__global__ void __launch_bounds__(320, quant_min_blocks(PRO, E)) fwht_quant_fast(const QuantParams p) {
+__global__ void __launch_bounds__(320, quant_min_blocks(PRO, E, KLOG, sizeof(InT) == 2)) fwht_quant_fast(const QuantParams p) {
     constexpr bool GN = PRO == 1 || PRO == 3;          // 3: GroupNorm without the SiLU
     constexpr bool GN_SILU = PRO == 1;
     constexpr bool LN = PRO == 2 || PRO == 4;
