@@ -1119,8 +1119,15 @@ static hq_status launch_quant_impl(const void* x, hq_dtype xdt, int64_t rows, in
         // With GroupNorm every CTA builds the table of its sample's channels, an eighth to a quarter of its work on wide pixels: twice the
         // rows there, where a sample's rows divide.  Statistics + transform, so many / twice: 64 x 16 x 16 x 1536 46.9 / 41.9 us, 64 x 8 x 8 x
         // 2048 19.1 / 17.3, 64 x 16 x 16 x 768 23.6 / 22.8, 64 x 32 x 32 x 1024 95.5 / 94.8; narrower ones lose resident CTAs (64 x 64 x 64 x
-        // 256 87.2 / 91.0, 64 x 32 x 32 x 512 44.8 / 46.4).
-        if (gn != nullptr && cols >= 768 && 2 * rpc * tr <= 256 && gn->rows_per_sample % (2 * rpc) == 0) rpc *= 2;
+        // 256 87.2 / 91.0, 64 x 32 x 32 x 512 44.8 / 46.4).  Four warps and more are doubled while 64 CTAs are left: below, fewer SMs work for
+        // longer (2 x 16 x 16 x 1024 in blocks of 1024 7.1 / 8.0, 1 x 8 x 8 x 2048 in blocks of 256 6.7 / 6.9, 1 x 16 x 16 x 4096 in blocks of
+        // 4096 11.9 / 10.8 with 64); three warps at any size (1 x 8 x 8 x 3072 9.6 / 8.8).  64 values a thread that wait for a row maximum up to two
+        // CTAs per SM, all that their registers admit (64 x 16 x 16 x 1024 33.3 / 34.4, 64 x 8 x 8 x 2048 20.6 / 22.2), from 3072 channels on beyond it too.
+        if (gn != nullptr && cols >= 768 && 2 * rpc * tr <= 256 && gn->rows_per_sample % (2 * rpc) == 0) {
+            const int64_t ctas = rows / (2 * rpc);
+            const bool few = rpc * tr >= 128 && ctas < 64, waits = mode == HQ_SCALE_PER_ROW && E == 64 && cols <= 2048 && ctas > 2 * int64_t(sm_count());
+            if (!few && !waits) rpc *= 2;
+        }
         p.threads_per_row = tr;
         p.row_magic = uint32_t(((1 << 20) + tr - 1) / tr);
         p.rows_per_cta = rpc;
