@@ -21,6 +21,9 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) { f32x2 r; asm("mul.rn.f
 
 // Two pairs to 16 bytes of shared memory, as four 32-bit operands: stored as a vector of two 64-bit values, every value was moved to
 // another register first (0.8 instructions per value; 32768 x 2048 bf16, two codes per byte, 43.3 -> 41.2 us).
+// The kernels that transform inside the product, as vectors / so, in a graph: hq_small.cu fp32 256 x 256 -> 256 block 256 3.46 / 3.42, 70 x 512 ->
+// 1024 block 512 5.31 / 5.15, 128 x 1024 -> 1024 block 128 6.21 / 6.04, 200 x 768 -> 640 block 256 4.69 / 4.67, bf16 70 x 512 -> 1024 block 512 5.11 /
+// 5.02; hq_fused.cu 8192 x 512 -> 512 fp32 block 512 30.2 / 29.5, block 128 29.0 / 28.0, bf16 block 512 29.3 / 28.4.
 __device__ __forceinline__ void st_shared_pairs(ulonglong2* to, f32x2 a, f32x2 b) {
     float x0, x1, x2, x3;
     upk2(a, x0, x1);
@@ -78,7 +81,9 @@ __host__ __device__ constexpr int ilog2_c(int v) { return v <= 1 ? 0 : 1 + ilog2
 // the scaled magic number off again (exact) and adding the other value (exact: the sum stays below 2^22 units) leaves
 // both biased codes side by side in the low bits of one float, on the floating-point pipe; byte permutes then gather
 // the fields of a word, and one XOR turns the biased fields into two's complement.  Bytes: the two values come from
-// neighbouring pairs, so that the additions are two-wide as well.
+// neighbouring pairs, so that the additions are two-wide as well (hq_small.cu, pairs of one value each / so: bf16 200 x 768 -> 640 block 128 4.84 /
+// 4.70, 256 x 256 -> 256 fp32 block 256 3.52 / 3.45; the exceptions are fp32 200 x 768 -> 640 block 256 4.49 / 4.68, 128 x 1024 -> 1024 block 128
+// 5.86 / 6.07).
 template <int E, bool INT8_OUT, bool CLAMP>
 __device__ __forceinline__ void round_pack(const f32x2 (&v)[E / 2], float inv, int bits, uint32_t (&out)[INT8_OUT ? E / 4 : E / 8]) {
     constexpr float F = INT8_OUT ? 256.0f : 16.0f;

@@ -556,6 +556,8 @@ __device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const void* tma
 // drained, scaled and added up in registers; 128 output channels a tile.  There a K block of two limbs is 48 KB for 536 cycles of MMAs, more
 // than an SM gets from L2, here 32.  Whole layer, one CTA / pairs: 8 x 32 x 32 x
 // 256 18.8 / 16.7 us, 64 x 16 x 16 x 768 (one limb) 127.6 / 97.1, 64 x 32 x 32 x 512 (one limb) 224.7 / 178.4, 2 x 32 x 32 x 256 16.7 / 14.9.
+// Products alone, 62 layers of two to 512 tiles of 128 pixels with either number of limbs: 0.72 to 0.92 of the one-CTA time, odd numbers of tiles and
+// tiles that overhang the image among them (3 x 8 x 16 x 256 13.6 / 11.5, 3 x 12 x 16 x 512 18.3 / 16.3, 1 x 6 x 160 x 256 13.8 / 11.6).
 template <int LIMBS, bool CONV, int KPS, int BN, bool HALVED, bool PERTAP = false>
 __global__ void __launch_bounds__(kPairThreads, 1)
 qgemm_pair_stream_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,

@@ -9,7 +9,7 @@
 // (rows 16 bytes apart from a multiple of 128: conflict-free), both limbs in accumulators of their own.
 // Launched as a programmatic dependent, and letting the next kernel in at its start: nothing is read before the wait, weights
 // included, since the kernel in front may be the one that writes them.
-// Two kernels / one, in a graph: 256 x 256 -> 256 5.4 / 3.2 us (a call 6.3 / 4.2), 70 x 512 -> 1024 6.5 / 5.3, 200 x 768 -> 640 6.4 / 4.6,
+// Two kernels / one, in a graph: 256 x 256 -> 256 5.4 / 3.2 us (a call 6.3 / 4.2), 70 x 512 -> 1024 6.5 / 5.3, 200 x 768 -> 640 6.4 / 4.7,
 // 2 x 1024 -> 1024 5.9 / 5.1, 128 x 1024 -> 1024 7.3 / 5.9, 2000 x 128 -> 64 5.1 / 3.6.  With a division per 16 bytes copied instead of
 // one per thread 4.2, 6.4, 5.7, 6.2, 6.9 and 4.6; with one bulk copy a channel and limb, 55 cycles each from the warp that
 // issues them, 6.3, 7.4, 7.1, 7.2, 7.8 and 6.8.

@@ -15,13 +15,14 @@ from paper_2512_05746_b200 import inputs
     (200, 1024, 512, 256, False),       # two rows of tiles
     (4096, 1024, 1024, 256, True),      # pairs of SMs, one limb
     (1001, 2304, 1160, 256, True),      # ... rows of the last tile missing, a column tile cut off inside a 32-column store
-    (16385, 768, 200, 256, True),       # ... narrower column tiles
+    (16385, 768, 200, 256, True),       # ... one column tile, cut off inside a store
+    (16001, 640, 1288, 128, True),      # ... tiles of 192 columns, six a pair
     (5000, 1024, 776, 256, False),      # ... two limbs
     (4096, 512, 512, 256, True),        # ... four K blocks, which a layer without a residual runs on one CTA
     (1001, 512, 200, 256, True),
     (9500, 512, 512, 256, True),        # ... beyond one round of tiles: a launch of its own, behind the one-CTA kernel that keeps the weights
     (20000, 256, 264, 256, True),       # two K blocks: likewise
-    (5000, 512, 776, 512, False),       # two limbs, weights kept by pairs of SMs: likewise
+    (6000, 512, 776, 512, False),       # two limbs, weights kept by pairs of SMs (168 tiles): likewise
     (8200, 2048, 520, 2048, True),      # halved weights: likewise
 ])
 def test_linear_with_a_residual_is_the_linear_and_an_addition(M, K, N, n, room):

@@ -40,7 +40,11 @@ def test_convolution_on_narrow_tiles(Nb, H, C, Cout):
                                                 dev_status=st), (Nb, H, H, Cout))
 
 
-@pytest.mark.parametrize("M,K,N", [(16001, 640, 1288), (32768, 640, 960), (9000, 1152, 3456)])
+@pytest.mark.parametrize("M,K,N", [
+    (16001, 640, 1288),       # 192 wide, six tiles a pair, five K blocks
+    (16001, 1152, 1288),      # ... nine
+    (50000, 640, 136),        # one column tile cut off inside a store, two to three tiles a pair
+])
 def test_narrow_tiles_one_after_the_other_keep_their_staging_apart(M, K, N):
     # three stores a tile and two staging buffers: the turn passes from tile to tile, and every pass gives the same bytes
     import torch
@@ -68,6 +72,12 @@ def test_narrow_tiles_one_after_the_other_keep_their_staging_apart(M, K, N):
     (5, 32, 32, 384, 264, 1, "folded"),      # ... three K blocks a tap, an odd number of row tiles, a column tile cut off
     (7, 16, 16, 256, 136, 2, "plain"),       # one limb, stride 2, two images a tile and one missing
     (40, 16, 16, 512, 520, 1, "plain"),      # ... several tiles a pair
+    (3, 12, 16, 256, 136, 1, "folded"),      # tiles of 8 rows: four of the second tile lie below the image
+    (3, 12, 16, 256, 264, 1, "plain"),
+    (1, 6, 160, 256, 136, 1, "folded"),      # tiles of 128 pixels of a row: 96 of the second lie past it
+    (1, 6, 160, 384, 264, 1, "plain"),
+    (2, 24, 32, 256, 136, 2, "folded"),      # 12 x 16 outputs at stride 2
+    (2, 6, 320, 256, 264, 2, "plain"),       # 3 x 160
 ])
 @pytest.mark.parametrize("f32", [False, True])
 def test_per_pixel_scales_on_pairs(Nb, H, W, C, Cout, stride, mode, f32):
@@ -80,7 +90,9 @@ def test_per_pixel_scales_on_pairs(Nb, H, W, C, Cout, stride, mode, f32):
     b = torch.from_numpy(inputs.bias(Cout, seed=1)).cuda()
     out = []
     for pair in (0, 2):
-        y = torch.full((Nb, H // stride, W // stride, Cout), 7.0, dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+        n = Nb * (H // stride) * (W // stride) * Cout
+        guard = torch.full((n + 1024,), 7.0, dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+        y = guard[512: 512 + n].view(Nb, H // stride, W // stride, Cout)
         status = torch.zeros((1,), dtype=torch.int32, device="cuda")
         before = hq.hq_set_pair_gemm(pair)
         try:
@@ -88,5 +100,6 @@ def test_per_pixel_scales_on_pairs(Nb, H, W, C, Cout, stride, mode, f32):
         finally:
             hq.hq_set_pair_gemm(before)
         assert int(status) == 0
+        assert bool((guard[:512] == 7).all()) and bool((guard[512 + n:] == 7).all())
         out.append(y)
     assert torch.equal(out[0], out[1])
